@@ -89,7 +89,7 @@ __device__ __forceinline__ void brow(const int* __restrict__ col, const MT* __re
     }
     for (; w < width; ++w) {
         const int c = col[base + w * C + r];
-        if (c < 0) break;
+        if (c < 0) continue;
         const VT a = Cv<VT>::f(val[base + w * C + r]);
         const XT* xr = x + (size_t)c * Kp + lane;
 #pragma unroll

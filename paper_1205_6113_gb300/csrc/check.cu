@@ -52,13 +52,15 @@ __global__ void k_chk_slots(int nslots, int C, int nrows, const int* perm, const
     }
 }
 
-// Chunk pointers ascending within [0, nelem] with widths a multiple of C; columns in [-1, ncols).
-__global__ void k_chk_entries(int nchunks, int C, int64_t nelem, int ncols, const int* cptr, const int* col,
+// Chunk pointers ascending within [0, nelem] with widths a multiple of C, each chunk's part boundary
+// (if it has one) inside it; columns in [-1, ncols).
+__global__ void k_chk_entries(int nchunks, int C, int64_t nelem, int ncols, const int* cptr, const int* cmid, const int* col,
                               unsigned long long* cnt) {
     const int64_t t0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, st = (int64_t)gridDim.x * blockDim.x;
     for (int64_t k = t0; k < nchunks; k += st) {
         const int a = cptr[k], b = cptr[k + 1];
         if (a < 0 || a > b || b > nelem || (b - a) % C != 0) atomicAdd(&cnt[C_RANGE], 1ull);
+        else if (cmid && (cmid[k] < a || cmid[k] > b || (cmid[k] - a) % C != 0)) atomicAdd(&cnt[C_RANGE], 1ull);
     }
     if (col)
         for (int64_t e = t0; e < nelem; e += st) {
@@ -123,7 +125,7 @@ struct Checker {
         k_chk_slots<<<cblk(S.nslots), CTPB, 0, s>>>(S.nslots, S.C, nrows, S.perm.p, dseg.get(), ng, seen.get(), grp, cnt.p);
         if (S.cptr.p)
             k_chk_entries<<<cblk(std::max<int64_t>(S.nchunks, S.nelem)), CTPB, 0, s>>>(S.nchunks, S.C, S.nelem, ncols,
-                                                                                     S.cptr.p, S.col.p, cnt.p);
+                                                                                     S.cptr.p, S.cmid.p, S.col.p, cnt.p);
         k_chk_seen<<<cblk(nrows), CTPB, 0, s>>>(nrows, seen.get(), exact ? 1 : 0, cnt.p);
         for (int d = 0; d < S.ndiag; ++d)
             if (S.doff.o[d] <= -nrows || S.doff.o[d] >= nrows) bump(C_RANGE);

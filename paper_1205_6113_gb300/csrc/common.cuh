@@ -142,7 +142,8 @@ struct DiaOff {
 //   warp with G = 32/C lanes per row; entry w of the row in slot Ck + r lives at
 //   val/col[cptr[k] + w*C + r], so that every warp-wide load covers 32 consecutive elements.
 //   With split_diag the diagonal is kept apart in diag[s] and val/col hold off-diagonals only.
-//   Padding entries have val 0 and col = -1; kernels skip them (no load is issued).
+//   Padding entries have val 0 and col = -1; kernels skip them (no load is issued).  In the
+//   smoother copy they end each of a chunk's two parts (cmid below), elsewhere each row.
 //   seg[] (host) gives chunk ranges: segment g is chunks [seg[g], seg[g+1]) -- a colour of a
 //   Gauss-Seidel sweep or a level of a triangular solve.
 struct Sell {
@@ -150,7 +151,11 @@ struct Sell {
     int nslots = 0, nchunks = 0;
     int64_t nelem = 0;
     int lanes = 0;                     // most entries one lane holds: ceil(widest chunk / 32)
-    DBuf<int> perm, cptr, col;
+    // Smoother copy (colour-grouped A_l): the entries of a chunk come in two parts, each padded to its
+    // widest row: columns of an earlier group than the row's in [cptr[k], cmid[k]), columns of a later
+    // group in [cmid[k], cptr[k+1]).  lanes_lo / lanes_up: most entries one lane holds of each part.
+    int lanes_lo = 0, lanes_up = 0;
+    DBuf<int> perm, cptr, cmid, col;
     DBuf<double> val, diag, dinv;      // FP64 copy (always); dinv = 1 / diag (split diagonal only)
     DBuf<float> val32, diag32, dinv32; // FP32 copy (mixed precision)
     DBuf<__nv_bfloat16> val16;         // BF16 copy of off-diagonals (coarse levels, mode 2)

@@ -3,6 +3,7 @@
 #pragma once
 
 #include <type_traits>
+#include <utility>
 
 #include "common.cuh"
 
@@ -49,6 +50,21 @@ inline SV<MT, DT> view(const Sell& S, const MT* val, const DT* diag) {
 // setup.  With read-only loads a kernel was seen to read values of the previous V-cycle.
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+// Launch with programmatic stream serialisation (see pdl_wait above).
+template <class... KArgs, class... Args>
+inline void launch(void (*k)(KArgs...), int grid, int block, cudaStream_t s, Args&&... args) {
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)grid, 1, 1);
+    cfg.blockDim = dim3((unsigned)block, 1, 1);
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    CPC_CK(cudaLaunchKernelEx(&cfg, k, std::forward<Args>(args)...));
+}
 
 // One batch of exactly M entries per lane (entries o, o + 32, ... with oo < e; the others load
 // nothing and add 0): loads, then (WAIT) the wait and the caller's hook, then the gathers, then the

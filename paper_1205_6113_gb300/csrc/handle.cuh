@@ -9,6 +9,7 @@ constexpr int CHUNK = 32;            // SELL chunk height = warp width
 constexpr int DENSE_MAX = 4096;      // largest coarsest level solved by the dense inverse
 constexpr int HIST_CAP = 100001;     // residual-history capacity on the device
 constexpr int NPART = 1024;          // partial-sum slots for deterministic reductions
+constexpr unsigned FLOW_RING = 256;  // counter slots of the flow launches
 constexpr int NPRECOND = 6;          // CPC_PRECOND_* values
 
 // One AMG level (0 = finest).
@@ -26,6 +27,10 @@ struct Level {
     DBuf<float> dnat32;
     DBuf<double> x64, f64, r64;
     DBuf<float> x32, f32, r32;
+    DBuf<double> xa64;      // forward sweep's result (the backward sweep's goes to x), flow sweeps only
+    DBuf<float> xa32;
+    bool flow = false;      // sweeps as one flow launch each (flow.cuh); else a launch per colour
+    bool red_black = false; // two colours in diagonal form (the structured fine level)
 };
 
 // Batched PCG state: block vectors [n][Kp] (Kp = K rounded up to 32), level vectors in the
@@ -50,7 +55,7 @@ struct Batched {
 // Device-side scalars of one PCG run (all reductions finish in fixed order).
 struct PcgState {
     double bnorm, rz, rz_old, pq, alpha, beta, rr, tol, res;
-    int k, maxit, status, pad;
+    int k, maxit, status, gave_up;   // gave_up: a flow launch's wait ran out
 };
 
 struct Handle {
@@ -73,6 +78,9 @@ struct Handle {
     DBuf<double> ic_uinv64;
     DBuf<float> ic_uinv32;
     Sell L, U;              // strictly-lower rows by forward level; upper rows by backward level
+    // Triangular solves as one flow launch each; y is unset between them.  Two levels (red-black) keep
+    // a launch per level.
+    bool ic_flow() const { return ic_levels_L > 2 || ic_levels_U > 2; }
     // coarsest level: dense inverse
     int nc = 0;
     DBuf<double> Ainv;
@@ -87,6 +95,11 @@ struct Handle {
     // reductions and PCG state
     DBuf<double> partial;
     DBuf<unsigned> counter;
+    // Chunk counters of the flow launches: a ring, a slot per recorded launch, so that a launch whose
+    // prologue starts early never draws on the counter of one still running.
+    DBuf<unsigned> flow_ctr;
+    unsigned flow_seq = 0;
+    unsigned* next_flow_ctr() { return flow_ctr.p + flow_seq++ % FLOW_RING; }
     DBuf<PcgState> state;
     DBuf<double> hist;
     DBuf<int> flags;        // [0] IC factor failure row + 1, [1] coarse Cholesky failure
@@ -141,15 +154,21 @@ void record_tail(Handle& h, int level, const void* f0, void* x0, cudaStream_t s)
 // solve.cu
 void record_precond(Handle& h, int which, const double* r, void* z, cudaStream_t s);
 void apply_precond(Handle& h, int which, const double* r, double* z);
+// Whether the sweeps of a level of n rows in g groups run as flow launches.  Wide colours fill the GPU
+// for longer than a launch takes to start, and their launches keep more warps resident than a flow's
+// waiting ones: 32,000 rows a colour (level 1 at 1M) take 49 us by launches and 50 by flow in FP64, 26
+// and 32 in FP32; 12,000 rows a colour 16.2 and 14.7 (FP32, 395,000 cells), 4,500 rows a colour 61 and 28.
+constexpr int FLOW_ROWS = 24000;
+inline bool gs_by_flow(int n, int g) { return n / g <= FLOW_ROWS; }
+// Warps resident at once at the colour steps' occupancy (8 blocks of 4 warps on each of 152 SMs).
+constexpr int GS_RESIDENT_WARPS = 152 * 32;
+// Marks the n elements of p unset (flow.cuh).
+template <class VT> void fill_unset(VT* p, int64_t n, cudaStream_t s);
 void spmv_fine(Handle& h, const double* x, double* y, cudaStream_t s);
 void solve_pcg(Handle& h, const double* b, double* x, double tol, int maxit, int* iters,
                double* res_hist, int hist_cap, int* status);
 void level_apply(Handle& h, int l, int op, const double* x, double* y);
 double sweep_time_us(Handle& h, int l, int reps);
-// Warps (SELL chunks) per block of the colour-step kernel, and how many of its blocks the GPU
-// holds at once (all SMs) for an operator whose lanes hold at most `lanes` entries (FP64).
-constexpr int GS_WARPS_PER_BLOCK = 4;
-int gs_resident_blocks(int lanes);
 void destroy_graphs(Handle& h);
 void ensure_solve_graph(Handle& h, int which);
 

@@ -1517,20 +1517,46 @@ __device__ __forceinline__ bool sell_keep(int mode, int j, int i) {
     }
 }
 
+// Entries of each chunk (padded to its widest row).  With a group key per row (smoother copy) the two
+// parts are padded apart: low[k] = entries of the part of earlier groups.  wmax[0..2]: the largest
+// chunk, low part and high part.  Columns of key 0 make the first part when by_col (the rows have no
+// key then: a transfer, its columns keyed by the fine colour).
 __global__ void k_sell_width(const int* perm, int nchunks, int C, const int* ptr, const int* col, int mode,
-                             int* width) {
+                             const int* key, bool by_col, int* width, int* low, int* wmax) {
     int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k > nchunks) return;
-    if (k == nchunks) { width[k] = 0; return; }
-    int w = 0;
-    for (int l = 0; l < C; ++l) {
-        const int i = perm[k * C + l];
-        if (i < 0) continue;
-        int c = 0;
-        for (int p = ptr[i]; p < ptr[i + 1]; ++p) c += sell_keep(mode, col[p], i) ? 1 : 0;
-        w = max(w, c);
+    int w = 0, wl = 0;
+    if (k < nchunks) {
+        for (int l = 0; l < C; ++l) {
+            const int i = perm[k * C + l];
+            if (i < 0) continue;
+            const int ki = !key ? 0 : by_col ? 1 : key[i];
+            int c = 0, cl = 0;
+            for (int p = ptr[i]; p < ptr[i + 1]; ++p)
+                if (sell_keep(mode, col[p], i)) {
+                    if (key && key[col[p]] < ki) ++cl;
+                    else ++c;
+                }
+            w = max(w, c);
+            wl = max(wl, cl);
+        }
+        width[k] = (w + wl) * C;
+        if (low) low[k] = wl * C;
+    } else if (k == nchunks) {
+        width[k] = 0;
     }
-    width[k] = w * C;
+    const int mt = __reduce_max_sync(0xffffffffu, (w + wl) * C), ml = __reduce_max_sync(0xffffffffu, wl * C),
+              mu = __reduce_max_sync(0xffffffffu, w * C);
+    if ((threadIdx.x & 31) == 0) {
+        atomicMax(wmax, mt);
+        atomicMax(wmax + 1, ml);
+        atomicMax(wmax + 2, mu);
+    }
+}
+
+// cmid[k] = cptr[k] + low[k].
+__global__ void k_sell_mid(int nchunks, const int* cptr, const int* low, int* cmid) {
+    int k = blockIdx.x * blockDim.x + threadIdx.x;
+    if (k < nchunks) cmid[k] = cptr[k] + low[k];
 }
 
 template <class T>
@@ -1543,30 +1569,36 @@ __global__ void k_slot_to_nat(int nslots, const int* perm, const T* v, T* out) {
 // Slots refer to rows of the CSR; imap (optional) renames rows and columns on output
 // (IC factor stored in its own ordering but applied to naturally ordered vectors).
 __global__ void k_sell_fill(const int* perm, int nslots, int C, const int* ptr, const int* col, const double* val,
-                            int mode, const int* cptr, const int* imap, int* perm_out, int* scol, double* sval,
-                            double* sdiag) {
+                            int mode, const int* key, bool by_col, const int* cptr, const int* cmid, const int* imap,
+                            int* perm_out, int* scol, double* sval, double* sdiag) {
     int s = blockIdx.x * blockDim.x + threadIdx.x;
     if (s >= nslots) return;
     const int k = s / C, lane = s % C;
     const int base = cptr[k];
     const int w = (cptr[k + 1] - base) / C;
+    const int wl = key ? (cmid[k] - base) / C : 0;
     const int i = perm[s];
     const int out_row = i < 0 ? -1 : (imap ? imap[i] : i);
     perm_out[s] = out_row;
-    int e = 0;
+    int el = 0, e = wl;
     double d = 1.0;
     if (i >= 0) {
+        const int ki = !key ? 0 : by_col ? 1 : key[i];
         for (int p = ptr[i]; p < ptr[i + 1]; ++p) {
             const int j = col[p];
             if (j == i) d = val[p];
             if (sell_keep(mode, j, i)) {
-                scol[base + e * C + lane] = imap ? imap[j] : j;
-                sval[base + e * C + lane] = val[p];
-                ++e;
+                const int o = key && key[j] < ki ? el++ : e++;
+                scol[base + o * C + lane] = imap ? imap[j] : j;
+                sval[base + o * C + lane] = val[p];
             }
         }
     }
-    for (; e < w; ++e) {                       // padding: column -1, skipped by every kernel
+    for (; el < wl; ++el) {                    // padding: column -1, skipped by every kernel
+        scol[base + el * C + lane] = -1;
+        sval[base + el * C + lane] = 0.0;
+    }
+    for (; e < w; ++e) {
         scol[base + e * C + lane] = -1;
         sval[base + e * C + lane] = 0.0;
     }
@@ -1648,30 +1680,37 @@ int choose_chunk(double avg) {
 }
 
 // Fill a Sell of chunk height C from CSR rows in the slot order `slots` (device, nslots entries).
+// key (device, may be null): the rows' group (by_col: the columns' group); splits each chunk by it
+// (Sell::cmid).
 void build_sell(const int* ptr, const int* col, const double* val, const DBuf<int>& slots, int nslots,
                 const std::vector<int>& seg, int C, int mode, bool split_diag, const int* imap, Sell& S,
-                cudaStream_t s) {
+                cudaStream_t s, const int* key = nullptr, bool by_col = false) {
     S.nslots = nslots;
     S.C = C;
     S.nchunks = nslots / C;
     S.seg = seg;
-    Tmp<int> width(S.nchunks + 1, s);
-    k_sell_width<<<nblk(S.nchunks + 1), TPB, 0, s>>>(slots.p, S.nchunks, C, ptr, col, mode, width.get());
-    {
-        Tmp<int> wmax(1, s);
-        CPC_CK(cudaMemsetAsync(wmax.get(), 0, sizeof(int), s));
-        k_max_int<<<nblk(S.nchunks + 1), TPB, 0, s>>>(width.get(), S.nchunks + 1, wmax.get());
-        S.lanes = (d2h(wmax.get(), s) + 31) / 32;
-    }
+    Tmp<int> width(S.nchunks + 1, s), low(key ? S.nchunks : 0, s), wmax(3, s);
+    CPC_CK(cudaMemsetAsync(wmax.get(), 0, 3 * sizeof(int), s));
+    k_sell_width<<<nblk(S.nchunks + 1), TPB, 0, s>>>(slots.p, S.nchunks, C, ptr, col, mode, key, by_col, width.get(),
+                                                     key ? low.get() : nullptr, wmax.get());
     S.cptr.alloc(S.nchunks + 1);
     exclusive_scan(width.get(), S.cptr.p, S.nchunks + 1, s);
+    int wm[3];
+    CPC_CK(cudaMemcpyAsync(wm, wmax.get(), sizeof wm, cudaMemcpyDeviceToHost, s));
     S.nelem = d2h(S.cptr.p + S.nchunks, s);
+    S.lanes = (wm[0] + 31) / 32;
+    S.lanes_lo = (wm[1] + 31) / 32;
+    S.lanes_up = (wm[2] + 31) / 32;
+    if (key) {
+        S.cmid.alloc(S.nchunks);
+        k_sell_mid<<<nblk(S.nchunks), TPB, 0, s>>>(S.nchunks, S.cptr.p, low.get(), S.cmid.p);
+    }
     S.perm.alloc(nslots);
     S.col.alloc(S.nelem);
     S.val.alloc(S.nelem);
     if (split_diag) S.diag.alloc(nslots);
-    k_sell_fill<<<nblk(nslots), TPB, 0, s>>>(slots.p, nslots, C, ptr, col, val, mode, S.cptr.p, imap, S.perm.p,
-                                             S.col.p, S.val.p, split_diag ? S.diag.p : nullptr);
+    k_sell_fill<<<nblk(nslots), TPB, 0, s>>>(slots.p, nslots, C, ptr, col, val, mode, key, by_col, S.cptr.p, S.cmid.p, imap,
+                                             S.perm.p, S.col.p, S.val.p, split_diag ? S.diag.p : nullptr);
     if (split_diag) {       // reciprocal diagonal: the sweeps multiply instead of dividing
         S.dinv.alloc(nslots);
         k_recip<<<nblk(nslots), TPB, 0, s>>>(nslots, S.diag.p, S.dinv.p);
@@ -2539,7 +2578,7 @@ void setup_ic_rb(Handle& h, bool colour_ic, cudaStream_t s) {
 // (within 4..32) around the row-length rule, each is timed on a forward Gauss-Seidel sweep replayed
 // from a graph (time_gs_sweep), and a candidate replaces the rule's layout only when it is more
 // than 3% faster.  C sets the threads per row (32 / C) of every kernel on that copy.
-void setup_level_sells(Level& L, cudaStream_t s, bool last, bool tune) {
+void setup_level_sells(Level& L, cudaStream_t s, bool last, bool tune, bool fp64) {
     // colour-grouped A_l (Gauss-Seidel and residual)
     if (!last) {
         auto build_grouped = [&](int C, Sell& out) {
@@ -2547,21 +2586,23 @@ void setup_level_sells(Level& L, cudaStream_t s, bool last, bool tune) {
             int nslots = 0;
             std::vector<int> seg;
             grouped_slots(L.n, L.colour.p, L.ncolours, C, s, slots, nslots, seg);
-            build_sell(L.A.ptr.p, L.A.col.p, L.A.val.p, slots, nslots, seg, C, SELL_OFFDIAG, true, nullptr, out, s);
+            build_sell(L.A.ptr.p, L.A.col.p, L.A.val.p, slots, nslots, seg, C, SELL_OFFDIAG, true, nullptr, out, s,
+                       L.colour.p);
             CPC_CK(cudaStreamSynchronize(s));
         };
         const int ca = choose_chunk((double)(L.A.nnz - L.n) / std::max(1, L.n));
         build_grouped(ca, L.S);
-        if (!tune && ca < 32) {
-            // One wave: a colour step whose CTAs do not all fit on the GPU at once runs in two
-            // waves, and only the first wave's matrix loads overlap the previous step.  If the
-            // widest colour needs more CTAs than fit and twice the chunk height (half the lanes
-            // per row, about twice the entries per lane) would fit, take twice the chunk height.
+        if (!tune && fp64 && ca < 32) {
+            // FP64 issue bounds a wide colour step on this part, and adding the partial sums of a row's
+            // lanes costs as much of it as a few entries: twice the chunk height (half the lanes per row)
+            // where a colour takes many waves of warps (level 1 at 8.4M: 300 -> 264 us a sweep), or where
+            // that brings a colour of rows of up to 18 entries into one wave (level 1 at 1M: 55 -> 49 us).
             int widest = 0;
             for (size_t c = 0; c + 1 < L.S.seg.size(); ++c) widest = std::max(widest, L.S.seg[c + 1] - L.S.seg[c]);
-            const int blocks = (widest + GS_WARPS_PER_BLOCK - 1) / GS_WARPS_PER_BLOCK;
-            const int blocks2 = (widest / 2 + GS_WARPS_PER_BLOCK) / GS_WARPS_PER_BLOCK;
-            if (blocks > gs_resident_blocks(L.S.lanes) && blocks2 <= gs_resident_blocks(16)) build_grouped(2 * ca, L.S);
+            const double per_lane = (double)(L.A.nnz - L.n) / L.n * 2 * ca / 32;
+            if (widest > 4 * GS_RESIDENT_WARPS ||
+                (widest > GS_RESIDENT_WARPS && widest <= 2 * GS_RESIDENT_WARPS && per_lane <= 9.0))
+                build_grouped(2 * ca, L.S);
         }
         if (tune) {
             float best = time_gs_sweep(L.S, L.n);
@@ -2576,18 +2617,23 @@ void setup_level_sells(Level& L, cudaStream_t s, bool last, bool tune) {
                 }
             }
         }
+        // On a two-colour level the red rows of P come first and the red columns of R make the first part:
+        // the cycle reads no others there (rec_vcycle).
+        const bool rb = L.ncolours == 2;
         DBuf<int> ps;
         int pn = 0;
         std::vector<int> pseg;
         const int cp = choose_chunk((double)L.P.nnz / std::max(1, L.P.n));
-        natural_slots(L.P.n, cp, s, ps, pn, pseg);
+        if (rb) grouped_slots(L.n, L.colour.p, 2, cp, s, ps, pn, pseg);
+        else natural_slots(L.P.n, cp, s, ps, pn, pseg);
         build_sell(L.P.ptr.p, L.P.col.p, L.P.val.p, ps, pn, pseg, cp, SELL_ALL, false, nullptr, L.SP, s);
         DBuf<int> rs;
         int rn = 0;
         std::vector<int> rseg;
         const int cr = choose_chunk((double)L.R.nnz / std::max(1, L.R.n));
         natural_slots(L.R.n, cr, s, rs, rn, rseg);
-        build_sell(L.R.ptr.p, L.R.col.p, L.R.val.p, rs, rn, rseg, cr, SELL_ALL, false, nullptr, L.SR, s);
+        build_sell(L.R.ptr.p, L.R.col.p, L.R.val.p, rs, rn, rseg, cr, SELL_ALL, false, nullptr, L.SR, s,
+                   rb ? L.colour.p : nullptr, true);
         CPC_CK(cudaStreamSynchronize(s));
     }
 }
@@ -2860,7 +2906,8 @@ void setup_handle(Handle& h, const cpc_csr& in) {
     CPC_CK(cudaStreamWaitEvent(s3, ph[1], 0));
     {
         AllocOn layouts_alloc(s3);
-        for (int l = 0; l < nl; ++l) setup_level_sells(h.lev[l], s3, l == nl - 1, h.opt.autotune == 1 && l > 0);
+        for (int l = 0; l < nl; ++l) setup_level_sells(h.lev[l], s3, l == nl - 1, h.opt.autotune == 1 && l > 0,
+                                                          h.opt.precision == CPC_PREC_FP64);
         // fine A in natural order for the SpMVs
         DBuf<int> slots;
         int nslots = 0;
@@ -2972,10 +3019,16 @@ void setup_handle(Handle& h, const cpc_csr& in) {
                 k_slot_to_nat<<<nblk(L.S.nslots), TPB, 0, s>>>(L.S.nslots, L.S.perm.p, L.S.dinv32.p, L.dnat32.p);
             }
             CPC_LAUNCH_CK();
+            L.red_black = L.S.ndiag && L.ncolours == 2;
+            L.flow = !L.red_black && gs_by_flow(L.n, L.ncolours);
         }
         const size_t n = L.n;
         if (L.vt == VT_F64) { L.x64.alloc(n); L.f64.alloc(n); L.r64.alloc(n); }
         else { L.x32.alloc(n); L.f32.alloc(n); L.r32.alloc(n); }
+        if (L.flow) {
+            if (L.vt == VT_F64) L.xa64.alloc(n);
+            else L.xa32.alloc(n);
+        }
     }
     if (prec != CPC_PREC_FP64) {
         sell_lowp(h.Anat, VT_F32, s);
@@ -2997,6 +3050,12 @@ void setup_handle(Handle& h, const cpc_csr& in) {
     h.state.alloc(1);
     CPC_CK(cudaMemsetAsync(h.state.p, 0, sizeof(PcgState), s));
     h.hist.alloc(HIST_CAP);
+    h.flow_ctr.alloc(FLOW_RING);
+    CPC_CK(cudaMemsetAsync(h.flow_ctr.p, 0, sizeof(unsigned) * h.flow_ctr.n, s));
+    if (h.ic_flow()) {
+        fill_unset(h.y.p, n, s);
+        if (prec != CPC_PREC_FP64) fill_unset(h.y32.p, n, s);
+    }
     h.flags.alloc(8);
     CPC_CK(cudaMemsetAsync(h.flags.p, 0, sizeof(int) * 8, s));
     CPC_CK(cudaStreamSynchronize(s));

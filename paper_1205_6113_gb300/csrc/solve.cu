@@ -14,31 +14,16 @@
 #include <type_traits>
 #include <utility>
 
-#include "device.cuh"
+#include "flow.cuh"
 #include "handle.cuh"
 
 namespace cpc {
 
 namespace {
 
-constexpr int WPB = GS_WARPS_PER_BLOCK;  // warps (= SELL chunks) per block
+constexpr int WPB = 4;                   // warps (= SELL chunks) per block
 constexpr int SELL_TPB = WPB * 32;
 constexpr int VEC_TPB = 256;
-
-// Launch with programmatic stream serialisation (see pdl_wait in device.cuh).
-template <class... KArgs, class... Args>
-void launch(void (*k)(KArgs...), int grid, int block, cudaStream_t s, Args&&... args) {
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3((unsigned)grid, 1, 1);
-    cfg.blockDim = dim3((unsigned)block, 1, 1);
-    cfg.stream = s;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    CPC_CK(cudaLaunchKernelEx(&cfg, k, std::forward<Args>(args)...));
-}
 
 // Calls f(std::integral_constant<int, U>{}) with the sell_dot batch width for an operator whose
 // lanes hold at most `lanes` entries.
@@ -50,11 +35,13 @@ void with_u(int lanes, F&& f) {
 }
 
 // As with_u for the Gauss-Seidel colour steps, with batches of up to 16: a colour step lasts as long
-// as its widest chunk, and one batch per lane keeps it to one round of dependent gathers.  The
-// products are added in the same entry order whatever the batch, so the results do not change.
+// as its widest chunk, and one batch per lane keeps it to one round of dependent gathers (level 1 at
+// 1M: 49 us a sweep, 67 with batches of 8).  A step of several waves of warps is bound by what it
+// keeps in flight instead, and the smaller batch lets more warps in (level 1 at 8.4M: 304 and 264).
+// The products are added in the same entry order whatever the batch, so the results do not change.
 template <class F>
-void with_u_gs(int lanes, F&& f) {
-    if (lanes <= 8) with_u(lanes, f);
+void with_u_gs(int lanes, int chunks, F&& f) {
+    if (lanes <= 8 || chunks > 4 * GS_RESIDENT_WARPS) with_u(lanes, f);
     else if (lanes <= 12) f(std::integral_constant<int, 12>{});
     else f(std::integral_constant<int, 16>{});
 }
@@ -203,8 +190,9 @@ __global__ void __launch_bounds__(SELL_TPB) k_resid_dia(DV<MT, DT> A, int s0, in
 // r = f - A x after a forward sweep on a two-colour level in diagonal form: slots below s1 (the
 // first colour) get the full residual; the rows of the last colour were just solved from their
 // current neighbours, so their residual is zero up to rounding and is written as 0 without
-// loading their matrix entries.
-template <class MT, class DT, class FT, class XT, class RT, int ND>
+// loading their matrix entries.  ZERO: the sweep started from zero, so f_i - a_ii x_i = 0 holds on the
+// first colour and r_i = -sum_j a_ij x_j.
+template <class MT, class DT, class FT, class XT, class RT, int ND, bool ZERO>
 __global__ void __launch_bounds__(SELL_TPB) k_resid_dia_first(DV<MT, DT> A, int s1, const FT* f, const XT* x, RT* r) {
     const int s = blockIdx.x * blockDim.x + threadIdx.x;
     if (s >= A.nslots) return;
@@ -217,13 +205,16 @@ __global__ void __launch_bounds__(SELL_TPB) k_resid_dia_first(DV<MT, DT> A, int 
     }
     RT v[ND];
     dia_load<ND, RT>(A, s, v);
-    const RT dg = Cv<RT>::f(A.diag[s]);
+    const RT dg = ZERO ? RT(0) : Cv<RT>::f(A.diag[s]);
     pdl_wait();
     if (row < 0) return;
-    const RT fr = Cv<RT>::f(f[row]);
-    const RT dx = dg * Cv<RT>::f(x[row]);
+    RT fr = RT(0), dx = RT(0);
+    if (!ZERO) {
+        fr = Cv<RT>::f(f[row]);
+        dx = dg * Cv<RT>::f(x[row]);
+    }
     const RT dot = dia_dot<ND, RT>(v, A.off, row, A.n, x);
-    r[row] = fr - (dx + dot);
+    r[row] = ZERO ? -dot : fr - (dx + dot);
 }
 
 // y = A x, diagonal form.
@@ -246,8 +237,11 @@ __global__ void __launch_bounds__(SELL_TPB) k_spmv_dia(DV<MT, DT> A, const XT* x
 // Gauss-Seidel over the rows of one colour (chunks [c0, c1)): x_i = (f_i - sum_{j!=i} a_ij x_j) / a_ii,
 // with the view's diagonal field holding 1 / a_ii (a multiply instead of an FP64 division).
 // Rows of one colour are not coupled, so they update in parallel exactly as in sequential order.
-template <class MT, class DT, class FT, class VT, int U>
-__global__ void __launch_bounds__(SELL_TPB) k_gs(SV<MT, DT> A, int c0, int c1, const FT* f, VT* x) {
+// LOW: in a forward sweep from a zero guess the rows of later colours are still zero, so only the
+// entries of earlier colours (up to cmid) are read.
+template <class MT, class DT, class FT, class VT, int U, bool LOW>
+__global__ void __launch_bounds__(SELL_TPB) k_gs(SV<MT, DT> A, const int* __restrict__ cmid, int c0, int c1, const FT* f,
+                                                 VT* x) {
     const int k = c0 + blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     if (k >= c1) return;
     pdl_launch_dependents();
@@ -257,32 +251,48 @@ __global__ void __launch_bounds__(SELL_TPB) k_gs(SV<MT, DT> A, int c0, int c1, c
     const bool own = g == 0 && row >= 0;
     const VT dinv = own ? Cv<VT>::f(A.diag[s]) : VT(0);
     VT fr = VT(0);
-    VT dot = sell_dot<VT, true, U>(A.col, A.val, A.cptr[k] + g * C + r, A.cptr[k + 1], x,
+    VT dot = sell_dot<VT, true, U>(A.col, A.val, A.cptr[k] + g * C + r, LOW ? cmid[k] : A.cptr[k + 1], x,
                                    [&] { if (own) fr = Cv<VT>::f(f[row]); });
     dot = sub_sum(dot, C);
     if (own) x[row] = (fr - dot) * dinv;
 }
 
-// r = f - A x over all chunks (grid-stride over chunks).
+// r = f - A x over all chunks, one per warp.
 template <class MT, class DT, class FT, class XT, class RT, int U>
 __global__ void __launch_bounds__(SELL_TPB) k_resid(SV<MT, DT> A, int nchunks, const FT* f,
                                                      const XT* x, RT* __restrict__ r) {
+    const int k = blockIdx.x * WPB + (threadIdx.x >> 5);
+    if (k >= nchunks) return;
     pdl_launch_dependents();
-    pdl_wait();
     const int lane = threadIdx.x & 31, C = A.C, rr = lane & (C - 1), g = lane / C;
-    for (int k = blockIdx.x * WPB + (threadIdx.x >> 5); k < nchunks; k += gridDim.x * WPB) {
-        const int s = k * C + rr;
-        const int row = A.perm[s];
-        const bool own = g == 0 && row >= 0;
-        RT fr = RT(0), dx = RT(0);
+    const int s = k * C + rr;
+    const int row = A.perm[s];
+    const bool own = g == 0 && row >= 0;
+    const RT dg = own ? Cv<RT>::f(A.diag[s]) : RT(0);
+    RT fr = RT(0), dx = RT(0);
+    RT dot = sell_dot<RT, true, U>(A.col, A.val, A.cptr[k] + g * C + rr, A.cptr[k + 1], x, [&] {
         if (own) {
             fr = Cv<RT>::f(f[row]);
-            dx = Cv<RT>::f(A.diag[s]) * Cv<RT>::f(x[row]);
+            dx = dg * Cv<RT>::f(x[row]);
         }
-        RT dot = sell_dot<RT, false, U>(A.col, A.val, A.cptr[k] + g * C + rr, A.cptr[k + 1], x);
-        dot = sub_sum(dot, C);
-        if (own) r[row] = fr - (dx + dot);
-    }
+    });
+    dot = sub_sum(dot, C);
+    if (own) r[row] = fr - (dx + dot);
+}
+
+// r = f - A x right after a forward sweep from a zero guess: (D + L) x = f holds row by row, so
+// r_i = -sum_up a_ij x_j and only the entries of later colours are read.
+template <class MT, class VT, int U>
+__global__ void __launch_bounds__(SELL_TPB) k_resid_up(SV<MT, VT> A, const int* __restrict__ cmid, int nchunks,
+                                                       const VT* x, VT* __restrict__ r) {
+    const int k = blockIdx.x * WPB + (threadIdx.x >> 5);
+    if (k >= nchunks) return;
+    pdl_launch_dependents();
+    const int lane = threadIdx.x & 31, C = A.C, rr = lane & (C - 1), g = lane / C;
+    const int row = A.perm[k * C + rr];
+    VT dot = sell_dot<VT, true, U>(A.col, A.val, cmid[k] + g * C + rr, A.cptr[k + 1], x);
+    dot = sub_sum(dot, C);
+    if (g == 0 && row >= 0) r[row] = -dot;
 }
 
 // y = A x (diagonal split) over all chunks.
@@ -303,103 +313,130 @@ __global__ void __launch_bounds__(SELL_TPB) k_spmv(SV<MT, DT> A, int nchunks, co
     }
 }
 
-// y = M x (full rows, no split diagonal): restriction f_c = R r.
-template <class MT, class VT, int U>
-__global__ void __launch_bounds__(SELL_TPB) k_apply_full(SV<MT, MT> M, int nchunks, const VT* x,
-                                                          VT* __restrict__ y) {
+// Restriction f_c = R r, one chunk per warp.  END: the entries of the chunk's first part only (cend =
+// cmid: the red columns of the finest R), else all (cend = cptr + 1).  FIRST selects what else the
+// next level's sweep needs: RF_NONE nothing (the coarsest level), RF_ZERO x_c = 0 (the cluster kernel),
+// RF_SWEEP the first colour step from a zero guess, x_c = f_c / a_ii on colour 0 (its rows see only
+// zeros; the sweep from zero never reads the others), RF_FLOW that with the other rows marked unset.
+enum RestrictNext { RF_NONE, RF_ZERO, RF_SWEEP, RF_FLOW };
+
+template <class MT, class VT, int U, int NEXT>
+__global__ void __launch_bounds__(SELL_TPB) k_restrict(SV<MT, MT> M, const int* __restrict__ cend, int nchunks,
+                                                       const VT* x, VT* __restrict__ y, VT* __restrict__ yx,
+                                                       const int* __restrict__ colour, const VT* __restrict__ dnat) {
+    const int k = blockIdx.x * WPB + (threadIdx.x >> 5);
+    if (k >= nchunks) return;
     pdl_launch_dependents();
-    pdl_wait();
     const int lane = threadIdx.x & 31, C = M.C, r = lane & (C - 1), g = lane / C;
-    for (int k = blockIdx.x * WPB + (threadIdx.x >> 5); k < nchunks; k += gridDim.x * WPB) {
-        const int row = M.perm[k * C + r];
-        VT dot = sell_dot<VT, false, U>(M.col, M.val, M.cptr[k] + g * C + r, M.cptr[k + 1], x);
-        dot = sub_sum(dot, C);
-        if (g == 0 && row >= 0) y[row] = dot;
+    const int row = M.perm[k * C + r];
+    const bool own = g == 0 && row >= 0;
+    int cr = 1;
+    VT dr = VT(0);
+    if ((NEXT == RF_SWEEP || NEXT == RF_FLOW) && own) {
+        cr = colour[row];
+        dr = dnat[row];
+    }
+    VT dot = sell_dot<VT, true, U>(M.col, M.val, M.cptr[k] + g * C + r, cend[k], x);
+    dot = sub_sum(dot, C);
+    if (own) {
+        y[row] = dot;
+        if (NEXT == RF_ZERO) yx[row] = VT(0);
+        if ((NEXT == RF_SWEEP || NEXT == RF_FLOW) && cr == 0) yx[row] = dot * dr;
+        else if (NEXT == RF_FLOW) flow_unset(yx + row);
     }
 }
 
-// f_c = R r and x_c = 0 (the next level starts from a zero guess).
-template <class MT, class VT, int U>
-__global__ void __launch_bounds__(SELL_TPB) k_restrict_zero(SV<MT, MT> M, int nchunks, const VT* x,
-                                                             VT* __restrict__ y, VT* __restrict__ yz) {
+// The first colour step with f given: x = f / a_ii on the slots [0, s1) of colour 0, 0 on the others
+// (the diagonal form gathers them with the value 0, and what a buffer held before may not be finite).
+template <class DT, class FT, class VT>
+__global__ void k_first(int s1, int nslots, const int* __restrict__ perm, const DT* __restrict__ dinv, const FT* f,
+                        VT* __restrict__ x) {
+    const int s = blockIdx.x * blockDim.x + threadIdx.x;
+    if (s >= nslots) return;
     pdl_launch_dependents();
+    const int row = perm[s];
+    const VT d = s < s1 ? Cv<VT>::f(dinv[s]) : VT(0);
     pdl_wait();
-    const int lane = threadIdx.x & 31, C = M.C, r = lane & (C - 1), g = lane / C;
-    for (int k = blockIdx.x * WPB + (threadIdx.x >> 5); k < nchunks; k += gridDim.x * WPB) {
-        const int row = M.perm[k * C + r];
-        VT dot = sell_dot<VT, false, U>(M.col, M.val, M.cptr[k] + g * C + r, M.cptr[k + 1], x);
-        dot = sub_sum(dot, C);
-        if (g == 0 && row >= 0) { y[row] = dot; yz[row] = VT(0); }
-    }
+    if (row >= 0) x[row] = s < s1 ? Cv<VT>::f(f[row]) * d : VT(0);
 }
 
-// f_c = R r, and the first colour step of the coarse sweep from a zero guess fused with the zero
-// fill: x_c = f_c / a_ii on colour 0 (its rows see only zeros), 0 elsewhere.
-template <class MT, class VT, int U>
-__global__ void __launch_bounds__(SELL_TPB) k_restrict_first(SV<MT, MT> M, int nchunks, const VT* x,
-                                                              VT* __restrict__ y, VT* __restrict__ yx,
-                                                              const int* __restrict__ colour,
-                                                              const VT* __restrict__ dnat) {
-    pdl_launch_dependents();
-    pdl_wait();
-    const int lane = threadIdx.x & 31, C = M.C, r = lane & (C - 1), g = lane / C;
-    for (int k = blockIdx.x * WPB + (threadIdx.x >> 5); k < nchunks; k += gridDim.x * WPB) {
-        const int row = M.perm[k * C + r];
-        const bool own = g == 0 && row >= 0;
-        int cr = 1;
-        VT dr = VT(0);
-        if (own) {
-            cr = colour[row];
-            dr = dnat[row];
-        }
-        VT dot = sell_dot<VT, false, U>(M.col, M.val, M.cptr[k] + g * C + r, M.cptr[k + 1], x);
-        dot = sub_sum(dot, C);
-        if (own) {
-            y[row] = dot;
-            yx[row] = cr == 0 ? dot * dr : VT(0);
-        }
-    }
-}
-
-// The same on the finest level (f given): x = f / a_ii on colour 0, 0 elsewhere.
+// The same over all rows in natural order, the others marked unset.
 template <class FT, class VT>
-__global__ void k_zero_first(int64_t n, const FT* f, const int* __restrict__ colour,
-                             const VT* __restrict__ dnat, VT* __restrict__ x) {
+__global__ void k_first_flow(int64_t n, const FT* f, const int* __restrict__ colour, const VT* __restrict__ dnat,
+                             VT* __restrict__ x) {
+    pdl_launch_dependents();
+    pdl_wait();
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+        if (colour[i] == 0) x[i] = Cv<VT>::f(f[i]) * dnat[i];
+        else flow_unset(x + i);
+    }
+}
+
+template <class VT>
+__global__ void k_fill_unset(int64_t n, VT* x) {
     pdl_launch_dependents();
     pdl_wait();
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        x[i] = colour[i] == 0 ? Cv<VT>::f(f[i]) * dnat[i] : VT(0);
+        flow_unset(x + i);
 }
 
-// x += P e (prolongation and correction).
+// x += P e (prolongation and correction) on the rows of chunks [0, nchunks); unset, if given, is marked
+// unset on them for the backward sweep.
 template <class MT, class VT, int U>
 __global__ void __launch_bounds__(SELL_TPB) k_prolong(SV<MT, MT> P, int nchunks, const VT* e,
-                                                       VT* __restrict__ x) {
+                                                       VT* __restrict__ x, VT* unset) {
+    const int k = blockIdx.x * WPB + (threadIdx.x >> 5);
+    if (k >= nchunks) return;
     pdl_launch_dependents();
-    pdl_wait();
     const int lane = threadIdx.x & 31, C = P.C, r = lane & (C - 1), g = lane / C;
-    for (int k = blockIdx.x * WPB + (threadIdx.x >> 5); k < nchunks; k += gridDim.x * WPB) {
-        const int row = P.perm[k * C + r];
-        const bool own = g == 0 && row >= 0;
-        const VT xr = own ? x[row] : VT(0);
-        VT dot = sell_dot<VT, false, U>(P.col, P.val, P.cptr[k] + g * C + r, P.cptr[k + 1], e);
-        dot = sub_sum(dot, C);
-        if (own) x[row] = xr + dot;
+    const int row = P.perm[k * C + r];
+    const bool own = g == 0 && row >= 0;
+    VT xr = VT(0);
+    VT dot = sell_dot<VT, true, U>(P.col, P.val, P.cptr[k] + g * C + r, P.cptr[k + 1], e,
+                                   [&] { if (own) xr = x[row]; });
+    dot = sub_sum(dot, C);
+    if (own) {
+        x[row] = xr + dot;
+        if (unset) flow_unset(unset + row);
     }
 }
 
-// x = A_c^{-1} f with the dense inverse (row-major), one warp per row.
+// x = A_c^{-1} f with the dense inverse (row-major), one warp per row.  A row is 1,823 entries at 1M: a
+// lane takes them in batches of 8 with all loads in flight (and the first batch's before the wait),
+// since a loop with one load in flight is a chain of 57 L2 trips.
 template <class AT, class FT, class VT>
-__global__ void k_coarse(int n, const AT* __restrict__ Ainv, const FT* f, VT* __restrict__ x) {
+__global__ void __launch_bounds__(128) k_coarse(int n, const AT* __restrict__ Ainv, const FT* f, VT* __restrict__ x) {
+    constexpr int B = 8;
+    const int i = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    if (i >= n) return;
     pdl_launch_dependents();
-    pdl_wait();
     const int lane = threadIdx.x & 31;
-    for (int i = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); i < n; i += gridDim.x * (blockDim.x >> 5)) {
-        VT acc = 0;
-        for (int j = lane; j < n; j += 32) acc += Cv<VT>::f(Ainv[(size_t)i * n + j]) * Cv<VT>::f(f[j]);
-        for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
-        if (lane == 0) x[i] = acc;
+    const AT* a = Ainv + (size_t)i * n;
+    VT av[B], fv[B], acc = VT(0);
+    auto load = [&](int j0) {
+#pragma unroll
+        for (int u = 0; u < B; ++u) {
+            const int j = j0 + u * 32 + lane;
+            av[u] = j < n ? Cv<VT>::f(a[j]) : VT(0);
+        }
+    };
+    load(0);
+    pdl_wait();
+    for (int j0 = 0; j0 < n; j0 += 32 * B) {
+#pragma unroll
+        for (int u = 0; u < B; ++u) {
+            const int j = j0 + u * 32 + lane;
+            fv[u] = j < n ? Cv<VT>::f(f[j]) : VT(0);
+        }
+        VT cur[B];
+#pragma unroll
+        for (int u = 0; u < B; ++u) cur[u] = av[u];
+        load(j0 + 32 * B);                                    // the next batch, in flight with the products
+#pragma unroll
+        for (int u = 0; u < B; ++u) acc += cur[u] * fv[u];
     }
+    for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
+    if (lane == 0) x[i] = acc;
 }
 
 template <class VT>
@@ -723,6 +760,10 @@ template <> float* lx<float>(Level& L) { return L.x32.p; }
 template <> float* lf<float>(Level& L) { return L.f32.p; }
 template <> float* lr<float>(Level& L) { return L.r32.p; }
 
+template <class VT> VT* lxa(Level& L);
+template <> double* lxa<double>(Level& L) { return L.xa64.p; }
+template <> float* lxa<float>(Level& L) { return L.xa32.p; }
+
 template <class VT> const VT* ainv(const Handle& h);
 template <> const double* ainv<double>(const Handle& h) { return h.Ainv.p; }
 template <> const float* ainv<float>(const Handle& h) { return h.Ainv32.p; }
@@ -744,7 +785,7 @@ int gs_block_warps(int chunks) {
 }
 
 template <class FT, class VT>
-void rec_gs(Level& L, int c, const FT* f, VT* x, cudaStream_t s) {
+void rec_gs(Level& L, int c, const FT* f, VT* x, cudaStream_t s, bool from_zero = false) {
     const int c0 = L.S.seg[c], c1 = L.S.seg[c + 1];
     if (c1 <= c0) return;
     if (L.S.ndiag) {
@@ -772,31 +813,61 @@ void rec_gs(Level& L, int c, const FT* f, VT* x, cudaStream_t s) {
     }
     const int w = gs_block_warps(c1 - c0);
     const int g = (c1 - c0 + w - 1) / w, tpb = 32 * w;
-    with_u_gs(L.S.lanes, [&](auto u) {
-        constexpr int U = decltype(u)::value;
-        if constexpr (std::is_same<VT, double>::value) {
-            launch(k_gs<double, double, FT, VT, U>, g, tpb, s, view(L.S, (const double*)L.S.val.p, (const double*)L.S.dinv.p), c0, c1, f, x);
-        } else {
-            if (L.vt == VT_BF16)
-                launch(k_gs<__nv_bfloat16, float, FT, VT, U>, g, tpb, s, view(L.S, (const __nv_bfloat16*)L.S.val16.p, (const float*)L.S.dinv32.p), c0, c1, f, x);
-            else
-                launch(k_gs<float, float, FT, VT, U>, g, tpb, s, view(L.S, (const float*)L.S.val32.p, (const float*)L.S.dinv32.p), c0, c1, f, x);
-        }
-    });
+    const int* cmid = L.S.cmid.p;
+    auto go = [&](auto low) {
+        constexpr bool LOW = decltype(low)::value;
+        with_u_gs(LOW ? L.S.lanes_lo : L.S.lanes, c1 - c0, [&](auto u) {
+            constexpr int U = decltype(u)::value;
+            if constexpr (std::is_same<VT, double>::value) {
+                launch(k_gs<double, double, FT, VT, U, LOW>, g, tpb, s, view(L.S, (const double*)L.S.val.p, (const double*)L.S.dinv.p), cmid, c0, c1, f, x);
+            } else {
+                if (L.vt == VT_BF16)
+                    launch(k_gs<__nv_bfloat16, float, FT, VT, U, LOW>, g, tpb, s, view(L.S, (const __nv_bfloat16*)L.S.val16.p, (const float*)L.S.dinv32.p), cmid, c0, c1, f, x);
+                else
+                    launch(k_gs<float, float, FT, VT, U, LOW>, g, tpb, s, view(L.S, (const float*)L.S.val32.p, (const float*)L.S.dinv32.p), cmid, c0, c1, f, x);
+            }
+        });
+    };
+    if (from_zero) go(std::true_type{});
+    else go(std::false_type{});
 }
 
 template <class FT, class VT>
-void rec_resid_level(Level& L, const FT* f, const VT* x, VT* r, cudaStream_t s, bool after_sweep = false) {
-    if (L.S.ndiag && after_sweep && L.ncolours == 2) {      // the last colour's residual is zero
+void rec_resid_level(Level& L, const FT* f, const VT* x, VT* r, cudaStream_t s, bool after_sweep, bool from_zero) {
+    if (L.red_black && after_sweep) {                       // the last colour's residual is zero
         const int s1 = L.S.seg[1] * L.S.C;
-        with_nd(L.S.ndiag, [&](auto nd) {
-            constexpr int ND = decltype(nd)::value;
-            if constexpr (std::is_same<VT, double>::value)
-                launch(k_resid_dia_first<double, double, FT, VT, VT, ND>, slot_blocks(L.S.nslots), SELL_TPB, s,
-                       dview(L.S, L.n, (const double*)L.S.dval.p, (const double*)L.S.diag.p, false), s1, f, x, r);
-            else
-                launch(k_resid_dia_first<float, float, FT, VT, VT, ND>, slot_blocks(L.S.nslots), SELL_TPB, s,
-                       dview(L.S, L.n, (const float*)L.S.dval32.p, (const float*)L.S.diag32.p, false), s1, f, x, r);
+        auto go = [&](auto zero) {
+            constexpr bool ZERO = decltype(zero)::value;
+            with_nd(L.S.ndiag, [&](auto nd) {
+                constexpr int ND = decltype(nd)::value;
+                if constexpr (std::is_same<VT, double>::value)
+                    launch(k_resid_dia_first<double, double, FT, VT, VT, ND, ZERO>, slot_blocks(L.S.nslots), SELL_TPB, s,
+                           dview(L.S, L.n, (const double*)L.S.dval.p, (const double*)L.S.diag.p, false), s1, f, x, r);
+                else
+                    launch(k_resid_dia_first<float, float, FT, VT, VT, ND, ZERO>, slot_blocks(L.S.nslots), SELL_TPB, s,
+                           dview(L.S, L.n, (const float*)L.S.dval32.p, (const float*)L.S.diag32.p, false), s1, f, x, r);
+            });
+        };
+        if (from_zero) go(std::true_type{});
+        else go(std::false_type{});
+        return;
+    }
+    if (after_sweep && from_zero && L.S.cmid.p) {
+        const int g = blocks_for_chunks(L.S.nchunks);
+        with_u(L.S.lanes_up, [&](auto w) {
+            constexpr int U = decltype(w)::value;
+            if constexpr (std::is_same<VT, double>::value) {
+                launch(k_resid_up<double, double, U>, g, SELL_TPB, s, view(L.S, (const double*)L.S.val.p, (const double*)nullptr),
+                       (const int*)L.S.cmid.p, L.S.nchunks, x, r);
+            } else {
+                if (L.vt == VT_BF16)
+                    launch(k_resid_up<__nv_bfloat16, float, U>, g, SELL_TPB, s,
+                           view(L.S, (const __nv_bfloat16*)L.S.val16.p, (const float*)nullptr), (const int*)L.S.cmid.p,
+                           L.S.nchunks, x, r);
+                else
+                    launch(k_resid_up<float, float, U>, g, SELL_TPB, s,
+                           view(L.S, (const float*)L.S.val32.p, (const float*)nullptr), (const int*)L.S.cmid.p, L.S.nchunks, x, r);
+            }
         });
         return;
     }
@@ -857,18 +928,37 @@ template <class VT> const VT* dnat(const Level& L);
 template <> const double* dnat<double>(const Level& L) { return L.dnat64.p; }
 template <> const float* dnat<float>(const Level& L) { return L.dnat32.p; }
 
+// One flow sweep of level l.
+template <class FT, class VT>
+void rec_sweep(Handle& h, int l, FlowMode mode, const FT* f, const VT* xo, VT* xn, cudaStream_t s) {
+    Level& L = h.lev[l];
+    rec_flow<FT, VT>(mode, L.S, L.vt, f, xo, xn, nullptr, nullptr, h.next_flow_ctr(), &h.state.p->gave_up, s);
+}
+
+// f_c = R r onto level l + 1, with what its sweep starts from (k_restrict).
+template <class VT, int NEXT>
+void rec_restrict(Handle& h, int l, bool red, const VT* r, VT* fc, VT* xc, cudaStream_t s) {
+    const Sell& R = h.lev[l].SR;
+    Level& C = h.lev[l + 1];
+    with_u(red ? R.lanes_lo : R.lanes, [&](auto w) {
+        launch(k_restrict<VT, VT, decltype(w)::value, NEXT>, blocks_for_chunks(R.nchunks), SELL_TPB, s, full_view<VT>(R),
+               red ? (const int*)R.cmid.p : (const int*)(R.cptr.p + 1), R.nchunks, r, fc, xc, (const int*)C.colour.p,
+               dnat<VT>(C));
+    });
+}
+
 // Algorithm 3.2 from level l: x <- V-cycle(f, initial guess x) (zero guess when zero_guess).  With
 // ilu, the finest level is smoothed by IC(0) steps instead of Gauss-Seidel sweeps.  With
-// first_done the caller has already applied the first colour step from the zero guess (and
-// zeroed the other rows), so the forward sweep starts at colour 1.  A Gauss-Seidel step from
-// zero on colour 0 reads only zeros, so x_i = (f_i - 0) / a_ii = f_i / a_ii exactly.
+// first_done the caller has already applied the first colour step from the zero guess to the vector
+// that the forward sweep writes (and, for a flow sweep, marked its other rows unset).  A Gauss-Seidel
+// step from zero on colour 0 reads only zeros, so x_i = (f_i - 0) / a_ii = f_i / a_ii exactly.
 template <class FT, class VT>
 void rec_vcycle(Handle& h, int l, const FT* f, VT* x, bool zero_guess, cudaStream_t s, bool ilu = false,
                 bool first_done = false) {
     const int nl = (int)h.lev.size();
     Level& L = h.lev[l];
     if (l == nl - 1) {                                          // step 2(b): exact coarsest solve
-        launch(k_coarse<VT, FT, VT>, std::max(1, (L.n + 7) / 8), 256, s, L.n, ainv<VT>(h), f, x);
+        launch(k_coarse<VT, FT, VT>, std::max(1, (L.n + 3) / 4), 128, s, L.n, ainv<VT>(h), f, x);
         return;
     }
     Level& C = h.lev[l + 1];
@@ -876,41 +966,43 @@ void rec_vcycle(Handle& h, int l, const FT* f, VT* x, bool zero_guess, cudaStrea
     if constexpr (std::is_same<FT, double>::value) {
         if (ilu_here) rec_ic_smooth<VT>(h, f, x, zero_guess, s);          // (1) IC(0) step
     }
-    if (!ilu_here) {
-        int c0 = 0;
-        if (first_done) {
-            c0 = 1;
-        } else if (zero_guess) {
-            launch(k_zero_first<FT, VT>, vec_blocks(L.n), VEC_TPB, s, (int64_t)L.n, f, (const int*)L.colour.p,
-                   dnat<VT>(L), x);
-            c0 = 1;
+    const bool flow = !ilu_here && L.flow;
+    VT* u = flow ? lxa<VT>(L) : x;                                       // the smoothed iterate
+    if (flow) {                                                          // (1) S_l: one launch
+        if (!zero_guess) launch(k_fill_unset<VT>, vec_blocks(L.n), VEC_TPB, s, (int64_t)L.n, u);
+        else if (!first_done)
+            launch(k_first_flow<FT, VT>, vec_blocks(L.n), VEC_TPB, s, (int64_t)L.n, f, (const int*)L.colour.p, dnat<VT>(L), u);
+        rec_sweep<FT, VT>(h, l, zero_guess ? FLOW_FWD0 : FLOW_FWD, f, x, u, s);
+    } else if (!ilu_here) {                                              // (1) S_l: colours ascending
+        if (zero_guess && !first_done) {
+            const int s1 = L.S.seg[1] * L.S.C, ns = L.S.nslots, g = std::max(1, (ns + VEC_TPB - 1) / VEC_TPB);
+            if constexpr (std::is_same<VT, double>::value)
+                launch(k_first<double, FT, VT>, g, VEC_TPB, s, s1, ns, (const int*)L.S.perm.p, (const double*)L.S.dinv.p, f, x);
+            else
+                launch(k_first<float, FT, VT>, g, VEC_TPB, s, s1, ns, (const int*)L.S.perm.p, (const float*)L.S.dinv32.p, f, x);
         }
-        for (int c = c0; c < L.ncolours; ++c) rec_gs(L, c, f, x, s);       // (1) S_l: colours ascending
+        for (int c = zero_guess ? 1 : 0; c < L.ncolours; ++c) rec_gs(L, c, f, x, s, zero_guess);
     }
-    rec_resid_level(L, f, x, lr<VT>(L), s, !ilu_here);                  // (2a) r = f - A u
+    rec_resid_level(L, f, u, lr<VT>(L), s, !ilu_here, zero_guess);       // (2a) r = f - A u
+    // On a red-black level the black residual is zero and the backward sweep overwrites the black rows
+    // before it reads them: only the red columns of R and the red rows of P count.
+    const bool red = L.red_black && !ilu_here;
+    const VT* r = lr<VT>(L);
     if (l + 1 >= h.tail_start) {                                         // (2a) f_c = R r, x_c = 0
-        with_u(L.SR.lanes, [&](auto u) {
-            launch(k_restrict_zero<VT, VT, decltype(u)::value>, blocks_for_chunks(L.SR.nchunks), SELL_TPB, s,
-                   full_view<VT>(L.SR), L.SR.nchunks, (const VT*)lr<VT>(L), lf<VT>(C), lx<VT>(C));
-        });
+        rec_restrict<VT, RF_ZERO>(h, l, red, r, lf<VT>(C), lx<VT>(C), s);
         record_tail(h, l + 1, lf<VT>(C), lx<VT>(C), s);                  // (2b) the coarser levels, one kernel
-    } else if (l + 1 == nl - 1) {                                       // (2a) f_c = R r
-        with_u(L.SR.lanes, [&](auto u) {
-            launch(k_apply_full<VT, VT, decltype(u)::value>, blocks_for_chunks(L.SR.nchunks), SELL_TPB, s,
-                   full_view<VT>(L.SR), L.SR.nchunks, (const VT*)lr<VT>(L), lf<VT>(C));
-        });
+    } else if (l + 1 == nl - 1) {                                        // (2a) f_c = R r
+        rec_restrict<VT, RF_NONE>(h, l, red, r, lf<VT>(C), (VT*)nullptr, s);
         rec_vcycle<VT, VT>(h, l + 1, lf<VT>(C), lx<VT>(C), true, s);     // (2b) exact coarsest solve
     } else {                                                             // (2a) f_c = R r, first colour step
-        with_u(L.SR.lanes, [&](auto u) {
-            launch(k_restrict_first<VT, VT, decltype(u)::value>, blocks_for_chunks(L.SR.nchunks), SELL_TPB, s,
-                   full_view<VT>(L.SR), L.SR.nchunks, (const VT*)lr<VT>(L), lf<VT>(C), lx<VT>(C),
-                   (const int*)C.colour.p, dnat<VT>(C));
-        });
+        if (C.flow) rec_restrict<VT, RF_FLOW>(h, l, red, r, lf<VT>(C), lxa<VT>(C), s);
+        else rec_restrict<VT, RF_SWEEP>(h, l, red, r, lf<VT>(C), lx<VT>(C), s);
         rec_vcycle<VT, VT>(h, l + 1, lf<VT>(C), lx<VT>(C), true, s, false, true);   // (2b) zero initial guess
     }
-    with_u(L.SP.lanes, [&](auto u) {                                     // (2c)
-        launch(k_prolong<VT, VT, decltype(u)::value>, blocks_for_chunks(L.SP.nchunks), SELL_TPB, s,
-               full_view<VT>(L.SP), L.SP.nchunks, (const VT*)lx<VT>(C), x);
+    const int pchunks = red ? L.SP.seg[1] : L.SP.nchunks;
+    with_u(L.SP.lanes, [&](auto w) {                                     // (2c)
+        launch(k_prolong<VT, VT, decltype(w)::value>, blocks_for_chunks(pchunks), SELL_TPB, s, full_view<VT>(L.SP), pchunks,
+               (const VT*)lx<VT>(C), u, flow ? x : (VT*)nullptr);
     });
     if constexpr (std::is_same<FT, double>::value) {
         if (ilu_here) {
@@ -918,7 +1010,9 @@ void rec_vcycle(Handle& h, int l, const FT* f, VT* x, bool zero_guess, cudaStrea
             return;
         }
     }
-    for (int c = L.ncolours - 1; c >= 0; --c) rec_gs(L, c, f, x, s);     // (3) S_l^T: colours descending
+    if (flow) rec_sweep<FT, VT>(h, l, FLOW_BWD, f, u, x, s);             // (3) S_l^T: one launch
+    else
+        for (int c = L.ncolours - 1; c >= 0; --c) rec_gs(L, c, f, x, s);  // (3) S_l^T: colours descending
 }
 
 // t = r - A z with the fine A in the preconditioner's precision.
@@ -947,7 +1041,7 @@ void rec_fine_resid(Handle& h, const double* r, const VT* z, VT* t, cudaStream_t
     });
 }
 
-// w = (LU)^{-1} t level by level; with zadd, z += w as well.
+// w = (LU)^{-1} t, by one flow launch per factor or level by level; with zadd, z += w as well.
 template <class TT, class VT>
 void rec_ic_solve(Handle& h, const TT* t, VT* y, VT* w, VT* zadd, cudaStream_t s) {
     const Sell& L = h.L;
@@ -959,6 +1053,12 @@ void rec_ic_solve(Handle& h, const TT* t, VT* y, VT* w, VT* zadd, cudaStream_t s
     } else {
         lv = view(L, (const float*)L.val32.p, (const float*)nullptr);
         uv = view(U, (const float*)U.val32.p, (const float*)U.dinv32.p);
+    }
+    if (h.ic_flow()) {
+        int* err = &h.state.p->gave_up;
+        rec_flow<TT, VT>(FLOW_LOWER, L, VT_F32, t, nullptr, y, w, nullptr, h.next_flow_ctr(), err, s);   // marks w unset
+        rec_flow<VT, VT>(FLOW_UPPER, U, VT_F32, y, nullptr, w, y, zadd, h.next_flow_ctr(), err, s);      // and y again
+        return;
     }
     for (int g = 0; g + 1 < (int)L.seg.size(); ++g) {
         const int c0 = L.seg[g], c1 = L.seg[g + 1];
@@ -1081,6 +1181,13 @@ void apply_precond(Handle& h, int which, const double* r, double* z) {
     CPC_LAUNCH_CK();
 }
 
+template <class VT>
+void fill_unset(VT* p, int64_t n, cudaStream_t s) {
+    launch(k_fill_unset<VT>, vec_blocks(n), VEC_TPB, s, n, p);
+}
+template void fill_unset<double>(double*, int64_t, cudaStream_t);
+template void fill_unset<float>(float*, int64_t, cudaStream_t);
+
 void spmv_fine(Handle& h, const double* x, double* y, cudaStream_t s) {
     const Sell& A = h.Anat;
     if (A.ndiag) {
@@ -1103,25 +1210,37 @@ float time_gs_sweep(const Sell& S, int n) {
     cudaStream_t cs;
     CPC_CK(cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking));
     struct SG { cudaStream_t s; ~SG() { cudaStreamSynchronize(s); cudaStreamDestroy(s); } } sg{cs};
-    DBuf<double> f, x;
+    constexpr int SWEEPS = 4;
+    DBuf<double> f, x, xa;
+    DBuf<unsigned> ctr;                     // a counter per launch and their error word
     f.alloc(n);
     x.alloc(n);
+    xa.alloc(n);
+    ctr.alloc(SWEEPS + 1);
     CPC_CK(cudaMemsetAsync(f.p, 0, sizeof(double) * n, cs));
     CPC_CK(cudaMemsetAsync(x.p, 0, sizeof(double) * n, cs));
+    CPC_CK(cudaMemsetAsync(ctr.p, 0, sizeof(unsigned) * ctr.n, cs));
     CPC_CK(cudaStreamSynchronize(cs));
-    constexpr int SWEEPS = 4;
+    const bool flow = gs_by_flow(n, (int)S.seg.size() - 1);
     cudaGraph_t g;
     CPC_CK(cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal));
-    for (int k = 0; k < SWEEPS; ++k)
+    for (int k = 0; k < SWEEPS; ++k) {      // the launches of the solve's sweeps
+        if (flow) {
+            launch(k_fill_unset<double>, vec_blocks(n), VEC_TPB, cs, (int64_t)n, xa.p);
+            rec_flow<double, double>(FLOW_FWD, S, VT_F64, f.p, x.p, xa.p, nullptr, nullptr, ctr.p + k, (int*)(ctr.p + SWEEPS), cs);
+            continue;
+        }
         for (size_t c = 0; c + 1 < S.seg.size(); ++c) {
             const int c0 = S.seg[c], c1 = S.seg[c + 1];
             if (c1 <= c0) continue;
             const int w = gs_block_warps(c1 - c0);
-            with_u_gs(S.lanes, [&](auto u) {         // the launch shapes of the solve's colour steps
-                launch(k_gs<double, double, double, double, decltype(u)::value>, (c1 - c0 + w - 1) / w, 32 * w,
-                       cs, view(S, (const double*)S.val.p, (const double*)S.dinv.p), c0, c1, (const double*)f.p, x.p);
+            with_u_gs(S.lanes, c1 - c0, [&](auto u) {
+                launch(k_gs<double, double, double, double, decltype(u)::value, false>, (c1 - c0 + w - 1) / w, 32 * w, cs,
+                       view(S, (const double*)S.val.p, (const double*)S.dinv.p), (const int*)S.cmid.p, c0, c1,
+                       (const double*)f.p, x.p);
             });
         }
+    }
     CPC_CK(cudaStreamEndCapture(cs, &g));
     cudaGraphExec_t ge;
     const cudaError_t ie = cudaGraphInstantiate(&ge, g, 0);
@@ -1165,16 +1284,34 @@ void level_apply(Handle& h, int l, int op, const double* x, double* y) {
         case 1:
         case 2:
             if (last) fail(CPC_EINVAL, "coarsest level has no smoother");
+            if (L.flow && op == 1) {
+                launch(k_first_flow<double, double>, vec_blocks(L.n), VEC_TPB, s, (int64_t)L.n, x, (const int*)L.colour.p,
+                       (const double*)L.dnat64.p, y);
+                rec_sweep<double, double>(h, l, FLOW_FWD0, x, nullptr, y, s);
+                break;
+            }
+            if (L.flow) {
+                launch(k_zero<double>, vec_blocks(L.n), VEC_TPB, s, (int64_t)L.n, L.xa64.p);
+                launch(k_fill_unset<double>, vec_blocks(L.n), VEC_TPB, s, (int64_t)L.n, y);
+                rec_sweep<double, double>(h, l, FLOW_BWD, x, L.xa64.p, y, s);
+                break;
+            }
             launch(k_zero<double>, vec_blocks(L.n), VEC_TPB, s, (int64_t)L.n, y);
-            if (op == 1) for (int c = 0; c < L.ncolours; ++c) rec_gs(L, c, x, y, s);
+            if (op == 1) for (int c = 0; c < L.ncolours; ++c) rec_gs(L, c, x, y, s, true);
             else for (int c = L.ncolours - 1; c >= 0; --c) rec_gs(L, c, x, y, s);
             break;
         case 3:
             if (!last) fail(CPC_EINVAL, "not the coarsest level");
-            launch(k_coarse<double, double, double>, std::max(1, (L.n + 7) / 8), 256, s, L.n, (const double*)h.Ainv.p, x, y);
+            launch(k_coarse<double, double, double>, std::max(1, (L.n + 3) / 4), 128, s, L.n, (const double*)h.Ainv.p, x, y);
             break;
         case 5:                                                   // sweep from the given y (no zeroing)
             if (last) fail(CPC_EINVAL, "coarsest level has no smoother");
+            if (L.flow) {
+                launch(k_copy<double, double>, vec_blocks(L.n), VEC_TPB, s, (int64_t)L.n, (const double*)y, L.xa64.p);
+                launch(k_fill_unset<double>, vec_blocks(L.n), VEC_TPB, s, (int64_t)L.n, y);
+                rec_sweep<double, double>(h, l, FLOW_FWD, x, L.xa64.p, y, s);
+                break;
+            }
             for (int c = 0; c < L.ncolours; ++c) rec_gs(L, c, x, y, s);
             break;
         case 4:
@@ -1194,17 +1331,6 @@ void level_apply(Handle& h, int l, int op, const double* x, double* y) {
 // Microseconds per forward Gauss-Seidel sweep (colours ascending) of level l in the
 // preconditioner's precision on the level's own work vectors, replayed from a CUDA graph as in the
 // solve: reps sweeps per replay, the best of three replays after one warm-up.
-int gs_resident_blocks(int lanes) {
-    int dev = 0, sms = 0, per_sm = 0;
-    CPC_CK(cudaGetDevice(&dev));
-    CPC_CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    with_u_gs(lanes, [&](auto u) {
-        CPC_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-            &per_sm, k_gs<double, double, double, double, decltype(u)::value>, SELL_TPB, 0));
-    });
-    return std::max(1, sms * per_sm);
-}
-
 double sweep_time_us(Handle& h, int l, int reps) {
     const int nl = (int)h.lev.size();
     if (l < 0 || l >= nl - 1) fail(CPC_EINVAL, "level has no smoother");
@@ -1214,13 +1340,28 @@ double sweep_time_us(Handle& h, int l, int reps) {
     CPC_CK(cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking));
     struct SG { cudaStream_t s; ~SG() { cudaStreamSynchronize(s); cudaStreamDestroy(s); } } sg{cs};
     CPC_CK(cudaStreamSynchronize(h.s));
+    // the old values of a flow sweep are read as they are: none may be unset
+    if (L.x64.p) CPC_CK(cudaMemsetAsync(L.x64.p, 0, sizeof(double) * L.n, cs));
+    if (L.x32.p) CPC_CK(cudaMemsetAsync(L.x32.p, 0, sizeof(float) * L.n, cs));
+    CPC_CK(cudaStreamSynchronize(cs));
     cudaGraph_t g;
     CPC_CK(cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal));
-    for (int k = 0; k < reps; ++k)
+    for (int k = 0; k < reps; ++k) {
+        if (L.flow) {
+            if (fp64(h)) {
+                launch(k_fill_unset<double>, vec_blocks(L.n), VEC_TPB, cs, (int64_t)L.n, L.xa64.p);
+                rec_sweep<double, double>(h, l, FLOW_FWD, L.f64.p, L.x64.p, L.xa64.p, cs);
+            } else {
+                launch(k_fill_unset<float>, vec_blocks(L.n), VEC_TPB, cs, (int64_t)L.n, L.xa32.p);
+                rec_sweep<float, float>(h, l, FLOW_FWD, L.f32.p, L.x32.p, L.xa32.p, cs);
+            }
+            continue;
+        }
         for (int c = 0; c < L.ncolours; ++c) {
             if (fp64(h)) rec_gs<double, double>(L, c, (const double*)L.f64.p, L.x64.p, cs);
             else rec_gs<float, float>(L, c, (const float*)L.f32.p, L.x32.p, cs);
         }
+    }
     CPC_CK(cudaStreamEndCapture(cs, &g));
     cudaGraphExec_t ge;
     const cudaError_t ie = cudaGraphInstantiate(&ge, g, 0);
@@ -1345,6 +1486,7 @@ void solve_pcg(Handle& h, const double* b, double* x, double tol, int maxit, int
     CPC_CK(cudaStreamSynchronize(s));
     *iters = out.k;
     *status = out.status;
+    if (out.gave_up) fail(CPC_ETIMEOUT, "a dependent row was not reached in time");
     if (res_hist && hist_cap > 0) {
         const int cnt = std::min(std::min(hist_cap, out.k + 1), HIST_CAP);
         CPC_CK(cudaMemcpy(res_hist, h.hist.p, sizeof(double) * cnt, cudaMemcpyDeviceToHost));

@@ -1,0 +1,82 @@
+"""Sweeps and triangular solves that run as one launch ordered by their data, and the sweeps by colour
+launches from a zero guess: every row of every level satisfies its own equation, to rounding.
+
+A row of a forward sweep from zero solves (D + L) y = x, of a backward sweep (D + U) y = x, of a forward
+sweep from y0 (D + L) y + U y0 = x, with L and U the couplings to earlier and later colours.  A sum of m
+products computed in any order, a difference and a product with the stored reciprocal of a_ii leave a
+residual of at most (m + 4) eps times the sum of the magnitudes of the row's terms.
+"""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+if not torch.cuda.is_available():
+    pytest.skip("needs a GPU", allow_module_level=True)
+
+from paper_1205_6113_gb300 import cpc, inputs  # noqa: E402
+
+pytestmark = pytest.mark.gpu
+DEV = torch.device("cuda:0")
+EPS = np.finfo(np.float64).eps
+
+
+def solver(p, **kw):
+    csr = cpc.tpfa_assemble(p.nx, p.ny, p.nz, torch.tensor(p.logk, device=DEV), p.kz_ratio, p.dirichlet)
+    return cpc.Solver(*csr, **kw)
+
+
+def worst(s, l, y, x, y0, forward):
+    """max over the rows of level l of |residual| / ((m + 4) eps sum of magnitudes)."""
+    ptr, col, val = s.level_matrix(l)
+    _, colour = s.level_splitting(l)
+    n = ptr.size - 1
+    rows = np.repeat(np.arange(n), np.diff(ptr))
+    earlier = colour[col] < colour[rows]
+    new = (rows == col) | (earlier if forward else colour[col] > colour[rows])
+    t = val * np.where(new, y[col], y0[col])
+    res = np.bincount(rows, weights=t, minlength=n) - x
+    mag = np.bincount(rows, weights=np.abs(t), minlength=n) + np.abs(x)
+    return float(np.max(np.abs(res) / ((np.diff(ptr) + 4) * EPS * mag)))
+
+
+# one colour and one row left over; few chunks per colour; blocks of four warps; colour launches on level 1
+@pytest.mark.parametrize("shape,kw", [((33, 1, 1), dict(coarse_max=8)), ((13, 11, 7), dict(coarse_max=16)),
+                                      ((13, 11, 7), dict(coarse_max=16, gs_order="natural")), ((61, 53, 37), {}),
+                                      ((101, 87, 45), {}), ((128, 128, 64), {})])
+def test_every_row_solves_its_equation(shape, kw):
+    s = solver(inputs.small_3d(*shape, seed=81), **kw)
+    for l in range(s.nlevels - 1):
+        n = s.level_info(l)["n"]
+        x, y0 = inputs.random_vector(n, 82 + l), inputs.random_vector(n, 92 + l)
+        xd, zero = torch.tensor(x, device=DEV), np.zeros(n)
+        assert worst(s, l, s.level_apply(l, 1, xd).cpu().numpy(), x, zero, True) <= 1.0
+        assert worst(s, l, s.level_apply(l, 2, xd).cpu().numpy(), x, zero, False) <= 1.0
+        y = s.level_apply(l, 5, xd, torch.tensor(y0, device=DEV)).cpu().numpy()
+        assert worst(s, l, y, x, y0, True) <= 1.0
+
+
+@pytest.mark.parametrize("precision", ["fp64", "fp32", "fp32_bf16"])
+@pytest.mark.parametrize("which", ["bco", "ic0", "amg_ilu"])
+def test_applications_repeat_to_the_bit(which, precision):
+    """Sums are taken in entry order whatever the order of arrival; and a NaN on one row spreads, it
+    does not hang or turn into a number."""
+    p = inputs.small_3d(40, 36, 20, seed=83)
+    s = solver(p, precond=which, precision=precision)
+    r = torch.tensor(inputs.random_vector(p.n, 84), device=DEV)
+    z = s.apply(r)
+    for _ in range(5):
+        assert torch.equal(s.apply(r), z)
+    bad = r.clone()
+    bad[p.n // 2] = float("nan")
+    assert bool(torch.isnan(s.apply(bad)).any())
+    assert torch.equal(s.apply(r), z)
+
+
+def test_in_place_ic0():
+    """z = r as one buffer: every row is read before it is written."""
+    p = inputs.small_3d(40, 36, 20, seed=85)
+    s = solver(p, precond="ic0")
+    r = torch.tensor(inputs.random_vector(p.n, 86), device=DEV)
+    z = s.apply(r)
+    buf = r.clone()
+    assert torch.equal(s.apply(buf, z=buf), z)
