@@ -1,13 +1,16 @@
 // batched.cu -- PCG on K right-hand sides at once (independent columns in lockstep).
 //
-// Block vectors are row-major [n][Kp] (Kp = K rounded up to a multiple of 32), so one warp owns a
-// row and its lanes own columns lane, lane + 32, ...: every matrix entry is one broadcast load
-// shared by all K columns, and every gathered vector row is one coalesced load.  The matrix is read
-// once per K solves instead of once per solve (SpMM).  Each column has its own alpha, beta and
-// convergence flag; a converged column is frozen (alpha = 0) while the others continue, so each
-// column reproduces the single-right-hand-side iteration.  Reductions are per column and finish in
-// a fixed order.  The preconditioner is the handle's, applied column-wise by the same algorithms
-// (Algorithm 2.1 with Algorithm 3.2 and the IC(0) solves).
+// Block vectors are row-major [n][Kp].  Kp = K rounded up to 8 or 16, or to a multiple of 32: a warp owns
+// one row of 32 J columns (lane l the J columns from l J on, one vector load), or for K <= 16 the R = 4
+// or 2 rows that fill its lanes, since a warp instruction costs the same with idle lanes and FP64 issue
+// is scarce on this part.  Every matrix entry is one broadcast load shared by all columns, and every
+// gathered vector row is one coalesced load.  The matrix is read once per K solves instead of once per
+// solve (SpMM).  Each column has its own alpha, beta and convergence flag; a converged column is frozen
+// (alpha = 0) while the others continue, so each column reproduces the single-right-hand-side
+// iteration.  Reductions are per column and finish in a fixed order.  The preconditioner is the
+// handle's, applied column-wise by the same algorithms (Algorithm 2.1 with Algorithm 3.2 and the IC(0)
+// solves); in FP32 it reads an FP32 copy of the residual, made once where the residual is updated
+// (FP64 to FP32 conversions issue at FP64 rate, and each application read the residual five times).
 #include <algorithm>
 #include <type_traits>
 #include <utility>
@@ -19,8 +22,17 @@ namespace cpc {
 
 namespace {
 
-constexpr int BWARPS = 4;                 // rows (warps) per block
+constexpr int BWARPS = 4;                 // warps per block of the SELL kernels, a row each
 constexpr int BTPB = BWARPS * 32;
+// Warps per block of the diagonal-form kernels and the vector passes.  Blocks start at about one a
+// nanosecond on this part, which bounded these short rows at four warps a block (131,072 blocks: a fine
+// colour step of 64 columns 135 us, 112 with 16 warps); the SELL kernels are slower in larger blocks
+// (a level-1 colour step 41 and 51 us).
+constexpr int DWARPS = 16;
+constexpr int DTPB = DWARPS * 32;
+constexpr int VWARPS = 8;                 // warps per block of the PCG vector kernels
+constexpr int VTPB = VWARPS * 32;
+constexpr int WSPLIT = 4;                 // warps that share a row in kb_gs_wide
 constexpr int NB_STATE = 12;              // per-column scalar slots
 
 // column-state layout: S[slot * Kp + col]
@@ -55,7 +67,60 @@ void blaunch(void (*k)(KArgs...), int grid, int block, cudaStream_t s, Args&&...
     CPC_CK(cudaLaunchKernelEx(&cfg, k, std::forward<Args>(args)...));
 }
 
-inline int rows_grid(int nrows) { return (nrows + BWARPS - 1) / BWARPS; }
+// The columns of a lane: 32 J columns on the 32 lanes of a warp (R = 1), or R rows of 32 / R columns.
+template <int J, int R>
+struct Cols {
+    static_assert(R == 1 || J == 1, "several rows per warp have one column per lane");
+    static constexpr int W = 32 / R, KP = 32 * J / R;
+    static __device__ __forceinline__ int sub() { return R == 1 ? 0 : (threadIdx.x & 31) / W; }
+    static __device__ __forceinline__ int col() { return R == 1 ? (threadIdx.x & 31) * J : (threadIdx.x & 31) % W; }
+    // element of (row, the lane's first column)
+    static __device__ __forceinline__ size_t at(int row) { return (size_t)row * KP + col(); }
+};
+
+template <int J, class VT, class T>
+__device__ __forceinline__ void ldv(const T* p, VT (&v)[J]) {
+    if constexpr (std::is_same<T, float>::value && J == 2) {
+        const float2 t = *reinterpret_cast<const float2*>(p);
+        v[0] = Cv<VT>::f(t.x);
+        v[1] = Cv<VT>::f(t.y);
+    } else if constexpr (std::is_same<T, float>::value && J == 4) {
+        const float4 t = *reinterpret_cast<const float4*>(p);
+        v[0] = Cv<VT>::f(t.x);
+        v[1] = Cv<VT>::f(t.y);
+        v[2] = Cv<VT>::f(t.z);
+        v[3] = Cv<VT>::f(t.w);
+    } else if constexpr (std::is_same<T, double>::value && J % 2 == 0) {
+#pragma unroll
+        for (int j = 0; j < J; j += 2) {
+            const double2 t = *reinterpret_cast<const double2*>(p + j);
+            v[j] = Cv<VT>::f(t.x);
+            v[j + 1] = Cv<VT>::f(t.y);
+        }
+    } else {
+#pragma unroll
+        for (int j = 0; j < J; ++j) v[j] = Cv<VT>::f(p[j]);
+    }
+}
+
+template <int J, class T>
+__device__ __forceinline__ void stv(T* p, const T (&v)[J]) {
+    if constexpr (std::is_same<T, float>::value && J == 2) {
+        *reinterpret_cast<float2*>(p) = make_float2(v[0], v[1]);
+    } else if constexpr (std::is_same<T, float>::value && J == 4) {
+        *reinterpret_cast<float4*>(p) = make_float4(v[0], v[1], v[2], v[3]);
+    } else if constexpr (std::is_same<T, double>::value && J % 2 == 0) {
+#pragma unroll
+        for (int j = 0; j < J; j += 2) *reinterpret_cast<double2*>(p + j) = make_double2(v[j], v[j + 1]);
+    } else {
+#pragma unroll
+        for (int j = 0; j < J; ++j) p[j] = v[j];
+    }
+}
+
+// Blocks for nrows rows, one row per warp lane group.
+template <int R>
+inline int rows_grid(int nrows, int warps = BWARPS) { return (nrows + warps * R - 1) / (warps * R); }
 
 // Calls f(std::integral_constant<int, ND>{}) with the padded diagonal count (4, 6 or 8).
 template <class F>
@@ -65,271 +130,355 @@ void bwith_nd(int nd, F&& f) {
     else f(std::integral_constant<int, 8>{});
 }
 
-// acc[j] += sum_w a_w x[col_w][lane + 32 j] over the entries of the row in slot s.  Padding entries
-// (col < 0) sit at the end of a row.  Four entries are loaded before their gathers.
-template <int J, class VT, class MT, class XT>
-__device__ __forceinline__ void brow(const int* __restrict__ col, const MT* __restrict__ val, int C, int base,
-                                     int width, int r, const XT* x, int Kp, int lane, VT (&acc)[J]) {
-    int w = 0;
-    for (; w + 4 <= width; w += 4) {
-        int c[4];
-        VT a[4];
+// The row in slot s of a SELL layout: entries base + w C + r, w < width.
+struct BRow {
+    int base, width, r, C;
+};
+template <class MT, class DT>
+__device__ __forceinline__ BRow brow_at(const BV<MT, DT>& A, int s, const int* end) {
+    const int k = s / A.C;
+    const int base = A.cptr[k];
+    return BRow{base, (end[k] - base) / A.C, s - k * A.C, A.C};
+}
+
+// acc[j] += sum_w a_w x[col_w][j] over entries w0, w0 + step, ... of a row, U entries' loads in flight
+// together.  Padding (-1) and marked columns (LATER) load nothing and add 0.
+template <int J, int R, int U, class VT, class MT, class XT>
+__device__ __forceinline__ void brow(const int* __restrict__ col, const MT* __restrict__ val, const BRow& t, int w0,
+                                     int step, const XT* x, VT (&acc)[J]) {
+    using L = Cols<J, R>;
+    for (int w = w0; w < t.width; w += U * step) {
+        int c[U];
+        VT a[U], xv[U][J];
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            c[u] = col[base + (w + u) * C + r];
-            a[u] = Cv<VT>::f(val[base + (w + u) * C + r]);
+        for (int u = 0; u < U; ++u) {
+            const bool on = w + u * step < t.width;
+            const int e = t.base + (w + u * step) * t.C + t.r;
+            c[u] = on ? col[e] : -1;
+            a[u] = on ? Cv<VT>::f(val[e]) : VT(0);
         }
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            if (c[u] < 0) continue;
-            const XT* xr = x + (size_t)c[u] * Kp + lane;
+        for (int u = 0; u < U; ++u) {
+            if ((unsigned)c[u] < (unsigned)LATER) {
+                ldv<J>(x + L::at(c[u]), xv[u]);
+            } else {
 #pragma unroll
-            for (int j = 0; j < J; ++j) acc[j] += a[u] * Cv<VT>::f(xr[32 * j]);
+                for (int j = 0; j < J; ++j) xv[u][j] = VT(0);
+            }
         }
-    }
-    for (; w < width; ++w) {
-        const int c = col[base + w * C + r];
-        if (c < 0) continue;
-        const VT a = Cv<VT>::f(val[base + w * C + r]);
-        const XT* xr = x + (size_t)c * Kp + lane;
 #pragma unroll
-        for (int j = 0; j < J; ++j) acc[j] += a * Cv<VT>::f(xr[32 * j]);
+        for (int u = 0; u < U; ++u)
+#pragma unroll
+            for (int j = 0; j < J; ++j) acc[j] += a[u] * xv[u][j];
     }
 }
 
-// brow with eight entries per batch (long rows): half the dependent rounds of brow.
-template <int J, class VT, class MT, class XT>
-__device__ __forceinline__ void brow8(const int* __restrict__ col, const MT* __restrict__ val, int C, int base,
-                                      int width, int r, const XT* x, int Kp, int lane, VT (&acc)[J]) {
-    int w = 0;
-    for (; w + 8 <= width; w += 8) {
-        int c[8];
-        VT a[8];
+template <int J, class VT>
+__device__ __forceinline__ void zero(VT (&v)[J]) {
 #pragma unroll
-        for (int u = 0; u < 8; ++u) {
-            c[u] = col[base + (w + u) * C + r];
-            a[u] = Cv<VT>::f(val[base + (w + u) * C + r]);
-        }
-#pragma unroll
-        for (int u = 0; u < 8; ++u) {
-            if (c[u] < 0) continue;
-            const XT* xr = x + (size_t)c[u] * Kp + lane;
-#pragma unroll
-            for (int j = 0; j < J; ++j) acc[j] += a[u] * Cv<VT>::f(xr[32 * j]);
-        }
-    }
-    brow<J, VT>(col, val, C, base + w * C, width - w, r, x, Kp, lane, acc);
+    for (int j = 0; j < J; ++j) v[j] = VT(0);
 }
 
-// Gauss-Seidel over the slots [s0, s1) of one colour, all columns.
-template <int J, class MT, class DT, class FT, class VT, bool LONG = false>
-__global__ void __launch_bounds__(BTPB) kb_gs(BV<MT, DT> A, int s0, int s1, const FT* f, VT* x, int Kp) {
-    const int s = s0 + blockIdx.x * BWARPS + (threadIdx.x >> 5);
+// Gauss-Seidel over the slots [s0, s1) of one colour, all columns; the entries of a row end at end[k]
+// (its chunk's last; in a sweep from a zero guess the entries of later colours, whose rows are zero, are
+// left out: by end in FP64, by their mark in FP32).
+template <int J, int R, class MT, class DT, class VT, int U>
+__global__ void __launch_bounds__(BTPB) kb_gs(BV<MT, DT> A, const int* __restrict__ end, int s0, int s1, const VT* f, VT* x) {
+    using L = Cols<J, R>;
+    const int s = s0 + (blockIdx.x * BWARPS + (threadIdx.x >> 5)) * R + L::sub();
     if (s >= s1) return;
     pdl_launch_dependents();
-    const int lane = threadIdx.x & 31;
     const int row = A.perm[s];                   // matrix data: before the wait
-    const int k = s / A.C, r = s % A.C;
-    const int base = A.cptr[k];
-    const int width = (A.cptr[k + 1] - base) / A.C;
+    const BRow t = brow_at(A, s, end);
     const VT dinv = Cv<VT>::f(A.diag[s]);        // the view's diagonal field holds 1 / a_ii
     pdl_wait();
     if (row < 0) return;
-    VT acc[J];
+    VT acc[J], fr[J];
+    zero(acc);
+    ldv<J>(f + L::at(row), fr);
+    brow<J, R, U>(A.col, A.val, t, 0, 1, x, acc);
 #pragma unroll
-    for (int j = 0; j < J; ++j) acc[j] = VT(0);
-    if (LONG) brow8<J, VT>(A.col, A.val, A.C, base, width, r, x, Kp, lane, acc);
-    else brow<J, VT>(A.col, A.val, A.C, base, width, r, x, Kp, lane, acc);
-#pragma unroll
-    for (int j = 0; j < J; ++j) {
-        const size_t o = (size_t)row * Kp + lane + 32 * j;
-        x[o] = (Cv<VT>::f(f[o]) - acc[j]) * dinv;
-    }
+    for (int j = 0; j < J; ++j) acc[j] = (fr[j] - acc[j]) * dinv;
+    stv<J>(x + L::at(row), acc);
 }
 
-// Gauss-Seidel for long rows in small colour groups (coarse levels): one block of BWARPS warps per
-// row, warp w taking the entries w, w + BWARPS, ...; the warps' partial sums are added in warp
-// order through shared memory.  A step of a few thousand rows then costs a quarter of a row's
-// chain of dependent loads instead of a whole one.
-template <int J, class MT, class DT, class FT, class VT>
-__global__ void __launch_bounds__(BTPB) kb_gs_wide(BV<MT, DT> A, int s0, const FT* f, VT* x, int Kp) {
-    __shared__ VT part[BWARPS][32 * J];
-    const int s = s0 + blockIdx.x;
+// Gauss-Seidel for long rows in small colour groups (coarse levels): WSPLIT warps per R rows, warp w
+// taking the entries w, w + WSPLIT, ...; the warps' partial sums are added in warp order through
+// shared memory.  A step of a few thousand rows then costs a quarter of a row's chain of dependent
+// loads instead of a whole one.  A block holds two such sets.
+template <int J, int R, class MT, class DT, class VT>
+__global__ void __launch_bounds__(64 * WSPLIT) kb_gs_wide(BV<MT, DT> A, const int* __restrict__ end, int s0, int s1,
+                                                          const VT* f, VT* x) {
+    using L = Cols<J, R>;
+    __shared__ VT part[2][WSPLIT][J][32];
+    const int lane = threadIdx.x & 31, w = (threadIdx.x >> 5) % WSPLIT, set = (threadIdx.x >> 5) / WSPLIT;
+    const int sr = s0 + ((int)blockIdx.x * 2 + set) * R + L::sub();
+    const int s = min(sr, s1 - 1);                           // (a repeated row is not written)
     pdl_launch_dependents();
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int row = A.perm[s];
-    const int k = s / A.C, r = s % A.C;
-    const int base = A.cptr[k];
-    const int width = (A.cptr[k + 1] - base) / A.C;
+    const BRow t = brow_at(A, s, end);
     const VT dinv = Cv<VT>::f(A.diag[s]);
     pdl_wait();
-    if (row < 0) return;                         // uniform over the block
-    VT acc[J];
+    VT acc[J], fr[J];
+    zero(acc);
+    zero(fr);
+    if (w == 0 && row >= 0) ldv<J>(f + L::at(row), fr);
+    brow<J, R, 4>(A.col, A.val, t, w, WSPLIT, x, acc);
 #pragma unroll
-    for (int j = 0; j < J; ++j) acc[j] = VT(0);
-    // entries w, w + BWARPS, ...: a strided view of the row (base + w C, step BWARPS C)
-    const int mine = width > w ? (width - w + BWARPS - 1) / BWARPS : 0;
-    brow<J, VT>(A.col, A.val, A.C * BWARPS, base + w * A.C, mine, r, x, Kp, lane, acc);
-#pragma unroll
-    for (int j = 0; j < J; ++j) part[w][lane + 32 * j] = acc[j];
+    for (int j = 0; j < J; ++j) part[set][w][j][lane] = acc[j];
     __syncthreads();
-    if (w != 0) return;
+    if (w != 0 || row < 0 || sr >= s1) return;
 #pragma unroll
     for (int j = 0; j < J; ++j) {
-        VT t = part[0][lane + 32 * j];
-        for (int q = 1; q < BWARPS; ++q) t += part[q][lane + 32 * j];
-        const size_t o = (size_t)row * Kp + lane + 32 * j;
-        x[o] = (Cv<VT>::f(f[o]) - t) * dinv;
+        VT v = part[set][0][j][lane];
+        for (int q = 1; q < WSPLIT; ++q) v += part[set][q][j][lane];
+        acc[j] = (fr[j] - v) * dinv;
     }
+    stv<J>(x + L::at(row), acc);
 }
 
-// out = f - A x (resid) over all slots; with DIAG the split diagonal is included.
-template <int J, class MT, class DT, class FT, class XT, class RT>
-__global__ void __launch_bounds__(BTPB) kb_resid(BV<MT, DT> A, int nslots, const FT* f,
-                                                  const XT* x, RT* __restrict__ out, int Kp) {
+// out = f - A x over all slots.
+template <int J, int R, class MT, class DT, class VT>
+__global__ void __launch_bounds__(BTPB) kb_resid(BV<MT, DT> A, int nslots, const VT* f, const VT* x, VT* __restrict__ out) {
+    using L = Cols<J, R>;
+    const int s = (blockIdx.x * BWARPS + (threadIdx.x >> 5)) * R + L::sub();
+    if (s >= nslots) return;
     pdl_launch_dependents();
+    const int row = A.perm[s];
+    const BRow t = brow_at(A, s, A.cptr + 1);
+    const VT d = Cv<VT>::f(A.diag[s]);
     pdl_wait();
-    const int lane = threadIdx.x & 31;
-    for (int s = blockIdx.x * BWARPS + (threadIdx.x >> 5); s < nslots; s += gridDim.x * BWARPS) {
-        const int row = A.perm[s];
-        if (row < 0) continue;
-        const int k = s / A.C, r = s % A.C;
-        const int base = A.cptr[k];
-        RT acc[J];
-        const RT d = Cv<RT>::f(A.diag[s]);
+    if (row < 0) return;
+    VT acc[J], fr[J];
+    ldv<J>(x + L::at(row), acc);
+    ldv<J>(f + L::at(row), fr);
 #pragma unroll
-        for (int j = 0; j < J; ++j) acc[j] = d * Cv<RT>::f(x[(size_t)row * Kp + lane + 32 * j]);
-        brow<J, RT>(A.col, A.val, A.C, base, (A.cptr[k + 1] - base) / A.C, r, x, Kp, lane, acc);
+    for (int j = 0; j < J; ++j) acc[j] *= d;
+    brow<J, R, 4>(A.col, A.val, t, 0, 1, x, acc);
 #pragma unroll
-        for (int j = 0; j < J; ++j) {
-            const size_t o = (size_t)row * Kp + lane + 32 * j;
-            out[o] = Cv<RT>::f(f[o]) - acc[j];
+    for (int j = 0; j < J; ++j) acc[j] = fr[j] - acc[j];
+    stv<J>(out + L::at(row), acc);
+}
+
+// out = f - A x after a forward sweep from a zero guess: (D + L) x = f holds row by row, so only the
+// entries of later colours (from cmid on) are read, out_i = -sum_up a_ij x_j.
+template <int J, int R, class MT, class DT, class VT>
+__global__ void __launch_bounds__(BTPB) kb_resid_up(BV<MT, DT> A, const int* __restrict__ cmid, int nslots, const VT* x,
+                                                    VT* __restrict__ out) {
+    using L = Cols<J, R>;
+    const int s = (blockIdx.x * BWARPS + (threadIdx.x >> 5)) * R + L::sub();
+    if (s >= nslots) return;
+    pdl_launch_dependents();
+    const int row = A.perm[s];
+    const int k = s / A.C, base = cmid[k];
+    const BRow t{base, (A.cptr[k + 1] - base) / A.C, s - k * A.C, A.C};
+    pdl_wait();
+    if (row < 0) return;
+    VT acc[J];
+    zero(acc);
+    brow<J, R, 4>(A.col, A.val, t, 0, 1, x, acc);
+#pragma unroll
+    for (int j = 0; j < J; ++j) acc[j] = -acc[j];
+    stv<J>(out + L::at(row), acc);
+}
+
+// f_c = R r (entries up to end[k]: all, or the red columns of the finest level) and, with yx, the coarse
+// level's first colour step from zero, x_c = f_c / a_ii on colour 0 (the sweep does not read the others).
+template <int J, int R, class MT, class VT>
+__global__ void __launch_bounds__(BTPB) kb_restrict(BV<MT, MT> M, const int* __restrict__ end, int nslots, const VT* x,
+                                                    VT* __restrict__ y, VT* __restrict__ yx,
+                                                    const int* __restrict__ colour, const VT* __restrict__ dnat) {
+    using L = Cols<J, R>;
+    const int s = (blockIdx.x * BWARPS + (threadIdx.x >> 5)) * R + L::sub();
+    if (s >= nslots) return;
+    pdl_launch_dependents();
+    const int row = M.perm[s];
+    const BRow t = brow_at(M, s, end);
+    const bool c0 = yx && row >= 0 && colour[row] == 0;
+    const VT dr = c0 ? dnat[row] : VT(0);
+    pdl_wait();
+    if (row < 0) return;
+    VT acc[J];
+    zero(acc);
+    brow<J, R, 4>(M.col, M.val, t, 0, 1, x, acc);
+    stv<J>(y + L::at(row), acc);
+    if (!c0) return;
+#pragma unroll
+    for (int j = 0; j < J; ++j) acc[j] *= dr;
+    stv<J>(yx + L::at(row), acc);
+}
+
+// x += P e on the rows of slots [0, nslots)
+template <int J, int R, class MT, class VT>
+__global__ void __launch_bounds__(BTPB) kb_prolong(BV<MT, MT> P, int nslots, const VT* e, VT* __restrict__ x) {
+    using L = Cols<J, R>;
+    const int s = (blockIdx.x * BWARPS + (threadIdx.x >> 5)) * R + L::sub();
+    if (s >= nslots) return;
+    pdl_launch_dependents();
+    const int row = P.perm[s];
+    const BRow t = brow_at(P, s, P.cptr + 1);
+    pdl_wait();
+    if (row < 0) return;
+    VT acc[J], xr[J];
+    zero(acc);
+    ldv<J>(x + L::at(row), xr);
+    brow<J, R, 4>(P.col, P.val, t, 0, 1, e, acc);
+#pragma unroll
+    for (int j = 0; j < J; ++j) acc[j] += xr[j];
+    stv<J>(x + L::at(row), acc);
+}
+
+// x = A_c^{-1} f (dense) in FP64: a block per R * CROWS rows, its warps sharing the columns of A_c^{-1} in
+// contiguous parts (one warp per row is a chain of 1,800 FP64 operations, 113 us; 17 this way), the partial
+// sums added in warp order.  A warp takes CROWS rows at a time, since f is read from L2 once per block.
+constexpr int CROWS = 4, CWARPS = 8;
+template <int J, int R, class AT, class FT, class VT>
+__global__ void __launch_bounds__(CWARPS * 32) kb_coarse(int n, const AT* __restrict__ Ainv, const FT* f, VT* __restrict__ x) {
+    using L = Cols<J, R>;
+    __shared__ VT part[CWARPS][CROWS][J][32];
+    pdl_launch_dependents();
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int i0 = (blockIdx.x * R + L::sub()) * CROWS;
+    const int per = (n + CWARPS - 1) / CWARPS, m0 = w * per, m1 = min(n, m0 + per);
+    pdl_wait();
+    VT acc[CROWS][J];
+#pragma unroll
+    for (int q = 0; q < CROWS; ++q) zero(acc[q]);
+#pragma unroll 4
+    for (int m = m0; m < m1; ++m) {
+        VT fv[J];
+        ldv<J>(f + L::at(m), fv);
+#pragma unroll
+        for (int q = 0; q < CROWS; ++q) {
+            const VT a = i0 + q < n ? Cv<VT>::f(Ainv[(size_t)(i0 + q) * n + m]) : VT(0);
+#pragma unroll
+            for (int j = 0; j < J; ++j) acc[q][j] += a * fv[j];
         }
     }
+#pragma unroll
+    for (int q = 0; q < CROWS; ++q)
+#pragma unroll
+        for (int j = 0; j < J; ++j) part[w][q][j][lane] = acc[q][j];
+    __syncthreads();
+    if (w >= CROWS || i0 + w >= n) return;                  // warp q adds up row q
+    VT v[J];
+#pragma unroll
+    for (int j = 0; j < J; ++j) {
+        v[j] = part[0][w][j][lane];
+        for (int q = 1; q < CWARPS; ++q) v[j] += part[q][w][j][lane];
+    }
+    stv<J>(x + L::at(i0 + w), v);
 }
 
-// y = M x for full rows (restriction), optionally zeroing yz (the next level's initial guess).
-template <int J, class MT, class VT>
-__global__ void __launch_bounds__(BTPB) kb_apply(BV<MT, MT> M, int nslots, const VT* x,
-                                                  VT* __restrict__ y, VT* __restrict__ yz, int Kp) {
+// The same in FP32, a warp per SROWS R rows, each sum taken in column order by one lane.  f (466 KB for 64 FP32 columns at 1M) and the block's rows of A_c^{-1} pass
+// through shared memory in tiles of CTILE columns, the next tile's loads in flight with the products: from
+// L2 the sum is a chain of 1,823 loads, read once per row (107 us; 50 this way, 45 in FP64's order).
+constexpr int SROWS = 2, CTILE = 32;
+template <int J, int R, class AT, class FT, class VT>
+__global__ void __launch_bounds__(CWARPS * 32) kb_coarse_seq(int n, const AT* __restrict__ Ainv, const FT* f, VT* __restrict__ x) {
+    using L = Cols<J, R>;
+    constexpr int KP = L::KP, ROWS = CWARPS * R * SROWS, TPB = CWARPS * 32;
+    constexpr int FPT = (CTILE * KP + TPB - 1) / TPB, APT = (ROWS * CTILE + TPB - 1) / TPB;
+    __shared__ VT fs[CTILE * KP];
+    __shared__ VT as[ROWS][CTILE + 1];
     pdl_launch_dependents();
+    const int t = threadIdx.x, b0 = blockIdx.x * ROWS;
+    const int r0 = ((t >> 5) * R + L::sub()) * SROWS;       // the lane's rows within the block
+    VT fv[FPT], av[APT], acc[SROWS][J];
+#pragma unroll
+    for (int q = 0; q < SROWS; ++q) zero(acc[q]);
+    auto load_a = [&](int m0) {
+#pragma unroll
+        for (int u = 0; u < APT; ++u) {
+            const int e = t + u * TPB, r = e / CTILE, c = e % CTILE;
+            av[u] = r < ROWS && b0 + r < n && m0 + c < n ? Cv<VT>::f(Ainv[(size_t)(b0 + r) * n + m0 + c]) : VT(0);
+        }
+    };
+    auto load_f = [&](int m0) {
+#pragma unroll
+        for (int u = 0; u < FPT; ++u) {
+            const int e = t + u * TPB;
+            fv[u] = e < CTILE * KP && m0 + e / KP < n ? Cv<VT>::f(f[(size_t)m0 * KP + e]) : VT(0);
+        }
+    };
+    load_a(0);
     pdl_wait();
-    const int lane = threadIdx.x & 31;
-    for (int s = blockIdx.x * BWARPS + (threadIdx.x >> 5); s < nslots; s += gridDim.x * BWARPS) {
-        const int row = M.perm[s];
-        if (row < 0) continue;
-        const int k = s / M.C, r = s % M.C;
-        const int base = M.cptr[k];
-        VT acc[J];
+    load_f(0);
+    for (int m0 = 0; m0 < n; m0 += CTILE) {
+        __syncthreads();
 #pragma unroll
-        for (int j = 0; j < J; ++j) acc[j] = VT(0);
-        brow<J, VT>(M.col, M.val, M.C, base, (M.cptr[k + 1] - base) / M.C, r, x, Kp, lane, acc);
+        for (int u = 0; u < FPT; ++u)
+            if (t + u * TPB < CTILE * KP) fs[t + u * TPB] = fv[u];
 #pragma unroll
-        for (int j = 0; j < J; ++j) {
-            const size_t o = (size_t)row * Kp + lane + 32 * j;
-            y[o] = acc[j];
-            if (yz) yz[o] = VT(0);
+        for (int u = 0; u < APT; ++u) {
+            const int e = t + u * TPB;
+            if (e / CTILE < ROWS) as[e / CTILE][e % CTILE] = av[u];
+        }
+        __syncthreads();
+        if (m0 + CTILE < n) {
+            load_a(m0 + CTILE);
+            load_f(m0 + CTILE);
+        }
+        const int mc = min(CTILE, n - m0);
+#pragma unroll 8
+        for (int m = 0; m < mc; ++m) {
+            VT v[J];
+            ldv<J>(fs + m * KP + L::col(), v);
+#pragma unroll
+            for (int q = 0; q < SROWS; ++q)
+#pragma unroll
+                for (int j = 0; j < J; ++j) acc[q][j] += as[r0 + q][m] * v[j];
         }
     }
-}
-
-// x += P e
-template <int J, class MT, class VT>
-__global__ void __launch_bounds__(BTPB) kb_prolong(BV<MT, MT> P, int nslots, const VT* e,
-                                                    VT* __restrict__ x, int Kp) {
-    pdl_launch_dependents();
-    pdl_wait();
-    const int lane = threadIdx.x & 31;
-    for (int s = blockIdx.x * BWARPS + (threadIdx.x >> 5); s < nslots; s += gridDim.x * BWARPS) {
-        const int row = P.perm[s];
-        if (row < 0) continue;
-        const int k = s / P.C, r = s % P.C;
-        const int base = P.cptr[k];
-        VT acc[J];
 #pragma unroll
-        for (int j = 0; j < J; ++j) acc[j] = VT(0);
-        brow<J, VT>(P.col, P.val, P.C, base, (P.cptr[k + 1] - base) / P.C, r, e, Kp, lane, acc);
-#pragma unroll
-        for (int j = 0; j < J; ++j) x[(size_t)row * Kp + lane + 32 * j] += acc[j];
-    }
-}
-
-// x = A_c^{-1} f (dense), one warp per row, lanes over columns.
-template <int J, class AT, class FT, class VT>
-__global__ void __launch_bounds__(BTPB) kb_coarse(int n, const AT* __restrict__ Ainv, const FT* f,
-                                                   VT* __restrict__ x, int Kp) {
-    pdl_launch_dependents();
-    pdl_wait();
-    const int lane = threadIdx.x & 31;
-    for (int i = blockIdx.x * BWARPS + (threadIdx.x >> 5); i < n; i += gridDim.x * BWARPS) {
-        VT acc[J];
-#pragma unroll
-        for (int j = 0; j < J; ++j) acc[j] = VT(0);
-        for (int m = 0; m < n; ++m) {
-            const VT a = Cv<VT>::f(Ainv[(size_t)i * n + m]);
-#pragma unroll
-            for (int j = 0; j < J; ++j) acc[j] += a * Cv<VT>::f(f[(size_t)m * Kp + lane + 32 * j]);
-        }
-#pragma unroll
-        for (int j = 0; j < J; ++j) x[(size_t)i * Kp + lane + 32 * j] = acc[j];
-    }
-}
-
-template <class VT>
-__global__ void kb_zero(int64_t n, VT* x) {
-    pdl_launch_dependents();
-    pdl_wait();
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        x[i] = VT(0);
+    for (int q = 0; q < SROWS; ++q)
+        if (b0 + r0 + q < n) stv<J>(x + L::at(b0 + r0 + q), acc[q]);
 }
 
 // Triangular solves of one IC(0) level, all columns: y = t - L y; w = (y - U w) / d, z += w.
-template <int J, class MT, class TT, class VT>
-__global__ void __launch_bounds__(BTPB) kb_lsolve(BV<MT, MT> L, int s0, int s1, const TT* t, VT* y, int Kp) {
-    pdl_launch_dependents();
-    pdl_wait();
-    const int s = s0 + blockIdx.x * BWARPS + (threadIdx.x >> 5);
+template <int J, int R, class MT, class VT>
+__global__ void __launch_bounds__(BTPB) kb_lsolve(BV<MT, MT> A, int s0, int s1, const VT* t, VT* y) {
+    using L = Cols<J, R>;
+    const int s = s0 + (blockIdx.x * BWARPS + (threadIdx.x >> 5)) * R + L::sub();
     if (s >= s1) return;
-    const int lane = threadIdx.x & 31;
-    const int row = L.perm[s];
+    pdl_launch_dependents();
+    const int row = A.perm[s];
+    const BRow b = brow_at(A, s, A.cptr + 1);
+    pdl_wait();
     if (row < 0) return;
-    const int k = s / L.C, r = s % L.C;
-    const int base = L.cptr[k];
-    VT acc[J];
+    VT acc[J], tr[J];
+    zero(acc);
+    ldv<J>(t + L::at(row), tr);
+    brow<J, R, 4>(A.col, A.val, b, 0, 1, y, acc);
 #pragma unroll
-    for (int j = 0; j < J; ++j) acc[j] = VT(0);
-    brow<J, VT>(L.col, L.val, L.C, base, (L.cptr[k + 1] - base) / L.C, r, y, Kp, lane, acc);
-#pragma unroll
-    for (int j = 0; j < J; ++j) {
-        const size_t o = (size_t)row * Kp + lane + 32 * j;
-        y[o] = Cv<VT>::f(t[o]) - acc[j];
-    }
+    for (int j = 0; j < J; ++j) acc[j] = tr[j] - acc[j];
+    stv<J>(y + L::at(row), acc);
 }
 
-template <int J, class MT, class VT>
-__global__ void __launch_bounds__(BTPB) kb_usolve(BV<MT, MT> U, int s0, int s1, const VT* y, VT* w,
-                                                   VT* zadd, int Kp) {
-    pdl_launch_dependents();
-    pdl_wait();
-    const int s = s0 + blockIdx.x * BWARPS + (threadIdx.x >> 5);
+template <int J, int R, class MT, class VT>
+__global__ void __launch_bounds__(BTPB) kb_usolve(BV<MT, MT> U, int s0, int s1, const VT* y, VT* w, VT* zadd) {
+    using L = Cols<J, R>;
+    const int s = s0 + (blockIdx.x * BWARPS + (threadIdx.x >> 5)) * R + L::sub();
     if (s >= s1) return;
-    const int lane = threadIdx.x & 31;
+    pdl_launch_dependents();
     const int row = U.perm[s];
-    if (row < 0) return;
-    const int k = s / U.C, r = s % U.C;
-    const int base = U.cptr[k];
-    VT acc[J];
-#pragma unroll
-    for (int j = 0; j < J; ++j) acc[j] = VT(0);
-    brow<J, VT>(U.col, U.val, U.C, base, (U.cptr[k + 1] - base) / U.C, r, w, Kp, lane, acc);
+    const BRow b = brow_at(U, s, U.cptr + 1);
     const VT dinv = Cv<VT>::f(U.diag[s]);        // 1 / u_ii
+    pdl_wait();
+    if (row < 0) return;
+    VT acc[J], yr[J];
+    zero(acc);
+    ldv<J>(y + L::at(row), yr);
+    brow<J, R, 4>(U.col, U.val, b, 0, 1, w, acc);
 #pragma unroll
-    for (int j = 0; j < J; ++j) {
-        const size_t o = (size_t)row * Kp + lane + 32 * j;
-        const VT v = (y[o] - acc[j]) * dinv;
-        w[o] = v;
-        if (zadd) zadd[o] += v;
-    }
+    for (int j = 0; j < J; ++j) acc[j] = (yr[j] - acc[j]) * dinv;
+    stv<J>(w + L::at(row), acc);
+    if (!zadd) return;
+    VT z[J];
+    ldv<J>(zadd + L::at(row), z);
+#pragma unroll
+    for (int j = 0; j < J; ++j) z[j] += acc[j];
+    stv<J>(zadd + L::at(row), z);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -357,18 +506,15 @@ __device__ __forceinline__ int bd_row(const BD<MT, DT>& A, int s) {
     return A.perm ? A.perm[s] : (s < A.n ? s : -1);
 }
 
-// acc[j] += sum_d v_d x[i + off_d][lane + 32 j] (all gathers issued before the products)
-template <int J, int ND, class VT, class XT>
-__device__ __forceinline__ void bd_dot(const VT (&v)[ND], const DiaOff& off, int row, int n, const XT* x, int Kp,
-                                       int lane, VT (&acc)[J]) {
+// acc[j] += sum_d v_d x[i + off_d][j] (all gathers issued before the products)
+template <int J, int R, int ND, class VT, class XT>
+__device__ __forceinline__ void bd_dot(const VT (&v)[ND], const DiaOff& off, int row, int n, const XT* x, VT (&acc)[J]) {
     VT xv[ND][J];
 #pragma unroll
     for (int d = 0; d < ND; ++d) {
         int jr = row + off.o[d];
         jr = jr < 0 ? 0 : (jr >= n ? n - 1 : jr);
-        const XT* xr = x + (size_t)jr * Kp + lane;
-#pragma unroll
-        for (int j = 0; j < J; ++j) xv[d][j] = Cv<VT>::f(xr[32 * j]);
+        ldv<J>(x + Cols<J, R>::at(jr), xv[d]);
     }
 #pragma unroll
     for (int d = 0; d < ND; ++d)
@@ -376,12 +522,12 @@ __device__ __forceinline__ void bd_dot(const VT (&v)[ND], const DiaOff& off, int
         for (int j = 0; j < J; ++j) acc[j] += v[d] * xv[d][j];
 }
 
-template <int J, class MT, class DT, class FT, class VT, int ND>
-__global__ void __launch_bounds__(BTPB) kb_gs_dia(BD<MT, DT> A, int s0, int s1, const FT* f, VT* x, int Kp) {
-    const int s = s0 + blockIdx.x * BWARPS + (threadIdx.x >> 5);
+template <int J, int R, class MT, class DT, class VT, int ND>
+__global__ void __launch_bounds__(DTPB) kb_gs_dia(BD<MT, DT> A, int s0, int s1, const VT* f, VT* x) {
+    using L = Cols<J, R>;
+    const int s = s0 + (blockIdx.x * DWARPS + (threadIdx.x >> 5)) * R + L::sub();
     if (s >= s1) return;
     pdl_launch_dependents();
-    const int lane = threadIdx.x & 31;
     const int row = bd_row(A, s);
     VT v[ND];
 #pragma unroll
@@ -390,51 +536,22 @@ __global__ void __launch_bounds__(BTPB) kb_gs_dia(BD<MT, DT> A, int s0, int s1, 
     pdl_wait();
     if (row < 0) return;
     VT fr[J], acc[J];
+    zero(acc);
+    ldv<J>(f + L::at(row), fr);
+    bd_dot<J, R, ND>(v, A.off, row, A.n, x, acc);
 #pragma unroll
-    for (int j = 0; j < J; ++j) {
-        fr[j] = Cv<VT>::f(f[(size_t)row * Kp + lane + 32 * j]);
-        acc[j] = VT(0);
-    }
-    bd_dot<J, ND>(v, A.off, row, A.n, x, Kp, lane, acc);
-#pragma unroll
-    for (int j = 0; j < J; ++j) x[(size_t)row * Kp + lane + 32 * j] = (fr[j] - acc[j]) * dinv;
+    for (int j = 0; j < J; ++j) acc[j] = (fr[j] - acc[j]) * dinv;
+    stv<J>(x + L::at(row), acc);
 }
 
-// out = f - A x, diagonal form (grid-stride over slots).
-template <int J, class MT, class DT, class FT, class XT, class RT, int ND>
-__global__ void __launch_bounds__(BTPB) kb_resid_dia(BD<MT, DT> A, const FT* f, const XT* x,
-                                                      RT* __restrict__ out, int Kp) {
-    pdl_launch_dependents();
-    pdl_wait();
-    const int lane = threadIdx.x & 31;
-    for (int s = blockIdx.x * BWARPS + (threadIdx.x >> 5); s < A.nslots; s += gridDim.x * BWARPS) {
-        const int row = bd_row(A, s);
-        if (row < 0) continue;
-        RT v[ND];
-#pragma unroll
-        for (int d = 0; d < ND; ++d) v[d] = Cv<RT>::f(A.val[(size_t)d * A.nslots + s]);
-        const RT dg = Cv<RT>::f(A.diag[s]);
-        RT acc[J];
-#pragma unroll
-        for (int j = 0; j < J; ++j) acc[j] = dg * Cv<RT>::f(x[(size_t)row * Kp + lane + 32 * j]);
-        bd_dot<J, ND>(v, A.off, row, A.n, x, Kp, lane, acc);
-#pragma unroll
-        for (int j = 0; j < J; ++j) {
-            const size_t o = (size_t)row * Kp + lane + 32 * j;
-            out[o] = Cv<RT>::f(f[o]) - acc[j];
-        }
-    }
-}
-
-// B_co step (2) with red-black IC(0), black rows only (see the single right-hand-side path):
-// z_b += (r_b - (A z)_b) / u_bb on the fine colour 1, diagonal form.
-template <int J, class MT, class DT, class VT, int ND>
-__global__ void __launch_bounds__(BTPB) kb_bco_black_dia(BD<MT, DT> A, int s0, int s1, const double* r,
-                                                          const VT* __restrict__ uinv, VT* __restrict__ z, int Kp) {
-    const int s = s0 + blockIdx.x * BWARPS + (threadIdx.x >> 5);
+// out = f - A x on slots [0, s1), diagonal form.  ZERO: after a forward sweep from a zero guess on the
+// first of two colours, whose f_i - a_ii x_i is 0.
+template <int J, int R, class MT, class DT, class FT, class VT, int ND, bool ZERO>
+__global__ void __launch_bounds__(DTPB) kb_resid_dia(BD<MT, DT> A, int s1, const FT* f, const VT* x, VT* __restrict__ out) {
+    using L = Cols<J, R>;
+    const int s = (blockIdx.x * DWARPS + (threadIdx.x >> 5)) * R + L::sub();
     if (s >= s1) return;
     pdl_launch_dependents();
-    const int lane = threadIdx.x & 31;
     const int row = bd_row(A, s);
     VT v[ND];
 #pragma unroll
@@ -442,80 +559,108 @@ __global__ void __launch_bounds__(BTPB) kb_bco_black_dia(BD<MT, DT> A, int s0, i
     const VT dg = Cv<VT>::f(A.diag[s]);
     pdl_wait();
     if (row < 0) return;
-    const VT ui = uinv[row];
-    VT zr[J], acc[J];
+    VT acc[J], fr[J];
+    zero(acc);
+    zero(fr);
+    if (!ZERO) {
+        ldv<J>(x + L::at(row), acc);
+        ldv<J>(f + L::at(row), fr);
 #pragma unroll
-    for (int j = 0; j < J; ++j) {
-        zr[j] = z[(size_t)row * Kp + lane + 32 * j];
-        acc[j] = dg * zr[j];
+        for (int j = 0; j < J; ++j) acc[j] *= dg;
     }
-    bd_dot<J, ND>(v, A.off, row, A.n, z, Kp, lane, acc);
+    bd_dot<J, R, ND>(v, A.off, row, A.n, x, acc);
 #pragma unroll
-    for (int j = 0; j < J; ++j) {
-        const size_t o = (size_t)row * Kp + lane + 32 * j;
-        z[o] = zr[j] + (Cv<VT>::f(r[o]) - acc[j]) * ui;
-    }
+    for (int j = 0; j < J; ++j) acc[j] = fr[j] - acc[j];
+    stv<J>(out + L::at(row), acc);
 }
 
-// First colour step of a sweep from a zero guess fused with the zero fill: x = f / a_ii on colour 0,
-// 0 elsewhere (colour-0 rows see only zeros).
-template <class FT, class VT>
-__global__ void kb_zero_first(int n, int Kp, const FT* f, const int* __restrict__ colour,
-                              const VT* __restrict__ dnat, VT* __restrict__ x) {
+// B_co step (2) with red-black IC(0), black rows only (see the single right-hand-side path):
+// z_b += (r_b - (A z)_b) / u_bb on the fine colour 1, diagonal form.
+template <int J, int R, class MT, class DT, class VT, int ND>
+__global__ void __launch_bounds__(DTPB) kb_bco_black_dia(BD<MT, DT> A, int s0, int s1, const VT* r,
+                                                          const VT* __restrict__ uinv, VT* __restrict__ z) {
+    using L = Cols<J, R>;
+    const int s = s0 + (blockIdx.x * DWARPS + (threadIdx.x >> 5)) * R + L::sub();
+    if (s >= s1) return;
     pdl_launch_dependents();
+    const int row = bd_row(A, s);
+    VT v[ND];
+#pragma unroll
+    for (int d = 0; d < ND; ++d) v[d] = Cv<VT>::f(A.val[(size_t)d * A.nslots + s]);
+    const VT dg = Cv<VT>::f(A.diag[s]);
+    const VT ui = row >= 0 ? uinv[row] : VT(0);
     pdl_wait();
-    for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < (int64_t)n * Kp;
-         t += (int64_t)gridDim.x * blockDim.x) {
-        const int i = (int)(t / Kp);
-        x[t] = colour[i] == 0 ? Cv<VT>::f(f[t]) * dnat[i] : VT(0);
-    }
+    if (row < 0) return;
+    VT zr[J], rr[J], acc[J];
+    ldv<J>(z + L::at(row), zr);
+    ldv<J>(r + L::at(row), rr);
+#pragma unroll
+    for (int j = 0; j < J; ++j) acc[j] = dg * zr[j];
+    bd_dot<J, R, ND>(v, A.off, row, A.n, z, acc);
+#pragma unroll
+    for (int j = 0; j < J; ++j) zr[j] += (rr[j] - acc[j]) * ui;
+    stv<J>(z + L::at(row), zr);
 }
 
-// f_c = R r and the coarse level's first colour step from zero: x_c = f_c / a_ii on colour 0, 0 elsewhere.
-template <int J, class MT, class VT>
-__global__ void __launch_bounds__(BTPB) kb_restrict_first(BV<MT, MT> M, int nslots, const VT* x,
-                                                           VT* __restrict__ y, VT* __restrict__ yx,
-                                                           const int* __restrict__ colour, const VT* __restrict__ dnat,
-                                                           int Kp) {
+// First colour step of a sweep from a zero guess: x = f / a_ii on colour 0; the other rows are set to 0
+// (the diagonal form gathers them with the value 0, and what a buffer held before may not be finite).
+template <int J, int R, class VT>
+__global__ void __launch_bounds__(DTPB) kb_first(int n, const VT* f, const int* __restrict__ colour,
+                                                 const VT* __restrict__ dnat, VT* __restrict__ x) {
+    using L = Cols<J, R>;
+    const int i = (blockIdx.x * DWARPS + (threadIdx.x >> 5)) * R + L::sub();
+    if (i >= n) return;
     pdl_launch_dependents();
+    const bool c0 = colour[i] == 0;
+    const VT d = dnat[i];
     pdl_wait();
-    const int lane = threadIdx.x & 31;
-    for (int s = blockIdx.x * BWARPS + (threadIdx.x >> 5); s < nslots; s += gridDim.x * BWARPS) {
-        const int row = M.perm[s];
-        if (row < 0) continue;
-        const int k = s / M.C, r = s % M.C;
-        const int base = M.cptr[k];
-        const bool c0 = colour[row] == 0;
-        const VT dr = dnat[row];
-        VT acc[J];
+    VT v[J];
+    zero(v);
+    if (c0) {
+        ldv<J>(f + L::at(i), v);
 #pragma unroll
-        for (int j = 0; j < J; ++j) acc[j] = VT(0);
-        brow<J, VT>(M.col, M.val, M.C, base, (M.cptr[k + 1] - base) / M.C, r, x, Kp, lane, acc);
-#pragma unroll
-        for (int j = 0; j < J; ++j) {
-            const size_t o = (size_t)row * Kp + lane + 32 * j;
-            y[o] = acc[j];
-            yx[o] = c0 ? acc[j] * dr : VT(0);
-        }
+        for (int j = 0; j < J; ++j) v[j] *= d;
     }
+    stv<J>(x + L::at(i), v);
 }
 
 // ---------------------------------------------------------------------------------------------
-// Per-column reductions: each block sums its rows per column (warps, then in order), writes a
-// partial row; the last block sums the partial rows in block order and runs `fin` per column.
+// Per-column reductions, in an order that depends on the number of rows alone: the rows are dealt to
+// 4 vblocks(n) lane groups (row i to group i mod 4 vblocks), the groups are added by fours in order, and
+// the last block adds these partial rows and runs `fin` per column.  How many groups a block holds (its
+// warps times the rows of a warp) does not show in the sums.  ordered (FP32 preconditioner, see
+// Level::skip_zeros): the partial rows are added one after another, a chain of 1,216 FP64 sums with the
+// loads of the next rows beside it; else in parts by all threads, the parts in order.  One thread per
+// column with one load in flight took 0.1 ms, three times an iteration.
 // ---------------------------------------------------------------------------------------------
-template <int J, class Fin>
-__device__ void col_finish(double (&v)[J], double* part, unsigned* ctr, int Kp, Fin fin) {
-    __shared__ double sh[BWARPS][128];
+constexpr int VBLOCKS = 152 * 8;
+__host__ __device__ inline int vblocks(int n) { return min(VBLOCKS, (n + 3) / 4); }
+// Blocks for a pass over n rows.
+template <int R>
+inline int vgrid(int n) { return (vblocks(n) * 4 + VWARPS * R - 1) / (VWARPS * R); }
+// The lane group's first row (none at or beyond n for a group past the last).
+template <int J, int R>
+__device__ __forceinline__ int vfirst(int n) {
+    const int g = (blockIdx.x * VWARPS + (threadIdx.x >> 5)) * R + Cols<J, R>::sub();
+    return g < vblocks(n) * 4 ? g : n;
+}
+
+template <int J, int R, class Fin>
+__device__ void col_finish(int n, bool ordered, double (&v)[J], double* part, unsigned* ctr, Fin fin) {
+    constexpr int KP = Cols<J, R>::KP, SETS = VWARPS * R / 4;
+    __shared__ double sh[VWARPS * 128];
     __shared__ bool last;
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int w = threadIdx.x >> 5, G = vblocks(n);
+    const int sub = Cols<J, R>::sub(), col = Cols<J, R>::col();
 #pragma unroll
-    for (int j = 0; j < J; ++j) sh[w][lane + 32 * j] = v[j];
+    for (int j = 0; j < J; ++j) sh[(w * R + sub) * KP + col + j] = v[j];
     __syncthreads();
-    for (int c = threadIdx.x; c < Kp; c += blockDim.x) {
+    for (int e = threadIdx.x; e < SETS * KP; e += VTPB) {
+        const int b = e / KP, c = e % KP;
+        if ((int)blockIdx.x * SETS + b >= G) break;
         double t = 0.0;
-        for (int q = 0; q < BWARPS; ++q) t += sh[q][c];
-        part[(size_t)blockIdx.x * Kp + c] = t;
+        for (int q = 0; q < 4; ++q) t += sh[(4 * b + q) * KP + c];
+        part[((size_t)blockIdx.x * SETS + b) * KP + c] = t;
     }
     __threadfence();
     __syncthreads();
@@ -523,35 +668,85 @@ __device__ void col_finish(double (&v)[J], double* part, unsigned* ctr, int Kp, 
     __syncthreads();
     if (!last) return;
     __threadfence();
-    for (int c = threadIdx.x; c < Kp; c += blockDim.x) {
+    constexpr int PER = 8;
+    if (!ordered) {
+        constexpr int PARTS = VTPB / KP;                     // (96 columns: some threads idle)
+        const int per = (G + PARTS - 1) / PARTS, c = threadIdx.x % KP, p = threadIdx.x / KP, b1 = min(G, (p + 1) * per);
         double t = 0.0;
-        for (int b = 0; b < (int)gridDim.x; ++b) t += __ldcg(&part[(size_t)b * Kp + c]);
-        fin(c, t);
+        if (p < PARTS)
+            for (int b = p * per; b < b1; b += 2 * PER) {
+                double u[2 * PER];
+#pragma unroll
+                for (int q = 0; q < 2 * PER; ++q) u[q] = b + q < b1 ? __ldcg(&part[(size_t)(b + q) * KP + c]) : 0.0;
+#pragma unroll
+                for (int q = 0; q < 2 * PER; ++q) t += u[q];
+            }
+        sh[threadIdx.x] = t;
+        __syncthreads();
+        if ((int)threadIdx.x < KP) {
+            for (int q = 1; q < PARTS; ++q) t += sh[q * KP + threadIdx.x];
+            fin(threadIdx.x, t);
+        }
+    } else {
+        // tiles of rows through shared memory, the next one's loads in flight with a column's chain of sums
+        constexpr int TILE = VTPB * PER / KP > VWARPS * 128 / KP ? VWARPS * 128 / KP : VTPB * PER / KP;
+        double u[PER], t = 0.0;
+        auto load = [&](int b) {
+#pragma unroll
+            for (int q = 0; q < PER; ++q) {
+                const int e = (int)threadIdx.x + q * VTPB;
+                u[q] = e < TILE * KP && b + e / KP < G ? __ldcg(&part[(size_t)b * KP + e]) : 0.0;
+            }
+        };
+        load(0);
+        for (int b = 0; b < G; b += TILE) {
+            __syncthreads();
+#pragma unroll
+            for (int q = 0; q < PER; ++q)
+                if ((int)threadIdx.x + q * VTPB < TILE * KP) sh[threadIdx.x + q * VTPB] = u[q];
+            __syncthreads();
+            if (b + TILE < G) load(b + TILE);
+            if ((int)threadIdx.x < KP) {                     // (rows past the last are 0: t + 0 = t)
+#pragma unroll
+                for (int q = 0; q < TILE; ++q) t += sh[q * KP + threadIdx.x];
+            }
+        }
+        if ((int)threadIdx.x < KP) fin(threadIdx.x, t);
     }
     __syncthreads();
     if (threadIdx.x == 0) *ctr = 0u;
 }
 
+// The residual in the preconditioner's precision (r32 null in FP64: the preconditioner reads r).
 template <int J>
-__global__ void __launch_bounds__(BTPB) kb_init(int n, int Kp, const double* b, double* __restrict__ x,
-                                                 double* __restrict__ r, double* part, unsigned* ctr, double* S) {
+__device__ __forceinline__ void st_r32(float* r32, size_t o, const double (&r)[J]) {
+    if (!r32) return;
+    float t[J];
+#pragma unroll
+    for (int j = 0; j < J; ++j) t[j] = (float)r[j];
+    stv<J>(r32 + o, t);
+}
+
+template <int J, int R>
+__global__ void __launch_bounds__(VTPB) kb_init(int n, const double* b, double* __restrict__ x, double* __restrict__ r,
+                                                 float* r32, double* part, unsigned* ctr, double* S, bool ordered) {
+    using L = Cols<J, R>;
+    constexpr int Kp = L::KP;
     pdl_launch_dependents();
     pdl_wait();
-    const int lane = threadIdx.x & 31;
-    double v[J];
+    double v[J], z[J];
+    zero(v);
+    zero(z);
+    for (int i = vfirst<J, R>(n); i < n; i += 4 * vblocks(n)) {
+        double bi[J];
+        ldv<J>(b + L::at(i), bi);
+        stv<J>(x + L::at(i), z);
+        stv<J>(r + L::at(i), bi);
+        st_r32<J>(r32, L::at(i), bi);
 #pragma unroll
-    for (int j = 0; j < J; ++j) v[j] = 0.0;
-    for (int i = blockIdx.x * BWARPS + (threadIdx.x >> 5); i < n; i += gridDim.x * BWARPS) {
-#pragma unroll
-        for (int j = 0; j < J; ++j) {
-            const size_t o = (size_t)i * Kp + lane + 32 * j;
-            const double bi = b[o];
-            x[o] = 0.0;
-            r[o] = bi;
-            v[j] += bi * bi;
-        }
+        for (int j = 0; j < J; ++j) v[j] += bi[j] * bi[j];
     }
-    col_finish<J>(v, part, ctr, Kp, [&](int c, double t) {
+    col_finish<J, R>(n, ordered, v, part, ctr, [&](int c, double t) {
         const double bn = sqrt(t);
         S[S_BNORM * Kp + c] = bn;
         S[S_K * Kp + c] = 0.0;
@@ -565,13 +760,14 @@ __global__ void __launch_bounds__(BTPB) kb_init(int n, int Kp, const double* b, 
     });
 }
 
-// Any column still active?  Sets the loop condition (one thread).
+// Any column still active?  Sets the loop condition (one warp).
 __global__ void kb_any_active(int Kp, const double* S, cudaGraphConditionalHandle cond) {
     pdl_launch_dependents();
     pdl_wait();
-    unsigned go = 0u;
-    for (int c = 0; c < Kp; ++c) go |= S[S_ACTIVE * Kp + c] > 0.0 ? 1u : 0u;
-    cudaGraphSetConditional(cond, go);
+    bool on = false;
+    for (int c = threadIdx.x; c < Kp; c += 32) on |= S[S_ACTIVE * Kp + c] > 0.0;
+    on = __any_sync(0xffffffffu, on);
+    if (threadIdx.x == 0) cudaGraphSetConditional(cond, on ? 1u : 0u);
 }
 
 __global__ void kb_guard(cudaGraphConditionalHandle cond) {
@@ -580,23 +776,22 @@ __global__ void kb_guard(cudaGraphConditionalHandle cond) {
     cudaGraphSetConditional(cond, 0u);
 }
 
-template <int J, class ZT>
-__global__ void __launch_bounds__(BTPB) kb_rz(int n, int Kp, const double* r, const ZT* z,
-                                               double* part, unsigned* ctr, double* S) {
+template <int J, int R, class ZT>
+__global__ void __launch_bounds__(VTPB) kb_rz(int n, const double* r, const ZT* z, double* part, unsigned* ctr, double* S, bool ordered) {
+    using L = Cols<J, R>;
+    constexpr int Kp = L::KP;
     pdl_launch_dependents();
     pdl_wait();
-    const int lane = threadIdx.x & 31;
     double v[J];
+    zero(v);
+    for (int i = vfirst<J, R>(n); i < n; i += 4 * vblocks(n)) {
+        double ri[J], zi[J];
+        ldv<J>(r + L::at(i), ri);
+        ldv<J>(z + L::at(i), zi);
 #pragma unroll
-    for (int j = 0; j < J; ++j) v[j] = 0.0;
-    for (int i = blockIdx.x * BWARPS + (threadIdx.x >> 5); i < n; i += gridDim.x * BWARPS) {
-#pragma unroll
-        for (int j = 0; j < J; ++j) {
-            const size_t o = (size_t)i * Kp + lane + 32 * j;
-            v[j] += r[o] * cvt_d(z[o]);
-        }
+        for (int j = 0; j < J; ++j) v[j] += ri[j] * zi[j];
     }
-    col_finish<J>(v, part, ctr, Kp, [&](int c, double t) {
+    col_finish<J, R>(n, ordered, v, part, ctr, [&](int c, double t) {
         const bool act = S[S_ACTIVE * Kp + c] > 0.0;
         if (act && (!(t > 0.0) || !isfinite(t))) {
             S[S_STATUS * Kp + c] = CPC_EBREAKDOWN;
@@ -608,127 +803,114 @@ __global__ void __launch_bounds__(BTPB) kb_rz(int n, int Kp, const double* r, co
     });
 }
 
-template <int J, class ZT>
-__global__ void __launch_bounds__(BTPB) kb_p(int n, int Kp, const ZT* z, double* __restrict__ p,
-                                              const double* S) {
+template <int J, int R, class ZT>
+__global__ void __launch_bounds__(VTPB) kb_p(int n, const ZT* z, double* __restrict__ p, const double* S) {
+    using L = Cols<J, R>;
+    constexpr int Kp = L::KP;
     pdl_launch_dependents();
     pdl_wait();
-    const int lane = threadIdx.x & 31;
-    double beta[J];
-    bool first[J];
+    double beta[J], k[J];
+    ldv<J>(S + S_BETA * Kp + L::col(), beta);
+    ldv<J>(S + S_K * Kp + L::col(), k);
+    for (int i = vfirst<J, R>(n); i < n; i += 4 * vblocks(n)) {
+        double zi[J], pi[J];
+        ldv<J>(z + L::at(i), zi);
+        ldv<J>(p + L::at(i), pi);
 #pragma unroll
-    for (int j = 0; j < J; ++j) {
-        beta[j] = S[S_BETA * Kp + lane + 32 * j];
-        first[j] = S[S_K * Kp + lane + 32 * j] == 0.0;
-    }
-    for (int i = blockIdx.x * BWARPS + (threadIdx.x >> 5); i < n; i += gridDim.x * BWARPS) {
-#pragma unroll
-        for (int j = 0; j < J; ++j) {
-            const size_t o = (size_t)i * Kp + lane + 32 * j;
-            p[o] = first[j] ? cvt_d(z[o]) : cvt_d(z[o]) + beta[j] * p[o];
-        }
+        for (int j = 0; j < J; ++j) pi[j] = k[j] == 0.0 ? zi[j] : zi[j] + beta[j] * pi[j];
+        stv<J>(p + L::at(i), pi);
     }
 }
 
-template <int J>
-__global__ void __launch_bounds__(BTPB) kb_spmv_pq(BV<double, double> A, int nslots, int Kp, const double* p,
-                                                    double* __restrict__ q, double* part, unsigned* ctr, double* S) {
+// p.q has been summed: alpha = (r.z) / (p.q), a column that is not positive stops.
+__device__ __forceinline__ void fin_pq(double* S, int Kp, int c, double t) {
+    const bool act = S[S_ACTIVE * Kp + c] > 0.0;
+    S[S_PQ * Kp + c] = t;
+    if (act && (!(t > 0.0) || !isfinite(t))) {
+        S[S_STATUS * Kp + c] = CPC_EBREAKDOWN;
+        S[S_ACTIVE * Kp + c] = 0.0;
+    }
+    S[S_ALPHA * Kp + c] = S[S_ACTIVE * Kp + c] > 0.0 ? S[S_RZ * Kp + c] / t : 0.0;
+}
+
+template <int J, int R>
+__global__ void __launch_bounds__(VTPB) kb_spmv_pq(BV<double, double> A, int nslots, const double* p,
+                                                    double* __restrict__ q, double* part, unsigned* ctr, double* S, bool ordered) {
+    using L = Cols<J, R>;
     pdl_launch_dependents();
     pdl_wait();
-    const int lane = threadIdx.x & 31;
     double v[J];
-#pragma unroll
-    for (int j = 0; j < J; ++j) v[j] = 0.0;
-    for (int s = blockIdx.x * BWARPS + (threadIdx.x >> 5); s < nslots; s += gridDim.x * BWARPS) {
+    zero(v);
+    for (int s = vfirst<J, R>(nslots); s < nslots; s += 4 * vblocks(nslots)) {
         const int row = A.perm[s];
         if (row < 0) continue;
-        const int k = s / A.C, r = s % A.C;
-        const int base = A.cptr[k];
-        double acc[J];
+        double acc[J], pr[J];
         const double d = A.diag[s];
+        ldv<J>(p + L::at(row), pr);
 #pragma unroll
-        for (int j = 0; j < J; ++j) acc[j] = d * p[(size_t)row * Kp + lane + 32 * j];
-        brow<J, double>(A.col, A.val, A.C, base, (A.cptr[k + 1] - base) / A.C, r, p, Kp, lane, acc);
+        for (int j = 0; j < J; ++j) acc[j] = d * pr[j];
+        brow<J, R, 4>(A.col, A.val, brow_at(A, s, A.cptr + 1), 0, 1, p, acc);
+        stv<J>(q + L::at(row), acc);
 #pragma unroll
-        for (int j = 0; j < J; ++j) {
-            const size_t o = (size_t)row * Kp + lane + 32 * j;
-            q[o] = acc[j];
-            v[j] += p[o] * acc[j];
-        }
+        for (int j = 0; j < J; ++j) v[j] += pr[j] * acc[j];
     }
-    col_finish<J>(v, part, ctr, Kp, [&](int c, double t) {
-        const bool act = S[S_ACTIVE * Kp + c] > 0.0;
-        S[S_PQ * Kp + c] = t;
-        if (act && (!(t > 0.0) || !isfinite(t))) {
-            S[S_STATUS * Kp + c] = CPC_EBREAKDOWN;
-            S[S_ACTIVE * Kp + c] = 0.0;
-        }
-        S[S_ALPHA * Kp + c] = S[S_ACTIVE * Kp + c] > 0.0 ? S[S_RZ * Kp + c] / t : 0.0;
-    });
+    col_finish<J, R>(nslots, ordered, v, part, ctr, [&](int c, double t) { fin_pq(S, L::KP, c, t); });
 }
 
-template <int J, int ND>
-__global__ void __launch_bounds__(BTPB) kb_spmv_pq_dia(BD<double, double> A, int Kp, const double* p,
-                                                        double* __restrict__ q, double* part, unsigned* ctr, double* S) {
+template <int J, int R, int ND>
+__global__ void __launch_bounds__(VTPB) kb_spmv_pq_dia(BD<double, double> A, const double* p, double* __restrict__ q,
+                                                        double* part, unsigned* ctr, double* S, bool ordered) {
+    using L = Cols<J, R>;
     pdl_launch_dependents();
     pdl_wait();
-    const int lane = threadIdx.x & 31;
     double v[J];
-#pragma unroll
-    for (int j = 0; j < J; ++j) v[j] = 0.0;
-    for (int s = blockIdx.x * BWARPS + (threadIdx.x >> 5); s < A.nslots; s += gridDim.x * BWARPS) {
+    zero(v);
+    for (int s = vfirst<J, R>(A.nslots); s < A.nslots; s += 4 * vblocks(A.nslots)) {
         const int row = bd_row(A, s);
         if (row < 0) continue;
         double w[ND];
 #pragma unroll
         for (int d = 0; d < ND; ++d) w[d] = A.val[(size_t)d * A.nslots + s];
         const double dg = A.diag[s];
-        double acc[J];
+        double acc[J], pr[J];
+        ldv<J>(p + L::at(row), pr);
 #pragma unroll
-        for (int j = 0; j < J; ++j) acc[j] = dg * p[(size_t)row * Kp + lane + 32 * j];
-        bd_dot<J, ND>(w, A.off, row, A.n, p, Kp, lane, acc);
+        for (int j = 0; j < J; ++j) acc[j] = dg * pr[j];
+        bd_dot<J, R, ND>(w, A.off, row, A.n, p, acc);
+        stv<J>(q + L::at(row), acc);
 #pragma unroll
-        for (int j = 0; j < J; ++j) {
-            const size_t o = (size_t)row * Kp + lane + 32 * j;
-            q[o] = acc[j];
-            v[j] += p[o] * acc[j];
-        }
+        for (int j = 0; j < J; ++j) v[j] += pr[j] * acc[j];
     }
-    col_finish<J>(v, part, ctr, Kp, [&](int c, double t) {
-        const bool act = S[S_ACTIVE * Kp + c] > 0.0;
-        S[S_PQ * Kp + c] = t;
-        if (act && (!(t > 0.0) || !isfinite(t))) {
-            S[S_STATUS * Kp + c] = CPC_EBREAKDOWN;
-            S[S_ACTIVE * Kp + c] = 0.0;
-        }
-        S[S_ALPHA * Kp + c] = S[S_ACTIVE * Kp + c] > 0.0 ? S[S_RZ * Kp + c] / t : 0.0;
-    });
+    col_finish<J, R>(A.nslots, ordered, v, part, ctr, [&](int c, double t) { fin_pq(S, L::KP, c, t); });
 }
 
-template <int J>
-__global__ void __launch_bounds__(BTPB) kb_update(int n, int Kp, double* __restrict__ x, double* __restrict__ r,
-                                                   const double* p, const double* q,
-                                                   double* part, unsigned* ctr, double* S) {
+template <int J, int R>
+__global__ void __launch_bounds__(VTPB) kb_update(int n, double* __restrict__ x, double* __restrict__ r, float* r32,
+                                                   const double* p, const double* q, double* part, unsigned* ctr, double* S, bool ordered) {
+    using L = Cols<J, R>;
+    constexpr int Kp = L::KP;
     pdl_launch_dependents();
     pdl_wait();
-    const int lane = threadIdx.x & 31;
     double alpha[J], v[J];
-#pragma unroll
-    for (int j = 0; j < J; ++j) {
-        alpha[j] = S[S_ALPHA * Kp + lane + 32 * j];
-        v[j] = 0.0;
-    }
-    for (int i = blockIdx.x * BWARPS + (threadIdx.x >> 5); i < n; i += gridDim.x * BWARPS) {
+    ldv<J>(S + S_ALPHA * Kp + L::col(), alpha);
+    zero(v);
+    for (int i = vfirst<J, R>(n); i < n; i += 4 * vblocks(n)) {
+        double xi[J], ri[J], pi[J], qi[J];
+        ldv<J>(x + L::at(i), xi);
+        ldv<J>(p + L::at(i), pi);
+        ldv<J>(r + L::at(i), ri);
+        ldv<J>(q + L::at(i), qi);
 #pragma unroll
         for (int j = 0; j < J; ++j) {
-            const size_t o = (size_t)i * Kp + lane + 32 * j;
-            x[o] += alpha[j] * p[o];
-            const double ri = r[o] - alpha[j] * q[o];
-            r[o] = ri;
-            v[j] += ri * ri;
+            xi[j] += alpha[j] * pi[j];
+            ri[j] -= alpha[j] * qi[j];
+            v[j] += ri[j] * ri[j];
         }
+        stv<J>(x + L::at(i), xi);
+        stv<J>(r + L::at(i), ri);
+        st_r32<J>(r32, L::at(i), ri);
     }
-    col_finish<J>(v, part, ctr, Kp, [&](int c, double t) {
+    col_finish<J, R>(n, ordered, v, part, ctr, [&](int c, double t) {
         if (S[S_ACTIVE * Kp + c] <= 0.0) return;
         const double k = S[S_K * Kp + c] + 1.0;
         S[S_K * Kp + c] = k;
@@ -740,25 +922,15 @@ __global__ void __launch_bounds__(BTPB) kb_update(int n, int Kp, double* __restr
     });
 }
 
-// [n][K] user layout <-> [n][Kp] internal layout
-__global__ void kb_pack(int n, int K, int Kp, const double* in, double* __restrict__ out) {
-    pdl_launch_dependents();
-    pdl_wait();
-    for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < (int64_t)n * Kp; t += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t i = t / Kp;
-        const int c = (int)(t % Kp);
-        out[t] = c < K ? in[i * K + c] : 0.0;
-    }
+// [n][K] user layout <-> [n][Kp] internal layout, 32 rows per block of 8 warps.
+__global__ void __launch_bounds__(256) kb_pack(int n, int K, int Kp, const double* in, double* __restrict__ out) {
+    for (int i = blockIdx.x * 8 + (threadIdx.x >> 5); i < n; i += gridDim.x * 8)
+        for (int c = threadIdx.x & 31; c < Kp; c += 32) out[(size_t)i * Kp + c] = c < K ? in[(size_t)i * K + c] : 0.0;
 }
 
-__global__ void kb_unpack(int n, int K, int Kp, const double* in, double* __restrict__ out) {
-    pdl_launch_dependents();
-    pdl_wait();
-    for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < (int64_t)n * K; t += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t i = t / K;
-        const int c = (int)(t % K);
-        out[t] = in[i * Kp + c];
-    }
+__global__ void __launch_bounds__(256) kb_unpack(int n, int K, int Kp, const double* in, double* __restrict__ out) {
+    for (int i = blockIdx.x * 8 + (threadIdx.x >> 5); i < n; i += gridDim.x * 8)
+        for (int c = threadIdx.x & 31; c < K; c += 32) out[(size_t)i * K + c] = in[(size_t)i * Kp + c];
 }
 
 // Adjoint sources from the forward solutions: b[i][c] = x[i][c] where b[i][c] != 0, else 0
@@ -782,55 +954,55 @@ __global__ void kb_adjoint_rhs(int64_t nk, double* __restrict__ b, const double*
 // arithmetic is FP64 and every sum finishes in a fixed order.
 // ------------------------------------------------------------------------------------------------
 constexpr int KK_TPB = 256;
-constexpr int KK_ROWS = 32;               // rows staged per step of kk_gram
+constexpr int KK_ELEMS = 2048;            // elements of U (and of V) staged per step of kk_gram
 constexpr int KK_GRID = 152 * 2;          // blocks of kk_gram / kk_update / kk_colnorm (fixed)
 enum { KM_PQ = 0, KM_GAMMA, KM_GAMMA_NEW, KM_ALPHA, KM_BETA, KM_COUNT };
 enum { KV_BNORM = 0, KV_RES, KV_COUNT };
 enum { KF_BAD = 0, KF_DONE, KF_COUNT };
 
 // part[block] = U^T V over the block's rows, on the 4 x 4 tiles (ti, tj) with ti <= tj of the
-// Kp x Kp result (Kp = 32 or 64); U is Z (preconditioner precision) or P, V is R or Q (FP64).
-// Thread t owns the t-th upper tile in row-major order, so the T (T + 1) / 2 active threads fill
-// whole warps: an FP64 warp instruction costs the same with idle lanes, and FP64 issue is the
-// bound of this kernel on this part.
-template <class UT>
-__global__ void __launch_bounds__(KK_TPB) kk_gram(int n, int Kp, const UT* U,
-                                                  const double* V, double* __restrict__ part) {
+// KP x KP result; U is Z (preconditioner precision) or P, V is R or Q (FP64).  The NT upper tiles in
+// row-major order belong to consecutive threads, and as many groups of NT threads as fit in the block
+// share the staged rows (25 groups of 10 tiles for 16 columns, one of 136 for 64), so that whole warps
+// work: an FP64 warp instruction costs the same with idle lanes, and FP64 issue is the bound of this
+// kernel on this part.  The groups' tiles are added in group order.
+template <int KP, class UT>
+__global__ void __launch_bounds__(KK_TPB) kk_gram(int n, const UT* U, const double* V, double* __restrict__ part) {
+    constexpr int T = KP / 4, NT = T * (T + 1) / 2, GROUPS = KK_TPB / NT, ROWS = KK_ELEMS / KP;
     extern __shared__ double ksm[];
-    double* us = ksm;                      // [KK_ROWS][Kp]
-    double* vs = ksm + KK_ROWS * Kp;       // [KK_ROWS][Kp]
-    const int T = Kp / 4, t = threadIdx.x;
-    int ti = 0, rem = t;
-    while (ti < T && rem >= T - ti) {
+    double* us = ksm;                      // [ROWS][KP]
+    double* vs = ksm + KK_ELEMS;           // [ROWS][KP]
+    const int t = threadIdx.x, grp = t / NT;
+    int ti = 0, rem = t - grp * NT;
+    while (rem >= T - ti) {
         rem -= T - ti;
         ++ti;
     }
     const int tj = ti + rem;
-    const bool act = ti < T;
+    const bool act = grp < GROUPS;
     double acc[4][4];
 #pragma unroll
     for (int a = 0; a < 4; ++a)
 #pragma unroll
         for (int c = 0; c < 4; ++c) acc[a][c] = 0.0;
     const int per = (n + gridDim.x - 1) / gridDim.x;
-    const int r0 = min(n, blockIdx.x * per), r1 = min(n, r0 + per);
-    for (int base = r0; base < r1; base += KK_ROWS) {
-        const int rows = min(KK_ROWS, r1 - base);
+    const int r0 = min(n, (int)blockIdx.x * per), r1 = min(n, r0 + per);
+    for (int base = r0; base < r1; base += ROWS) {
+        const int rows = min(ROWS, r1 - base);
         __syncthreads();
-        for (int e = t; e < KK_ROWS * Kp; e += KK_TPB) {
-            const int rr = e / Kp;
-            const size_t g = (size_t)base * Kp + e;
-            us[e] = rr < rows ? (double)U[g] : 0.0;
-            vs[e] = rr < rows ? V[g] : 0.0;
+        for (int e = t; e < KK_ELEMS; e += KK_TPB) {
+            const size_t g = (size_t)base * KP + e;
+            us[e] = e < rows * KP ? (double)U[g] : 0.0;
+            vs[e] = e < rows * KP ? V[g] : 0.0;
         }
         __syncthreads();
         if (act) {
-            for (int rr = 0; rr < rows; ++rr) {
+            for (int rr = grp; rr < rows; rr += GROUPS) {
                 double a[4], c[4];
 #pragma unroll
                 for (int q = 0; q < 4; ++q) {
-                    a[q] = us[rr * Kp + ti * 4 + q];
-                    c[q] = vs[rr * Kp + tj * 4 + q];
+                    a[q] = us[rr * KP + ti * 4 + q];
+                    c[q] = vs[rr * KP + tj * 4 + q];
                 }
 #pragma unroll
                 for (int q = 0; q < 4; ++q)
@@ -839,23 +1011,42 @@ __global__ void __launch_bounds__(KK_TPB) kk_gram(int n, int Kp, const UT* U,
             }
         }
     }
-    if (act)
+    // the groups in turn add their tiles in shared memory (KP x KP <= 2 KK_ELEMS)
+    for (int g = 0; g < GROUPS; ++g) {
+        __syncthreads();
+        if (grp == g)
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+#pragma unroll
+                for (int w = 0; w < 4; ++w) {
+                    double& o = ksm[(ti * 4 + q) * KP + tj * 4 + w];
+                    o = g == 0 ? acc[q][w] : o + acc[q][w];
+                }
+    }
+    __syncthreads();
+    if (grp == 0)
 #pragma unroll
         for (int q = 0; q < 4; ++q)
 #pragma unroll
-            for (int w = 0; w < 4; ++w) part[((size_t)blockIdx.x * Kp + ti * 4 + q) * Kp + tj * 4 + w] = acc[q][w];
+            for (int w = 0; w < 4; ++w) {
+                const int e = (ti * 4 + q) * KP + tj * 4 + w;
+                part[(size_t)blockIdx.x * KP * KP + e] = ksm[e];
+            }
 }
 
-// out = sum over blocks of part, in block order; entry (i, j) and (j, i) both take the computed
-// upper entry (min, max), so the result is exactly symmetric.
-__global__ void kk_gram_sum(int G, int Kp, const double* part, double* __restrict__ out) {
-    for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < Kp * Kp; e += gridDim.x * blockDim.x) {
-        const int i = e / Kp, j = e - (e / Kp) * Kp;
-        const int a = min(i, j), b = max(i, j);
-        double s = 0.0;
-        for (int g = 0; g < G; ++g) s += part[((size_t)g * Kp + a) * Kp + b];
-        out[e] = s;
-    }
+// out = sum over blocks of part, a warp per entry (each lane its blocks in order, then a fixed tree);
+// entry (i, j) and (j, i) both take the computed upper entry (min, max), so the result is exactly
+// symmetric.
+__global__ void __launch_bounds__(256) kk_gram_sum(int G, int Kp, const double* part, double* __restrict__ out) {
+    const int e = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    if (e >= Kp * Kp) return;
+    const int i = e / Kp, j = e - i * Kp;
+    const double* p = part + (size_t)min(i, j) * Kp + max(i, j);
+    double s = 0.0;
+#pragma unroll 8
+    for (int g = lane; g < G; g += 32) s += p[(size_t)g * Kp * Kp];
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (lane == 0) out[e] = s;
 }
 
 // Y = S^{-1} W on the leading K x K blocks by Cholesky S = L L^T (one block; S symmetric).  out is
@@ -914,91 +1105,115 @@ __global__ void __launch_bounds__(KK_TPB) kk_solve(int K, int Kp, const double* 
     if (t == 0 && bad) flag[KF_BAD] = 1;
 }
 
-// Entry k of a row held across the warp (lane k mod 32 of register k / 32).
-template <int J>
+// Entry k of a row held across its lanes.
+template <int J, int R>
 __device__ __forceinline__ double kk_lane(const double (&v)[J], int k) {
-    if constexpr (J == 1) return __shfl_sync(0xffffffffu, v[0], k & 31);
-    else return __shfl_sync(0xffffffffu, k < 32 ? v[0] : v[1], k & 31);
+    if constexpr (R > 1) return __shfl_sync(0xffffffffu, v[0], Cols<J, R>::sub() * Cols<J, R>::W + k);
+    else if constexpr (J == 1) return __shfl_sync(0xffffffffu, v[0], k);
+    else return __shfl_sync(0xffffffffu, k % J ? v[1] : v[0], k / J);
 }
 
-// X += P alpha and R -= Q alpha (warp per row, lanes over columns, alpha in shared memory), and
-// per block the column sums of r_ij^2 in warp order into part[block][Kp].
-template <int J>
-__global__ void __launch_bounds__(BTPB) kk_update(int n, int Kp, int K, double* __restrict__ X, double* __restrict__ R,
-                                                  const double* P, const double* Q,
-                                                  const double* alpha, double* __restrict__ part,
-                                                  const int* flag) {
+// Per block, the column sums of v over the lanes in warp order, into part[block][KP].
+template <int J, int R>
+__device__ __forceinline__ void kk_block_cols(const double (&v)[J], double* ws, double* __restrict__ part) {
+    using L = Cols<J, R>;
+    const int w = threadIdx.x >> 5;
+#pragma unroll
+    for (int m = 0; m < J; ++m) ws[(w * R + L::sub()) * L::KP + L::col() + m] = v[m];
+    __syncthreads();
+    for (int c = threadIdx.x; c < L::KP; c += BTPB) {
+        double s = 0.0;
+        for (int q = 0; q < BWARPS * R; ++q) s += ws[q * L::KP + c];
+        part[(size_t)blockIdx.x * L::KP + c] = s;
+    }
+}
+
+// X += P alpha and R -= Q alpha (alpha in shared memory), and per block the column sums of r_ij^2.
+template <int J, int R>
+__global__ void __launch_bounds__(BTPB) kk_update(int n, int K, double* __restrict__ X, double* __restrict__ Rv, float* r32,
+                                                  const double* P, const double* Q, const double* alpha,
+                                                  double* __restrict__ part, const int* flag) {
+    using L = Cols<J, R>;
+    constexpr int Kp = L::KP;
     if (flag[KF_BAD]) return;              // a K x K solve failed: keep the last good iterate
     extern __shared__ double ksm[];
     double* al = ksm;                      // [Kp][Kp]
-    double* ws = ksm + Kp * Kp;            // [BWARPS][Kp]
-    for (int e = threadIdx.x; e < Kp * Kp; e += blockDim.x) al[e] = alpha[e];
+    double* ws = ksm + Kp * Kp;            // [BWARPS R][Kp]
+    for (int e = threadIdx.x; e < Kp * Kp; e += BTPB) al[e] = alpha[e];
     __syncthreads();
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     double rr[J];
-#pragma unroll
-    for (int m = 0; m < J; ++m) rr[m] = 0.0;
-    for (int i = blockIdx.x * BWARPS + w; i < n; i += gridDim.x * BWARPS) {
-        const size_t o = (size_t)i * Kp + lane;
+    zero(rr);
+    for (int i0 = (blockIdx.x * BWARPS + (threadIdx.x >> 5)) * R; i0 < n; i0 += gridDim.x * BWARPS * R) {
+        const bool on = i0 + L::sub() < n;
+        const size_t o = L::at(i0 + L::sub());
         double p[J], q[J], dx[J], dr[J];
-#pragma unroll
-        for (int m = 0; m < J; ++m) {
-            p[m] = P[o + 32 * m];
-            q[m] = Q[o + 32 * m];
-            dx[m] = 0.0;
-            dr[m] = 0.0;
+        zero(p);
+        zero(q);
+        zero(dx);
+        zero(dr);
+        if (on) {
+            ldv<J>(P + o, p);
+            ldv<J>(Q + o, q);
         }
         for (int k = 0; k < K; ++k) {
-            const double pk = kk_lane<J>(p, k), qk = kk_lane<J>(q, k);
+            const double pk = kk_lane<J, R>(p, k), qk = kk_lane<J, R>(q, k);
+            double a[J];
+            ldv<J>(al + k * Kp + L::col(), a);
 #pragma unroll
             for (int m = 0; m < J; ++m) {
-                const double a = al[k * Kp + lane + 32 * m];
-                dx[m] = __fma_rn(pk, a, dx[m]);
-                dr[m] = __fma_rn(qk, a, dr[m]);
+                dx[m] = __fma_rn(pk, a[m], dx[m]);
+                dr[m] = __fma_rn(qk, a[m], dr[m]);
             }
         }
+        if (!on) continue;
+        double x[J], r[J];
+        ldv<J>(X + o, x);
+        ldv<J>(Rv + o, r);
 #pragma unroll
         for (int m = 0; m < J; ++m) {
-            X[o + 32 * m] += dx[m];
-            const double r = R[o + 32 * m] - dr[m];
-            R[o + 32 * m] = r;
-            rr[m] = __fma_rn(r, r, rr[m]);
+            x[m] += dx[m];
+            r[m] -= dr[m];
+            rr[m] = __fma_rn(r[m], r[m], rr[m]);
         }
+        stv<J>(X + o, x);
+        stv<J>(Rv + o, r);
+        st_r32<J>(r32, o, r);
     }
-#pragma unroll
-    for (int m = 0; m < J; ++m) ws[w * Kp + lane + 32 * m] = rr[m];
-    __syncthreads();
-    for (int c = threadIdx.x; c < Kp; c += blockDim.x) {
-        double s = 0.0;
-        for (int v = 0; v < BWARPS; ++v) s += ws[v * Kp + c];
-        part[(size_t)blockIdx.x * Kp + c] = s;
-    }
+    kk_block_cols<J, R>(rr, ws, part);
 }
 
-// P = Z + P beta, in place (a warp reads its whole row of P before writing it).
-template <int J, class ZT>
-__global__ void __launch_bounds__(BTPB) kk_pupdate(int n, int Kp, int K, const ZT* Z, double* __restrict__ P,
-                                                   const double* beta, const int* flag) {
+// P = Z + P beta, in place (a row is read by its own lanes before they write it).
+template <int J, int R, class ZT>
+__global__ void __launch_bounds__(BTPB) kk_pupdate(int n, int K, const ZT* Z, double* __restrict__ P, const double* beta,
+                                                   const int* flag) {
+    using L = Cols<J, R>;
+    constexpr int Kp = L::KP;
     if (flag[KF_BAD]) return;
     extern __shared__ double ksm[];
-    for (int e = threadIdx.x; e < Kp * Kp; e += blockDim.x) ksm[e] = beta[e];
+    for (int e = threadIdx.x; e < Kp * Kp; e += BTPB) ksm[e] = beta[e];
     __syncthreads();
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    for (int i = blockIdx.x * BWARPS + w; i < n; i += gridDim.x * BWARPS) {
-        const size_t o = (size_t)i * Kp + lane;
-        double p[J], acc[J];
-#pragma unroll
-        for (int m = 0; m < J; ++m) {
-            p[m] = P[o + 32 * m];
-            acc[m] = 0.0;
+    for (int i0 = (blockIdx.x * BWARPS + (threadIdx.x >> 5)) * R; i0 < n; i0 += gridDim.x * BWARPS * R) {
+        const bool on = i0 + L::sub() < n;
+        const size_t o = L::at(i0 + L::sub());
+        double p[J], z[J], acc[J];
+        zero(p);
+        zero(z);
+        zero(acc);
+        if (on) {
+            ldv<J>(P + o, p);
+            ldv<J>(Z + o, z);
         }
         for (int k = 0; k < K; ++k) {
-            const double pk = kk_lane<J>(p, k);
+            const double pk = kk_lane<J, R>(p, k);
+            double b[J];
+            ldv<J>(ksm + k * Kp + L::col(), b);
 #pragma unroll
-            for (int m = 0; m < J; ++m) acc[m] = __fma_rn(pk, ksm[k * Kp + lane + 32 * m], acc[m]);
+            for (int m = 0; m < J; ++m) acc[m] = __fma_rn(pk, b[m], acc[m]);
         }
+        if (!on) continue;
 #pragma unroll
-        for (int m = 0; m < J; ++m) P[o + 32 * m] = (double)Z[o + 32 * m] + acc[m];
+        for (int m = 0; m < J; ++m) z[m] += acc[m];
+        stv<J>(P + o, z);
     }
 }
 
@@ -1008,62 +1223,57 @@ __global__ void kk_copy(int64_t nk, const ZT* z, double* __restrict__ p) {
         p[e] = (double)z[e];
 }
 
-// Q = A P with A in CSR (warp per row, lanes over columns).
-template <int J>
-__global__ void __launch_bounds__(BTPB) kk_spmm(int n, int Kp, const int* __restrict__ ptr, const int* __restrict__ col,
-                                                const double* __restrict__ val, const double* P,
-                                                double* __restrict__ Q) {
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    for (int i = blockIdx.x * BWARPS + w; i < n; i += gridDim.x * BWARPS) {
-        double acc[J];
-#pragma unroll
-        for (int m = 0; m < J; ++m) acc[m] = 0.0;
-        for (int e = ptr[i]; e < ptr[i + 1]; ++e) {
-            const double a = val[e];
-            const size_t o = (size_t)col[e] * Kp + lane;
-#pragma unroll
-            for (int m = 0; m < J; ++m) acc[m] = __fma_rn(a, P[o + 32 * m], acc[m]);
-        }
-#pragma unroll
-        for (int m = 0; m < J; ++m) Q[(size_t)i * Kp + lane + 32 * m] = acc[m];
-    }
+// Q = A P with A in CSR.
+template <int J, int R>
+__global__ void __launch_bounds__(BTPB) kk_spmm(int n, const int* __restrict__ ptr, const int* __restrict__ col,
+                                                const double* __restrict__ val, const double* P, double* __restrict__ Q) {
+    using L = Cols<J, R>;
+    const int i = (blockIdx.x * BWARPS + (threadIdx.x >> 5)) * R + L::sub();
+    if (i >= n) return;
+    double acc[J];
+    zero(acc);
+    const int e0 = ptr[i];
+    brow<J, R, 4>(col, val, BRow{e0, ptr[i + 1] - e0, 0, 1}, 0, 1, P, acc);
+    stv<J>(Q + L::at(i), acc);
 }
 
-// Per block, the column sums of v_ij^2 in warp order into part[block][Kp].
-template <int J>
-__global__ void __launch_bounds__(BTPB) kk_colnorm(int n, int Kp, const double* V, double* __restrict__ part) {
-    __shared__ double ws[BWARPS * 128];
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    double s[J];
+// R = B (and its copy in the preconditioner's precision), X = 0, and per block the column sums of b_ij^2.
+template <int J, int R>
+__global__ void __launch_bounds__(BTPB) kk_init(int n, const double* B, double* __restrict__ X, double* __restrict__ Rv,
+                                                float* r32, double* __restrict__ part) {
+    using L = Cols<J, R>;
+    __shared__ double ws[BWARPS * R * L::KP];
+    double s[J], z[J];
+    zero(s);
+    zero(z);
+    for (int i = (blockIdx.x * BWARPS + (threadIdx.x >> 5)) * R + L::sub(); i < n; i += gridDim.x * BWARPS * R) {
+        double v[J];
+        ldv<J>(B + L::at(i), v);
+        stv<J>(Rv + L::at(i), v);
+        stv<J>(X + L::at(i), z);
+        st_r32<J>(r32, L::at(i), v);
 #pragma unroll
-    for (int m = 0; m < J; ++m) s[m] = 0.0;
-    for (int i = blockIdx.x * BWARPS + w; i < n; i += gridDim.x * BWARPS)
-#pragma unroll
-        for (int m = 0; m < J; ++m) {
-            const double v = V[(size_t)i * Kp + lane + 32 * m];
-            s[m] = __fma_rn(v, v, s[m]);
-        }
-#pragma unroll
-    for (int m = 0; m < J; ++m) ws[w * Kp + lane + 32 * m] = s[m];
-    __syncthreads();
-    for (int c = threadIdx.x; c < Kp; c += blockDim.x) {
-        double t = 0.0;
-        for (int v = 0; v < BWARPS; ++v) t += ws[v * Kp + c];
-        part[(size_t)blockIdx.x * Kp + c] = t;
+        for (int m = 0; m < J; ++m) s[m] = __fma_rn(v[m], v[m], s[m]);
     }
+    kk_block_cols<J, R>(s, ws, part);
 }
 
-// One block.  Column norms from the partials (block order).  init: bnorm_k = ||b_k||, a zero column
-// sets KF_BAD.  Otherwise res_k = ||r_k|| / ||b_k||; KF_DONE = 1 when every column is below tol,
-// and a residual that is not finite sets KF_BAD.
-__global__ void kk_check(int G, int Kp, int K, const double* part, double* __restrict__ vec, double tol,
-                         int init, int* flag) {
+// One block of 8 warps, a warp per column.  Column norms from the partials (each lane its blocks in
+// order, then a fixed tree).  init: bnorm_k = ||b_k||, a zero column sets KF_BAD.  Otherwise res_k =
+// ||r_k|| / ||b_k||; KF_DONE = 1 when every column is below tol, and a residual that is not finite
+// sets KF_BAD.
+__global__ void __launch_bounds__(256) kk_check(int G, int Kp, int K, const double* part, double* __restrict__ vec, double tol,
+                                                int init, int* flag) {
     __shared__ int all;
     if (threadIdx.x == 0) all = 1;
     __syncthreads();
-    for (int c = threadIdx.x; c < K; c += blockDim.x) {
+    const int lane = threadIdx.x & 31;
+    for (int c = threadIdx.x >> 5; c < K; c += 8) {
         double s = 0.0;
-        for (int g = 0; g < G; ++g) s += part[(size_t)g * Kp + c];
+#pragma unroll 8
+        for (int g = lane; g < G; g += 32) s += part[(size_t)g * Kp + c];
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        if (lane != 0) continue;
         const double nrm = sqrt(s);
         if (init) {
             vec[KV_BNORM * Kp + c] = nrm;
@@ -1083,68 +1293,76 @@ template <class VT> VT* bx(Batched& B, int l) { return (VT*)B.lx[l].p; }
 template <class VT> VT* bf(Batched& B, int l) { return (VT*)B.lf[l].p; }
 template <class VT> VT* br(Batched& B, int l) { return (VT*)B.lr[l].p; }
 
-template <int J, class FT, class VT>
-void brec_gs(Level& L, int c, const FT* f, VT* x, int Kp, cudaStream_t s) {
+// One colour of a level; from_zero: in a forward sweep from a zero guess.
+template <int J, int R, class VT>
+void brec_gs(Level& L, int c, const VT* f, VT* x, cudaStream_t s, bool from_zero) {
     const int s0 = L.S.seg[c] * L.S.C, s1 = L.S.seg[c + 1] * L.S.C;
     if (s1 <= s0) return;
-    const int g = rows_grid(s1 - s0);
+    const int g = rows_grid<R>(s1 - s0);
     if (L.S.ndiag) {
         bwith_nd(L.S.ndiag, [&](auto nd) {
             constexpr int ND = decltype(nd)::value;
             if constexpr (std::is_same<VT, double>::value)
-                blaunch(kb_gs_dia<J, double, double, FT, VT, ND>, g, BTPB, s,
-                        bdview(L.S, L.n, (const double*)L.S.dval.p, (const double*)L.S.dinv.p, false), s0, s1, f, x, Kp);
+                blaunch(kb_gs_dia<J, R, double, double, VT, ND>, rows_grid<R>(s1 - s0, DWARPS), DTPB, s,
+                        bdview(L.S, L.n, (const double*)L.S.dval.p, (const double*)L.S.dinv.p, false), s0, s1, f, x);
             else
-                blaunch(kb_gs_dia<J, float, float, FT, VT, ND>, g, BTPB, s,
-                        bdview(L.S, L.n, (const float*)L.S.dval32.p, (const float*)L.S.dinv32.p, false), s0, s1, f, x, Kp);
+                blaunch(kb_gs_dia<J, R, float, float, VT, ND>, rows_grid<R>(s1 - s0, DWARPS), DTPB, s,
+                        bdview(L.S, L.n, (const float*)L.S.dval32.p, (const float*)L.S.dinv32.p, false), s0, s1, f, x);
         });
         return;
     }
-    // long rows in a small colour group: a block per row (kb_gs_wide), else a warp per row
-    const bool wide = L.A.nnz >= (int64_t)16 * L.n && (s1 - s0) <= 16384;
-    if (wide) {
-        if constexpr (std::is_same<VT, double>::value)
-            blaunch(kb_gs_wide<J, double, double, FT, VT>, s1 - s0, BTPB, s, bview(L.S, (const double*)L.S.val.p, (const double*)L.S.dinv.p), s0, f, x, Kp);
-        else if (L.vt == VT_BF16)
-            blaunch(kb_gs_wide<J, __nv_bfloat16, float, FT, VT>, s1 - s0, BTPB, s, bview(L.S, (const __nv_bfloat16*)L.S.val16.p, (const float*)L.S.dinv32.p), s0, f, x, Kp);
-        else
-            blaunch(kb_gs_wide<J, float, float, FT, VT>, s1 - s0, BTPB, s, bview(L.S, (const float*)L.S.val32.p, (const float*)L.S.dinv32.p), s0, f, x, Kp);
-        return;
-    }
-    auto go = [&](auto longrows) {
-        constexpr bool LG = decltype(longrows)::value;
-        if constexpr (std::is_same<VT, double>::value)
-            blaunch(kb_gs<J, double, double, FT, VT, LG>, g, BTPB, s, bview(L.S, (const double*)L.S.val.p, (const double*)L.S.dinv.p), s0, s1, f, x, Kp);
-        else if (L.vt == VT_BF16)
-            blaunch(kb_gs<J, __nv_bfloat16, float, FT, VT, LG>, g, BTPB, s, bview(L.S, (const __nv_bfloat16*)L.S.val16.p, (const float*)L.S.dinv32.p), s0, s1, f, x, Kp);
-        else
-            blaunch(kb_gs<J, float, float, FT, VT, LG>, g, BTPB, s, bview(L.S, (const float*)L.S.val32.p, (const float*)L.S.dinv32.p), s0, s1, f, x, Kp);
+    const int* end = from_zero && L.skip_zeros() ? (const int*)L.S.cmid.p : (const int*)(L.S.cptr.p + 1);
+    auto go = [&](auto view) {
+        if (from_zero && !L.skip_zeros()) view.col = L.S.fcol.p;
+        using V = decltype(view);
+        using MT = std::remove_cv_t<std::remove_reference_t<decltype(*view.val)>>;
+        using DT = std::remove_cv_t<std::remove_reference_t<decltype(*view.diag)>>;
+        static_assert(std::is_same<V, BV<MT, DT>>::value, "");
+        // long rows: in a small colour group a block per R rows, else eight entries per batch
+        const bool lng = L.A.nnz >= (int64_t)16 * L.n;
+        if (lng && (s1 - s0) <= 16384) blaunch(kb_gs_wide<J, R, MT, DT, VT>, (s1 - s0 + 2 * R - 1) / (2 * R), 64 * WSPLIT, s, view, end, s0, s1, f, x);
+        else if (lng) blaunch(kb_gs<J, R, MT, DT, VT, 8>, g, BTPB, s, view, end, s0, s1, f, x);
+        else blaunch(kb_gs<J, R, MT, DT, VT, 4>, g, BTPB, s, view, end, s0, s1, f, x);
     };
-    if (L.A.nnz >= (int64_t)16 * L.n) go(std::true_type{});   // long rows: eight entries per batch
-    else go(std::false_type{});
+    if constexpr (std::is_same<VT, double>::value) go(bview(L.S, (const double*)L.S.val.p, (const double*)L.S.dinv.p));
+    else if (L.vt == VT_BF16) go(bview(L.S, (const __nv_bfloat16*)L.S.val16.p, (const float*)L.S.dinv32.p));
+    else go(bview(L.S, (const float*)L.S.val32.p, (const float*)L.S.dinv32.p));
 }
 
-template <int J, class FT, class VT>
-void brec_resid(Level& L, const FT* f, const VT* x, VT* r, int Kp, cudaStream_t s) {
-    const int g = std::min(rows_grid(L.S.nslots), 152 * 32);
+// r = f - A x after a forward sweep (from a zero guess with from_zero).  In FP64, on a red-black level
+// only the red rows are written: the black residual is zero up to rounding, and no transfer reads it.
+template <int J, int R, class VT>
+void brec_resid(Level& L, const VT* f, const VT* x, VT* r, cudaStream_t s, bool from_zero) {
+    from_zero = from_zero && L.skip_zeros();
     if (L.S.ndiag) {
+        const int s1 = L.red_black && L.skip_zeros() ? L.S.seg[1] * L.S.C : L.S.nslots;
         bwith_nd(L.S.ndiag, [&](auto nd) {
             constexpr int ND = decltype(nd)::value;
+            auto go = [&](auto view, auto zero) {
+                using MT = std::remove_cv_t<std::remove_reference_t<decltype(*view.val)>>;
+                blaunch(kb_resid_dia<J, R, MT, MT, VT, VT, ND, decltype(zero)::value>, rows_grid<R>(s1, DWARPS), DTPB, s, view, s1, f, x, r);
+            };
+            auto both = [&](auto view) {
+                if (from_zero && L.red_black) go(view, std::true_type{});
+                else go(view, std::false_type{});
+            };
             if constexpr (std::is_same<VT, double>::value)
-                blaunch(kb_resid_dia<J, double, double, FT, VT, VT, ND>, g, BTPB, s,
-                        bdview(L.S, L.n, (const double*)L.S.dval.p, (const double*)L.S.diag.p, false), f, x, r, Kp);
+                both(bdview(L.S, L.n, (const double*)L.S.dval.p, (const double*)L.S.diag.p, false));
             else
-                blaunch(kb_resid_dia<J, float, float, FT, VT, VT, ND>, g, BTPB, s,
-                        bdview(L.S, L.n, (const float*)L.S.dval32.p, (const float*)L.S.diag32.p, false), f, x, r, Kp);
+                both(bdview(L.S, L.n, (const float*)L.S.dval32.p, (const float*)L.S.diag32.p, false));
         });
         return;
     }
-    if constexpr (std::is_same<VT, double>::value)
-        blaunch(kb_resid<J, double, double, FT, VT, VT>, g, BTPB, s, bview(L.S, (const double*)L.S.val.p, (const double*)L.S.diag.p), L.S.nslots, f, x, r, Kp);
-    else if (L.vt == VT_BF16)
-        blaunch(kb_resid<J, __nv_bfloat16, float, FT, VT, VT>, g, BTPB, s, bview(L.S, (const __nv_bfloat16*)L.S.val16.p, (const float*)L.S.diag32.p), L.S.nslots, f, x, r, Kp);
-    else
-        blaunch(kb_resid<J, float, float, FT, VT, VT>, g, BTPB, s, bview(L.S, (const float*)L.S.val32.p, (const float*)L.S.diag32.p), L.S.nslots, f, x, r, Kp);
+    const int g = rows_grid<R>(L.S.nslots);
+    auto go = [&](auto view) {
+        using MT = std::remove_cv_t<std::remove_reference_t<decltype(*view.val)>>;
+        using DT = std::remove_cv_t<std::remove_reference_t<decltype(*view.diag)>>;
+        if (from_zero) blaunch(kb_resid_up<J, R, MT, DT, VT>, g, BTPB, s, view, (const int*)L.S.cmid.p, L.S.nslots, x, r);
+        else blaunch(kb_resid<J, R, MT, DT, VT>, g, BTPB, s, view, L.S.nslots, f, x, r);
+    };
+    if constexpr (std::is_same<VT, double>::value) go(bview(L.S, (const double*)L.S.val.p, (const double*)L.S.diag.p));
+    else if (L.vt == VT_BF16) go(bview(L.S, (const __nv_bfloat16*)L.S.val16.p, (const float*)L.S.diag32.p));
+    else go(bview(L.S, (const float*)L.S.val32.p, (const float*)L.S.diag32.p));
 }
 
 template <class VT>
@@ -1158,45 +1376,37 @@ template <> const double* bdnat<double>(const Level& L) { return L.dnat64.p; }
 template <> const float* bdnat<float>(const Level& L) { return L.dnat32.p; }
 
 // As rec_vcycle: with first_done the caller has applied the first colour step from the zero guess.
-template <int J, class FT, class VT>
-void brec_vcycle(Handle& h, int l, const FT* f, VT* x, bool zero_guess, cudaStream_t s, bool first_done = false) {
+template <int J, int R, class VT>
+void brec_vcycle(Handle& h, int l, const VT* f, VT* x, bool zero_guess, cudaStream_t s, bool first_done = false) {
     Batched& B = h.bat;
-    const int Kp = B.Kp;
     const int nl = (int)h.lev.size();
     Level& L = h.lev[l];
     if (l == nl - 1) {
         const VT* ai = std::is_same<VT, double>::value ? (const VT*)h.Ainv.p : (const VT*)h.Ainv32.p;
-        blaunch(kb_coarse<J, VT, FT, VT>, rows_grid(L.n), BTPB, s, L.n, ai, f, x, Kp);
+        if constexpr (std::is_same<VT, double>::value)
+            blaunch(kb_coarse<J, R, VT, VT, VT>, (L.n + R * CROWS - 1) / (R * CROWS), CWARPS * 32, s, L.n, ai, f, x);
+        else
+            blaunch(kb_coarse_seq<J, R, VT, VT, VT>, (L.n + CWARPS * R * SROWS - 1) / (CWARPS * R * SROWS), CWARPS * 32, s, L.n,
+                    ai, f, x);
         return;
     }
-    int c0 = 0;
-    if (first_done) {
-        c0 = 1;
-    } else if (zero_guess) {
-        blaunch(kb_zero_first<FT, VT>, 2048, 256, s, L.n, Kp, f, (const int*)L.colour.p, bdnat<VT>(L), x);
-        c0 = 1;
-    }
-    for (int c = c0; c < L.ncolours; ++c) brec_gs<J>(L, c, f, x, Kp, s);
-    brec_resid<J>(L, f, (const VT*)x, br<VT>(B, l), Kp, s);
+    if (zero_guess && !first_done)
+        blaunch(kb_first<J, R, VT>, rows_grid<R>(L.n, DWARPS), DTPB, s, L.n, f, (const int*)L.colour.p, bdnat<VT>(L), x);
+    for (int c = zero_guess ? 1 : 0; c < L.ncolours; ++c) brec_gs<J, R>(L, c, f, x, s, zero_guess);
+    brec_resid<J, R>(L, f, (const VT*)x, br<VT>(B, l), s, zero_guess);
     Level& C = h.lev[l + 1];
-    if (l + 1 == nl - 1) {
-        blaunch(kb_apply<J, VT, VT>, std::min(rows_grid(L.SR.nslots), 152 * 32), BTPB, s, bfull<VT>(L.SR), L.SR.nslots,
-                (const VT*)br<VT>(B, l), bf<VT>(B, l + 1), bx<VT>(B, l + 1), Kp);
-        brec_vcycle<J, VT, VT>(h, l + 1, bf<VT>(B, l + 1), bx<VT>(B, l + 1), false, s);
-    } else {
-        blaunch(kb_restrict_first<J, VT, VT>, std::min(rows_grid(L.SR.nslots), 152 * 32), BTPB, s, bfull<VT>(L.SR),
-                L.SR.nslots, (const VT*)br<VT>(B, l), bf<VT>(B, l + 1), bx<VT>(B, l + 1), (const int*)C.colour.p,
-                bdnat<VT>(C), Kp);
-        brec_vcycle<J, VT, VT>(h, l + 1, bf<VT>(B, l + 1), bx<VT>(B, l + 1), true, s, true);
-    }
-    blaunch(kb_prolong<J, VT, VT>, std::min(rows_grid(L.SP.nslots), 152 * 32), BTPB, s, bfull<VT>(L.SP), L.SP.nslots,
-            (const VT*)bx<VT>(B, l + 1), x, Kp);
-    for (int c = L.ncolours - 1; c >= 0; --c) brec_gs<J>(L, c, f, x, Kp, s);
+    const bool last = l + 1 == nl - 1;
+    blaunch(kb_restrict<J, R, VT, VT>, rows_grid<R>(L.SR.nslots), BTPB, s, bfull<VT>(L.SR),
+            L.red_black && L.skip_zeros() ? (const int*)L.SR.cmid.p : (const int*)(L.SR.cptr.p + 1), L.SR.nslots, (const VT*)br<VT>(B, l),
+            bf<VT>(B, l + 1), last ? (VT*)nullptr : bx<VT>(B, l + 1), (const int*)C.colour.p, bdnat<VT>(C));
+    brec_vcycle<J, R, VT>(h, l + 1, bf<VT>(B, l + 1), bx<VT>(B, l + 1), !last, s, !last);
+    const int ps = L.red_black ? L.SP.seg[1] * L.SP.C : L.SP.nslots;
+    blaunch(kb_prolong<J, R, VT, VT>, rows_grid<R>(ps), BTPB, s, bfull<VT>(L.SP), ps, (const VT*)bx<VT>(B, l + 1), x);
+    for (int c = L.ncolours - 1; c >= 0; --c) brec_gs<J, R>(L, c, f, x, s, false);
 }
 
-template <int J, class TT, class VT>
-void brec_ic(Handle& h, const TT* t, VT* y, VT* w, VT* zadd, cudaStream_t s) {
-    const int Kp = h.bat.Kp;
+template <int J, int R, class VT>
+void brec_ic(Handle& h, const VT* t, VT* y, VT* w, VT* zadd, cudaStream_t s) {
     BV<VT, VT> lv, uv;
     if constexpr (std::is_same<VT, double>::value) {
         lv = bview(h.L, (const double*)h.L.val.p, (const double*)nullptr);
@@ -1207,43 +1417,42 @@ void brec_ic(Handle& h, const TT* t, VT* y, VT* w, VT* zadd, cudaStream_t s) {
     }
     for (int g = 0; g + 1 < (int)h.L.seg.size(); ++g) {
         const int s0 = h.L.seg[g] * h.L.C, s1 = h.L.seg[g + 1] * h.L.C;
-        blaunch(kb_lsolve<J, VT, TT, VT>, rows_grid(s1 - s0), BTPB, s, lv, s0, s1, t, y, Kp);
+        blaunch(kb_lsolve<J, R, VT, VT>, rows_grid<R>(s1 - s0), BTPB, s, lv, s0, s1, t, y);
     }
     for (int g = 0; g + 1 < (int)h.U.seg.size(); ++g) {
         const int s0 = h.U.seg[g] * h.U.C, s1 = h.U.seg[g + 1] * h.U.C;
-        blaunch(kb_usolve<J, VT, VT>, rows_grid(s1 - s0), BTPB, s, uv, s0, s1, (const VT*)y, w, zadd, Kp);
+        blaunch(kb_usolve<J, R, VT, VT>, rows_grid<R>(s1 - s0), BTPB, s, uv, s0, s1, (const VT*)y, w, zadd);
     }
 }
 
-template <int J, class VT>
-void brec_precond(Handle& h, int which, const double* r, VT* z, cudaStream_t s) {
+template <int J, int R, class VT>
+void brec_precond(Handle& h, int which, const VT* r, VT* z, cudaStream_t s) {
     Batched& B = h.bat;
-    const int Kp = B.Kp;
     VT* t = (VT*)B.t.p;
     VT* y = (VT*)B.y.p;
     const Sell& A = h.Anat;
     auto fine_resid = [&]() {
-        const int g = std::min(rows_grid(A.nslots), 152 * 32);
+        const int g = rows_grid<R>(A.nslots);
         if (A.ndiag) {
             bwith_nd(A.ndiag, [&](auto nd) {
                 constexpr int ND = decltype(nd)::value;
                 if constexpr (std::is_same<VT, double>::value)
-                    blaunch(kb_resid_dia<J, double, double, double, VT, VT, ND>, g, BTPB, s,
-                            bdview(A, h.n, (const double*)A.dval.p, (const double*)A.diag.p, true), r, (const VT*)z, t, Kp);
+                    blaunch(kb_resid_dia<J, R, double, double, VT, VT, ND, false>, rows_grid<R>(A.nslots, DWARPS), DTPB, s,
+                            bdview(A, h.n, (const double*)A.dval.p, (const double*)A.diag.p, true), A.nslots, r, (const VT*)z, t);
                 else
-                    blaunch(kb_resid_dia<J, float, float, double, VT, VT, ND>, g, BTPB, s,
-                            bdview(A, h.n, (const float*)A.dval32.p, (const float*)A.diag32.p, true), r, (const VT*)z, t, Kp);
+                    blaunch(kb_resid_dia<J, R, float, float, VT, VT, ND, false>, rows_grid<R>(A.nslots, DWARPS), DTPB, s,
+                            bdview(A, h.n, (const float*)A.dval32.p, (const float*)A.diag32.p, true), A.nslots, r, (const VT*)z, t);
             });
             return;
         }
         if constexpr (std::is_same<VT, double>::value)
-            blaunch(kb_resid<J, double, double, double, VT, VT>, g, BTPB, s, bview(A, (const double*)A.val.p, (const double*)A.diag.p), A.nslots, r, (const VT*)z, t, Kp);
+            blaunch(kb_resid<J, R, double, double, VT>, g, BTPB, s, bview(A, (const double*)A.val.p, (const double*)A.diag.p), A.nslots, r, (const VT*)z, t);
         else
-            blaunch(kb_resid<J, float, float, double, VT, VT>, g, BTPB, s, bview(A, (const float*)A.val32.p, (const float*)A.diag32.p), A.nslots, r, (const VT*)z, t, Kp);
+            blaunch(kb_resid<J, R, float, float, VT>, g, BTPB, s, bview(A, (const float*)A.val32.p, (const float*)A.diag32.p), A.nslots, r, (const VT*)z, t);
     };
     switch (which) {
         case CPC_PRECOND_BCO:
-            brec_vcycle<J, double, VT>(h, 0, r, z, true, s);
+            brec_vcycle<J, R, VT>(h, 0, r, z, true, s);
             if (h.ic_rb && h.lev[0].S.ndiag) {                   // step (2): black rows, one pass
                 const Sell& S0 = h.lev[0].S;
                 const int s0 = S0.seg[1] * S0.C, s1 = S0.seg[2] * S0.C;
@@ -1251,38 +1460,43 @@ void brec_precond(Handle& h, int which, const double* r, VT* z, cudaStream_t s) 
                     bwith_nd(S0.ndiag, [&](auto nd) {
                         constexpr int ND = decltype(nd)::value;
                         if constexpr (std::is_same<VT, double>::value)
-                            blaunch(kb_bco_black_dia<J, double, double, VT, ND>, rows_grid(s1 - s0), BTPB, s,
+                            blaunch(kb_bco_black_dia<J, R, double, double, VT, ND>, rows_grid<R>(s1 - s0, DWARPS), DTPB, s,
                                     bdview(S0, h.n, (const double*)S0.dval.p, (const double*)S0.diag.p, false), s0, s1,
-                                    r, (const VT*)h.ic_uinv64.p, z, Kp);
+                                    r, (const VT*)h.ic_uinv64.p, z);
                         else
-                            blaunch(kb_bco_black_dia<J, float, float, VT, ND>, rows_grid(s1 - s0), BTPB, s,
+                            blaunch(kb_bco_black_dia<J, R, float, float, VT, ND>, rows_grid<R>(s1 - s0, DWARPS), DTPB, s,
                                     bdview(S0, h.n, (const float*)S0.dval32.p, (const float*)S0.diag32.p, false), s0,
-                                    s1, r, (const VT*)h.ic_uinv32.p, z, Kp);
+                                    s1, r, (const VT*)h.ic_uinv32.p, z);
                     });
             } else {
                 fine_resid();
-                brec_ic<J, VT, VT>(h, t, y, t, z, s);
+                brec_ic<J, R, VT>(h, t, y, t, z, s);
             }
-            brec_vcycle<J, double, VT>(h, 0, r, z, false, s);
+            brec_vcycle<J, R, VT>(h, 0, r, z, false, s);
             break;
         case CPC_PRECOND_AMG:
-            brec_vcycle<J, double, VT>(h, 0, r, z, true, s);
-            brec_vcycle<J, double, VT>(h, 0, r, z, false, s);
+            brec_vcycle<J, R, VT>(h, 0, r, z, true, s);
+            brec_vcycle<J, R, VT>(h, 0, r, z, false, s);
             break;
         case CPC_PRECOND_IC0:
-            brec_ic<J, double, VT>(h, r, y, z, (VT*)nullptr, s);
+            brec_ic<J, R, VT>(h, r, y, z, (VT*)nullptr, s);
             break;
         case CPC_PRECOND_BHAT:
-            brec_vcycle<J, double, VT>(h, 0, r, z, true, s);
-            brec_vcycle<J, double, VT>(h, 0, r, z, false, s);
-            brec_ic<J, double, VT>(h, r, y, t, z, s);
+            brec_vcycle<J, R, VT>(h, 0, r, z, true, s);
+            brec_vcycle<J, R, VT>(h, 0, r, z, false, s);
+            brec_ic<J, R, VT>(h, r, y, t, z, s);
             break;
         default:
             fail(CPC_EINVAL, "batched solve supports B_co, AMG, IC(0) and B^");
     }
 }
 
-template <int J, class VT>
+// The residual as the preconditioner reads it.
+template <class VT> const VT* bres(const Batched& B);
+template <> const double* bres<double>(const Batched& B) { return B.r.p; }
+template <> const float* bres<float>(const Batched& B) { return B.r32.p; }
+
+template <int J, int R, class VT>
 void brec_loop(Handle& h, cudaGraph_t g, cudaStream_t cs, cudaGraphNode_t* dep, size_t ndep, cudaGraphNode_t* out_node) {
     Batched& B = h.bat;
     const int Kp = B.Kp;
@@ -1299,28 +1513,30 @@ void brec_loop(Handle& h, cudaGraph_t g, cudaStream_t cs, cudaGraphNode_t* dep, 
     CPC_CK(cudaStreamBeginCaptureToGraph(cs, body, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal));
     blaunch(kb_guard, 1, 32, cs, cond);
     VT* z = (VT*)B.z.p;
-    brec_precond<J, VT>(h, h.opt.precond, B.r.p, z, cs);
-    const int vg = std::min(rows_grid(n), 152 * 8);
-    blaunch(kb_rz<J, VT>, vg, BTPB, cs, n, Kp, (const double*)B.r.p, (const VT*)z, B.partial.p, h.counter.p + 1, B.S.p);
-    blaunch(kb_p<J, VT>, vg, BTPB, cs, n, Kp, (const VT*)z, B.p.p, (const double*)B.S.p);
+    brec_precond<J, R, VT>(h, h.opt.precond, bres<VT>(B), z, cs);
+    const int vg = vgrid<R>(n);
+    const bool ord = !std::is_same<VT, double>::value;
+    blaunch(kb_rz<J, R, VT>, vg, VTPB, cs, n, (const double*)B.r.p, (const VT*)z, B.partial.p, h.counter.p + 1, B.S.p, ord);
+    blaunch(kb_p<J, R, VT>, vg, VTPB, cs, n, (const VT*)z, B.p.p, (const double*)B.S.p);
     const Sell& A = h.Anat;
     if (A.ndiag)
         bwith_nd(A.ndiag, [&](auto nd) {
-            blaunch(kb_spmv_pq_dia<J, decltype(nd)::value>, std::min(rows_grid(A.nslots), 152 * 8), BTPB, cs,
-                    bdview(A, n, (const double*)A.dval.p, (const double*)A.diag.p, true), Kp, (const double*)B.p.p,
-                    B.q.p, B.partial.p, h.counter.p + 1, B.S.p);
+            blaunch(kb_spmv_pq_dia<J, R, decltype(nd)::value>, vgrid<R>(A.nslots), VTPB, cs,
+                    bdview(A, n, (const double*)A.dval.p, (const double*)A.diag.p, true), (const double*)B.p.p,
+                    B.q.p, B.partial.p, h.counter.p + 1, B.S.p, ord);
         });
     else
-        blaunch(kb_spmv_pq<J>, std::min(rows_grid(A.nslots), 152 * 8), BTPB, cs, bview(A, (const double*)A.val.p, (const double*)A.diag.p),
-                A.nslots, Kp, (const double*)B.p.p, B.q.p, B.partial.p, h.counter.p + 1, B.S.p);
-    blaunch(kb_update<J>, vg, BTPB, cs, n, Kp, B.x.p, B.r.p, (const double*)B.p.p, (const double*)B.q.p, B.partial.p,
-            h.counter.p + 1, B.S.p);
+        blaunch(kb_spmv_pq<J, R>, vgrid<R>(A.nslots), VTPB, cs, bview(A, (const double*)A.val.p, (const double*)A.diag.p),
+                A.nslots, (const double*)B.p.p, B.q.p, B.partial.p, h.counter.p + 1, B.S.p, ord);
+    blaunch(kb_update<J, R>, vg, VTPB, cs, n, B.x.p, B.r.p, B.r32.p, (const double*)B.p.p, (const double*)B.q.p, B.partial.p,
+            h.counter.p + 1, B.S.p, ord);
     blaunch(kb_any_active, 1, 32, cs, Kp, (const double*)B.S.p, cond);
     CPC_CK(cudaStreamEndCapture(cs, &body));
 }
 
-// One graph: pack B, init, while(any active) { iteration }, [adjoint: sources, init, while {...}].
-template <int J, class VT>
+// One graph: init, while(any active) { iteration }, [adjoint: sources, init, while {...}].  It works on the
+// internal block vectors alone, so calls with other buffers replay it.
+template <int J, int R, class VT>
 void build_batched_graph(Handle& h, bool with_adjoint) {
     Batched& B = h.bat;
     const int Kp = B.Kp;
@@ -1330,7 +1546,8 @@ void build_batched_graph(Handle& h, bool with_adjoint) {
     struct SG { cudaStream_t s; ~SG() { cudaStreamDestroy(s); } } sg{cs};
     cudaGraph_t g;
     CPC_CK(cudaGraphCreate(&g, 0));
-    const int vg = std::min(rows_grid(n), 152 * 8);
+    const int vg = vgrid<R>(n);
+    const bool ord = !std::is_same<VT, double>::value;
     auto capture_into = [&](cudaGraphNode_t* deps, size_t ndeps, auto&& body) -> std::vector<cudaGraphNode_t> {
         std::vector<cudaGraphNode_t> before;
         size_t nn = 0;
@@ -1356,27 +1573,20 @@ void build_batched_graph(Handle& h, bool with_adjoint) {
         return leaves;
     };
     auto l1 = capture_into(nullptr, 0, [&] {
-        blaunch(kb_pack, 2048, 256, cs, n, B.K, Kp, (const double*)B.user_b, B.b.p);
-        blaunch(kb_init<J>, vg, BTPB, cs, n, Kp, (const double*)B.b.p, B.x.p, B.r.p, B.partial.p, h.counter.p + 1, B.S.p);
+        blaunch(kb_init<J, R>, vg, VTPB, cs, n, (const double*)B.b.p, B.x.p, B.r.p, B.r32.p, B.partial.p, h.counter.p + 1, B.S.p, ord);
     });
     cudaGraphNode_t w1;
-    brec_loop<J, VT>(h, g, cs, l1.data(), l1.size(), &w1);
-    cudaGraphNode_t tail = w1;
+    brec_loop<J, R, VT>(h, g, cs, l1.data(), l1.size(), &w1);
     if (with_adjoint) {
         auto l2 = capture_into(&w1, 1, [&] {
             blaunch(kb_adjoint_rhs, 2048, 256, cs, (int64_t)n * Kp, B.b.p, (const double*)B.x.p, B.xfwd.p);
-            blaunch(kb_unpack, 2048, 256, cs, n, B.K, Kp, (const double*)B.xfwd.p, B.user_x);
             CPC_CK(cudaMemcpyAsync(B.kfwd.p, B.S.p + (size_t)S_K * Kp, sizeof(double) * Kp, cudaMemcpyDeviceToDevice, cs));
             CPC_CK(cudaMemcpyAsync(B.kfwd.p + Kp, B.S.p + (size_t)S_STATUS * Kp, sizeof(double) * Kp, cudaMemcpyDeviceToDevice, cs));
-            blaunch(kb_init<J>, vg, BTPB, cs, n, Kp, (const double*)B.b.p, B.x.p, B.r.p, B.partial.p, h.counter.p + 1, B.S.p);
+            blaunch(kb_init<J, R>, vg, VTPB, cs, n, (const double*)B.b.p, B.x.p, B.r.p, B.r32.p, B.partial.p, h.counter.p + 1, B.S.p, ord);
         });
         cudaGraphNode_t w2;
-        brec_loop<J, VT>(h, g, cs, l2.data(), l2.size(), &w2);
-        tail = w2;
+        brec_loop<J, R, VT>(h, g, cs, l2.data(), l2.size(), &w2);
     }
-    capture_into(&tail, 1, [&] {
-        blaunch(kb_unpack, 2048, 256, cs, n, B.K, Kp, (const double*)B.x.p, with_adjoint ? B.user_lambda : B.user_x);
-    });
     cudaGraphExec_t ge;
     CPC_CK(cudaGraphInstantiate(&ge, g, 0));
     B.graph = g;
@@ -1388,24 +1598,24 @@ void build_batched_graph(Handle& h, bool with_adjoint) {
 //   Q = A P;  alpha = (P^T Q)^{-1} gamma;  X += P alpha, R -= Q alpha;  stop when every column
 //   has ||r_k|| / ||b_k|| < tol;  Z = M R;  beta = gamma^{-1} (Z^T R);  gamma = Z^T R;  P = Z + P beta.
 // The host reads two flags per iteration (one stream synchronisation).
-template <int J, class VT>
-int solve_block_t(Handle& h, int K, double tol, int maxit, int* iters, double* res) {
+template <int J, int R, class VT>
+int solve_block_t(Handle& h, int K, const double* b, double* x, double tol, int maxit, int* iters, double* res) {
     Batched& B = h.bat;
     const int Kp = B.Kp, n = h.n;
     cudaStream_t s = h.s;
     const int64_t nk = (int64_t)n * Kp;
     auto km = [&](int i) { return B.kmat.p + (size_t)i * Kp * Kp; };
-    const size_t gram_smem = 2 * (size_t)KK_ROWS * Kp * sizeof(double);
+    constexpr int KP = Cols<J, R>::KP;
+    const size_t gram_smem = 2 * (size_t)KK_ELEMS * sizeof(double);
     const size_t solve_smem = 2 * (size_t)K * K * sizeof(double);
-    const size_t upd_smem = ((size_t)Kp * Kp + BWARPS * Kp) * sizeof(double);
+    const size_t upd_smem = ((size_t)Kp * Kp + BWARPS * R * Kp) * sizeof(double);
     const size_t pup_smem = (size_t)Kp * Kp * sizeof(double);
     CPC_CK(cudaFuncSetAttribute(kk_solve, cudaFuncAttributeMaxDynamicSharedMemorySize, 2 * 64 * 64 * (int)sizeof(double)));
     const Csr& A = h.lev[0].A;
-    const int rg = std::min(rows_grid(n), 152 * 8);
     VT* z = (VT*)B.z.p;
     auto gram = [&](const auto* U, const double* V, double* out) {
-        kk_gram<<<KK_GRID, KK_TPB, gram_smem, s>>>(n, Kp, U, V, B.kpart.p);
-        kk_gram_sum<<<16, 256, 0, s>>>(KK_GRID, Kp, B.kpart.p, out);
+        kk_gram<KP><<<KK_GRID, KK_TPB, gram_smem, s>>>(n, U, V, B.kpart.p);
+        kk_gram_sum<<<(Kp * Kp + 7) / 8, 256, 0, s>>>(KK_GRID, Kp, B.kpart.p, out);
     };
     int flags[KF_COUNT] = {0, 0};
     auto read_flags = [&]() {
@@ -1415,24 +1625,22 @@ int solve_block_t(Handle& h, int K, double tol, int maxit, int* iters, double* r
     };
     CPC_CK(cudaMemsetAsync(B.kflag.p, 0, sizeof(int) * KF_COUNT, s));
     CPC_CK(cudaMemsetAsync(B.kmat.p, 0, sizeof(double) * KM_COUNT * Kp * Kp, s));
-    kb_pack<<<2048, 256, 0, s>>>(n, K, Kp, (const double*)B.user_b, B.b.p);
-    CPC_CK(cudaMemcpyAsync(B.r.p, B.b.p, sizeof(double) * nk, cudaMemcpyDeviceToDevice, s));
-    CPC_CK(cudaMemsetAsync(B.x.p, 0, sizeof(double) * nk, s));
-    kk_colnorm<J><<<KK_GRID, BTPB, 0, s>>>(n, Kp, B.r.p, B.kpart.p);
-    kk_check<<<1, 64, 0, s>>>(KK_GRID, Kp, K, B.kpart.p, B.kvec.p, tol, 1, B.kflag.p);
+    kb_pack<<<152 * 8, 256, 0, s>>>(n, K, Kp, b, B.b.p);
+    kk_init<J, R><<<KK_GRID, BTPB, 0, s>>>(n, B.b.p, B.x.p, B.r.p, B.r32.p, B.kpart.p);
+    kk_check<<<1, 256, 0, s>>>(KK_GRID, Kp, K, B.kpart.p, B.kvec.p, tol, 1, B.kflag.p);
     read_flags();
     if (flags[KF_BAD]) fail(CPC_EINVAL, "a right-hand-side column is zero or not finite");
-    brec_precond<J, VT>(h, h.opt.precond, B.r.p, z, s);              // Z = M R
+    brec_precond<J, R, VT>(h, h.opt.precond, bres<VT>(B), z, s);       // Z = M R
     kk_copy<VT><<<2048, 256, 0, s>>>(nk, (const VT*)z, B.p.p);         // P = Z
     gram((const VT*)z, B.r.p, km(KM_GAMMA));                           // gamma = Z^T R
     int status = CPC_ENOCONV, it = 0;
     for (int k = 1; k <= maxit; ++k) {
-        kk_spmm<J><<<rg, BTPB, 0, s>>>(n, Kp, A.ptr.p, A.col.p, A.val.p, (const double*)B.p.p, B.q.p);
+        kk_spmm<J, R><<<rows_grid<R>(n), BTPB, 0, s>>>(n, A.ptr.p, A.col.p, A.val.p, (const double*)B.p.p, B.q.p);
         gram((const double*)B.p.p, B.q.p, km(KM_PQ));
         kk_solve<<<1, KK_TPB, solve_smem, s>>>(K, Kp, km(KM_PQ), km(KM_GAMMA), km(KM_ALPHA), nullptr, B.kflag.p);
-        kk_update<J><<<KK_GRID, BTPB, upd_smem, s>>>(n, Kp, K, B.x.p, B.r.p, B.p.p, B.q.p, km(KM_ALPHA), B.kpart.p,
-                                                    B.kflag.p);
-        kk_check<<<1, 64, 0, s>>>(KK_GRID, Kp, K, B.kpart.p, B.kvec.p, tol, 0, B.kflag.p);
+        kk_update<J, R><<<KK_GRID, BTPB, upd_smem, s>>>(n, K, B.x.p, B.r.p, B.r32.p, B.p.p, B.q.p, km(KM_ALPHA), B.kpart.p,
+                                                       B.kflag.p);
+        kk_check<<<1, 256, 0, s>>>(KK_GRID, Kp, K, B.kpart.p, B.kvec.p, tol, 0, B.kflag.p);
         read_flags();
         if (flags[KF_BAD]) {                                           // X holds iteration k - 1
             status = CPC_EBREAKDOWN;
@@ -1445,13 +1653,13 @@ int solve_block_t(Handle& h, int K, double tol, int maxit, int* iters, double* r
             break;
         }
         if (k == maxit) break;
-        brec_precond<J, VT>(h, h.opt.precond, B.r.p, z, s);          // Z = M R
+        brec_precond<J, R, VT>(h, h.opt.precond, bres<VT>(B), z, s);   // Z = M R
         gram((const VT*)z, B.r.p, km(KM_GAMMA_NEW));                   // Z^T R
         kk_solve<<<1, KK_TPB, solve_smem, s>>>(K, Kp, km(KM_GAMMA), km(KM_GAMMA_NEW), km(KM_BETA), km(KM_GAMMA),
                                                B.kflag.p);
-        kk_pupdate<J, VT><<<KK_GRID, BTPB, pup_smem, s>>>(n, Kp, K, (const VT*)z, B.p.p, km(KM_BETA), B.kflag.p);
+        kk_pupdate<J, R, VT><<<KK_GRID, BTPB, pup_smem, s>>>(n, K, (const VT*)z, B.p.p, km(KM_BETA), B.kflag.p);
     }
-    kb_unpack<<<2048, 256, 0, s>>>(n, K, Kp, (const double*)B.x.p, B.user_x);
+    kb_unpack<<<152 * 8, 256, 0, s>>>(n, K, Kp, (const double*)B.x.p, x);
     CPC_LAUNCH_CK();
     std::vector<double> hv((size_t)KV_COUNT * Kp);
     CPC_CK(cudaMemcpyAsync(hv.data(), B.kvec.p, sizeof(double) * hv.size(), cudaMemcpyDeviceToHost, s));
@@ -1472,20 +1680,37 @@ void destroy_batched(Handle& h) {
     B.graph = nullptr;
 }
 
+// Columns the block vectors are padded to.
+static int padded(int K) { return K <= 8 ? 8 : K <= 16 ? 16 : (K + 31) / 32 * 32; }
+
+// Calls f(J, R) with the layout of Kp columns.
+template <class F>
+static auto with_cols(int Kp, F&& f) {
+    using std::integral_constant;
+    switch (Kp) {
+        case 8: return f(integral_constant<int, 1>{}, integral_constant<int, 4>{});
+        case 16: return f(integral_constant<int, 1>{}, integral_constant<int, 2>{});
+        case 32: return f(integral_constant<int, 1>{}, integral_constant<int, 1>{});
+        case 64: return f(integral_constant<int, 2>{}, integral_constant<int, 1>{});
+        case 96: return f(integral_constant<int, 3>{}, integral_constant<int, 1>{});
+        default: return f(integral_constant<int, 4>{}, integral_constant<int, 1>{});
+    }
+}
+
 // Allocate the block vectors for K columns (kept across calls with the same padded width).
-static void ensure_batched(Handle& h, int K, bool adjoint, double* user_b, double* user_x, double* user_lambda) {
+static void ensure_batched(Handle& h, int K, bool adjoint) {
     Batched& B = h.bat;
-    const int Kp = (K + 31) / 32 * 32;
+    const int Kp = padded(K);
     if (Kp > 128) fail(CPC_EINVAL, "at most 128 right-hand sides per batched call");
     const bool fp64 = h.opt.precision == CPC_PREC_FP64;
     const size_t vsz = fp64 ? sizeof(double) : sizeof(float);
     if (B.Kp != Kp) {
         destroy_batched(h);
         B = Batched{};
-        B.Kp = Kp;
         const size_t nk = (size_t)h.n * Kp;
         B.b.alloc(nk); B.x.alloc(nk); B.r.alloc(nk); B.p.alloc(nk); B.q.alloc(nk); B.xfwd.alloc(nk);
         B.z.alloc(nk * vsz); B.t.alloc(nk * vsz); B.y.alloc(nk * vsz);
+        if (!fp64) B.r32.alloc(nk);
         const int nl = (int)h.lev.size();
         B.lx.resize(nl); B.lf.resize(nl); B.lr.resize(nl);
         for (int l = 0; l < nl; ++l) {
@@ -1501,37 +1726,23 @@ static void ensure_batched(Handle& h, int K, bool adjoint, double* user_b, doubl
             B.kvec.alloc((size_t)KV_COUNT * Kp);
             B.kflag.alloc(KF_COUNT);
         }
+        B.Kp = Kp;                          // only now: a failed allocation leaves no layout behind
     }
-    if (B.gexec && (B.K != K || B.adjoint != adjoint || B.user_b != user_b || B.user_x != user_x ||
-                    B.user_lambda != user_lambda)) destroy_batched(h);
-    B.K = K;
+    if (B.gexec && B.adjoint != adjoint) destroy_batched(h);
     B.adjoint = adjoint;
-    B.user_b = user_b;
-    B.user_x = user_x;
-    B.user_lambda = user_lambda;
 }
 
 void solve_batched(Handle& h, int K, const double* b, double* x, double* lambda, double tol, int maxit,
                    int* iters, int* status, int* iters_adj, int* status_adj) {
-    ensure_batched(h, K, lambda != nullptr, (double*)b, x, lambda);
+    ensure_batched(h, K, lambda != nullptr);
     Batched& B = h.bat;
-    const int Kp = B.Kp;
-    if (!B.gexec) {
-        const bool fp64 = h.opt.precision == CPC_PREC_FP64;
-        const int J = Kp / 32;
-        const bool adj = lambda != nullptr;
-        if (fp64) {
-            if (J == 1) build_batched_graph<1, double>(h, adj);
-            else if (J == 2) build_batched_graph<2, double>(h, adj);
-            else if (J == 3) build_batched_graph<3, double>(h, adj);
-            else build_batched_graph<4, double>(h, adj);
-        } else {
-            if (J == 1) build_batched_graph<1, float>(h, adj);
-            else if (J == 2) build_batched_graph<2, float>(h, adj);
-            else if (J == 3) build_batched_graph<3, float>(h, adj);
-            else build_batched_graph<4, float>(h, adj);
-        }
-    }
+    const int Kp = B.Kp, n = h.n;
+    if (!B.gexec)
+        with_cols(Kp, [&](auto j, auto r) {
+            constexpr int J = decltype(j)::value, R = decltype(r)::value;
+            if (h.opt.precision == CPC_PREC_FP64) build_batched_graph<J, R, double>(h, lambda != nullptr);
+            else build_batched_graph<J, R, float>(h, lambda != nullptr);
+        });
     cudaStream_t s = h.s;
     std::vector<double> st((size_t)NB_STATE * Kp, 0.0);
     for (int c = 0; c < Kp; ++c) {
@@ -1539,7 +1750,11 @@ void solve_batched(Handle& h, int K, const double* b, double* x, double* lambda,
         st[(size_t)S_MAXIT * Kp + c] = c < K ? (double)maxit : 0.0;
     }
     CPC_CK(cudaMemcpyAsync(B.S.p, st.data(), sizeof(double) * st.size(), cudaMemcpyHostToDevice, s));
+    kb_pack<<<152 * 8, 256, 0, s>>>(n, K, Kp, b, B.b.p);
     CPC_CK(cudaGraphLaunch(B.gexec, s));
+    kb_unpack<<<152 * 8, 256, 0, s>>>(n, K, Kp, (const double*)(lambda ? B.xfwd.p : B.x.p), x);
+    if (lambda) kb_unpack<<<152 * 8, 256, 0, s>>>(n, K, Kp, (const double*)B.x.p, lambda);
+    CPC_LAUNCH_CK();
     CPC_CK(cudaMemcpyAsync(st.data(), B.S.p, sizeof(double) * st.size(), cudaMemcpyDeviceToHost, s));
     std::vector<double> kf(2 * (size_t)Kp, 0.0);
     if (lambda) CPC_CK(cudaMemcpyAsync(kf.data(), B.kfwd.p, sizeof(double) * 2 * Kp, cudaMemcpyDeviceToHost, s));
@@ -1562,12 +1777,16 @@ void solve_batched(Handle& h, int K, const double* b, double* x, double* lambda,
 int solve_block(Handle& h, int K, const double* b, double* x, double tol, int maxit, int* iters, double* res) {
     if (K < 1 || K > 64) fail(CPC_EINVAL, "block CG takes 1 to 64 right-hand sides");
     if (h.opt.precond == CPC_PRECOND_AMG_ILU) fail(CPC_EINVAL, "block CG supports B_co, AMG, IC(0) and B^");
-    ensure_batched(h, K, false, (double*)b, x, nullptr);
-    const bool fp64 = h.opt.precision == CPC_PREC_FP64;
-    if (h.bat.Kp == 32) return fp64 ? solve_block_t<1, double>(h, K, tol, maxit, iters, res)
-                                    : solve_block_t<1, float>(h, K, tol, maxit, iters, res);
-    return fp64 ? solve_block_t<2, double>(h, K, tol, maxit, iters, res)
-                : solve_block_t<2, float>(h, K, tol, maxit, iters, res);
+    ensure_batched(h, K, false);
+    return with_cols(h.bat.Kp, [&](auto j, auto r) {
+        constexpr int J = decltype(j)::value, R = decltype(r)::value;
+        if constexpr (J <= 2) {
+            if (h.opt.precision == CPC_PREC_FP64) return solve_block_t<J, R, double>(h, K, b, x, tol, maxit, iters, res);
+            return solve_block_t<J, R, float>(h, K, b, x, tol, maxit, iters, res);
+        } else {
+            return (int)CPC_EINVAL;
+        }
+    });
 }
 
 }  // namespace cpc

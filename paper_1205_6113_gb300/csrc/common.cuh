@@ -133,6 +133,11 @@ struct Csr {
 // Value storage types of the preconditioner data.
 enum VType { VT_F64 = 0, VT_F32 = 1, VT_BF16 = 2 };
 
+// An FP64 smoother layout keeps a row's entries of earlier and of later groups apart (Sell::cmid).  In an
+// FP32 one they stay in column order, so that a sum is rounded the same whichever of them it takes, and
+// Sell::fcol marks the columns of later groups with this bit: a sweep from a zero guess skips them.
+constexpr int LATER = 1 << 30;
+
 struct DiaOff {
     int o[8];
 };
@@ -151,11 +156,12 @@ struct Sell {
     int nslots = 0, nchunks = 0;
     int64_t nelem = 0;
     int lanes = 0;                     // most entries one lane holds: ceil(widest chunk / 32)
-    // Smoother copy (colour-grouped A_l): the entries of a chunk come in two parts, each padded to its
+    // FP64 smoother copy (colour-grouped A_l): the entries of a chunk come in two parts, each padded to its
     // widest row: columns of an earlier group than the row's in [cptr[k], cmid[k]), columns of a later
     // group in [cmid[k], cptr[k+1]).  lanes_lo / lanes_up: most entries one lane holds of each part.
     int lanes_lo = 0, lanes_up = 0;
     DBuf<int> perm, cptr, cmid, col;
+    DBuf<int> fcol;                    // FP32 smoother copy: col with the columns of later groups marked
     DBuf<double> val, diag, dinv;      // FP64 copy (always); dinv = 1 / diag (split diagonal only)
     DBuf<float> val32, diag32, dinv32; // FP32 copy (mixed precision)
     DBuf<__nv_bfloat16> val16;         // BF16 copy of off-diagonals (coarse levels, mode 2)

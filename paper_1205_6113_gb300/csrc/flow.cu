@@ -98,6 +98,39 @@ struct FlowBatch {
             acc += v[u] * flow_val(b[u]);
         }
     }
+    // The same over a row whose entries keep their order: the new values of one part, the old ones of
+    // the other, told apart by LATER.  MODE FLOW_FWD0 takes no old ones (they are zero).
+    template <int MODE>
+    __device__ __forceinline__ void add_mixed(const VT* xo, const VT* xn, VT& acc, int* err) {
+        using U = Unset<VT>;
+        typename U::B b[M];
+        auto from = [&](int u) {
+            const bool later = c[u] & LATER;
+            return (later == (MODE == FLOW_BWD) ? xn : xo) + (c[u] & ~LATER);
+        };
+#pragma unroll
+        for (int u = 0; u < M; ++u) {
+            if (c[u] < 0 || (MODE == FLOW_FWD0 && (c[u] & LATER))) c[u] = -1;
+            b[u] = 0;
+            flow_ld(b[u], c[u] >= 0 ? from(u) : xn, c[u] >= 0);
+        }
+        for (int spin = 0;; ++spin) {
+            bool miss = false;
+#pragma unroll
+            for (int u = 0; u < M; ++u) miss |= b[u] == U::bits;
+            if (!__any_sync(0xffffffffu, miss)) break;
+            if (spin == FLOW_SPINS) {
+                if (miss) *err = 1;
+#pragma unroll
+                for (int u = 0; u < M; ++u) b[u] = b[u] == U::bits ? U::nan : b[u];
+                break;
+            }
+#pragma unroll
+            for (int u = 0; u < M; ++u) flow_ld(b[u], c[u] >= 0 ? from(u) : xn, b[u] == U::bits);
+        }
+#pragma unroll
+        for (int u = 0; u < M; ++u) acc += v[u] * flow_val(b[u]);
+    }
 };
 
 // WIDE: blocks of four warps, one chunk each.  Else blocks of one warp, which takes one chunk after
@@ -106,8 +139,11 @@ struct FlowBatch {
 template <class MT, class DT, class FT, class VT, int MODE, int M, bool WIDE>
 __global__ void __launch_bounds__(WIDE ? 128 : 32) k_flow(SV<MT, DT> A, const int* __restrict__ cmid, int nchunks, const FT* f,
                                              const VT* xo, VT* xn, VT* unset, VT* zadd, unsigned* ctr, int* err) {
-    constexpr bool UP = MODE == FLOW_BWD, OLD = MODE == FLOW_FWD || MODE == FLOW_BWD;
+    constexpr bool UP = MODE == FLOW_BWD;
     constexpr bool TRI = MODE == FLOW_LOWER || MODE == FLOW_UPPER;
+    // FP32 rows keep their entries in column order, the two parts mixed
+    constexpr bool MIX = std::is_same<VT, float>::value && !TRI;
+    constexpr bool OLD = !MIX && (MODE == FLOW_FWD || MODE == FLOW_BWD);
     const int lane = threadIdx.x & 31, C = A.C, r = lane & (C - 1), g = lane / C, o = g * C + r;
     bool waited = false;
     do {
@@ -128,8 +164,8 @@ __global__ void __launch_bounds__(WIDE ? 128 : 32) k_flow(SV<MT, DT> A, const in
         const int row = A.perm[s];
         const bool own = g == 0 && row >= 0;
         // [nb, ne): the entries with new values, [ob, oe): those with old values
-        const int b0 = A.cptr[k], b2 = A.cptr[k + 1], b1 = TRI ? b2 : cmid[k];
-        const int nb = UP ? b1 : b0, ne = UP ? b2 : b1, ob = UP ? b0 : b1, oe = UP ? b1 : b2;
+        const int b0 = A.cptr[k], b2 = A.cptr[k + 1], b1 = TRI || MIX ? b2 : cmid[k];
+        const int nb = UP && !MIX ? b1 : b0, ne = UP ? b2 : b1, ob = UP ? b0 : b1, oe = UP ? b1 : b2;
         FlowBatch<M, VT, MT> bn, bo;
         bn.load(A.col, A.val, nb + o, ne, (ne - nb + 31) >> 5);
         if (OLD) bo.load(A.col, A.val, ob + o, oe, (oe - ob + 31) >> 5);
@@ -152,10 +188,14 @@ __global__ void __launch_bounds__(WIDE ? 128 : 32) k_flow(SV<MT, DT> A, const in
                 bo.add_old(xo, acc);
             }
         }
-        bn.add_new(xn, acc, err);
+        auto add = [&] {
+            if constexpr (MIX) bn.template add_mixed<MODE>(xo, xn, acc, err);
+            else bn.add_new(xn, acc, err);
+        };
+        add();
         for (int p = 32 * M; p < ne - nb; p += 32 * M) {
             bn.load(A.col, A.val, nb + p + o, ne, (ne - nb - p + 31) >> 5);
-            bn.add_new(xn, acc, err);
+            add();
         }
         for (int w = C; w < 32; w <<= 1) acc += __shfl_xor_sync(0xffffffffu, acc, w);
         if (own) {
@@ -187,7 +227,7 @@ void flow_mode(const Sell& S, SV<MT, DT> v, const FT* f, const VT* xo, VT* xn, V
     // a draw, once per chunk (18,000 chunks: 24 us against 15).
     const int ahead = std::max(2 * flow_sms(), (int)(4 * (int64_t)S.nchunks / std::max<int>(1, (int)S.seg.size() - 1)));
     const bool wide = ahead > 16 * flow_sms();
-    const int lanes = (MODE == FLOW_LOWER || MODE == FLOW_UPPER) ? S.lanes : std::max(S.lanes_lo, S.lanes_up);
+    const int lanes = MODE == FLOW_LOWER || MODE == FLOW_UPPER || std::is_same<VT, float>::value ? S.lanes : std::max(S.lanes_lo, S.lanes_up);
     auto go = [&](auto m) {
         constexpr int M = decltype(m)::value;
         if (wide)
@@ -220,6 +260,10 @@ void rec_flow(FlowMode mode, const Sell& S, VType vt, const FT* f, const VT* xo,
         if (mode == FLOW_LOWER) go(v, std::integral_constant<int, FLOW_LOWER>{});
         else go(v, std::integral_constant<int, FLOW_UPPER>{});
     };
+    auto flagged = [&](auto v) {
+        v.col = S.fcol.p;
+        return v;
+    };
     const bool tri = mode == FLOW_LOWER || mode == FLOW_UPPER;
     if constexpr (std::is_same<VT, double>::value) {
         const auto v = view(S, (const double*)S.val.p, (const double*)S.dinv.p);
@@ -228,10 +272,9 @@ void rec_flow(FlowMode mode, const Sell& S, VType vt, const FT* f, const VT* xo,
     } else {
         if (tri) solve(view(S, (const float*)S.val32.p, (const float*)S.dinv32.p));
         else if (vt == VT_BF16) {
-            if constexpr (std::is_same<FT, float>::value)
-                sweep(view(S, (const __nv_bfloat16*)S.val16.p, (const float*)S.dinv32.p));
+            if constexpr (std::is_same<FT, float>::value) sweep(flagged(view(S, (const __nv_bfloat16*)S.val16.p, (const float*)S.dinv32.p)));
         } else {
-            sweep(view(S, (const float*)S.val32.p, (const float*)S.dinv32.p));
+            sweep(flagged(view(S, (const float*)S.val32.p, (const float*)S.dinv32.p)));
         }
     }
     CPC_LAUNCH_CK();

@@ -31,23 +31,25 @@ struct Level {
     DBuf<float> xa32;
     bool flow = false;      // sweeps as one flow launch each (flow.cuh); else a launch per colour
     bool red_black = false; // two colours in diagonal form (the structured fine level)
+    // FP64: sweeps, residuals and transfers leave out the entries that multiply values known to be zero.
+    // FP32 ones add every term in the order of the full sums: a preconditioner rounded otherwise moves the
+    // solution by 1e-11 to 5e-9 of its norm, inside the error of a solve to 1e-6 but not repeatable to it.
+    bool skip_zeros() const { return vt == VT_F64; }
 };
 
-// Batched PCG state: block vectors [n][Kp] (Kp = K rounded up to 32), level vectors in the
+// Batched PCG state: block vectors [n][Kp] (Kp = K rounded up to 8, 16 or a multiple of 32), level vectors in the
 // preconditioner's precision (raw bytes), per-column scalars, and the captured graph.
 struct Batched {
-    int K = 0, Kp = 0;
+    int Kp = 0;
     bool adjoint = false;
     DBuf<double> b, x, r, p, q, xfwd;
+    DBuf<float> r32;        // the residual in the preconditioner's precision (FP32 modes)
     DBuf<char> z, t, y;
     std::vector<DBuf<char>> lx, lf, lr;
     DBuf<double> S, partial, kfwd;
     // block CG: K x K matrices [KM_COUNT][Kp][Kp], Gram partials, column vectors [KV_COUNT][Kp], flags
     DBuf<double> kmat, kpart, kvec;
     DBuf<int> kflag;
-    double* user_b = nullptr;
-    double* user_x = nullptr;
-    double* user_lambda = nullptr;
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t gexec = nullptr;
 };

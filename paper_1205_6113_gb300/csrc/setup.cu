@@ -1605,6 +1605,17 @@ __global__ void k_sell_fill(const int* perm, int nslots, int C, const int* ptr, 
     if (sdiag) sdiag[s] = d;
 }
 
+// fcol = col with the columns of later groups than the row's marked.
+__global__ void k_flag_later(int nslots, int C, const int* perm, const int* cptr, const int* col, const int* key, int* fcol) {
+    int s = blockIdx.x * blockDim.x + threadIdx.x;
+    if (s >= nslots) return;
+    const int i = perm[s], k = s / C;
+    for (int e = cptr[k] + s % C; e < cptr[k + 1]; e += C) {
+        const int j = col[e];
+        fcol[e] = i >= 0 && j >= 0 && key[j] > key[i] ? j | LATER : j;
+    }
+}
+
 // Slot order from a per-row group key (colour or level): rows sorted by (key, row), each group
 // padded to a multiple of the chunk height C.  Returns the chunk boundaries of the groups in seg.
 __global__ void k_group_count(int n, const int* key, int* cnt) {
@@ -2587,22 +2598,26 @@ void setup_level_sells(Level& L, cudaStream_t s, bool last, bool tune, bool fp64
             std::vector<int> seg;
             grouped_slots(L.n, L.colour.p, L.ncolours, C, s, slots, nslots, seg);
             build_sell(L.A.ptr.p, L.A.col.p, L.A.val.p, slots, nslots, seg, C, SELL_OFFDIAG, true, nullptr, out, s,
-                       L.colour.p);
+                       fp64 ? L.colour.p : nullptr);
             CPC_CK(cudaStreamSynchronize(s));
         };
         const int ca = choose_chunk((double)(L.A.nnz - L.n) / std::max(1, L.n));
         build_grouped(ca, L.S);
-        if (!tune && fp64 && ca < 32) {
-            // FP64 issue bounds a wide colour step on this part, and adding the partial sums of a row's
-            // lanes costs as much of it as a few entries: twice the chunk height (half the lanes per row)
-            // where a colour takes many waves of warps (level 1 at 8.4M: 300 -> 264 us a sweep), or where
-            // that brings a colour of rows of up to 18 entries into one wave (level 1 at 1M: 55 -> 49 us).
-            int widest = 0;
+        if (!tune && ca < 32) {
+            // One wave: a colour step whose blocks do not all fit on the GPU at once runs in two waves, and
+            // only the first wave's matrix loads overlap the previous step.  If the widest colour needs more
+            // blocks than fit (by the registers of the batch width) and twice the chunk height (half the
+            // lanes per row, about twice the entries per lane) would fit, take twice the chunk height
+            // (level 1 at 1M, FP64: 55 -> 49 us a sweep).  In FP64 also where a colour takes many waves: FP64
+            // issue bounds it then, and adding the partial sums of a row's lanes costs as much of it as a
+            // few entries (level 1 at 8.4M: 300 -> 264 us).
+            int widest = 0, sms = 0, dev = 0;
             for (size_t c = 0; c + 1 < L.S.seg.size(); ++c) widest = std::max(widest, L.S.seg[c + 1] - L.S.seg[c]);
-            const double per_lane = (double)(L.A.nnz - L.n) / L.n * 2 * ca / 32;
-            if (widest > 4 * GS_RESIDENT_WARPS ||
-                (widest > GS_RESIDENT_WARPS && widest <= 2 * GS_RESIDENT_WARPS && per_lane <= 9.0))
-                build_grouped(2 * ca, L.S);
+            CPC_CK(cudaGetDevice(&dev));
+            CPC_CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+            const int per_sm = L.S.lanes <= 4 ? 16 : L.S.lanes <= 6 ? 12 : L.S.lanes <= 8 ? 9 : L.S.lanes <= 12 ? 8 : 6;
+            const bool one_wave = (widest + 3) / 4 > per_sm * sms && (widest / 2 + 4) / 4 <= 6 * sms;
+            if (one_wave || (fp64 && widest > 4 * GS_RESIDENT_WARPS)) build_grouped(2 * ca, L.S);
         }
         if (tune) {
             float best = time_gs_sweep(L.S, L.n);
@@ -2619,7 +2634,7 @@ void setup_level_sells(Level& L, cudaStream_t s, bool last, bool tune, bool fp64
         }
         // On a two-colour level the red rows of P come first and the red columns of R make the first part:
         // the cycle reads no others there (rec_vcycle).
-        const bool rb = L.ncolours == 2;
+        const bool rb = L.ncolours == 2;     // (R in FP64 only: FP32 sums keep their order)
         DBuf<int> ps;
         int pn = 0;
         std::vector<int> pseg;
@@ -2633,7 +2648,7 @@ void setup_level_sells(Level& L, cudaStream_t s, bool last, bool tune, bool fp64
         const int cr = choose_chunk((double)L.R.nnz / std::max(1, L.R.n));
         natural_slots(L.R.n, cr, s, rs, rn, rseg);
         build_sell(L.R.ptr.p, L.R.col.p, L.R.val.p, rs, rn, rseg, cr, SELL_ALL, false, nullptr, L.SR, s,
-                   rb ? L.colour.p : nullptr, true);
+                   rb && fp64 ? L.colour.p : nullptr, true);
         CPC_CK(cudaStreamSynchronize(s));
     }
 }
@@ -3028,6 +3043,12 @@ void setup_handle(Handle& h, const cpc_csr& in) {
         if (L.flow) {
             if (L.vt == VT_F64) L.xa64.alloc(n);
             else L.xa32.alloc(n);
+        }
+        if (l < nl - 1 && !L.skip_zeros() && !L.red_black) {
+            L.S.fcol.alloc(L.S.nelem);
+            k_flag_later<<<nblk(L.S.nslots), TPB, 0, s>>>(L.S.nslots, L.S.C, L.S.perm.p, L.S.cptr.p, L.S.col.p, L.colour.p,
+                                                          L.S.fcol.p);
+            CPC_LAUNCH_CK();
         }
     }
     if (prec != CPC_PREC_FP64) {

@@ -238,7 +238,7 @@ __global__ void __launch_bounds__(SELL_TPB) k_spmv_dia(DV<MT, DT> A, const XT* x
 // with the view's diagonal field holding 1 / a_ii (a multiply instead of an FP64 division).
 // Rows of one colour are not coupled, so they update in parallel exactly as in sequential order.
 // LOW: in a forward sweep from a zero guess the rows of later colours are still zero, so only the
-// entries of earlier colours (up to cmid) are read.
+// entries of earlier colours are taken: up to cmid in FP64, those not marked LATER in FP32.
 template <class MT, class DT, class FT, class VT, int U, bool LOW>
 __global__ void __launch_bounds__(SELL_TPB) k_gs(SV<MT, DT> A, const int* __restrict__ cmid, int c0, int c1, const FT* f,
                                                  VT* x) {
@@ -251,7 +251,7 @@ __global__ void __launch_bounds__(SELL_TPB) k_gs(SV<MT, DT> A, const int* __rest
     const bool own = g == 0 && row >= 0;
     const VT dinv = own ? Cv<VT>::f(A.diag[s]) : VT(0);
     VT fr = VT(0);
-    VT dot = sell_dot<VT, true, U>(A.col, A.val, A.cptr[k] + g * C + r, LOW ? cmid[k] : A.cptr[k + 1], x,
+    VT dot = sell_dot<VT, true, U>(A.col, A.val, A.cptr[k] + g * C + r, LOW && std::is_same<VT, double>::value ? cmid[k] : A.cptr[k + 1], x,
                                    [&] { if (own) fr = Cv<VT>::f(f[row]); });
     dot = sub_sum(dot, C);
     if (own) x[row] = (fr - dot) * dinv;
@@ -317,7 +317,7 @@ __global__ void __launch_bounds__(SELL_TPB) k_spmv(SV<MT, DT> A, int nchunks, co
 // cmid: the red columns of the finest R), else all (cend = cptr + 1).  FIRST selects what else the
 // next level's sweep needs: RF_NONE nothing (the coarsest level), RF_ZERO x_c = 0 (the cluster kernel),
 // RF_SWEEP the first colour step from a zero guess, x_c = f_c / a_ii on colour 0 (its rows see only
-// zeros; the sweep from zero never reads the others), RF_FLOW that with the other rows marked unset.
+// zeros; the sweep from zero does not read the others), RF_FLOW that with the others marked unset.
 enum RestrictNext { RF_NONE, RF_ZERO, RF_SWEEP, RF_FLOW };
 
 template <class MT, class VT, int U, int NEXT>
@@ -816,17 +816,20 @@ void rec_gs(Level& L, int c, const FT* f, VT* x, cudaStream_t s, bool from_zero 
     const int* cmid = L.S.cmid.p;
     auto go = [&](auto low) {
         constexpr bool LOW = decltype(low)::value;
-        with_u_gs(LOW ? L.S.lanes_lo : L.S.lanes, c1 - c0, [&](auto u) {
-            constexpr int U = decltype(u)::value;
-            if constexpr (std::is_same<VT, double>::value) {
-                launch(k_gs<double, double, FT, VT, U, LOW>, g, tpb, s, view(L.S, (const double*)L.S.val.p, (const double*)L.S.dinv.p), cmid, c0, c1, f, x);
-            } else {
-                if (L.vt == VT_BF16)
-                    launch(k_gs<__nv_bfloat16, float, FT, VT, U, LOW>, g, tpb, s, view(L.S, (const __nv_bfloat16*)L.S.val16.p, (const float*)L.S.dinv32.p), cmid, c0, c1, f, x);
-                else
-                    launch(k_gs<float, float, FT, VT, U, LOW>, g, tpb, s, view(L.S, (const float*)L.S.val32.p, (const float*)L.S.dinv32.p), cmid, c0, c1, f, x);
-            }
-        });
+        auto run = [&](auto v, int lanes) {
+            if (LOW && !L.skip_zeros()) v.col = L.S.fcol.p;
+            using MT = std::remove_cv_t<std::remove_reference_t<decltype(*v.val)>>;
+            using DT = std::remove_cv_t<std::remove_reference_t<decltype(*v.diag)>>;
+            with_u_gs(lanes, c1 - c0, [&](auto u) {
+                launch(k_gs<MT, DT, FT, VT, decltype(u)::value, LOW>, g, tpb, s, v, cmid, c0, c1, f, x);
+            });
+        };
+        if constexpr (std::is_same<VT, double>::value)
+            run(view(L.S, (const double*)L.S.val.p, (const double*)L.S.dinv.p), LOW ? L.S.lanes_lo : L.S.lanes);
+        else if (L.vt == VT_BF16)
+            run(view(L.S, (const __nv_bfloat16*)L.S.val16.p, (const float*)L.S.dinv32.p), L.S.lanes);
+        else
+            run(view(L.S, (const float*)L.S.val32.p, (const float*)L.S.dinv32.p), L.S.lanes);
     };
     if (from_zero) go(std::true_type{});
     else go(std::false_type{});
@@ -834,6 +837,7 @@ void rec_gs(Level& L, int c, const FT* f, VT* x, cudaStream_t s, bool from_zero 
 
 template <class FT, class VT>
 void rec_resid_level(Level& L, const FT* f, const VT* x, VT* r, cudaStream_t s, bool after_sweep, bool from_zero) {
+    from_zero = from_zero && L.skip_zeros();
     if (L.red_black && after_sweep) {                       // the last colour's residual is zero
         const int s1 = L.S.seg[1] * L.S.C;
         auto go = [&](auto zero) {
@@ -852,24 +856,14 @@ void rec_resid_level(Level& L, const FT* f, const VT* x, VT* r, cudaStream_t s, 
         else go(std::false_type{});
         return;
     }
-    if (after_sweep && from_zero && L.S.cmid.p) {
-        const int g = blocks_for_chunks(L.S.nchunks);
-        with_u(L.S.lanes_up, [&](auto w) {
-            constexpr int U = decltype(w)::value;
-            if constexpr (std::is_same<VT, double>::value) {
-                launch(k_resid_up<double, double, U>, g, SELL_TPB, s, view(L.S, (const double*)L.S.val.p, (const double*)nullptr),
-                       (const int*)L.S.cmid.p, L.S.nchunks, x, r);
-            } else {
-                if (L.vt == VT_BF16)
-                    launch(k_resid_up<__nv_bfloat16, float, U>, g, SELL_TPB, s,
-                           view(L.S, (const __nv_bfloat16*)L.S.val16.p, (const float*)nullptr), (const int*)L.S.cmid.p,
-                           L.S.nchunks, x, r);
-                else
-                    launch(k_resid_up<float, float, U>, g, SELL_TPB, s,
-                           view(L.S, (const float*)L.S.val32.p, (const float*)nullptr), (const int*)L.S.cmid.p, L.S.nchunks, x, r);
-            }
-        });
-        return;
+    if constexpr (std::is_same<VT, double>::value) {
+        if (after_sweep && from_zero && L.S.cmid.p) {
+            with_u(L.S.lanes_up, [&](auto w) {
+                launch(k_resid_up<double, double, decltype(w)::value>, blocks_for_chunks(L.S.nchunks), SELL_TPB, s,
+                       view(L.S, (const double*)L.S.val.p, (const double*)nullptr), (const int*)L.S.cmid.p, L.S.nchunks, x, r);
+            });
+            return;
+        }
     }
     if (L.S.ndiag) {
         with_nd(L.S.ndiag, [&](auto nd) {
@@ -986,17 +980,17 @@ void rec_vcycle(Handle& h, int l, const FT* f, VT* x, bool zero_guess, cudaStrea
     rec_resid_level(L, f, u, lr<VT>(L), s, !ilu_here, zero_guess);       // (2a) r = f - A u
     // On a red-black level the black residual is zero and the backward sweep overwrites the black rows
     // before it reads them: only the red columns of R and the red rows of P count.
-    const bool red = L.red_black && !ilu_here;
+    const bool red = L.red_black && !ilu_here, red_cols = red && L.SR.cmid.p;
     const VT* r = lr<VT>(L);
     if (l + 1 >= h.tail_start) {                                         // (2a) f_c = R r, x_c = 0
-        rec_restrict<VT, RF_ZERO>(h, l, red, r, lf<VT>(C), lx<VT>(C), s);
+        rec_restrict<VT, RF_ZERO>(h, l, red_cols, r, lf<VT>(C), lx<VT>(C), s);
         record_tail(h, l + 1, lf<VT>(C), lx<VT>(C), s);                  // (2b) the coarser levels, one kernel
     } else if (l + 1 == nl - 1) {                                        // (2a) f_c = R r
-        rec_restrict<VT, RF_NONE>(h, l, red, r, lf<VT>(C), (VT*)nullptr, s);
+        rec_restrict<VT, RF_NONE>(h, l, red_cols, r, lf<VT>(C), (VT*)nullptr, s);
         rec_vcycle<VT, VT>(h, l + 1, lf<VT>(C), lx<VT>(C), true, s);     // (2b) exact coarsest solve
     } else {                                                             // (2a) f_c = R r, first colour step
-        if (C.flow) rec_restrict<VT, RF_FLOW>(h, l, red, r, lf<VT>(C), lxa<VT>(C), s);
-        else rec_restrict<VT, RF_SWEEP>(h, l, red, r, lf<VT>(C), lx<VT>(C), s);
+        if (C.flow) rec_restrict<VT, RF_FLOW>(h, l, red_cols, r, lf<VT>(C), lxa<VT>(C), s);
+        else rec_restrict<VT, RF_SWEEP>(h, l, red_cols, r, lf<VT>(C), lx<VT>(C), s);
         rec_vcycle<VT, VT>(h, l + 1, lf<VT>(C), lx<VT>(C), true, s, false, true);   // (2b) zero initial guess
     }
     const int pchunks = red ? L.SP.seg[1] : L.SP.nchunks;
@@ -1221,7 +1215,7 @@ float time_gs_sweep(const Sell& S, int n) {
     CPC_CK(cudaMemsetAsync(x.p, 0, sizeof(double) * n, cs));
     CPC_CK(cudaMemsetAsync(ctr.p, 0, sizeof(unsigned) * ctr.n, cs));
     CPC_CK(cudaStreamSynchronize(cs));
-    const bool flow = gs_by_flow(n, (int)S.seg.size() - 1);
+    const bool flow = S.cmid.p && gs_by_flow(n, (int)S.seg.size() - 1);   // (an FP32 layout is timed by launches)
     cudaGraph_t g;
     CPC_CK(cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal));
     for (int k = 0; k < SWEEPS; ++k) {      // the launches of the solve's sweeps
