@@ -834,17 +834,6 @@ __global__ void k_interp_fill(int n, const int* ptr, const int* col, const doubl
 // row i; in round r every remaining point with deg_i <= 2 min_{remaining} deg takes round r, then
 // each remaining point loses one degree per entry of its row taken in round r.
 // ============================================================================================
-// ============================================================================================
-// Jones-Plassmann colouring with priority (peel round, fmix32(i ^ COLOUR_SEED)): a point whose
-// neighbours of higher priority are all coloured takes the smallest colour they leave free.  Its
-// neighbours of lower priority cannot be coloured before it, so the result is the greedy colouring
-// in decreasing priority.  Colours written during a round by other threads may or may not be seen
-// (volatile reads): seeing one only lets a point finish in an earlier round, with the same colour.
-// ============================================================================================
-__device__ __forceinline__ bool jp_beats(int rj, int j, int ri, uint32_t hi) {
-    return rj > ri || (rj == ri && fmix32((uint32_t)j ^ COLOUR_SEED) > hi);
-}
-
 // Grid-wide barrier of a cooperative launch (every CTA resident).  Arrivals count up on *ctr (zero
 // before the launch); barrier number e completes when it reaches e * gridDim.x.  The wait gives up
 // after GBAR_NS or as soon as another CTA has given up (*err != 0), setting *err = 1; then every
@@ -903,18 +892,6 @@ __device__ int block_reduce(int v, Op op, int identity) {
     return v;                                                   // valid in thread 0
 }
 
-// blk[i]: the uncoloured neighbour of higher priority that stopped point i last time (-1: none
-// yet).  While that neighbour stays uncoloured the point is skipped.  Once it
-// is coloured, the point's row is examined again by a group of COL_G lanes (gl = lane in the
-// group, gm = the group's lane mask, gs = its first lane in the warp), COL_U entries per lane per
-// pass, with all loads of a pass in flight together: the first uncoloured neighbour of higher
-// priority in row order is recorded and false returned; if there is none, the point takes the
-// smallest colour left free by its neighbours of higher priority (from the colours just loaded
-// when the row fits one pass) and true is returned (group-uniform).  Entries before the old
-// blocking one are examined again although they cannot block (lower priority, or coloured for
-// good): with the loads in flight together that costs nothing, and their colours are needed.
-constexpr int COL_U = 4;
-
 // The lowest 32 / COL_G set bits of a warp-uniform mask go to the groups of the warp, one each in
 // order: returns group g's bit (-1: none left for it) and clears them all.
 __device__ __forceinline__ int take_group_bit(unsigned& bits, int g) {
@@ -928,65 +905,12 @@ __device__ __forceinline__ int take_group_bit(unsigned& bits, int g) {
     return mine;
 }
 
-__device__ bool jp_group(int i, int p0, int p1, int ri, const int* col, const int* rnd, volatile int* vc, int* blk,
-                         int gl, unsigned gm, int gs) {
-    const uint32_t hi = fmix32((uint32_t)i ^ COLOUR_SEED);
-    constexpr int W = COL_U * COL_G;                             // entries per pass
-    int cj[COL_U];
-    bool up[COL_U];                                             // neighbour of higher priority
-    for (int base = p0; base < p1; base += W) {
-        int j[COL_U];
-#pragma unroll
-        for (int u = 0; u < COL_U; ++u) {
-            const int p = base + u * COL_G + gl;
-            j[u] = p < p1 ? col[p] : -1;
-        }
-#pragma unroll
-        for (int u = 0; u < COL_U; ++u) {
-            const bool e = j[u] >= 0 && j[u] != i;
-            const int rj = e ? rnd[j[u]] : 0;                   // both loads in flight together
-            cj[u] = e ? vc[j[u]] : 0;
-            up[u] = e && jp_beats(rj, j[u], ri, hi);
-        }
-#pragma unroll
-        for (int u = 0; u < COL_U; ++u) {
-            const unsigned bits = (__ballot_sync(gm, up[u] && cj[u] < 0) >> gs) & ((1u << COL_G) - 1u);
-            if (bits) {
-                const int q = __ffs(bits) - 1;                  // first blocking entry of this batch
-                const int jq = __shfl_sync(gm, j[u], gs + q);
-                if (gl == 0) blk[i] = jq;
-                return false;
-            }
-        }
-    }
-    const bool one = p1 - p0 <= W;                              // colours of the only pass still at hand
-    for (int cb = 0;; cb += 64) {
-        unsigned long long used = 0ull;
-        if (one) {
-#pragma unroll
-            for (int u = 0; u < COL_U; ++u)
-                if (up[u] && cj[u] >= cb && cj[u] < cb + 64) used |= 1ull << (cj[u] - cb);
-        } else {
-            for (int p = p0 + gl; p < p1; p += COL_G) {
-                const int j = col[p];
-                if (j == i || !jp_beats(rnd[j], j, ri, hi)) continue;
-                const int c = vc[j];
-                if (c >= cb && c < cb + 64) used |= 1ull << (c - cb);
-            }
-        }
-        for (int o = COL_G / 2; o > 0; o >>= 1) used |= __shfl_xor_sync(gm, used, o);
-        if (used != ~0ull) {
-            if (gl == 0) vc[i] = cb + __ffsll((long long)~used) - 1;
-            return true;
-        }
-    }
-}
-
 // ---------------------------------------------------------------------------------------------
-// All levels are coloured by one cooperative launch of k_colour.  Each level runs its own state
+// The parity colourings and peel rounds of all levels run in one cooperative launch of k_colour; the
+// greedy colouring of the levels that are not bipartite follows (k_greedy).  Each level runs its own state
 // machine, and all advance one step per grid barrier, so that the setup waits for the longest
 // chain of rounds, not their sum:
-//   init       degrees, round -1, colour -1, blocking entry -1, parity word, triangle probe
+//   init       degrees, round -1, colour -1, parity word, triangle probe
 //   parity     the breadth-first parity 2-colouring (only if no triangle was found): colour =
 //              distance parity from the smallest index of the component.  A union-find over the
 //              entries, each word (parent, parity relative to it), joins the two ends of every
@@ -999,7 +923,6 @@ __device__ bool jp_group(int i, int p0, int p1, int ri, const int* col, const in
 //              each neighbour in dec[]; step 2: the remaining points apply their decrements and
 //              the next dmin is their minimum (decrements counted on points taken in the same
 //              round are never read)
-//   colour     Jones-Plassmann rounds (jp_group)
 // The CTAs of a step are shared among the levels with work in that step, in proportion to their
 // points (at least one each); a CTA works on one level.
 // ---------------------------------------------------------------------------------------------
@@ -1010,16 +933,15 @@ struct ColLev {
     const int* ptr;
     const int* col;
     int* colour;
-    int *deg, *dec, *rnd, *blk;
+    int *deg, *dec, *rnd;
     unsigned* w;                              // union-find words
     int* scal;                                // COL_NS counters, see below
 };
 
-// scal of a level: [0], [1] dmin of even / odd peel rounds; [2..4] points coloured in colour
-// round t (slot t % 3: a slot is cleared one round before it is added to and read one barrier
-// after); [5] triangle found; [6] not bipartite; [7] peel rounds; [8] colour rounds.
-enum { CS_DMIN = 0, CS_JP = 2, CS_TRI = 5, CS_BAD = 6, CS_PEEL_ROUNDS = 7, CS_JP_ROUNDS = 8, COL_NS = 12 };
-enum { CP_INIT, CP_UNION, CP_FIND, CP_CHECK, CP_RESET, CP_MARK, CP_MIN, CP_JP, CP_DONE };
+// scal of a level: [0], [1] dmin of even / odd peel rounds; [2] 1 when the peel rounds are done: the
+// level is not bipartite; [3] triangle found; [4] not bipartite or a join failed.
+enum { CS_DMIN = 0, CS_GREEDY = 2, CS_TRI = 3, CS_BAD = 4, COL_NS = 6 };
+enum { CP_INIT, CP_UNION, CP_FIND, CP_CHECK, CP_RESET, CP_MARK, CP_MIN, CP_DONE };
 
 // Union-find words: parent << 1 | parity relative to the parent (a root: itself, parity 0).
 // Returns the root of x and x's parity relative to it, halving the path on the way (a point is
@@ -1103,7 +1025,6 @@ __device__ void col_step(const ColLev& V, int phase, int rnd_no, int dm, int t, 
             V.dec[i] = 0;
             V.rnd[i] = -1;
             V.colour[i] = -1;
-            V.blk[i] = -1;
             V.w[i] = (unsigned)i << 1;
             m = imin(m, d);
             if (!tri) tri = tri_probe(i, ptr, col);
@@ -1184,47 +1105,10 @@ __device__ void col_step(const ColLev& V, int phase, int rnd_no, int dm, int t, 
         }
         m = block_reduce(m, imin, INT_MAX);
         if (threadIdx.x == 0 && m != INT_MAX) atomicMin(&V.scal[CS_DMIN + ((rnd_no + 1) & 1)], m);
-    } else if (phase == CP_JP) {
-        volatile int* vc = V.colour;
-        int cnt = 0;
-        for (int b0 = t - lane; b0 < n; b0 += COL_K * T) {     // warp-uniform trip count
-            int cv[COL_K], bv[COL_K], vb[COL_K];
-#pragma unroll
-            for (int k = 0; k < COL_K; ++k) {                   // loads of COL_K points in flight
-                const int i = b0 + k * T + lane;
-                cv[k] = i < n ? vc[i] : 0;
-                bv[k] = i < n ? V.blk[i] : -1;
-            }
-#pragma unroll
-            for (int k = 0; k < COL_K; ++k) vb[k] = cv[k] < 0 && bv[k] >= 0 ? vc[bv[k]] : -1;
-#pragma unroll
-            for (int k = 0; k < COL_K; ++k) {
-                const int base = b0 + k * T;
-                // uncoloured, and either never examined or its blocker has been coloured since
-                const bool ready = cv[k] < 0 && (bv[k] < 0 || vb[k] >= 0);
-                int q0 = 0, q1 = 0, qr = 0;                     // row bounds and round of a ready point
-                if (ready) {
-                    q0 = ptr[base + lane];
-                    q1 = ptr[base + lane + 1];
-                    qr = V.rnd[base + lane];
-                }
-                unsigned bits = __ballot_sync(0xffffffffu, ready);
-                while (bits) {                                  // a ready point per group at a time
-                    const int mine = take_group_bit(bits, gs / COL_G);
-                    const int src = mine < 0 ? 0 : mine;
-                    const int m0 = __shfl_sync(0xffffffffu, q0, src), m1 = __shfl_sync(0xffffffffu, q1, src);
-                    const int mr = __shfl_sync(0xffffffffu, qr, src);
-                    if (mine >= 0 && jp_group(base + mine, m0, m1, mr, col, V.rnd, vc, V.blk, gl, gm, gs) && gl == 0) ++cnt;
-                }
-            }
-        }
-        cnt = block_reduce(cnt, iadd, 0);
-        if (threadIdx.x == 0 && cnt) atomicAdd(&V.scal[CS_JP + rnd_no % 3], cnt);
     }
 }
 
-// *err: 1 a barrier gave up, 2 peel rounds or 3 colour rounds beyond their bound, 4 a union-find
-// join kept losing its race.
+// *err: 1 a barrier gave up, 2 peel rounds beyond their bound, 4 a union-find join kept losing its race.
 // Each CTA keeps the level descriptors and the levels' phases in shared memory; at each step its
 // threads load every level's counters at once (they change only before a barrier), thread 0 takes
 // the phase decisions (the same in every CTA) and picks the CTA's level, and the CTA works on it.
@@ -1232,7 +1116,6 @@ __global__ void __launch_bounds__(COL_TPB) k_colour(const ColLev* levs, int nlev
     __shared__ ColLev lv[COL_MAXL];
     __shared__ int sc[COL_MAXL * COL_NS];
     __shared__ int ph[COL_MAXL], rr[COL_MAXL], work[COL_MAXL], dmv[COL_MAXL];
-    __shared__ long long done[COL_MAXL];
     __shared__ int mine, c0s, cns, quit;
     unsigned long long epoch = 0;
     const bool lead = threadIdx.x == 0, first = lead && blockIdx.x == 0;
@@ -1240,7 +1123,6 @@ __global__ void __launch_bounds__(COL_TPB) k_colour(const ColLev* levs, int nlev
         lv[l] = levs[l];
         ph[l] = CP_INIT;
         rr[l] = 0;
-        done[l] = 0;
     }
     __syncthreads();
     for (int step = 0;; ++step) {
@@ -1286,10 +1168,9 @@ __global__ void __launch_bounds__(COL_TPB) k_colour(const ColLev* levs, int nlev
                     } else if (p == CP_MARK) {
                         dmv[l] = c[CS_DMIN + (rr[l] & 1)];
                         if (dmv[l] == INT_MAX) {
-                            if (first) g[CS_PEEL_ROUNDS] = rr[l];
-                            ph[l] = CP_JP;
-                            rr[l] = 0;
-                            continue;
+                            if (first) g[CS_GREEDY] = 1;
+                            ph[l] = CP_DONE;
+                            break;
                         }
                         if (rr[l] > n + 16) { if (first) atomicCAS(err, 0, 2); quit = 1; break; }
                         if (first) g[CS_DMIN + ((rr[l] + 1) & 1)] = INT_MAX;
@@ -1297,19 +1178,6 @@ __global__ void __launch_bounds__(COL_TPB) k_colour(const ColLev* levs, int nlev
                         break;
                     } else if (p == CP_MIN) {
                         work[l] = CP_MIN;
-                        break;
-                    } else if (p == CP_JP) {
-                        if (rr[l] > 0) {
-                            done[l] += c[CS_JP + (rr[l] - 1) % 3];
-                            if (done[l] >= n) {
-                                if (first) g[CS_JP_ROUNDS] = rr[l];
-                                ph[l] = CP_DONE;
-                                break;
-                            }
-                        }
-                        if (rr[l] > n + 32) { if (first) atomicCAS(err, 0, 3); quit = 1; break; }
-                        if (first) g[CS_JP + (rr[l] + 1) % 3] = 0;
-                        work[l] = CP_JP;
                         break;
                     } else {
                         break;                                  // done
@@ -1356,8 +1224,7 @@ __global__ void __launch_bounds__(COL_TPB) k_colour(const ColLev* levs, int nlev
         __syncthreads();
         if (lead) {                                             // advance the phases worked in this step
             for (int l = 0; l < nlev; ++l) {
-                if (work[l] == CP_JP) ++rr[l];
-                else if (work[l] == CP_MARK) ph[l] = CP_MIN;
+                if (work[l] == CP_MARK) ph[l] = CP_MIN;
                 else if (work[l] == CP_MIN) {
                     ph[l] = CP_MARK;
                     ++rr[l];
@@ -1365,6 +1232,88 @@ __global__ void __launch_bounds__(COL_TPB) k_colour(const ColLev* levs, int nlev
             }
         }
         if (!grid_bar(bar, epoch, err)) return;
+    }
+}
+
+// ============================================================================================
+// Greedy colouring in decreasing priority (peel round, fmix32(i ^ COLOUR_SEED)): each point takes the
+// smallest colour its neighbours of higher priority leave free.  The points of a level are sorted by
+// priority and handed out in that order by a counter, GREEDY_WARPS to a block; a warp takes a point and
+// loads the colours of its neighbours of higher priority until all are there.  A point only waits for
+// points handed out before it, to blocks that are running, so the earliest one without a colour never
+// waits for one that has not started.  The chain is as long as the longest path of the priorities (554
+// points at 1M); a step is a trip through L2, about 1.2 us, where a round over all points with a
+// grid barrier took 12 (colouring of all levels at 1M 13.5 ms, 6.0 with this).
+// ============================================================================================
+constexpr int GREEDY_WARPS = 4;
+constexpr int GREEDY_SPINS = 1 << 21;
+
+struct GreedyLev {
+    int n, blk0, blk1;                        // points; blocks [blk0, blk1) work on the level
+    const int *ptr, *col, *order, *rank;      // order[q]: the q-th point, rank: its inverse
+    int* colour;                              // -1 on entry
+    unsigned* ctr;
+};
+
+// Keys of a level's points, ascending in decreasing priority: level, complement of (round, hash).
+__global__ void k_greedy_key(int n, int lev, const int* rnd, int base, uint64_t* key, int* idx) {
+    int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    const uint64_t pr = ((uint64_t)(uint32_t)rnd[i] << 32) | fmix32((uint32_t)i ^ COLOUR_SEED);
+    key[base + i] = ((uint64_t)lev << 58) | (~pr & ((1ull << 58) - 1ull));
+    idx[base + i] = i;
+}
+
+__global__ void k_greedy_rank(int n, const int* order, int* rank) {
+    int q = blockIdx.x * blockDim.x + threadIdx.x;
+    if (q < n) rank[order[q]] = q;
+}
+
+__device__ __forceinline__ int colour_ld(const int* p) {
+    int v;
+    asm volatile("ld.relaxed.gpu.global.b32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
+
+__global__ void __launch_bounds__(GREEDY_WARPS * 32) k_greedy(const GreedyLev* levs, int nlev, int* err) {
+    __shared__ unsigned ticket;
+    int l = 0;
+    while (l + 1 < nlev && (int)blockIdx.x >= levs[l].blk1) ++l;
+    const GreedyLev V = levs[l];
+    const int lane = threadIdx.x & 31;
+    for (;;) {
+        __syncthreads();
+        if (threadIdx.x == 0) ticket = atomicAdd(V.ctr, 1u);
+        __syncthreads();
+        const int64_t q0 = (int64_t)ticket * GREEDY_WARPS;
+        if (q0 >= V.n) return;
+        const int q = (int)q0 + (threadIdx.x >> 5);
+        if (q >= V.n) continue;
+        const int i = V.order[q], p0 = V.ptr[i], p1 = V.ptr[i + 1];
+        for (int cb = 0;; cb += 64) {                          // colours [cb, cb + 64)
+            unsigned lo = 0u, hi = 0u;
+            for (int p = p0 + lane; p - lane < p1; p += 32) {
+                const int j = p < p1 ? V.col[p] : i;
+                const bool up = j != i && V.rank[j] < q;
+                int c = up ? colour_ld(V.colour + j) : 0;
+                for (int spin = 0; __any_sync(0xffffffffu, c < 0); ++spin) {
+                    if (spin == GREEDY_SPINS) {                // gives up: setup reports it
+                        if (c < 0) *err = 3;
+                        c = max(c, 0);
+                        break;
+                    }
+                    if (c < 0) c = colour_ld(V.colour + j);
+                }
+                if (up && c >= cb && c < cb + 32) lo |= 1u << (c - cb);
+                if (up && c >= cb + 32 && c < cb + 64) hi |= 1u << (c - cb - 32);
+            }
+            lo = __reduce_or_sync(0xffffffffu, lo);
+            hi = __reduce_or_sync(0xffffffffu, hi);
+            if (lo == ~0u && hi == ~0u) continue;
+            const int c = cb + (lo != ~0u ? __ffs((int)~lo) - 1 : 32 + __ffs((int)~hi) - 1);
+            if (lane == 0) asm volatile("st.relaxed.gpu.global.b32 [%0], %1;" ::"l"(V.colour + i), "r"(c) : "memory");
+            break;
+        }
     }
 }
 
@@ -2668,8 +2617,7 @@ void wavefront_levels(Handle& h, cudaStream_t s) {
 }
 
 // Smoothing colours of levels [0, nl - 1): the breadth-first parity 2-colouring if the pattern
-// graph is bipartite, else Jones-Plassmann with peel-round priority; all levels in one cooperative
-// launch of k_colour.
+// graph is bipartite, else the greedy colouring with peel-round priority.
 void colour_levels(Handle& h, cudaStream_t s) {
     const int nl = (int)h.lev.size();
     if (nl < 2) return;
@@ -2677,7 +2625,7 @@ void colour_levels(Handle& h, cudaStream_t s) {
     if (nj > COL_MAXL) fail(CPC_ESETUP, "too many levels to colour");
     int64_t tot = 0;
     for (int l = 0; l < nj; ++l) tot += h.lev[l].n;
-    Tmp<int> work((size_t)5 * tot, s), scal((size_t)COL_NS * nj, s), err(1, s);
+    Tmp<int> work((size_t)4 * tot, s), scal((size_t)COL_NS * nj, s), err(1, s);
     Tmp<unsigned long long> bar(1, s);
     Tmp<ColLev> dlev(nj, s);
     std::vector<ColLev> hl(nj);
@@ -2694,10 +2642,9 @@ void colour_levels(Handle& h, cudaStream_t s) {
         V.deg = work.get() + off;
         V.dec = V.deg + L.n;
         V.rnd = V.dec + L.n;
-        V.blk = V.rnd + L.n;
-        V.w = (unsigned*)(V.blk + L.n);
+        V.w = (unsigned*)(V.rnd + L.n);
         V.scal = scal.get() + (size_t)COL_NS * l;
-        off += (int64_t)5 * L.n;
+        off += (int64_t)4 * L.n;
         hs[(size_t)COL_NS * l + CS_DMIN] = INT_MAX;
         hs[(size_t)COL_NS * l + CS_DMIN + 1] = INT_MAX;
     }
@@ -2719,11 +2666,56 @@ void colour_levels(Handle& h, cudaStream_t s) {
     void* args[] = {(void*)&pl, &nn, &pbar, &perr};
     CPC_CK(cudaLaunchCooperativeKernel((void*)k_colour, grid, COL_TPB, args, 0, s));
     CPC_LAUNCH_CK();
+    CPC_CK(cudaMemcpyAsync(hs.data(), scal.get(), sizeof(int) * hs.size(), cudaMemcpyDeviceToHost, s));
     const int e = d2h(err.get(), s);
     if (e == 1) fail(CPC_ESETUP, "colouring: a grid barrier gave up");
     if (e == 2) fail(CPC_ESETUP, "peel rounds did not terminate");
-    if (e == 3) fail(CPC_ESETUP, "colouring did not terminate");
     if (e == 4) fail(CPC_ESETUP, "colouring: a union-find join did not complete");
+    // the levels that are not bipartite, sorted by priority together
+    std::vector<int> gl;
+    int64_t gn = 0;
+    for (int l = 0; l < nj; ++l)
+        if (hs[(size_t)COL_NS * l + CS_GREEDY]) {
+            gl.push_back(l);
+            gn += h.lev[l].n;
+        }
+    if (!gl.empty()) {
+        const int ng = (int)gl.size();
+        Tmp<uint64_t> key(gn, s), skey(gn, s);
+        Tmp<int> idx(gn, s), order(gn, s), rank(gn, s);
+        Tmp<unsigned> ctr(ng, s);
+        Tmp<GreedyLev> dg(ng, s);
+        std::vector<GreedyLev> hg(ng);
+        CPC_CK(cudaMemsetAsync(ctr.get(), 0, sizeof(unsigned) * ng, s));
+        int base = 0, blk = 0;
+        for (int g = 0; g < ng; ++g) {
+            const Level& L = h.lev[gl[g]];
+            k_greedy_key<<<nblk(L.n), TPB, 0, s>>>(L.n, g, hl[gl[g]].rnd, base, key.get(), idx.get());
+            GreedyLev& V = hg[g];
+            V.n = L.n;
+            V.ptr = L.A.ptr.p;
+            V.col = L.A.col.p;
+            V.order = order.get() + base;
+            V.rank = rank.get() + base;
+            V.colour = L.colour.p;
+            V.ctr = ctr.get() + g;
+            // points in flight: a few steps' worth of a level of 400,000 (700 points a step)
+            V.blk0 = blk;
+            blk += std::min(6 * sms, nblk(L.n, GREEDY_WARPS));
+            V.blk1 = blk;
+            base += L.n;
+        }
+        sort_pairs(key.get(), skey.get(), idx.get(), order.get(), gn, 64, s);
+        base = 0;
+        for (int g = 0; g < ng; ++g) {
+            k_greedy_rank<<<nblk(hg[g].n), TPB, 0, s>>>(hg[g].n, order.get() + base, rank.get() + base);
+            base += hg[g].n;
+        }
+        h2d(dg.get(), hg.data(), ng, s);
+        k_greedy<<<blk, GREEDY_WARPS * 32, 0, s>>>(dg.get(), ng, err.get());
+        CPC_LAUNCH_CK();
+        if (d2h(err.get(), s) == 3) fail(CPC_ESETUP, "colouring did not terminate");
+    }
     Tmp<int> mx(nj, s);
     CPC_CK(cudaMemsetAsync(mx.get(), 0, sizeof(int) * nj, s));
     for (int l = 0; l < nj; ++l) k_max_int<<<nblk(h.lev[l].n), TPB, 0, s>>>(h.lev[l].colour.p, h.lev[l].n, mx.get() + l);

@@ -1,0 +1,42 @@
+"""The greedy colouring at the edges of its kernel: equal to the oracle's, colour for colour.
+
+A block takes four points and a warp one, 32 entries of its row at a time and 64 colours at a time.
+"""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+if not torch.cuda.is_available():
+    pytest.skip("needs a GPU", allow_module_level=True)
+
+import oracle as O  # noqa: E402
+from paper_1205_6113_gb300 import cpc  # noqa: E402
+
+pytestmark = pytest.mark.gpu
+
+
+def cliques(sizes, seed):
+    """Disjoint complete graphs of the given sizes in a random order, a chain through their first points."""
+    n = int(np.sum(sizes))
+    name = np.random.default_rng(seed).permutation(n)
+    D = np.zeros((n, n))
+    first = np.cumsum(sizes) - sizes
+    for f, m in zip(first, sizes):
+        q = name[f:f + m]
+        D[np.ix_(q, q)] = -1.0
+    D[name[first[1:]], name[first[:-1]]] = D[name[first[:-1]], name[first[1:]]] = -0.5
+    np.fill_diagonal(D, 0.0)
+    np.fill_diagonal(D, 0.5 - D.sum(1))
+    r, c = np.nonzero(D)
+    ptr = np.concatenate(([0], np.cumsum(np.bincount(r, minlength=n))))
+    return n, ptr.astype(np.int32), c.astype(np.int32), D[r, c]
+
+
+@pytest.mark.parametrize("sizes", [[3], [3, 1], [4, 3, 2], [32, 1], [33, 2], [34, 31], [64, 1], [65, 3], [66, 129, 2]])
+def test_greedy_colours_match_the_oracle(sizes):
+    n, ptr, col, val = cliques(np.array(sizes), seed=sum(sizes))
+    s = cpc.Solver(ptr, col, val, coarse_max=1)
+    orc = O.Oracle(O.Csr(n, ptr, col, val), coarse_max=1)
+    _, colour = s.level_splitting(0)
+    assert np.array_equal(colour, orc.level_cf_colour(0)[1])
+    assert colour.max() + 1 == max(sizes)
