@@ -251,9 +251,15 @@ __global__ void k_max_int(const int* a, int n, int* out) {
     if (i < n) atomicMax(out, a[i]);
 }
 
+// One atomic per warp that could raise the maximum: one per entry took 670 us for 1M entries.
 __global__ void k_max_i64(const int64_t* a, int n, int64_t* out) {
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) atomicMax((unsigned long long*)out, (unsigned long long)a[i]);
+    int64_t m = 0;
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) m = a[i] > m ? a[i] : m;
+    for (int o = 16; o > 0; o >>= 1) {
+        const int64_t v = __shfl_xor_sync(0xffffffffu, m, o);
+        m = v > m ? v : m;
+    }
+    if ((threadIdx.x & 31) == 0 && m > 0) atomicMax((unsigned long long*)out, (unsigned long long)m);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -712,7 +718,7 @@ void spgemm(const Csr& A, const Csr& B, Csr& C, cudaStream_t s) {
     Tmp<int64_t> cnt(n + 1, s), off(n + 1, s), mx(1, s);
     k_prod_count<<<nblk(n + 1), TPB, 0, s>>>(n, A.ptr.p, A.col.p, B.ptr.p, cnt.get());
     CPC_CK(cudaMemsetAsync(mx.get(), 0, sizeof(int64_t), s));
-    k_max_i64<<<nblk(n), TPB, 0, s>>>(cnt.get(), n, mx.get());
+    k_max_i64<<<std::min(nblk(n), 304), TPB, 0, s>>>(cnt.get(), n, mx.get());
     exclusive_scan(cnt.get(), off.get(), n + 1, s);
     CPC_LAUNCH_CK();
     const int64_t most = d2h(mx.get(), s);
@@ -855,12 +861,12 @@ __device__ bool grid_bar(unsigned long long* ctr, unsigned long long& epoch, int
         asm volatile("red.release.gpu.global.add.u64 [%0], 1;" ::"l"(ctr) : "memory");
         const unsigned long long target = epoch * gridDim.x;
         const unsigned long long t0 = gtime_ns();
-        int good = 1;
+        int good = 1, polls = 0;
         for (;;) {
             unsigned long long v;
             asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(ctr) : "memory");
             if (v >= target) break;
-            if (*(volatile int*)err != 0 || gtime_ns() - t0 > GBAR_NS) {
+            if ((++polls & 15) == 0 && (*(volatile int*)err != 0 || gtime_ns() - t0 > GBAR_NS)) {
                 atomicCAS(err, 0, 1);
                 good = 0;
                 break;
@@ -892,19 +898,6 @@ __device__ int block_reduce(int v, Op op, int identity) {
     return v;                                                   // valid in thread 0
 }
 
-// The lowest 32 / COL_G set bits of a warp-uniform mask go to the groups of the warp, one each in
-// order: returns group g's bit (-1: none left for it) and clears them all.
-__device__ __forceinline__ int take_group_bit(unsigned& bits, int g) {
-    int mine = -1;
-#pragma unroll
-    for (int q = 0; q < 32 / COL_G; ++q) {
-        const int b = bits ? __ffs(bits) - 1 : -1;
-        if (q == g) mine = b;
-        if (bits) bits &= bits - 1;
-    }
-    return mine;
-}
-
 // ---------------------------------------------------------------------------------------------
 // The parity colourings and peel rounds of all levels run in one cooperative launch of k_colour; the
 // greedy colouring of the levels that are not bipartite follows (k_greedy).  Each level runs its own state
@@ -919,10 +912,10 @@ __device__ __forceinline__ int take_group_bit(unsigned& bits, int g) {
 //              parity of a point relative to it is its distance parity (all paths agree)
 //   check      any entry joining two points of equal parity: not bipartite, colours reset, go to
 //              peel rounds
-//   peel       round r, step 1: points with deg <= 2 dmin take round r and count a decrement on
-//              each neighbour in dec[]; step 2: the remaining points apply their decrements and
-//              the next dmin is their minimum (decrements counted on points taken in the same
-//              round are never read)
+//   peel       round r: points with deg <= 2 dmin take round r and take one off the degree of each
+//              neighbour that remains; the next dmin is the minimum of the remaining points'
+//              degrees as they were and of every decremented one (one step per round, where a step to
+//              mark and a step to count took two: 197 rounds of level 1 at 1M, with the list below 4.3 -> 2.1 ms)
 // The CTAs of a step are shared among the levels with work in that step, in proportion to their
 // points (at least one each); a CTA works on one level.
 // ---------------------------------------------------------------------------------------------
@@ -933,15 +926,17 @@ struct ColLev {
     const int* ptr;
     const int* col;
     int* colour;
-    int *deg, *dec, *rnd;
+    int4* cnt;                                // degrees while the rounds run, see below
+    int* rnd;
     unsigned* w;                              // union-find words
     int* scal;                                // COL_NS counters, see below
 };
 
-// scal of a level: [0], [1] dmin of even / odd peel rounds; [2] 1 when the peel rounds are done: the
-// level is not bipartite; [3] triangle found; [4] not bipartite or a join failed.
-enum { CS_DMIN = 0, CS_GREEDY = 2, CS_TRI = 3, CS_BAD = 4, COL_NS = 6 };
-enum { CP_INIT, CP_UNION, CP_FIND, CP_CHECK, CP_RESET, CP_MARK, CP_MIN, CP_DONE };
+// scal of a level: [0..2] dmin of peel round r in slot r % 3 (a slot is cleared one round before it is
+// added to and read one barrier after); [3] 1 when the peel rounds are done: the level is not bipartite;
+// [4] triangle found; [5] not bipartite or a join failed.
+enum { CS_DMIN = 0, CS_GREEDY = 3, CS_TRI = 4, CS_BAD = 5, COL_NS = 6 };
+enum { CP_INIT, CP_UNION, CP_FIND, CP_CHECK, CP_RESET, CP_PEEL, CP_DONE };
 
 // Union-find words: parent << 1 | parity relative to the parent (a root: itself, parity 0).
 // Returns the root of x and x's parity relative to it, halving the path on the way (a point is
@@ -1014,15 +1009,13 @@ __device__ void col_step(const ColLev& V, int phase, int rnd_no, int dm, int t, 
     const int n = V.n;
     const int* ptr = V.ptr;
     const int* col = V.col;
-    const int lane = threadIdx.x & 31, gl = lane % COL_G, gs = lane - gl;
-    const unsigned gm = ((1u << COL_G) - 1u) << gs;
+    const int gl = threadIdx.x % COL_G;
     if (phase == CP_INIT) {
         int m = INT_MAX, tri = 0;
         for (int i = t; i < n; i += T) {
             int d = 0;
             for (int p = ptr[i]; p < ptr[i + 1]; ++p) d += col[p] != i;
-            V.deg[i] = d;
-            V.dec[i] = 0;
+            V.cnt[i] = make_int4(d, 0, d, 0);
             V.rnd[i] = -1;
             V.colour[i] = -1;
             V.w[i] = (unsigned)i << 1;
@@ -1059,52 +1052,67 @@ __device__ void col_step(const ColLev& V, int phase, int rnd_no, int dm, int t, 
         if (threadIdx.x == 0 && bad) atomicOr(&V.scal[CS_BAD], 1);
     } else if (phase == CP_RESET) {
         for (int i = t; i < n; i += T) V.colour[i] = -1;
-    } else if (phase == CP_MARK) {
-        for (int b0 = t - lane; b0 < n; b0 += COL_K * T) {     // warp-uniform trip count
-            bool take[COL_K];
+    } else if (phase == CP_PEEL) {
+        // cnt = (c0, c1, s0, s1), degree = c0 + c1: round r takes its decrements off c_p, p = r & 1, while
+        // c_q of the other parity and s_p = c_p as the round began stand still, so that c_q + s_p is the
+        // degree at the round's beginning to whoever asks; the owner keeps s_q = c_q for the next round.
+        // The taken points of a batch go through a list to all groups of the CTA: few are taken in most rounds,
+        // and a warp that went through its own one after the other held up everyone (26 us a round, 9 now).
+        __shared__ int list[COL_K * COL_TPB], nlist;
+        const bool odd = rnd_no & 1;
+        int m = INT_MAX;
+        for (int b0 = t - threadIdx.x; b0 < n; b0 += COL_K * T) {   // CTA-uniform trip count
+            int rv[COL_K];
+            int4 cv[COL_K];
+            if (threadIdx.x == 0) nlist = 0;
+            __syncthreads();
 #pragma unroll
             for (int k = 0; k < COL_K; ++k) {                   // loads of COL_K points in flight
-                const int i = b0 + k * T + lane;
-                take[k] = i < n && __ldcg(&V.rnd[i]) < 0 && __ldcg(&V.deg[i]) <= 2 * dm;
+                const int i = b0 + k * T + threadIdx.x;
+                rv[k] = i < n ? __ldcg(&V.rnd[i]) : 0;
             }
 #pragma unroll
+            for (int k = 0; k < COL_K; ++k)
+                if (rv[k] < 0) cv[k] = __ldcg(&V.cnt[b0 + k * T + threadIdx.x]);
+#pragma unroll
             for (int k = 0; k < COL_K; ++k) {
-                const int base = b0 + k * T;
-                if (take[k]) V.rnd[base + lane] = rnd_no;
-                unsigned bits = __ballot_sync(0xffffffffu, take[k]);
-                while (bits) {                                  // a taken point per group at a time
-                    const int mine = take_group_bit(bits, gs / COL_G);
-                    if (mine >= 0) {
-                        const int ip = base + mine;
-                        for (int p = ptr[ip] + gl; p < ptr[ip + 1]; p += COL_G)
-                            if (col[p] != ip) atomicSub(&V.dec[col[p]], 1);
+                const int i = b0 + k * T + threadIdx.x;
+                if (rv[k] >= 0) continue;
+                const int cq = odd ? cv[k].x : cv[k].y, d = cq + (odd ? cv[k].w : cv[k].z);
+                if (d <= 2 * dm) {
+                    V.rnd[i] = rnd_no;
+                    list[atomicAdd(&nlist, 1)] = i;
+                } else {
+                    m = imin(m, d);
+                    (odd ? V.cnt[i].z : V.cnt[i].w) = cq;
+                }
+            }
+            __syncthreads();
+            for (int q = threadIdx.x / COL_G; q < nlist; q += COL_TPB / COL_G) {
+                const int ip = list[q], p1 = ptr[ip + 1];
+                for (int p = ptr[ip] + gl; p < p1; p += 2 * COL_G) {
+                    int j[2], rj[2];
+                    int4 cj[2];
+#pragma unroll
+                    for (int u = 0; u < 2; ++u) j[u] = p + u * COL_G < p1 ? col[p + u * COL_G] : ip;
+#pragma unroll
+                    for (int u = 0; u < 2; ++u) {
+                        rj[u] = j[u] != ip ? __ldcg(&V.rnd[j[u]]) : 0;
+                        cj[u] = __ldcg(&V.cnt[j[u]]);
+                    }
+#pragma unroll
+                    for (int u = 0; u < 2; ++u) {
+                        const int cq = odd ? cj[u].x : cj[u].y, d = cq + (odd ? cj[u].w : cj[u].z);
+                        // remaining after this round: the last of its decrements returns its next degree
+                        if (rj[u] < 0 && d > 2 * dm)
+                            m = imin(m, cq + atomicSub(odd ? &V.cnt[j[u]].y : &V.cnt[j[u]].x, 1) - 1);
                     }
                 }
             }
-        }
-    } else if (phase == CP_MIN) {
-        int m = INT_MAX;
-        for (int i0 = t; i0 < n; i0 += COL_K * T) {
-            int rv[COL_K], dv[COL_K], ev[COL_K];
-#pragma unroll
-            for (int k = 0; k < COL_K; ++k) {                   // loads of COL_K points in flight
-                const int i = i0 + k * T;
-                rv[k] = i < n ? __ldcg(&V.rnd[i]) : 0;
-                dv[k] = i < n ? __ldcg(&V.deg[i]) : 0;
-                ev[k] = i < n ? __ldcg(&V.dec[i]) : 0;
-            }
-#pragma unroll
-            for (int k = 0; k < COL_K; ++k) {
-                const int i = i0 + k * T;
-                if (i >= n || rv[k] >= 0) continue;
-                const int d = dv[k] + ev[k];
-                V.deg[i] = d;
-                V.dec[i] = 0;
-                m = imin(m, d);
-            }
+            __syncthreads();
         }
         m = block_reduce(m, imin, INT_MAX);
-        if (threadIdx.x == 0 && m != INT_MAX) atomicMin(&V.scal[CS_DMIN + ((rnd_no + 1) & 1)], m);
+        if (threadIdx.x == 0 && m != INT_MAX) atomicMin(&V.scal[CS_DMIN + (rnd_no + 1) % 3], m);
     }
 }
 
@@ -1142,7 +1150,7 @@ __global__ void __launch_bounds__(COL_TPB) k_colour(const ColLev* levs, int nlev
                     const int p = ph[l];
                     if (p == CP_INIT) {
                         if (step == 0) { work[l] = CP_INIT; break; }
-                        ph[l] = c[CS_TRI] ? CP_MARK : CP_UNION;
+                        ph[l] = c[CS_TRI] ? CP_PEEL : CP_UNION;
                         rr[l] = 0;
                         if (ph[l] == CP_UNION) { work[l] = CP_UNION; break; }
                     } else if (p == CP_UNION) {
@@ -1163,21 +1171,18 @@ __global__ void __launch_bounds__(COL_TPB) k_colour(const ColLev* levs, int nlev
                         }
                         break;
                     } else if (p == CP_RESET) {
-                        ph[l] = CP_MARK;
+                        ph[l] = CP_PEEL;
                         rr[l] = 0;
-                    } else if (p == CP_MARK) {
-                        dmv[l] = c[CS_DMIN + (rr[l] & 1)];
+                    } else if (p == CP_PEEL) {
+                        dmv[l] = c[CS_DMIN + rr[l] % 3];
                         if (dmv[l] == INT_MAX) {
                             if (first) g[CS_GREEDY] = 1;
                             ph[l] = CP_DONE;
                             break;
                         }
                         if (rr[l] > n + 16) { if (first) atomicCAS(err, 0, 2); quit = 1; break; }
-                        if (first) g[CS_DMIN + ((rr[l] + 1) & 1)] = INT_MAX;
-                        work[l] = CP_MARK;
-                        break;
-                    } else if (p == CP_MIN) {
-                        work[l] = CP_MIN;
+                        if (first) g[CS_DMIN + (rr[l] + 2) % 3] = INT_MAX;
+                        work[l] = CP_PEEL;
                         break;
                     } else {
                         break;                                  // done
@@ -1202,7 +1207,7 @@ __global__ void __launch_bounds__(COL_TPB) k_colour(const ColLev* levs, int nlev
                 for (int l = 0; l < nlev && mine < 0; ++l) {
                     if (work[l] < 0) continue;
                     wacc += lv[l].n;
-                    const int c1 = (int)(((long long)spare * wacc) / wsum) + (++cs);
+                    const int c1 = (wacc == wsum ? spare : (int)(((long long)spare * wacc) / wsum)) + (++cs);
                     if ((int)blockIdx.x >= c0 && (int)blockIdx.x < c1) {
                         mine = l;
                         c0s = c0;
@@ -1218,17 +1223,13 @@ __global__ void __launch_bounds__(COL_TPB) k_colour(const ColLev* levs, int nlev
         if (quit == 3) continue;
         if (mine >= 0) {
             const int l = mine;
-            col_step(lv[l], work[l], rr[l], work[l] == CP_MARK ? dmv[l] : 0, ((int)blockIdx.x - c0s) * COL_TPB + threadIdx.x,
+            col_step(lv[l], work[l], rr[l], work[l] == CP_PEEL ? dmv[l] : 0, ((int)blockIdx.x - c0s) * COL_TPB + threadIdx.x,
                      cns * COL_TPB);
         }
         __syncthreads();
         if (lead) {                                             // advance the phases worked in this step
             for (int l = 0; l < nlev; ++l) {
-                if (work[l] == CP_MARK) ph[l] = CP_MIN;
-                else if (work[l] == CP_MIN) {
-                    ph[l] = CP_MARK;
-                    ++rr[l];
-                }
+                if (work[l] == CP_PEEL) ++rr[l];
             }
         }
         if (!grid_bar(bar, epoch, err)) return;
@@ -1466,39 +1467,43 @@ __device__ __forceinline__ bool sell_keep(int mode, int j, int i) {
     }
 }
 
-// Entries of each chunk (padded to its widest row).  With a group key per row (smoother copy) the two
-// parts are padded apart: low[k] = entries of the part of earlier groups.  wmax[0..2]: the largest
-// chunk, low part and high part.  Columns of key 0 make the first part when by_col (the rows have no
-// key then: a transfer, its columns keyed by the fine colour).
-__global__ void k_sell_width(const int* perm, int nchunks, int C, const int* ptr, const int* col, int mode,
-                             const int* key, bool by_col, int* width, int* low, int* wmax) {
-    int k = blockIdx.x * blockDim.x + threadIdx.x;
-    int w = 0, wl = 0;
-    if (k < nchunks) {
-        for (int l = 0; l < C; ++l) {
-            const int i = perm[k * C + l];
-            if (i < 0) continue;
-            const int ki = !key ? 0 : by_col ? 1 : key[i];
-            int c = 0, cl = 0;
-            for (int p = ptr[i]; p < ptr[i + 1]; ++p)
-                if (sell_keep(mode, col[p], i)) {
-                    if (key && key[col[p]] < ki) ++cl;
-                    else ++c;
-                }
-            w = max(w, c);
-            wl = max(wl, cl);
-        }
-        width[k] = (w + wl) * C;
-        if (low) low[k] = wl * C;
-    } else if (k == nchunks) {
-        width[k] = 0;
+// Entries of each chunk (padded to its widest row), a warp per chunk and 32 / C lanes per row.  With a
+// group key per row (smoother copy) the two parts are padded apart: low[k] = entries of the part of earlier
+// groups.  wmax[0..2]: the largest chunk, low part and high part.  Columns of key 0 make the first part when
+// by_col (the rows have no key then: a transfer, its columns keyed by the fine colour).  (A thread per chunk
+// walked C rows one after the other: 100 us for 1M entries, 10 with this.)
+__global__ void __launch_bounds__(TPB) k_sell_width(const int* perm, int nchunks, int C, const int* ptr, const int* col,
+                                                    int mode, const int* key, bool by_col, int* width, int* low,
+                                                    int* wmax) {
+    __shared__ int part[3][TPB / 32];
+    const int k = blockIdx.x * (TPB / 32) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    int c = 0, cl = 0;
+    const int i = k < nchunks ? perm[k * C + lane % C] : -1;
+    if (i >= 0) {
+        const int ki = !key ? 0 : by_col ? 1 : key[i];
+        for (int p = ptr[i] + lane / C; p < ptr[i + 1]; p += 32 / C)
+            if (sell_keep(mode, col[p], i)) {
+                if (key && key[col[p]] < ki) ++cl;
+                else ++c;
+            }
     }
-    const int mt = __reduce_max_sync(0xffffffffu, (w + wl) * C), ml = __reduce_max_sync(0xffffffffu, wl * C),
-              mu = __reduce_max_sync(0xffffffffu, w * C);
-    if ((threadIdx.x & 31) == 0) {
-        atomicMax(wmax, mt);
-        atomicMax(wmax + 1, ml);
-        atomicMax(wmax + 2, mu);
+    for (int o = C; o < 32; o <<= 1) {                          // a row's lanes: lane, lane + C, ...
+        c += __shfl_xor_sync(0xffffffffu, c, o);
+        cl += __shfl_xor_sync(0xffffffffu, cl, o);
+    }
+    const int w = __reduce_max_sync(0xffffffffu, c), wl = __reduce_max_sync(0xffffffffu, cl);
+    if (lane == 0) {
+        if (k <= nchunks) width[k] = (w + wl) * C;              // width[nchunks] = 0
+        if (low && k < nchunks) low[k] = wl * C;
+        part[0][threadIdx.x >> 5] = (w + wl) * C;
+        part[1][threadIdx.x >> 5] = wl * C;
+        part[2][threadIdx.x >> 5] = w * C;
+    }
+    __syncthreads();
+    if (threadIdx.x < 3) {
+        int m = 0;
+        for (int q = 0; q < TPB / 32; ++q) m = max(m, part[threadIdx.x][q]);
+        if (m > 0) atomicMax(wmax + threadIdx.x, m);
     }
 }
 
@@ -1567,9 +1572,11 @@ __global__ void k_flag_later(int nslots, int C, const int* perm, const int* cptr
 
 // Slot order from a per-row group key (colour or level): rows sorted by (key, row), each group
 // padded to a multiple of the chunk height C.  Returns the chunk boundaries of the groups in seg.
-__global__ void k_group_count(int n, const int* key, int* cnt) {
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) atomicAdd(&cnt[key[i]], 1);
+// The first row of each group among the sorted keys (-1 where the group has none): no counting by atomics,
+// which a few groups of many rows serialise (two colours of 1M rows: 330 us).
+__global__ void k_group_start(int n, const int* skey, int* start) {
+    int t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t < n && (t == 0 || skey[t] != skey[t - 1])) start[skey[t]] = t;
 }
 
 __global__ void k_group_scatter(int n, const int* skey, const int* srow, const int* gstart, const int* sstart,
@@ -1582,25 +1589,28 @@ __global__ void k_group_scatter(int n, const int* skey, const int* srow, const i
 
 // Build perm (device, nslots) from a group key per row; ngroups known.
 void grouped_slots(int n, const int* key, int ngroups, int C, cudaStream_t s, DBuf<int>& perm, int& nslots,
-                   std::vector<int>& seg, DBuf<int>* sorted_rows = nullptr) {
-    Tmp<int> rows(n, s), skey(n, s), srow(n, s), cnt(ngroups, s);
+                   std::vector<int>& seg, DBuf<int>* sorted_rows = nullptr, std::vector<int>* counts = nullptr) {
+    Tmp<int> rows(n, s), skey(n, s), srow(n, s), first(ngroups, s);
     k_iota<<<nblk(n), TPB, 0, s>>>(rows.get(), n);
     sort_pairs(key, skey.get(), rows.get(), srow.get(), n, bits_for((uint64_t)std::max(1, ngroups)), s);
-    CPC_CK(cudaMemsetAsync(cnt.get(), 0, sizeof(int) * ngroups, s));
-    k_group_count<<<nblk(n), TPB, 0, s>>>(n, key, cnt.get());
-    std::vector<int> hc(ngroups);
-    CPC_CK(cudaMemcpyAsync(hc.data(), cnt.get(), sizeof(int) * ngroups, cudaMemcpyDeviceToHost, s));
+    k_fill_int<<<nblk(ngroups), TPB, 0, s>>>(first.get(), ngroups, -1);
+    k_group_start<<<nblk(n), TPB, 0, s>>>(n, skey.get(), first.get());
+    std::vector<int> gstart(ngroups), sstart(ngroups), hc(ngroups);
+    CPC_CK(cudaMemcpyAsync(gstart.data(), first.get(), sizeof(int) * ngroups, cudaMemcpyDeviceToHost, s));
     CPC_CK(cudaStreamSynchronize(s));
-    std::vector<int> gstart(ngroups), sstart(ngroups);
+    for (int g = ngroups - 1, end = n; g >= 0; --g) {
+        if (gstart[g] < 0) gstart[g] = end;
+        hc[g] = end - gstart[g];
+        end = gstart[g];
+    }
     seg.assign(ngroups + 1, 0);
-    int g0 = 0, s0 = 0;
+    int s0 = 0;
     for (int g = 0; g < ngroups; ++g) {
-        gstart[g] = g0;
         sstart[g] = s0;
         seg[g] = s0 / C;
-        g0 += hc[g];
         s0 += (hc[g] + C - 1) / C * C;
     }
+    if (counts) *counts = hc;
     seg[ngroups] = s0 / C;
     nslots = s0;
     perm.alloc_async(nslots, s);                                // a temporary slot order
@@ -1651,7 +1661,7 @@ void build_sell(const int* ptr, const int* col, const double* val, const DBuf<in
     S.seg = seg;
     Tmp<int> width(S.nchunks + 1, s), low(key ? S.nchunks : 0, s), wmax(3, s);
     CPC_CK(cudaMemsetAsync(wmax.get(), 0, 3 * sizeof(int), s));
-    k_sell_width<<<nblk(S.nchunks + 1), TPB, 0, s>>>(slots.p, S.nchunks, C, ptr, col, mode, key, by_col, width.get(),
+    k_sell_width<<<nblk(S.nchunks + 1, TPB / 32), TPB, 0, s>>>(slots.p, S.nchunks, C, ptr, col, mode, key, by_col, width.get(),
                                                      key ? low.get() : nullptr, wmax.get());
     S.cptr.alloc(S.nchunks + 1);
     exclusive_scan(width.get(), S.cptr.p, S.nchunks + 1, s);
@@ -1678,24 +1688,31 @@ void build_sell(const int* ptr, const int* col, const double* val, const DBuf<in
     CPC_LAUNCH_CK();
 }
 
-// Distinct off-diagonal offsets col - row of the rows, into a table of 8 (EMPTY = INT_MIN: no offset
-// can be INT_MIN); *over = 1 when there are more than 8.
-__global__ void k_dia_offsets(int n, const int* ptr, const int* col, int* table, int* over) {
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
+// The offset's place in a table of 8 (EMPTY = INT_MIN: no offset can be INT_MIN); false when it is full.
+__device__ __forceinline__ bool dia_insert(int* table, int off) {
     volatile int* vt = table;
-    for (int p = ptr[i]; p < ptr[i + 1]; ++p) {
-        const int j = col[p];
-        if (j == i) continue;
-        const int off = j - i;
-        bool found = false;
-        for (int t = 0; t < 8 && !found; ++t) {
-            int cur = vt[t];
-            if (cur == INT_MIN) cur = atomicCAS(table + t, INT_MIN, off);
-            found = cur == INT_MIN || cur == off;
-        }
-        if (!found) *over = 1;
+    for (int t = 0; t < 8; ++t) {
+        int cur = vt[t];
+        if (cur == INT_MIN) cur = atomicCAS(table + t, INT_MIN, off);
+        if (cur == INT_MIN || cur == off) return true;
     }
+    return false;
+}
+
+// Distinct off-diagonal offsets col - row of the rows into the table; *over = 1 when there are more than 8.
+// Each block collects its rows' in shared memory first: with all threads on the one table in L2 1M rows
+// took 230 us, 35 with this.
+__global__ void k_dia_offsets(int n, const int* ptr, const int* col, int* table, int* over) {
+    __shared__ int tab[8];
+    if (threadIdx.x < 8) tab[threadIdx.x] = INT_MIN;
+    __syncthreads();
+    bool fit = true;
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n && fit; i += gridDim.x * blockDim.x)
+        for (int p = ptr[i]; p < ptr[i + 1] && fit; ++p)
+            if (col[p] != i) fit = dia_insert(tab, col[p] - i);
+    __syncthreads();
+    if (threadIdx.x < 8 && tab[threadIdx.x] != INT_MIN) fit = dia_insert(table, tab[threadIdx.x]) && fit;
+    if (!fit) *over = 1;
 }
 
 // dval[d * nslots + s] = a_{i, i + off_d} for slot s = row i (0 where absent or padding).
@@ -1726,7 +1743,7 @@ void build_dia(int n, const int* ptr, const int* col, const double* val, Sell& S
     Tmp<int> table(8, s), over(1, s);
     k_fill_int<<<1, 32, 0, s>>>(table.get(), 8, INT_MIN);
     CPC_CK(cudaMemsetAsync(over.get(), 0, sizeof(int), s));
-    k_dia_offsets<<<nblk(n), TPB, 0, s>>>(n, ptr, col, table.get(), over.get());
+    k_dia_offsets<<<std::min(nblk(n), 1216), TPB, 0, s>>>(n, ptr, col, table.get(), over.get());
     CPC_LAUNCH_CK();
     int t[8];
     CPC_CK(cudaMemcpyAsync(t, table.get(), sizeof(t), cudaMemcpyDeviceToHost, s));
@@ -2446,16 +2463,8 @@ void setup_ic0(Handle& h, cudaStream_t s) {
     DBuf<int> slotsL, rowsL;
     int nslotsL = 0;
     std::vector<int> segL;
-    grouped_slots(n, lvl.get(), h.ic_levels_L, CHUNK, s, slotsL, nslotsL, segL, &rowsL);
-    // level g has rows rowsL[gstart..], count from segments: recompute counts from the slot layout
-    std::vector<int> hc(h.ic_levels_L);
-    {
-        Tmp<int> cnt(h.ic_levels_L, s);
-        CPC_CK(cudaMemsetAsync(cnt.get(), 0, sizeof(int) * h.ic_levels_L, s));
-        k_group_count<<<nblk(n), TPB, 0, s>>>(n, lvl.get(), cnt.get());
-        CPC_CK(cudaMemcpyAsync(hc.data(), cnt.get(), sizeof(int) * h.ic_levels_L, cudaMemcpyDeviceToHost, s));
-        CPC_CK(cudaStreamSynchronize(s));
-    }
+    std::vector<int> hc;
+    grouped_slots(n, lvl.get(), h.ic_levels_L, CHUNK, s, slotsL, nslotsL, segL, &rowsL, &hc);
     h.ic_rows_L1 = h.ic_levels_L > 1 ? hc[1] : 0;
     Tmp<int> failrow(1, s);
     k_fill_int<<<1, 1, 0, s>>>(failrow.get(), 1, INT_MAX);
@@ -2541,32 +2550,38 @@ void setup_ic_rb(Handle& h, bool colour_ic, cudaStream_t s) {
 void setup_level_sells(Level& L, cudaStream_t s, bool last, bool tune, bool fp64) {
     // colour-grouped A_l (Gauss-Seidel and residual)
     if (!last) {
-        auto build_grouped = [&](int C, Sell& out) {
-            DBuf<int> slots;
-            int nslots = 0;
-            std::vector<int> seg;
-            grouped_slots(L.n, L.colour.p, L.ncolours, C, s, slots, nslots, seg);
+        DBuf<int> slots;
+        int nslots = 0;
+        std::vector<int> seg;
+        auto group = [&](int C) { grouped_slots(L.n, L.colour.p, L.ncolours, C, s, slots, nslots, seg); };
+        auto build = [&](int C, Sell& out) {
             build_sell(L.A.ptr.p, L.A.col.p, L.A.val.p, slots, nslots, seg, C, SELL_OFFDIAG, true, nullptr, out, s,
                        fp64 ? L.colour.p : nullptr);
             CPC_CK(cudaStreamSynchronize(s));
         };
-        const int ca = choose_chunk((double)(L.A.nnz - L.n) / std::max(1, L.n));
-        build_grouped(ca, L.S);
-        if (!tune && ca < 32) {
+        auto build_grouped = [&](int C, Sell& out) {
+            group(C);
+            build(C, out);
+        };
+        int ca = choose_chunk((double)(L.A.nnz - L.n) / std::max(1, L.n)), widest = 0;
+        group(ca);
+        for (size_t c = 0; c + 1 < seg.size(); ++c) widest = std::max(widest, seg[c + 1] - seg[c]);
+        // FP64 issue bounds a colour that takes many waves of warps, and adding the partial sums of a row's
+        // lanes costs as much of it as a few entries: twice the chunk height, half the lanes per row
+        // (level 1 at 8.4M: 300 -> 264 us a sweep).
+        const bool many = !tune && fp64 && ca < 32 && widest > 4 * GS_RESIDENT_WARPS;
+        if (many) group(ca *= 2);
+        build(ca, L.S);
+        if (!tune && !many && ca < 32) {
             // One wave: a colour step whose blocks do not all fit on the GPU at once runs in two waves, and
             // only the first wave's matrix loads overlap the previous step.  If the widest colour needs more
-            // blocks than fit (by the registers of the batch width) and twice the chunk height (half the
-            // lanes per row, about twice the entries per lane) would fit, take twice the chunk height
-            // (level 1 at 1M, FP64: 55 -> 49 us a sweep).  In FP64 also where a colour takes many waves: FP64
-            // issue bounds it then, and adding the partial sums of a row's lanes costs as much of it as a
-            // few entries (level 1 at 8.4M: 300 -> 264 us).
-            int widest = 0, sms = 0, dev = 0;
-            for (size_t c = 0; c + 1 < L.S.seg.size(); ++c) widest = std::max(widest, L.S.seg[c + 1] - L.S.seg[c]);
+            // blocks than fit (by the registers of the batch width) and twice the chunk height would fit,
+            // take twice the chunk height (level 1 at 1M, FP64: 55 -> 49 us a sweep).
+            int sms = 0, dev = 0;
             CPC_CK(cudaGetDevice(&dev));
             CPC_CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
             const int per_sm = L.S.lanes <= 4 ? 16 : L.S.lanes <= 6 ? 12 : L.S.lanes <= 8 ? 9 : L.S.lanes <= 12 ? 8 : 6;
-            const bool one_wave = (widest + 3) / 4 > per_sm * sms && (widest / 2 + 4) / 4 <= 6 * sms;
-            if (one_wave || (fp64 && widest > 4 * GS_RESIDENT_WARPS)) build_grouped(2 * ca, L.S);
+            if ((widest + 3) / 4 > per_sm * sms && (widest / 2 + 4) / 4 <= 6 * sms) build_grouped(2 * ca, L.S);
         }
         if (tune) {
             float best = time_gs_sweep(L.S, L.n);
@@ -2625,7 +2640,8 @@ void colour_levels(Handle& h, cudaStream_t s) {
     if (nj > COL_MAXL) fail(CPC_ESETUP, "too many levels to colour");
     int64_t tot = 0;
     for (int l = 0; l < nj; ++l) tot += h.lev[l].n;
-    Tmp<int> work((size_t)4 * tot, s), scal((size_t)COL_NS * nj, s), err(1, s);
+    Tmp<int4> cnts(tot, s);
+    Tmp<int> work((size_t)2 * tot, s), scal((size_t)COL_NS * nj, s), err(1, s);
     Tmp<unsigned long long> bar(1, s);
     Tmp<ColLev> dlev(nj, s);
     std::vector<ColLev> hl(nj);
@@ -2639,14 +2655,12 @@ void colour_levels(Handle& h, cudaStream_t s) {
         V.ptr = L.A.ptr.p;
         V.col = L.A.col.p;
         V.colour = L.colour.p;
-        V.deg = work.get() + off;
-        V.dec = V.deg + L.n;
-        V.rnd = V.dec + L.n;
+        V.cnt = cnts.get() + off / 2;
+        V.rnd = work.get() + off;
         V.w = (unsigned*)(V.rnd + L.n);
         V.scal = scal.get() + (size_t)COL_NS * l;
-        off += (int64_t)4 * L.n;
-        hs[(size_t)COL_NS * l + CS_DMIN] = INT_MAX;
-        hs[(size_t)COL_NS * l + CS_DMIN + 1] = INT_MAX;
+        off += (int64_t)2 * L.n;
+        for (int q = 0; q < 3; ++q) hs[(size_t)COL_NS * l + CS_DMIN + q] = INT_MAX;
     }
     CPC_CK(cudaMemcpyAsync(dlev.get(), hl.data(), sizeof(ColLev) * nj, cudaMemcpyHostToDevice, s));
     CPC_CK(cudaMemcpyAsync(scal.get(), hs.data(), sizeof(int) * hs.size(), cudaMemcpyHostToDevice, s));
