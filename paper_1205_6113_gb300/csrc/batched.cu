@@ -645,6 +645,11 @@ __device__ __forceinline__ int vfirst(int n) {
     return g < vblocks(n) * 4 ? g : n;
 }
 
+// Rows whose loads a warp keeps in flight together: u of them, fewer where a lane has more columns.  The
+// order of the sums is that of one row after another.  (64 columns at 1M, 608 blocks, one row against u:
+// r.z 0.53 -> 0.31 ms, p 0.57 -> 0.24 ms, an iteration 9.84 -> 9.16 ms.)
+__host__ __device__ constexpr int vrows(int J, int u) { return J <= 2 ? u : u / 2; }
+
 template <int J, int R, class Fin>
 __device__ void col_finish(int n, bool ordered, double (&v)[J], double* part, unsigned* ctr, Fin fin) {
     constexpr int KP = Cols<J, R>::KP, SETS = VWARPS * R / 4;
@@ -777,19 +782,30 @@ __global__ void kb_guard(cudaGraphConditionalHandle cond) {
 }
 
 template <int J, int R, class ZT>
-__global__ void __launch_bounds__(VTPB) kb_rz(int n, const double* r, const ZT* z, double* part, unsigned* ctr, double* S, bool ordered) {
+__global__ void __launch_bounds__(VTPB, 4) kb_rz(int n, const double* r, const ZT* z, double* part, unsigned* ctr, double* S, bool ordered) {
     using L = Cols<J, R>;
     constexpr int Kp = L::KP;
     pdl_launch_dependents();
     pdl_wait();
+    constexpr int U = vrows(J, 4);
+    const int step = 4 * vblocks(n);
     double v[J];
     zero(v);
-    for (int i = vfirst<J, R>(n); i < n; i += 4 * vblocks(n)) {
-        double ri[J], zi[J];
-        ldv<J>(r + L::at(i), ri);
-        ldv<J>(z + L::at(i), zi);
+    for (int i0 = vfirst<J, R>(n); i0 < n; i0 += U * step) {
+        double ri[U][J], zi[U][J];
 #pragma unroll
-        for (int j = 0; j < J; ++j) v[j] += ri[j] * zi[j];
+        for (int u = 0; u < U; ++u) {
+            const int i = i0 + u * step;
+            if (i >= n) break;
+            ldv<J>(r + L::at(i), ri[u]);
+            ldv<J>(z + L::at(i), zi[u]);
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            if (i0 + u * step >= n) break;
+#pragma unroll
+            for (int j = 0; j < J; ++j) v[j] += ri[u][j] * zi[u][j];
+        }
     }
     col_finish<J, R>(n, ordered, v, part, ctr, [&](int c, double t) {
         const bool act = S[S_ACTIVE * Kp + c] > 0.0;
@@ -804,7 +820,7 @@ __global__ void __launch_bounds__(VTPB) kb_rz(int n, const double* r, const ZT* 
 }
 
 template <int J, int R, class ZT>
-__global__ void __launch_bounds__(VTPB) kb_p(int n, const ZT* z, double* __restrict__ p, const double* S) {
+__global__ void __launch_bounds__(VTPB, 4) kb_p(int n, const ZT* z, double* __restrict__ p, const double* S) {
     using L = Cols<J, R>;
     constexpr int Kp = L::KP;
     pdl_launch_dependents();
@@ -812,13 +828,25 @@ __global__ void __launch_bounds__(VTPB) kb_p(int n, const ZT* z, double* __restr
     double beta[J], k[J];
     ldv<J>(S + S_BETA * Kp + L::col(), beta);
     ldv<J>(S + S_K * Kp + L::col(), k);
-    for (int i = vfirst<J, R>(n); i < n; i += 4 * vblocks(n)) {
-        double zi[J], pi[J];
-        ldv<J>(z + L::at(i), zi);
-        ldv<J>(p + L::at(i), pi);
+    constexpr int U = vrows(J, 4);
+    const int step = 4 * vblocks(n);
+    for (int i0 = vfirst<J, R>(n); i0 < n; i0 += U * step) {
+        double zi[U][J], pi[U][J];
 #pragma unroll
-        for (int j = 0; j < J; ++j) pi[j] = k[j] == 0.0 ? zi[j] : zi[j] + beta[j] * pi[j];
-        stv<J>(p + L::at(i), pi);
+        for (int u = 0; u < U; ++u) {
+            const int i = i0 + u * step;
+            if (i >= n) break;
+            ldv<J>(z + L::at(i), zi[u]);
+            ldv<J>(p + L::at(i), pi[u]);
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int i = i0 + u * step;
+            if (i >= n) break;
+#pragma unroll
+            for (int j = 0; j < J; ++j) pi[u][j] = k[j] == 0.0 ? zi[u][j] : zi[u][j] + beta[j] * pi[u][j];
+            stv<J>(p + L::at(i), pi[u]);
+        }
     }
 }
 
@@ -885,7 +913,7 @@ __global__ void __launch_bounds__(VTPB) kb_spmv_pq_dia(BD<double, double> A, con
 }
 
 template <int J, int R>
-__global__ void __launch_bounds__(VTPB) kb_update(int n, double* __restrict__ x, double* __restrict__ r, float* r32,
+__global__ void __launch_bounds__(VTPB, 4) kb_update(int n, double* __restrict__ x, double* __restrict__ r, float* r32,
                                                    const double* p, const double* q, double* part, unsigned* ctr, double* S, bool ordered) {
     using L = Cols<J, R>;
     constexpr int Kp = L::KP;
@@ -894,21 +922,33 @@ __global__ void __launch_bounds__(VTPB) kb_update(int n, double* __restrict__ x,
     double alpha[J], v[J];
     ldv<J>(S + S_ALPHA * Kp + L::col(), alpha);
     zero(v);
-    for (int i = vfirst<J, R>(n); i < n; i += 4 * vblocks(n)) {
-        double xi[J], ri[J], pi[J], qi[J];
-        ldv<J>(x + L::at(i), xi);
-        ldv<J>(p + L::at(i), pi);
-        ldv<J>(r + L::at(i), ri);
-        ldv<J>(q + L::at(i), qi);
+    constexpr int U = vrows(J, 2);
+    const int step = 4 * vblocks(n);
+    for (int i0 = vfirst<J, R>(n); i0 < n; i0 += U * step) {
+        double xi[U][J], ri[U][J], pi[U][J], qi[U][J];
 #pragma unroll
-        for (int j = 0; j < J; ++j) {
-            xi[j] += alpha[j] * pi[j];
-            ri[j] -= alpha[j] * qi[j];
-            v[j] += ri[j] * ri[j];
+        for (int u = 0; u < U; ++u) {
+            const int i = i0 + u * step;
+            if (i >= n) break;
+            ldv<J>(x + L::at(i), xi[u]);
+            ldv<J>(p + L::at(i), pi[u]);
+            ldv<J>(r + L::at(i), ri[u]);
+            ldv<J>(q + L::at(i), qi[u]);
         }
-        stv<J>(x + L::at(i), xi);
-        stv<J>(r + L::at(i), ri);
-        st_r32<J>(r32, L::at(i), ri);
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int i = i0 + u * step;
+            if (i >= n) break;
+#pragma unroll
+            for (int j = 0; j < J; ++j) {
+                xi[u][j] += alpha[j] * pi[u][j];
+                ri[u][j] -= alpha[j] * qi[u][j];
+                v[j] += ri[u][j] * ri[u][j];
+            }
+            stv<J>(x + L::at(i), xi[u]);
+            stv<J>(r + L::at(i), ri[u]);
+            st_r32<J>(r32, L::at(i), ri[u]);
+        }
     }
     col_finish<J, R>(n, ordered, v, part, ctr, [&](int c, double t) {
         if (S[S_ACTIVE * Kp + c] <= 0.0) return;

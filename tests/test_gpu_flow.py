@@ -100,3 +100,24 @@ def test_batched_paddings_repeat_single_solves(K, precision):
             x, iters, status, _ = s.solve(B[:, k].contiguous(), tol=1e-6, maxit=100)
             assert status == 0 and iters == it[k]
             assert float((X[:, k] - x).norm() / x.norm()) <= bound
+
+
+# one row per lane group and a few left over; a full batch of four rows and one left over
+@pytest.mark.parametrize("shape", [(19, 16, 16), (33, 33, 18)])
+@pytest.mark.parametrize("K,precision", [(8, "fp64"), (16, "fp32"), (31, "fp32"), (33, "fp32"), (64, "fp64"), (90, "fp32"), (128, "fp32")])
+def test_batched_rows_left_over(shape, K, precision):
+    """Every column reaches the tolerance in its true residual (which differs from the recurrence's by
+    rounding, far less than the tolerance), in as many iterations as its own solve to one."""
+    p = inputs.small_3d(*shape, seed=85)
+    csr = cpc.tpfa_assemble(p.nx, p.ny, p.nz, torch.tensor(p.logk, device=DEV), p.kz_ratio, p.dirichlet)
+    s = cpc.Solver(*csr, precision=precision, ic_order="colour")
+    n = p.nx * p.ny * p.nz
+    B = torch.tensor(inputs.random_vector(n * K, 86).reshape(n, K), device=DEV)
+    X, it, st = s.solve_batched(B, tol=1e-8, maxit=500)
+    assert np.all(st == 0)
+    A = torch.sparse_csr_tensor(*csr, size=(n, n))
+    res = (torch.linalg.vector_norm(B - A @ X, dim=0) / torch.linalg.vector_norm(B, dim=0)).cpu().numpy()
+    assert np.all(res <= 2e-8)
+    for k in (0, K // 2, K - 1):
+        _, its, sts, _ = s.solve(B[:, k].contiguous(), tol=1e-8, maxit=500)
+        assert sts == 0 and abs(int(it[k]) - its) <= 1
