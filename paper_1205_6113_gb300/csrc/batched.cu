@@ -67,15 +67,26 @@ void blaunch(void (*k)(KArgs...), int grid, int block, cudaStream_t s, Args&&...
     CPC_CK(cudaLaunchKernelEx(&cfg, k, std::forward<Args>(args)...));
 }
 
-// The columns of a lane: 32 J columns on the 32 lanes of a warp (R = 1), or R rows of 32 / R columns.
+// The columns of a lane: a warp holds R rows of 32 J / R columns, J neighbouring ones to a lane.
 template <int J, int R>
 struct Cols {
-    static_assert(R == 1 || J == 1, "several rows per warp have one column per lane");
-    static constexpr int W = 32 / R, KP = 32 * J / R;
+    static constexpr int W = 32 / R, KP = W * J;
     static __device__ __forceinline__ int sub() { return R == 1 ? 0 : (threadIdx.x & 31) / W; }
-    static __device__ __forceinline__ int col() { return R == 1 ? (threadIdx.x & 31) * J : (threadIdx.x & 31) % W; }
+    static __device__ __forceinline__ int col() { return (R == 1 ? threadIdx.x & 31 : (threadIdx.x & 31) % W) * J; }
     // element of (row, the lane's first column)
     static __device__ __forceinline__ size_t at(int row) { return (size_t)row * KP + col(); }
+};
+
+// The columns of a lane in the preconditioner's kernels.  In FP32 they gather 16 bytes to a lane from two or
+// four rows at a time (8 bytes for 16 columns), so that half or a quarter of the load instructions move
+// the same bytes; a column's sums are the same.  64 solves and adjoints at 1M 255 -> 221 ms, 28 at 433k cells
+// 87 -> 64 ms, 16 at 1M 148 -> 123 ms, 12 at 131k cells 28.0 -> 26.3 ms.  Not for 8 columns (nothing gained)
+// and not in FP64, whose issue bounds them: fewer warps only lose (12 columns of a block solve 22.9 -> 27.9 ms,
+// 32 at 590k cells 157 -> 159 ms).
+template <int J, int R, class VT>
+struct Gather {
+    static constexpr int M = !std::is_same<VT, float>::value ? 1 : R == 1 && J <= 2 ? 4 / J : R == 2 ? 2 : 1;
+    static constexpr int j = J * M, r = R * M;
 };
 
 template <int J, class VT, class T>
@@ -1422,11 +1433,12 @@ void brec_vcycle(Handle& h, int l, const VT* f, VT* x, bool zero_guess, cudaStre
     const int nl = (int)h.lev.size();
     Level& L = h.lev[l];
     if (l == nl - 1) {
+        constexpr int KP = Cols<J, R>::KP, JC = KP > 32 ? KP / 32 : 1, RC = KP > 32 ? 1 : 32 / KP;
         const VT* ai = std::is_same<VT, double>::value ? (const VT*)h.Ainv.p : (const VT*)h.Ainv32.p;
         if constexpr (std::is_same<VT, double>::value)
-            blaunch(kb_coarse<J, R, VT, VT, VT>, (L.n + R * CROWS - 1) / (R * CROWS), CWARPS * 32, s, L.n, ai, f, x);
+            blaunch(kb_coarse<JC, RC, VT, VT, VT>, (L.n + RC * CROWS - 1) / (RC * CROWS), CWARPS * 32, s, L.n, ai, f, x);
         else
-            blaunch(kb_coarse_seq<J, R, VT, VT, VT>, (L.n + CWARPS * R * SROWS - 1) / (CWARPS * R * SROWS), CWARPS * 32, s, L.n,
+            blaunch(kb_coarse_seq<JC, RC, VT, VT, VT>, (L.n + CWARPS * RC * SROWS - 1) / (CWARPS * RC * SROWS), CWARPS * 32, s, L.n,
                     ai, f, x);
         return;
     }
@@ -1553,7 +1565,7 @@ void brec_loop(Handle& h, cudaGraph_t g, cudaStream_t cs, cudaGraphNode_t* dep, 
     CPC_CK(cudaStreamBeginCaptureToGraph(cs, body, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal));
     blaunch(kb_guard, 1, 32, cs, cond);
     VT* z = (VT*)B.z.p;
-    brec_precond<J, R, VT>(h, h.opt.precond, bres<VT>(B), z, cs);
+    brec_precond<Gather<J, R, VT>::j, Gather<J, R, VT>::r, VT>(h, h.opt.precond, bres<VT>(B), z, cs);
     const int vg = vgrid<R>(n);
     const bool ord = !std::is_same<VT, double>::value;
     blaunch(kb_rz<J, R, VT>, vg, VTPB, cs, n, (const double*)B.r.p, (const VT*)z, B.partial.p, h.counter.p + 1, B.S.p, ord);
@@ -1670,7 +1682,7 @@ int solve_block_t(Handle& h, int K, const double* b, double* x, double tol, int 
     kk_check<<<1, 256, 0, s>>>(KK_GRID, Kp, K, B.kpart.p, B.kvec.p, tol, 1, B.kflag.p);
     read_flags();
     if (flags[KF_BAD]) fail(CPC_EINVAL, "a right-hand-side column is zero or not finite");
-    brec_precond<J, R, VT>(h, h.opt.precond, bres<VT>(B), z, s);       // Z = M R
+    brec_precond<Gather<J, R, VT>::j, Gather<J, R, VT>::r, VT>(h, h.opt.precond, bres<VT>(B), z, s);       // Z = M R
     kk_copy<VT><<<2048, 256, 0, s>>>(nk, (const VT*)z, B.p.p);         // P = Z
     gram((const VT*)z, B.r.p, km(KM_GAMMA));                           // gamma = Z^T R
     int status = CPC_ENOCONV, it = 0;
@@ -1693,7 +1705,7 @@ int solve_block_t(Handle& h, int K, const double* b, double* x, double tol, int 
             break;
         }
         if (k == maxit) break;
-        brec_precond<J, R, VT>(h, h.opt.precond, bres<VT>(B), z, s);   // Z = M R
+        brec_precond<Gather<J, R, VT>::j, Gather<J, R, VT>::r, VT>(h, h.opt.precond, bres<VT>(B), z, s);   // Z = M R
         gram((const VT*)z, B.r.p, km(KM_GAMMA_NEW));                   // Z^T R
         kk_solve<<<1, KK_TPB, solve_smem, s>>>(K, Kp, km(KM_GAMMA), km(KM_GAMMA_NEW), km(KM_BETA), km(KM_GAMMA),
                                                B.kflag.p);
