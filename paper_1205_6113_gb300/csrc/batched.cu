@@ -78,14 +78,14 @@ struct Cols {
 };
 
 // The columns of a lane in the preconditioner's kernels.  In FP32 they gather 16 bytes to a lane from two or
-// four rows at a time (8 bytes for 16 columns), so that half or a quarter of the load instructions move
-// the same bytes; a column's sums are the same.  64 solves and adjoints at 1M 255 -> 221 ms, 28 at 433k cells
-// 87 -> 64 ms, 16 at 1M 148 -> 123 ms, 12 at 131k cells 28.0 -> 26.3 ms.  Not for 8 columns (nothing gained)
-// and not in FP64, whose issue bounds them: fewer warps only lose (12 columns of a block solve 22.9 -> 27.9 ms,
-// 32 at 590k cells 157 -> 159 ms).
+// four rows at a time (8 bytes for up to 16 columns), so that half or a quarter of the load instructions
+// move the same bytes; a column's sums are the same.  64 solves and adjoints at 1M 255 -> 221 ms, 28 at 433k
+// cells 87 -> 64 ms, 16 at 1M 148 -> 123 ms, 8 at 1M 98 -> 91 ms, 12 at 131k cells 28.0 -> 26.3 ms (with four
+// columns to a lane 29.9).  Not in FP64, whose issue bounds them: fewer warps only lose (12 columns of a block
+// solve 22.9 -> 27.9 ms, 32 at 590k cells 157 -> 159 ms).
 template <int J, int R, class VT>
 struct Gather {
-    static constexpr int M = !std::is_same<VT, float>::value ? 1 : R == 1 && J <= 2 ? 4 / J : R == 2 ? 2 : 1;
+    static constexpr int M = !std::is_same<VT, float>::value ? 1 : R == 1 && J <= 2 ? 4 / J : R >= 2 ? 2 : 1;
     static constexpr int j = J * M, r = R * M;
 };
 
