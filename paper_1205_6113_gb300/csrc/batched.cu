@@ -152,15 +152,13 @@ __device__ __forceinline__ BRow brow_at(const BV<MT, DT>& A, int s, const int* e
     return BRow{base, (end[k] - base) / A.C, s - k * A.C, A.C};
 }
 
-// acc[j] += sum_w a_w x[col_w][j] over entries w0, w0 + step, ... of a row, U entries' loads in flight
-// together.  Padding (-1) and marked columns (LATER) load nothing and add 0.
-template <int J, int R, int U, class VT, class MT, class XT>
-__device__ __forceinline__ void brow(const int* __restrict__ col, const MT* __restrict__ val, const BRow& t, int w0,
-                                     int step, const XT* x, VT (&acc)[J]) {
-    using L = Cols<J, R>;
-    for (int w = w0; w < t.width; w += U * step) {
-        int c[U];
-        VT a[U], xv[U][J];
+// Columns and values of U entries w, w + step, ... of a row (past its end: column -1, value 0).
+template <int U, class VT>
+struct Entries {
+    int c[U];
+    VT a[U];
+    template <class MT>
+    __device__ __forceinline__ void load(const int* __restrict__ col, const MT* __restrict__ val, const BRow& t, int w, int step) {
 #pragma unroll
         for (int u = 0; u < U; ++u) {
             const bool on = w + u * step < t.width;
@@ -168,19 +166,36 @@ __device__ __forceinline__ void brow(const int* __restrict__ col, const MT* __re
             c[u] = on ? col[e] : -1;
             a[u] = on ? Cv<VT>::f(val[e]) : VT(0);
         }
+    }
+};
+
+// acc[j] += sum_w a_w x[col_w][j] over entries w0, w0 + step, ... of a row, U entries' gathers in flight
+// together and the next entries' columns beside them; m holds the first ones, loaded by the caller before it
+// waits for x.  Padding (-1) and marked columns (LATER) load nothing and add 0.  (With each batch's columns
+// loaded before its own gathers a row cost two trips through L2 per batch and one more after the wait:
+// 64 solves and adjoints at 1M 220 -> 203 ms, 28 at 433k cells 63.6 -> 53.2, a block solve of 12 22.9 -> 20.7.)
+template <int J, int R, int U, class VT, class MT, class XT>
+__device__ __forceinline__ void brow(const int* __restrict__ col, const MT* __restrict__ val, const BRow& t, int w0,
+                                     int step, Entries<U, VT>& m, const XT* x, VT (&acc)[J]) {
+    using L = Cols<J, R>;
+    for (int w = w0; w < t.width; w += U * step) {
+        VT xv[U][J];
 #pragma unroll
         for (int u = 0; u < U; ++u) {
-            if ((unsigned)c[u] < (unsigned)LATER) {
-                ldv<J>(x + L::at(c[u]), xv[u]);
+            if ((unsigned)m.c[u] < (unsigned)LATER) {
+                ldv<J>(x + L::at(m.c[u]), xv[u]);
             } else {
 #pragma unroll
                 for (int j = 0; j < J; ++j) xv[u][j] = VT(0);
             }
         }
+        Entries<U, VT> next;
+        next.load(col, val, t, w + U * step, step);
 #pragma unroll
         for (int u = 0; u < U; ++u)
 #pragma unroll
-            for (int j = 0; j < J; ++j) acc[j] += a[u] * xv[u][j];
+            for (int j = 0; j < J; ++j) acc[j] += m.a[u] * xv[u][j];
+        m = next;
     }
 }
 
@@ -193,7 +208,7 @@ __device__ __forceinline__ void zero(VT (&v)[J]) {
 // Gauss-Seidel over the slots [s0, s1) of one colour, all columns; the entries of a row end at end[k]
 // (its chunk's last; in a sweep from a zero guess the entries of later colours, whose rows are zero, are
 // left out: by end in FP64, by their mark in FP32).
-template <int J, int R, class MT, class DT, class VT, int U>
+template <int J, int R, class MT, class DT, class VT>
 __global__ void __launch_bounds__(BTPB) kb_gs(BV<MT, DT> A, const int* __restrict__ end, int s0, int s1, const VT* f, VT* x) {
     using L = Cols<J, R>;
     const int s = s0 + (blockIdx.x * BWARPS + (threadIdx.x >> 5)) * R + L::sub();
@@ -202,12 +217,14 @@ __global__ void __launch_bounds__(BTPB) kb_gs(BV<MT, DT> A, const int* __restric
     const int row = A.perm[s];                   // matrix data: before the wait
     const BRow t = brow_at(A, s, end);
     const VT dinv = Cv<VT>::f(A.diag[s]);        // the view's diagonal field holds 1 / a_ii
+    Entries<4, VT> m;
+    m.load(A.col, A.val, t, 0, 1);
     pdl_wait();
     if (row < 0) return;
     VT acc[J], fr[J];
     zero(acc);
     ldv<J>(f + L::at(row), fr);
-    brow<J, R, U>(A.col, A.val, t, 0, 1, x, acc);
+    brow<J, R, 4>(A.col, A.val, t, 0, 1, m, x, acc);
 #pragma unroll
     for (int j = 0; j < J; ++j) acc[j] = (fr[j] - acc[j]) * dinv;
     stv<J>(x + L::at(row), acc);
@@ -229,12 +246,14 @@ __global__ void __launch_bounds__(64 * WSPLIT) kb_gs_wide(BV<MT, DT> A, const in
     const int row = A.perm[s];
     const BRow t = brow_at(A, s, end);
     const VT dinv = Cv<VT>::f(A.diag[s]);
+    Entries<4, VT> m;
+    m.load(A.col, A.val, t, w, WSPLIT);
     pdl_wait();
     VT acc[J], fr[J];
     zero(acc);
     zero(fr);
     if (w == 0 && row >= 0) ldv<J>(f + L::at(row), fr);
-    brow<J, R, 4>(A.col, A.val, t, w, WSPLIT, x, acc);
+    brow<J, R, 4>(A.col, A.val, t, w, WSPLIT, m, x, acc);
 #pragma unroll
     for (int j = 0; j < J; ++j) part[set][w][j][lane] = acc[j];
     __syncthreads();
@@ -258,6 +277,8 @@ __global__ void __launch_bounds__(BTPB) kb_resid(BV<MT, DT> A, int nslots, const
     const int row = A.perm[s];
     const BRow t = brow_at(A, s, A.cptr + 1);
     const VT d = Cv<VT>::f(A.diag[s]);
+    Entries<4, VT> m;
+    m.load(A.col, A.val, t, 0, 1);
     pdl_wait();
     if (row < 0) return;
     VT acc[J], fr[J];
@@ -265,7 +286,7 @@ __global__ void __launch_bounds__(BTPB) kb_resid(BV<MT, DT> A, int nslots, const
     ldv<J>(f + L::at(row), fr);
 #pragma unroll
     for (int j = 0; j < J; ++j) acc[j] *= d;
-    brow<J, R, 4>(A.col, A.val, t, 0, 1, x, acc);
+    brow<J, R, 4>(A.col, A.val, t, 0, 1, m, x, acc);
 #pragma unroll
     for (int j = 0; j < J; ++j) acc[j] = fr[j] - acc[j];
     stv<J>(out + L::at(row), acc);
@@ -283,11 +304,13 @@ __global__ void __launch_bounds__(BTPB) kb_resid_up(BV<MT, DT> A, const int* __r
     const int row = A.perm[s];
     const int k = s / A.C, base = cmid[k];
     const BRow t{base, (A.cptr[k + 1] - base) / A.C, s - k * A.C, A.C};
+    Entries<4, VT> m;
+    m.load(A.col, A.val, t, 0, 1);
     pdl_wait();
     if (row < 0) return;
     VT acc[J];
     zero(acc);
-    brow<J, R, 4>(A.col, A.val, t, 0, 1, x, acc);
+    brow<J, R, 4>(A.col, A.val, t, 0, 1, m, x, acc);
 #pragma unroll
     for (int j = 0; j < J; ++j) acc[j] = -acc[j];
     stv<J>(out + L::at(row), acc);
@@ -307,11 +330,13 @@ __global__ void __launch_bounds__(BTPB) kb_restrict(BV<MT, MT> M, const int* __r
     const BRow t = brow_at(M, s, end);
     const bool c0 = yx && row >= 0 && colour[row] == 0;
     const VT dr = c0 ? dnat[row] : VT(0);
+    Entries<4, VT> m;
+    m.load(M.col, M.val, t, 0, 1);
     pdl_wait();
     if (row < 0) return;
     VT acc[J];
     zero(acc);
-    brow<J, R, 4>(M.col, M.val, t, 0, 1, x, acc);
+    brow<J, R, 4>(M.col, M.val, t, 0, 1, m, x, acc);
     stv<J>(y + L::at(row), acc);
     if (!c0) return;
 #pragma unroll
@@ -328,12 +353,14 @@ __global__ void __launch_bounds__(BTPB) kb_prolong(BV<MT, MT> P, int nslots, con
     pdl_launch_dependents();
     const int row = P.perm[s];
     const BRow t = brow_at(P, s, P.cptr + 1);
+    Entries<4, VT> m;
+    m.load(P.col, P.val, t, 0, 1);
     pdl_wait();
     if (row < 0) return;
     VT acc[J], xr[J];
     zero(acc);
     ldv<J>(x + L::at(row), xr);
-    brow<J, R, 4>(P.col, P.val, t, 0, 1, e, acc);
+    brow<J, R, 4>(P.col, P.val, t, 0, 1, m, e, acc);
 #pragma unroll
     for (int j = 0; j < J; ++j) acc[j] += xr[j];
     stv<J>(x + L::at(row), acc);
@@ -455,12 +482,14 @@ __global__ void __launch_bounds__(BTPB) kb_lsolve(BV<MT, MT> A, int s0, int s1, 
     pdl_launch_dependents();
     const int row = A.perm[s];
     const BRow b = brow_at(A, s, A.cptr + 1);
+    Entries<4, VT> m;
+    m.load(A.col, A.val, b, 0, 1);
     pdl_wait();
     if (row < 0) return;
     VT acc[J], tr[J];
     zero(acc);
     ldv<J>(t + L::at(row), tr);
-    brow<J, R, 4>(A.col, A.val, b, 0, 1, y, acc);
+    brow<J, R, 4>(A.col, A.val, b, 0, 1, m, y, acc);
 #pragma unroll
     for (int j = 0; j < J; ++j) acc[j] = tr[j] - acc[j];
     stv<J>(y + L::at(row), acc);
@@ -475,12 +504,14 @@ __global__ void __launch_bounds__(BTPB) kb_usolve(BV<MT, MT> U, int s0, int s1, 
     const int row = U.perm[s];
     const BRow b = brow_at(U, s, U.cptr + 1);
     const VT dinv = Cv<VT>::f(U.diag[s]);        // 1 / u_ii
+    Entries<4, VT> m;
+    m.load(U.col, U.val, b, 0, 1);
     pdl_wait();
     if (row < 0) return;
     VT acc[J], yr[J];
     zero(acc);
     ldv<J>(y + L::at(row), yr);
-    brow<J, R, 4>(U.col, U.val, b, 0, 1, w, acc);
+    brow<J, R, 4>(U.col, U.val, b, 0, 1, m, w, acc);
 #pragma unroll
     for (int j = 0; j < J; ++j) acc[j] = (yr[j] - acc[j]) * dinv;
     stv<J>(w + L::at(row), acc);
@@ -888,7 +919,10 @@ __global__ void __launch_bounds__(VTPB) kb_spmv_pq(BV<double, double> A, int nsl
         ldv<J>(p + L::at(row), pr);
 #pragma unroll
         for (int j = 0; j < J; ++j) acc[j] = d * pr[j];
-        brow<J, R, 4>(A.col, A.val, brow_at(A, s, A.cptr + 1), 0, 1, p, acc);
+        const BRow t = brow_at(A, s, A.cptr + 1);
+        Entries<4, double> m;
+        m.load(A.col, A.val, t, 0, 1);
+        brow<J, R, 4>(A.col, A.val, t, 0, 1, m, p, acc);
         stv<J>(q + L::at(row), acc);
 #pragma unroll
         for (int j = 0; j < J; ++j) v[j] += pr[j] * acc[j];
@@ -1284,7 +1318,10 @@ __global__ void __launch_bounds__(BTPB) kk_spmm(int n, const int* __restrict__ p
     double acc[J];
     zero(acc);
     const int e0 = ptr[i];
-    brow<J, R, 4>(col, val, BRow{e0, ptr[i + 1] - e0, 0, 1}, 0, 1, P, acc);
+    const BRow t{e0, ptr[i + 1] - e0, 0, 1};
+    Entries<4, double> m;
+    m.load(col, val, t, 0, 1);
+    brow<J, R, 4>(col, val, t, 0, 1, m, P, acc);
     stv<J>(Q + L::at(i), acc);
 }
 
@@ -1369,11 +1406,10 @@ void brec_gs(Level& L, int c, const VT* f, VT* x, cudaStream_t s, bool from_zero
         using MT = std::remove_cv_t<std::remove_reference_t<decltype(*view.val)>>;
         using DT = std::remove_cv_t<std::remove_reference_t<decltype(*view.diag)>>;
         static_assert(std::is_same<V, BV<MT, DT>>::value, "");
-        // long rows: in a small colour group a block per R rows, else eight entries per batch
+        // long rows in a small colour group: a block per 2 R rows
         const bool lng = L.A.nnz >= (int64_t)16 * L.n;
         if (lng && (s1 - s0) <= 16384) blaunch(kb_gs_wide<J, R, MT, DT, VT>, (s1 - s0 + 2 * R - 1) / (2 * R), 64 * WSPLIT, s, view, end, s0, s1, f, x);
-        else if (lng) blaunch(kb_gs<J, R, MT, DT, VT, 8>, g, BTPB, s, view, end, s0, s1, f, x);
-        else blaunch(kb_gs<J, R, MT, DT, VT, 4>, g, BTPB, s, view, end, s0, s1, f, x);
+        else blaunch(kb_gs<J, R, MT, DT, VT>, g, BTPB, s, view, end, s0, s1, f, x);
     };
     if constexpr (std::is_same<VT, double>::value) go(bview(L.S, (const double*)L.S.val.p, (const double*)L.S.dinv.p));
     else if (L.vt == VT_BF16) go(bview(L.S, (const __nv_bfloat16*)L.S.val16.p, (const float*)L.S.dinv32.p));
