@@ -362,8 +362,8 @@ def gpu_arm(args, rank, world):
     headline_ms = float(np.mean(ms))
     roofline = dict(bound="hbm", achieved=round(coarse_achieved, 1), peak=peak, unit="GB/s",
                     frac=round(coarse_achieved / peak, 4), traffic=TRAFFIC_COARSE_SWEEP,
-                    kernel="k_gs (Gauss-Seidel colour steps of the coarse levels 1..%d, FP64): one forward sweep per "
-                           "level, aggregated; dependent-launch latency bounds these steps" % (s_bco.nlevels - 2),
+                    kernel="k_gs, k_flow (Gauss-Seidel sweeps of the coarse levels 1..%d, FP64): one forward sweep per "
+                           "level, aggregated; the latency of their dependent steps bounds them" % (s_bco.nlevels - 2),
                     bytes_per_sweep=int(cbytes), us_per_sweep=round(cus, 2), peak_kind=peak_kind, levels=coarse,
                     fine_gs=fine, spmv=spmv)
     out.update(dict(p=p, arms=arms, matrices=matrices, clocks=clk, e2e_ms=e2e_ms, true_res=true_res,

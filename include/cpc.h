@@ -67,8 +67,8 @@ enum {
                             /* sequential sweep i = 0..n-1 (and n-1..0 for S_l^T).  Far more steps.   */
 };
 
-/* Largest accepted cpc_options.max_levels: the smoothing colourings of all levels but the
-   coarsest are computed in one launch that holds per-level state for 24 levels. */
+/* Largest accepted cpc_options.max_levels: the colouring launches of all levels but the coarsest
+   hold per-level state for 24 levels. */
 #define CPC_MAX_LEVELS 25
 
 /* CSR matrix, caller-owned; cpc_setup copies what it needs. */
@@ -191,7 +191,8 @@ const char* cpc_last_error(const cpc_handle* h);
  * b[n], x[n]: device pointers (x is output only).  *iters = iterations taken;
  * res_hist[k] = ||r_k|| / ||b|| for k = 0..*iters (at most hist_cap values written; res_hist
  * may be NULL).  Runs the whole iteration loop on the device; synchronises the stream.
- * Returns CPC_OK, CPC_ENOCONV, CPC_EBREAKDOWN, CPC_ECUDA or CPC_EINVAL.
+ * Returns CPC_OK, CPC_ENOCONV, CPC_EBREAKDOWN, CPC_ECUDA, CPC_EINVAL or CPC_ETIMEOUT (a wait
+ * between the parts of a sweep or triangular solve gave up: x is not a solution).
  */
 int cpc_solve(cpc_handle* h, const double* b, double* x, double tol, int32_t maxit,
               int32_t* iters, double* res_hist, int32_t hist_cap);
@@ -272,8 +273,8 @@ int cpc_coarse_inverse_info(const cpc_handle* h, int32_t* method, double* residu
  * graph if it does not exist yet. */
 int cpc_solve_launches(cpc_handle* h, int64_t* per_iteration, int64_t* fixed);
 
-/* Profiling: *us = microseconds per forward Gauss-Seidel sweep (colours ascending, one dependent
- * launch per colour, Section 3.3) of level `level` (0 <= level < levels - 1), in the handle's
+/* Profiling: *us = microseconds per forward Gauss-Seidel sweep (colours ascending, Section 3.3: one
+ * dependent launch per colour, or on a small level one launch ordered by its data) of level `level` (0 <= level < levels - 1), in the handle's
  * preconditioner precision, replayed from a CUDA graph as inside the solve: `reps` sweeps
  * (1..1000) per replay, best of three replays after a warm-up.  Overwrites the level's work
  * vectors.  Synchronous. */
@@ -324,7 +325,7 @@ int cpc_ic0_values(const cpc_handle* h, double* lu);
 /* Level operators on device vectors, for parity tests: op 0 y = A_l x; 1 y = S_l x (forward
  * Gauss-Seidel sweep, zero guess); 2 y = S_l^T x (backward sweep); 3 y = A_l^{-1} x (coarsest
  * level); 4 y = V-cycle from level l with zero initial guess; 5 one forward Gauss-Seidel sweep on
- * A_l y = x starting from the given y (one launch per colour, nothing else).  Asynchronous. */
+ * A_l y = x starting from the given y (the sweep's launches, nothing else).  Asynchronous. */
 int cpc_level_apply(cpc_handle* h, int32_t level, int32_t op, const double* x, double* y);
 
 #ifdef __cplusplus

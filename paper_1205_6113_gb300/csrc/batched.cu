@@ -3,7 +3,7 @@
 // Block vectors are row-major [n][Kp].  Kp = K rounded up to 8 or 16, or to a multiple of 32: a warp owns
 // one row of 32 J columns (lane l the J columns from l J on, one vector load), or for K <= 16 the R = 4
 // or 2 rows that fill its lanes, since a warp instruction costs the same with idle lanes and FP64 issue
-// is scarce on this part.  Every matrix entry is one broadcast load shared by all columns, and every
+// is scarce on this part (the FP32 preconditioner's kernels take more rows to a warp, see Gather).  Every matrix entry is one broadcast load shared by all columns, and every
 // gathered vector row is one coalesced load.  The matrix is read once per K solves instead of once per
 // solve (SpMM).  Each column has its own alpha, beta and convergence flag; a converged column is frozen
 // (alpha = 0) while the others continue, so each column reproduces the single-right-hand-side

@@ -7,8 +7,8 @@
 //   AMG     strength theta, PMIS splitting with weight (|S^T_i|, fmix32(i)), direct
 //           interpolation, R = P^T, Galerkin A_c = R (A P) (Section 3.2);
 //   colour  breadth-first parity 2-colouring when the level graph is bipartite (red-black on a
-//           structured grid), else Jones-Plassmann with priority (peel round, fmix32(i ^
-//           0x5bd1e995)) and the smallest free colour; peel rounds are a smallest-last style
+//           structured grid), else greedy in decreasing priority (peel round, fmix32(i ^
+//           0x5bd1e995)) with the smallest free colour; peel rounds are a smallest-last style
 //           ordering that needs fewer colours than a random one; with natural-order
 //           Gauss-Seidel, the wavefronts of the lower-triangular graph of A_l instead.
 // Sums that define matrix entries are accumulated in a fixed order (the order the products are
@@ -1244,7 +1244,8 @@ __global__ void __launch_bounds__(COL_TPB) k_colour(const ColLev* levs, int nlev
 // points handed out before it, to blocks that are running, so the earliest one without a colour never
 // waits for one that has not started.  The chain is as long as the longest path of the priorities (554
 // points at 1M); a step is a trip through L2, about 1.2 us, where a round over all points with a
-// grid barrier took 12 (colouring of all levels at 1M 13.5 ms, 6.0 with this).
+// grid barrier took 12 (colouring of all levels at 1M 13.5 ms, 6.0 with this, 4.0
+// with the peel rounds of one step).
 // ============================================================================================
 constexpr int GREEDY_WARPS = 4;
 constexpr int GREEDY_SPINS = 1 << 21;
@@ -1471,7 +1472,7 @@ __device__ __forceinline__ bool sell_keep(int mode, int j, int i) {
 // group key per row (smoother copy) the two parts are padded apart: low[k] = entries of the part of earlier
 // groups.  wmax[0..2]: the largest chunk, low part and high part.  Columns of key 0 make the first part when
 // by_col (the rows have no key then: a transfer, its columns keyed by the fine colour).  (A thread per chunk
-// walked C rows one after the other: 100 us for 1M entries, 10 with this.)
+// walked C rows one after the other: 60-190 us a layout, whatever the level's size.)
 __global__ void __launch_bounds__(TPB) k_sell_width(const int* perm, int nchunks, int C, const int* ptr, const int* col,
                                                     int mode, const int* key, bool by_col, int* width, int* low,
                                                     int* wmax) {
@@ -1701,7 +1702,7 @@ __device__ __forceinline__ bool dia_insert(int* table, int off) {
 
 // Distinct off-diagonal offsets col - row of the rows into the table; *over = 1 when there are more than 8.
 // Each block collects its rows' in shared memory first: with all threads on the one table in L2 1M rows
-// took 230 us, 35 with this.
+// took 230 us.
 __global__ void k_dia_offsets(int n, const int* ptr, const int* col, int* table, int* over) {
     __shared__ int tab[8];
     if (threadIdx.x < 8) tab[threadIdx.x] = INT_MIN;
