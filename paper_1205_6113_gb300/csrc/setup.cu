@@ -934,8 +934,8 @@ struct ColLev {
 
 // scal of a level: [0..2] dmin of peel round r in slot r % 3 (a slot is cleared one round before it is
 // added to and read one barrier after); [3] 1 when the peel rounds are done: the level is not bipartite;
-// [4] triangle found; [5] not bipartite or a join failed.
-enum { CS_DMIN = 0, CS_GREEDY = 3, CS_TRI = 4, CS_BAD = 5, COL_NS = 6 };
+// [4] triangle found; [5] not bipartite or a join failed; [6] the largest degree.
+enum { CS_DMIN = 0, CS_GREEDY = 3, CS_TRI = 4, CS_BAD = 5, CS_DMAX = 6, COL_NS = 7 };
 enum { CP_INIT, CP_UNION, CP_FIND, CP_CHECK, CP_RESET, CP_PEEL, CP_DONE };
 
 // Union-find words: parent << 1 | parity relative to the parent (a root: itself, parity 0).
@@ -1005,13 +1005,14 @@ __device__ bool tri_probe(int i, const int* ptr, const int* col) {
 // index; whole CTAs, so that the block reductions see every thread of the CTA).
 __device__ void col_step(const ColLev& V, int phase, int rnd_no, int dm, int t, int T) {
     auto imin = [](int a, int b) { return a < b ? a : b; };
+    auto imax = [](int a, int b) { return a > b ? a : b; };
     auto iadd = [](int a, int b) { return a + b; };
     const int n = V.n;
     const int* ptr = V.ptr;
     const int* col = V.col;
     const int gl = threadIdx.x % COL_G;
     if (phase == CP_INIT) {
-        int m = INT_MAX, tri = 0;
+        int m = INT_MAX, most = 0, tri = 0;
         for (int i = t; i < n; i += T) {
             int d = 0;
             for (int p = ptr[i]; p < ptr[i + 1]; ++p) d += col[p] != i;
@@ -1020,12 +1021,15 @@ __device__ void col_step(const ColLev& V, int phase, int rnd_no, int dm, int t, 
             V.colour[i] = -1;
             V.w[i] = (unsigned)i << 1;
             m = imin(m, d);
+            most = imax(most, d);
             if (!tri) tri = tri_probe(i, ptr, col);
         }
         m = block_reduce(m, imin, INT_MAX);
+        most = block_reduce(most, imax, 0);
         tri = block_reduce(tri, iadd, 0);
         if (threadIdx.x == 0) {
             if (m != INT_MAX) atomicMin(&V.scal[CS_DMIN], m);
+            if (most) atomicMax(&V.scal[CS_DMAX], most);
             if (tri) atomicOr(&V.scal[CS_TRI], 1);
         }
     } else if (phase == CP_UNION) {
@@ -1248,10 +1252,19 @@ __global__ void __launch_bounds__(COL_TPB) k_colour(const ColLev* levs, int nlev
 // with the peel rounds of one step).
 // ============================================================================================
 constexpr int GREEDY_WARPS = 4;
-constexpr int GREEDY_SPINS = 1 << 21;
+
+// Polls (a quarter of a microsecond each) after which a wait gives up.  A point waits at most for the points in
+// flight (warps), one after another, each (dmax / 32 + 1) batches of neighbours on (dmax / 64 + 1) passes, a
+// batch three trips through L2 or some ten polls; three times that, and at least half a second (2^21).  (Half a
+// second alone was not enough for 2,000 points that are all coupled.)
+inline int greedy_polls(int64_t warps, int64_t dmax) {
+    const double w = 32.0 * (double)warps * (double)(dmax / 32 + 1) * (double)(dmax / 64 + 1);
+    return (int)std::min(std::max(w, (double)(1 << 21)), (double)(1 << 30));
+}
 
 struct GreedyLev {
     int n, blk0, blk1;                        // points; blocks [blk0, blk1) work on the level
+    int polls;                                // greedy_polls
     const int *ptr, *col, *order, *rank;      // order[q]: the q-th point, rank: its inverse
     int* colour;                              // -1 on entry
     unsigned* ctr;
@@ -1299,7 +1312,7 @@ __global__ void __launch_bounds__(GREEDY_WARPS * 32) k_greedy(const GreedyLev* l
                 const bool up = j != i && V.rank[j] < q;
                 int c = up ? colour_ld(V.colour + j) : 0;
                 for (int spin = 0; __any_sync(0xffffffffu, c < 0); ++spin) {
-                    if (spin == GREEDY_SPINS) {                // gives up: setup reports it
+                    if (spin == V.polls) {                     // gives up: setup reports it
                         if (c < 0) *err = 3;
                         c = max(c, 0);
                         break;
@@ -2719,6 +2732,7 @@ void colour_levels(Handle& h, cudaStream_t s) {
             V.blk0 = blk;
             blk += std::min(6 * sms, nblk(L.n, GREEDY_WARPS));
             V.blk1 = blk;
+            V.polls = greedy_polls(std::min(L.n, (blk - V.blk0) * GREEDY_WARPS), hs[(size_t)COL_NS * gl[g] + CS_DMAX]);
             base += L.n;
         }
         sort_pairs(key.get(), skey.get(), idx.get(), order.get(), gn, 64, s);

@@ -40,3 +40,22 @@ def test_greedy_colours_match_the_oracle(sizes):
     _, colour = s.level_splitting(0)
     assert np.array_equal(colour, orc.level_cf_colour(0)[1])
     assert colour.max() + 1 == max(sizes)
+
+
+def test_greedy_colours_a_long_chain_of_long_rows():
+    """A coarse level whose points are all coupled: each takes its colour after all before it, half a
+    second later for the last.  The fine level has a point for each pair of the first m, so that those
+    m become the coarse points."""
+    m = 2200
+    a, b = np.triu_indices(m, 1)
+    f = m + np.arange(a.size)
+    r, c = np.concatenate((a, b, f, f)), np.concatenate((f, f, a, b))
+    n = m + a.size
+    r, c = np.concatenate((r, np.arange(n))), np.concatenate((c, np.arange(n)))
+    v = np.where(r == c, np.where(r < m, float(m), 2.5), -1.0)
+    o = np.lexsort((c, r))
+    ptr = np.concatenate(([0], np.cumsum(np.bincount(r, minlength=n)))).astype(np.int32)
+    s = cpc.Solver(ptr, c[o].astype(np.int32), v[o], coarse_max=64)
+    i = s.level_info(1)
+    assert i["n"] == m and i["nnz"] == m * m
+    assert np.array_equal(np.sort(s.level_splitting(1)[1]), np.arange(m))
