@@ -1,6 +1,8 @@
 // handle.cuh -- the solver handle: hierarchy, IC(0) factor, work vectors, captured graphs.
 #pragma once
 
+#include <algorithm>
+
 #include "common.cuh"
 
 namespace cpc {
@@ -81,8 +83,15 @@ struct Handle {
     DBuf<float> ic_uinv32;
     Sell L, U;              // strictly-lower rows by forward level; upper rows by backward level
     // Triangular solves as one flow launch each; y is unset between them.  Two levels (red-black) keep
-    // a launch per level.
-    bool ic_flow() const { return ic_levels_L > 2 || ic_levels_U > 2; }
+    // a launch per level, and so do levels so wide that a launch is over in no time beside its work, as in
+    // the colour order of a large matrix without a red-black colouring: both solves by launches and by flow
+    // at 189,000 rows a level 29.3 and 25.2 us, 258,000 35.2 and 36.9, 707,000 87 and 104 (mixed-hybrid
+    // systems, FP64; in FP32 28.3 and 28.4 at 258,000), 27 points a row 140,000 327 and 310, 218,000 467 and 510.
+    static constexpr int IC_FLOW_ROWS = 200000;
+    bool ic_flow() const {
+        const int g = std::max(ic_levels_L, ic_levels_U);
+        return g > 2 && n / g <= IC_FLOW_ROWS;
+    }
     // coarsest level: dense inverse
     int nc = 0;
     DBuf<double> Ainv;

@@ -121,3 +121,29 @@ def test_batched_rows_left_over(shape, K, precision):
     for k in (0, K // 2, K - 1):
         _, its, sts, _ = s.solve(B[:, k].contiguous(), tol=1e-8, maxit=500)
         assert sts == 0 and abs(int(it[k]) - its) <= 1
+
+
+def test_wide_ic0_levels_keep_their_launches():
+    """IC(0) of a mixed-hybrid system in its four colours, 258,000 rows each: a launch per level and factor,
+    where the natural order's narrow levels take one per factor.  The solve of L (U z) = r, rows of at
+    most m products, leaves a residual of at most 2 (m + 5) eps (|L| |U| |z| + |r|) per row."""
+    import scipy.sparse as sp
+    nx, ny, nz = 80, 80, 40
+    logk = torch.tensor(inputs.random_vector(nx * ny * nz, 89), device=DEV)
+    csr = cpc.mhfem_assemble(nx, ny, nz, logk, 0.1, inputs.FACE_X0)
+    s = cpc.Solver(*csr, precond="ic0", ic_order="colour")
+    t = cpc.Solver(*csr, precond="ic0")
+    levels = s.level_info(0)["ic_levels"]
+    assert 2 < levels and s.n // levels > 200000 > t.n // t.level_info(0)["ic_levels"]
+    assert s.solve_launches()[0] == t.solve_launches()[0] - 2 + 2 * levels
+    r = inputs.random_vector(s.n, 90)
+    z = s.apply(torch.tensor(r, device=DEV)).cpu().numpy()
+    ptr, col, val = (a.cpu().numpy() for a in csr)
+    order = np.argsort(s.level_splitting(0)[1], kind="stable")
+    F = sp.csr_matrix((val, col, ptr), shape=(s.n, s.n))[order][:, order]
+    F.sort_indices()
+    F.data = s.ic0_values()
+    L, U = sp.tril(F, -1) + sp.identity(s.n), sp.triu(F)
+    r, z = r[order], z[order]
+    bound = 2 * (np.diff(F.indptr).max() + 5) * EPS * (abs(L) @ (abs(U) @ abs(z)) + abs(r))
+    assert np.all(np.abs(L @ (U @ z) - r) <= bound)
