@@ -217,6 +217,17 @@ int flow_sms() {
     return sms;
 }
 
+// Calls f(std::integral_constant<int, M>{}) with the batch of a kernel whose lanes hold at most `lanes` entries.
+template <class F>
+void with_m(int lanes, F&& f) {
+    if (lanes <= 4) f(std::integral_constant<int, 4>{});
+    else if (lanes <= 8) f(std::integral_constant<int, 8>{});
+    else f(std::integral_constant<int, 16>{});
+}
+
+// Most entries that a lane takes of a row's new or old values: of one part in FP64, of the mixed row in FP32.
+inline int sweep_lanes(const Sell& S, bool fp64) { return fp64 ? std::max(S.lanes_lo, S.lanes_up) : S.lanes; }
+
 template <int MODE, class MT, class DT, class FT, class VT>
 void flow_mode(const Sell& S, SV<MT, DT> v, const FT* f, const VT* xo, VT* xn, VT* unset, VT* zadd, unsigned* ctr,
                int* err, cudaStream_t s) {
@@ -227,7 +238,7 @@ void flow_mode(const Sell& S, SV<MT, DT> v, const FT* f, const VT* xo, VT* xn, V
     // a draw, once per chunk (18,000 chunks: 24 us against 15).
     const int ahead = std::max(2 * flow_sms(), (int)(4 * (int64_t)S.nchunks / std::max<int>(1, (int)S.seg.size() - 1)));
     const bool wide = ahead > 16 * flow_sms();
-    const int lanes = MODE == FLOW_LOWER || MODE == FLOW_UPPER || std::is_same<VT, float>::value ? S.lanes : std::max(S.lanes_lo, S.lanes_up);
+    const int lanes = MODE == FLOW_LOWER || MODE == FLOW_UPPER ? S.lanes : sweep_lanes(S, std::is_same<VT, double>::value);
     auto go = [&](auto m) {
         constexpr int M = decltype(m)::value;
         if (wide)
@@ -237,12 +248,40 @@ void flow_mode(const Sell& S, SV<MT, DT> v, const FT* f, const VT* xo, VT* xn, V
             launch(k_flow<MT, DT, FT, VT, MODE, M, false>, std::min(S.nchunks, ahead), 32, s, v, (const int*)S.cmid.p,
                    S.nchunks, f, xo, xn, unset, zadd, ctr, err);
     };
-    if (lanes <= 4) go(std::integral_constant<int, 4>{});
-    else if (lanes <= 8) go(std::integral_constant<int, 8>{});
-    else go(std::integral_constant<int, 16>{});
+    with_m(lanes, go);
+}
+
+// Warps of a level's sweep that the GPU holds at once.
+template <class MT, class VT>
+int flow_resident(int lanes) {
+    int blocks = 0;
+    with_m(lanes, [&](auto m) {
+        CPC_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, k_flow<MT, VT, VT, VT, FLOW_FWD, decltype(m)::value, true>, 128, 0));
+    });
+    return 4 * blocks * flow_sms();
 }
 
 }  // namespace
+
+// Wide colours fill the GPU for longer than a launch takes to start, and their launches keep more warps
+// resident than a flow's waiting ones: 32,000 rows a colour (level 1 at 1M) take 49 us by launches and 50 by
+// flow in FP64, 26 and 32 in FP32; 12,000 rows a colour 16.2 and 14.7 (FP32, 395,000 cells), 4,500 rows a colour
+// 61 and 28.  Below that the chunks of a colour count, against the warps that the GPU holds (fewer where a
+// lane takes 16 entries at a time): once they are not all resident a flow waits for its own chunks.  Launches and
+// flow, us a full sweep, at chunks a colour per resident warp: FP64 0.83 68 and 57, 0.94 76 and 70, 1.02 59 and
+// 53, 1.12 75 and 77, 1.49 67 and 85, 2.6 103 and 161 (with the sweep from zero, half a row, two cycles at 1.12
+// 1,884 and 1,858, at 1.25 2,048 and 2,042, at 1.40 2,217 and 2,225); FP32, which polls every entry of a row, 0.42
+// 19 and 16, 0.66 47 and 42, 0.71 46 and 45, 0.84 46 and 54, 1.25 36 and 59, 2.0 52 and 115, and 83 and 109 at
+// 0.55 with 30 entries to a lane, two batches.
+bool gs_by_flow(const Sell& S, int n, VType vt) {
+    constexpr int FLOW_ROWS = 24000;
+    const int g = std::max(1, (int)S.seg.size() - 1), lanes = sweep_lanes(S, vt == VT_F64);
+    if (n / g > FLOW_ROWS) return false;
+    const double per = (double)S.nchunks / g;
+    if (vt == VT_F64) return per <= 1.25 * flow_resident<double, double>(lanes);
+    const int res = vt == VT_BF16 ? flow_resident<__nv_bfloat16, float>(lanes) : flow_resident<float, float>(lanes);
+    return per * std::max(1.0, lanes / 16.0) <= 0.75 * res;
+}
 
 template <class FT, class VT>
 void rec_flow(FlowMode mode, const Sell& S, VType vt, const FT* f, const VT* xo, VT* xn, VT* unset, VT* zadd,

@@ -165,12 +165,8 @@ void record_tail(Handle& h, int level, const void* f0, void* x0, cudaStream_t s)
 // solve.cu
 void record_precond(Handle& h, int which, const double* r, void* z, cudaStream_t s);
 void apply_precond(Handle& h, int which, const double* r, double* z);
-// Whether the sweeps of a level of n rows in g groups run as flow launches.  Wide colours fill the GPU
-// for longer than a launch takes to start, and their launches keep more warps resident than a flow's
-// waiting ones: 32,000 rows a colour (level 1 at 1M) take 49 us by launches and 50 by flow in FP64, 26
-// and 32 in FP32; 12,000 rows a colour 16.2 and 14.7 (FP32, 395,000 cells), 4,500 rows a colour 61 and 28.
-constexpr int FLOW_ROWS = 24000;
-inline bool gs_by_flow(int n, int g) { return n / g <= FLOW_ROWS; }
+// Whether the sweeps of a level of n rows run as flow launches (flow.cu).
+bool gs_by_flow(const Sell& S, int n, VType vt);
 // Warps resident at once at the colour steps' occupancy (8 blocks of 4 warps on each of 152 SMs).
 constexpr int GS_RESIDENT_WARPS = 152 * 32;
 // Marks the n elements of p unset (flow.cuh).

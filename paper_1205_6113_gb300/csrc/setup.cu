@@ -3057,7 +3057,7 @@ void setup_handle(Handle& h, const cpc_csr& in) {
             }
             CPC_LAUNCH_CK();
             L.red_black = L.S.ndiag && L.ncolours == 2;
-            L.flow = !L.red_black && gs_by_flow(L.n, L.ncolours);
+            L.flow = !L.red_black && gs_by_flow(L.S, L.n, L.vt);
         }
         const size_t n = L.n;
         if (L.vt == VT_F64) { L.x64.alloc(n); L.f64.alloc(n); L.r64.alloc(n); }

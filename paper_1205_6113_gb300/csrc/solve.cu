@@ -1215,7 +1215,7 @@ float time_gs_sweep(const Sell& S, int n) {
     CPC_CK(cudaMemsetAsync(x.p, 0, sizeof(double) * n, cs));
     CPC_CK(cudaMemsetAsync(ctr.p, 0, sizeof(unsigned) * ctr.n, cs));
     CPC_CK(cudaStreamSynchronize(cs));
-    const bool flow = S.cmid.p && gs_by_flow(n, (int)S.seg.size() - 1);   // (an FP32 layout is timed by launches)
+    const bool flow = S.cmid.p && gs_by_flow(S, n, VT_F64);   // (an FP32 layout is timed by launches)
     cudaGraph_t g;
     CPC_CK(cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal));
     for (int k = 0; k < SWEEPS; ++k) {      // the launches of the solve's sweeps

@@ -147,3 +147,20 @@ def test_wide_ic0_levels_keep_their_launches():
     r, z = r[order], z[order]
     bound = 2 * (np.diff(F.indptr).max() + 5) * EPS * (abs(L) @ (abs(U) @ abs(z)) + abs(r))
     assert np.all(np.abs(L @ (U @ z) - r) <= bound)
+
+
+def test_sweeps_of_more_chunks_than_the_gpu_holds_keep_their_launches():
+    """Level 2 of 5 million cells in FP32, 18,000 rows a colour in chunks of 8 rows: more than three quarters of
+    the 2,432 warps that the GPU holds of a sweep with 16 entries to a lane.  An iteration has five kernels
+    of the loop and two cycles of at least 7 launches on the red-black level 0, on levels 1 and 2 of g colours
+    g - 1 forward from zero (the first colour comes with the restriction), g backward and 3 for residual and
+    transfers, and the coarsest solve."""
+    nx, ny, nz = 216, 216, 108
+    gen = torch.Generator(device=DEV)
+    gen.manual_seed(91)
+    logk = torch.randn(nx * ny * nz, generator=gen, device=DEV, dtype=torch.float64)
+    s = cpc.Solver(*cpc.tpfa_assemble(nx, ny, nz, logk, 0.1, inputs.FACE_X0), precond="amg", precision="fp32")
+    i = s.level_info(2)
+    assert i["n"] // i["ncolours"] <= 24000 and i["n"] / (s.level_layout(2)["C"] * i["ncolours"]) > 0.75 * 2432
+    by_colours = sum(2 * s.level_info(l)["ncolours"] - 1 + 3 for l in (1, 2))
+    assert s.solve_launches()[0] >= 5 + 2 * (7 + by_colours + 1)
