@@ -192,7 +192,8 @@ const char* cpc_last_error(const cpc_handle* h);
  * res_hist[k] = ||r_k|| / ||b|| for k = 0..*iters (at most hist_cap values written; res_hist
  * may be NULL).  Runs the whole iteration loop on the device; synchronises the stream.
  * Returns CPC_OK, CPC_ENOCONV, CPC_EBREAKDOWN, CPC_ECUDA, CPC_EINVAL or CPC_ETIMEOUT (a wait
- * between the parts of a sweep or triangular solve gave up: x is not a solution).
+ * for a row of a sweep or triangular solve gave up, in this call or in an application before it, see
+ * cpc_set_wait_polls: x may not be a solution; the next call starts anew).
  */
 int cpc_solve(cpc_handle* h, const double* b, double* x, double tol, int32_t maxit,
               int32_t* iters, double* res_hist, int32_t hist_cap);
@@ -239,7 +240,9 @@ int cpc_solve_batched_adjoint(cpc_handle* h, int32_t nrhs, const double* B, doub
                               double tol, int32_t maxit, int32_t* iters_fwd, int32_t* iters_adj);
 
 /* z = M r for one application of a preconditioner (which = CPC_PRECOND_*; -1 = the handle's).
- * r[n], z[n] device.  Asynchronous.  cpc_apply_Bcom is which = CPC_PRECOND_BCO. */
+ * r[n], z[n] device.  Asynchronous.  cpc_apply_Bcom is which = CPC_PRECOND_BCO.  If a wait inside gives
+ * up (cpc_set_wait_polls), z holds NaN and the next cpc_solve, cpc_solve_host or cpc_sweep_time_us on the
+ * handle returns CPC_ETIMEOUT, once. */
 int cpc_apply_precond(cpc_handle* h, int32_t which, const double* r, double* z);
 int cpc_apply_Bcom(cpc_handle* h, const double* r, double* z);
 
@@ -265,6 +268,13 @@ int cpc_setup_phases_ms(const cpc_handle* h, double* ms, int32_t cap);
  * max_ij |(I - A_c X)_ij|, computed on the device in FP64.  Either pointer may be NULL.  Host
  * memory.  Returns CPC_OK, or CPC_EINVAL if h is NULL. */
 int cpc_coarse_inverse_info(const cpc_handle* h, int32_t* method, double* residual);
+
+/* Limit of the waits between the rows of a sweep or triangular solve that run as one launch, in polls of
+ * about a quarter of a microsecond; 0 (default): a limit that follows from the layout, at least 2^21.  A
+ * wait that gives up takes NaN for the row it waited for, and its launch ends; CPC_ETIMEOUT reports it.  For
+ * callers that share the GPU with work that can hold a launch up for longer, or that want to hear of
+ * it sooner.  Synchronises the stream. */
+int cpc_set_wait_polls(cpc_handle* h, int32_t polls);
 
 /* ---- inspection (tests and diagnostics; all synchronous, outputs in HOST memory) ---------- */
 
@@ -325,7 +335,8 @@ int cpc_ic0_values(const cpc_handle* h, double* lu);
 /* Level operators on device vectors, for parity tests: op 0 y = A_l x; 1 y = S_l x (forward
  * Gauss-Seidel sweep, zero guess); 2 y = S_l^T x (backward sweep); 3 y = A_l^{-1} x (coarsest
  * level); 4 y = V-cycle from level l with zero initial guess; 5 one forward Gauss-Seidel sweep on
- * A_l y = x starting from the given y (the sweep's launches, nothing else).  Asynchronous. */
+ * A_l y = x starting from the given y (the sweep's launches, nothing else).  Asynchronous; a wait that
+ * gives up is reported as for cpc_apply_precond. */
 int cpc_level_apply(cpc_handle* h, int32_t level, int32_t op, const double* x, double* y);
 
 #ifdef __cplusplus

@@ -67,6 +67,7 @@ SIGNATURES = [
     ("cpc_spmv", _I32, [_P, _P, _P]),
     ("cpc_setup_time_ms", _I32, [_P, _P, _P]),
     ("cpc_solve_launches", _I32, [_P, _P, _P]),
+    ("cpc_set_wait_polls", _I32, [_P, _I32]),
     ("cpc_sweep_time_us", _I32, [_P, _I32, _I32, _P]),
     ("cpc_setup_phases_ms", _I32, [_P, _P, _I32]),
     ("cpc_coarse_inverse_info", _I32, [_P, _P, _P]),
@@ -336,6 +337,10 @@ class Solver:
         a, b = ctypes.c_double(), ctypes.c_double()
         _check(load().cpc_setup_time_ms(self._h, ctypes.byref(a), ctypes.byref(b)), self._h)
         return a.value, b.value
+
+    def set_wait_polls(self, polls=0):
+        """Polls after which a wait between the rows of a sweep gives up (cpc_set_wait_polls); 0: the default."""
+        _check(load().cpc_set_wait_polls(self._h, int(polls)), self._h)
 
     # -- inspection ------------------------------------------------------------------------------
     def solve_launches(self):

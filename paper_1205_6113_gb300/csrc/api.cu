@@ -253,6 +253,15 @@ int cpc_coarse_inverse_info(const cpc_handle* h, int32_t* method, double* residu
     return CPC_OK;
 }
 
+int cpc_set_wait_polls(cpc_handle* h, int32_t polls) {
+    if (!h || polls < 0) return CPC_EINVAL;
+    return guarded(h, [&] {
+        CPC_CK(cudaStreamSynchronize(h->h.s));
+        if (polls != h->h.wait_polls) cpc::destroy_graphs(h->h);     // the solve's graph holds the limit
+        h->h.wait_polls = polls;
+    });
+}
+
 int cpc_sweep_time_us(cpc_handle* h, int32_t level, int32_t reps, double* us) {
     if (!h || !us) return CPC_EINVAL;
     return guarded(h, [&] { *us = cpc::sweep_time_us(h->h, level, reps); });

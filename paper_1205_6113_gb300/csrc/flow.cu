@@ -11,7 +11,7 @@
 // rows of earlier groups, hence on chunks that running warps already hold; so whatever the
 // scheduling, the earliest unfinished chunk never waits for one that has not started.  Sums are
 // taken in entry order whatever the order of arrival, so results are reproducible to the bit.
-// A wait gives up after FLOW_SPINS polls: it takes NaN for what is missing and sets *err.
+// A wait gives up after a number of polls: it takes NaN for what is missing and sets *err.
 #include "flow.cuh"
 #include "handle.cuh"
 
@@ -19,7 +19,12 @@ namespace cpc {
 
 namespace {
 
-constexpr int FLOW_SPINS = 1 << 21;      // about a second of polls
+// Polls (a quarter of a microsecond each) after which a wait gives up: a chunk waits at most for the chunks
+// in flight, one after another, each of `batches` batches of some ten polls; three times that, and at
+// least half a second.
+inline int flow_polls(int64_t chunks, int64_t batches) {
+    return (int)std::min<int64_t>(std::max<int64_t>(32 * chunks * batches, 1 << 21), 1 << 30);
+}
 
 // v = *p if on, else v unchanged: a predicated load and no branch, so that the loads of a batch are
 // all in flight before the first value is looked at (with a branch per load a poll took a round
@@ -70,7 +75,7 @@ struct FlowBatch {
             acc += v[u] * xv[u];
         }
     }
-    __device__ __forceinline__ void add_new(const VT* x, VT& acc, int* err) {
+    __device__ __forceinline__ void add_new(const VT* x, VT& acc, int* err, int polls) {
         using U = Unset<VT>;
         typename U::B b[M];
 #pragma unroll
@@ -83,7 +88,7 @@ struct FlowBatch {
 #pragma unroll
             for (int u = 0; u < M; ++u) miss |= b[u] == U::bits;
             if (!__any_sync(0xffffffffu, miss)) break;
-            if (spin == FLOW_SPINS) {
+            if (spin == polls) {
                 if (miss) *err = 1;
 #pragma unroll
                 for (int u = 0; u < M; ++u) b[u] = b[u] == U::bits ? U::nan : b[u];
@@ -101,7 +106,7 @@ struct FlowBatch {
     // The same over a row whose entries keep their order: the new values of one part, the old ones of
     // the other, told apart by LATER.  MODE FLOW_FWD0 takes no old ones (they are zero).
     template <int MODE>
-    __device__ __forceinline__ void add_mixed(const VT* xo, const VT* xn, VT& acc, int* err) {
+    __device__ __forceinline__ void add_mixed(const VT* xo, const VT* xn, VT& acc, int* err, int polls) {
         using U = Unset<VT>;
         typename U::B b[M];
         auto from = [&](int u) {
@@ -119,7 +124,7 @@ struct FlowBatch {
 #pragma unroll
             for (int u = 0; u < M; ++u) miss |= b[u] == U::bits;
             if (!__any_sync(0xffffffffu, miss)) break;
-            if (spin == FLOW_SPINS) {
+            if (spin == polls) {
                 if (miss) *err = 1;
 #pragma unroll
                 for (int u = 0; u < M; ++u) b[u] = b[u] == U::bits ? U::nan : b[u];
@@ -138,7 +143,7 @@ struct FlowBatch {
 // waits for an SM to empty before it can start (the IC(0) solves above: 190 us more an application).
 template <class MT, class DT, class FT, class VT, int MODE, int M, bool WIDE>
 __global__ void __launch_bounds__(WIDE ? 128 : 32) k_flow(SV<MT, DT> A, const int* __restrict__ cmid, int nchunks, const FT* f,
-                                             const VT* xo, VT* xn, VT* unset, VT* zadd, unsigned* ctr, int* err) {
+                                             const VT* xo, VT* xn, VT* unset, VT* zadd, unsigned* ctr, int* err, int polls) {
     constexpr bool UP = MODE == FLOW_BWD;
     constexpr bool TRI = MODE == FLOW_LOWER || MODE == FLOW_UPPER;
     // FP32 rows keep their entries in column order, the two parts mixed
@@ -189,8 +194,8 @@ __global__ void __launch_bounds__(WIDE ? 128 : 32) k_flow(SV<MT, DT> A, const in
             }
         }
         auto add = [&] {
-            if constexpr (MIX) bn.template add_mixed<MODE>(xo, xn, acc, err);
-            else bn.add_new(xn, acc, err);
+            if constexpr (MIX) bn.template add_mixed<MODE>(xo, xn, acc, err, polls);
+            else bn.add_new(xn, acc, err, polls);
         };
         add();
         for (int p = 32 * M; p < ne - nb; p += 32 * M) {
@@ -230,7 +235,7 @@ inline int sweep_lanes(const Sell& S, bool fp64) { return fp64 ? std::max(S.lane
 
 template <int MODE, class MT, class DT, class FT, class VT>
 void flow_mode(const Sell& S, SV<MT, DT> v, const FT* f, const VT* xo, VT* xn, VT* unset, VT* zadd, unsigned* ctr,
-               int* err, cudaStream_t s) {
+               int* err, int polls, cudaStream_t s) {
     // Chunks in flight: four groups' worth, enough to have the matrix data of a chunk on hand when its
     // turn comes, and no more, since waiting warps slow the working ones down (IC(0) of 120,000 cells,
     // 25 chunks a level: 250 us with every chunk in flight, 150 with 304).  Where that is most of what
@@ -241,12 +246,13 @@ void flow_mode(const Sell& S, SV<MT, DT> v, const FT* f, const VT* xo, VT* xn, V
     const int lanes = MODE == FLOW_LOWER || MODE == FLOW_UPPER ? S.lanes : sweep_lanes(S, std::is_same<VT, double>::value);
     auto go = [&](auto m) {
         constexpr int M = decltype(m)::value;
+        if (polls <= 0) polls = flow_polls(std::min(S.nchunks, wide ? 64 * flow_sms() : ahead), (lanes + M - 1) / M);
         if (wide)
             launch(k_flow<MT, DT, FT, VT, MODE, M, true>, (S.nchunks + 3) / 4, 128, s, v, (const int*)S.cmid.p, S.nchunks, f,
-                   xo, xn, unset, zadd, ctr, err);
+                   xo, xn, unset, zadd, ctr, err, polls);
         else
             launch(k_flow<MT, DT, FT, VT, MODE, M, false>, std::min(S.nchunks, ahead), 32, s, v, (const int*)S.cmid.p,
-                   S.nchunks, f, xo, xn, unset, zadd, ctr, err);
+                   S.nchunks, f, xo, xn, unset, zadd, ctr, err, polls);
     };
     with_m(lanes, go);
 }
@@ -285,10 +291,10 @@ bool gs_by_flow(const Sell& S, int n, VType vt) {
 
 template <class FT, class VT>
 void rec_flow(FlowMode mode, const Sell& S, VType vt, const FT* f, const VT* xo, VT* xn, VT* unset, VT* zadd,
-              unsigned* ctr, int* err, cudaStream_t s) {
+              unsigned* ctr, int* err, int polls, cudaStream_t s) {
     if (S.nchunks == 0) return;
     auto go = [&](auto v, auto md) {
-        flow_mode<decltype(md)::value>(S, v, f, xo, xn, unset, zadd, ctr, err, s);
+        flow_mode<decltype(md)::value>(S, v, f, xo, xn, unset, zadd, ctr, err, polls, s);
     };
     auto sweep = [&](auto v) {
         if (mode == FLOW_FWD0) go(v, std::integral_constant<int, FLOW_FWD0>{});
@@ -320,10 +326,10 @@ void rec_flow(FlowMode mode, const Sell& S, VType vt, const FT* f, const VT* xo,
 }
 
 template void rec_flow<double, double>(FlowMode, const Sell&, VType, const double*, const double*, double*, double*,
-                                       double*, unsigned*, int*, cudaStream_t);
+                                       double*, unsigned*, int*, int, cudaStream_t);
 template void rec_flow<double, float>(FlowMode, const Sell&, VType, const double*, const float*, float*, float*, float*,
-                                      unsigned*, int*, cudaStream_t);
+                                      unsigned*, int*, int, cudaStream_t);
 template void rec_flow<float, float>(FlowMode, const Sell&, VType, const float*, const float*, float*, float*, float*,
-                                     unsigned*, int*, cudaStream_t);
+                                     unsigned*, int*, int, cudaStream_t);
 
 }  // namespace cpc

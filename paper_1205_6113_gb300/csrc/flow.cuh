@@ -36,9 +36,10 @@ __device__ __forceinline__ void flow_unset(VT* p) {
 // Records a flow launch over all chunks of S.  f: right-hand side; xo: old values; xn: new values,
 // unset on entry except where a row is already known; unset: own-row elements marked unset once f
 // has been read (may be null, may be f's own storage); zadd: += the new value (may be null).
-// ctr: a counter of this launch's own, 0 on entry and on exit; err: set to 1 when a wait gave up.
+// ctr: a counter of this launch's own, 0 on entry and on exit; err: set to 1 when a wait gave up, after
+// polls polls (0: a number that follows from S, flow.cu).  Every element of xn is written all the same.
 template <class FT, class VT>
 void rec_flow(FlowMode mode, const Sell& S, VType vt, const FT* f, const VT* xo, VT* xn, VT* unset, VT* zadd,
-              unsigned* ctr, int* err, cudaStream_t s);
+              unsigned* ctr, int* err, int polls, cudaStream_t s);
 
 }  // namespace cpc

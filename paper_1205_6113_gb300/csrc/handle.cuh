@@ -59,7 +59,8 @@ struct Batched {
 // Device-side scalars of one PCG run (all reductions finish in fixed order).
 struct PcgState {
     double bnorm, rz, rz_old, pq, alpha, beta, rr, tol, res;
-    int k, maxit, status, gave_up;   // gave_up: a flow launch's wait ran out
+    int k, maxit, status;
+    int gave_up;            // a flow launch's wait ran out; stays set until a synchronising call reports it
 };
 
 struct Handle {
@@ -110,6 +111,7 @@ struct Handle {
     // prologue starts early never draws on the counter of one still running.
     DBuf<unsigned> flow_ctr;
     unsigned flow_seq = 0;
+    int wait_polls = 0;     // polls of their waits (0: by the layout)
     unsigned* next_flow_ctr() { return flow_ctr.p + flow_seq++ % FLOW_RING; }
     DBuf<PcgState> state;
     DBuf<double> hist;
@@ -176,6 +178,8 @@ void solve_pcg(Handle& h, const double* b, double* x, double tol, int maxit, int
                double* res_hist, int hist_cap, int* status);
 void level_apply(Handle& h, int l, int op, const double* x, double* y);
 double sweep_time_us(Handle& h, int l, int reps);
+// Throws CPC_ETIMEOUT if gave_up, after clearing the handle's flag.
+void report_gave_up(Handle& h, int gave_up);
 void destroy_graphs(Handle& h);
 void ensure_solve_graph(Handle& h, int which);
 

@@ -11,6 +11,7 @@
 // block partials in index order), so iteration counts are reproducible run to run.
 #include <algorithm>
 #include <cstdio>
+#include <cstddef>
 #include <type_traits>
 #include <utility>
 
@@ -926,7 +927,8 @@ template <> const float* dnat<float>(const Level& L) { return L.dnat32.p; }
 template <class FT, class VT>
 void rec_sweep(Handle& h, int l, FlowMode mode, const FT* f, const VT* xo, VT* xn, cudaStream_t s) {
     Level& L = h.lev[l];
-    rec_flow<FT, VT>(mode, L.S, L.vt, f, xo, xn, nullptr, nullptr, h.next_flow_ctr(), &h.state.p->gave_up, s);
+    rec_flow<FT, VT>(mode, L.S, L.vt, f, xo, xn, nullptr, nullptr, h.next_flow_ctr(), &h.state.p->gave_up,
+                     h.wait_polls, s);
 }
 
 // f_c = R r onto level l + 1, with what its sweep starts from (k_restrict).
@@ -1050,8 +1052,9 @@ void rec_ic_solve(Handle& h, const TT* t, VT* y, VT* w, VT* zadd, cudaStream_t s
     }
     if (h.ic_flow()) {
         int* err = &h.state.p->gave_up;
-        rec_flow<TT, VT>(FLOW_LOWER, L, VT_F32, t, nullptr, y, w, nullptr, h.next_flow_ctr(), err, s);   // marks w unset
-        rec_flow<VT, VT>(FLOW_UPPER, U, VT_F32, y, nullptr, w, y, zadd, h.next_flow_ctr(), err, s);      // and y again
+        const int polls = h.wait_polls;
+        rec_flow<TT, VT>(FLOW_LOWER, L, VT_F32, t, nullptr, y, w, nullptr, h.next_flow_ctr(), err, polls, s);  // marks w unset
+        rec_flow<VT, VT>(FLOW_UPPER, U, VT_F32, y, nullptr, w, y, zadd, h.next_flow_ctr(), err, polls, s);     // and y again
         return;
     }
     for (int g = 0; g + 1 < (int)L.seg.size(); ++g) {
@@ -1221,7 +1224,7 @@ float time_gs_sweep(const Sell& S, int n) {
     for (int k = 0; k < SWEEPS; ++k) {      // the launches of the solve's sweeps
         if (flow) {
             launch(k_fill_unset<double>, vec_blocks(n), VEC_TPB, cs, (int64_t)n, xa.p);
-            rec_flow<double, double>(FLOW_FWD, S, VT_F64, f.p, x.p, xa.p, nullptr, nullptr, ctr.p + k, (int*)(ctr.p + SWEEPS), cs);
+            rec_flow<double, double>(FLOW_FWD, S, VT_F64, f.p, x.p, xa.p, nullptr, nullptr, ctr.p + k, (int*)(ctr.p + SWEEPS), 0, cs);
             continue;
         }
         for (size_t c = 0; c + 1 < S.seg.size(); ++c) {
@@ -1256,7 +1259,9 @@ float time_gs_sweep(const Sell& S, int n) {
         CPC_CK(cudaEventElapsedTime(&ms, e0, e1));
         best = std::min(best, ms / SWEEPS);
     }
-    return best;
+    unsigned gave_up = 0;                   // a layout whose sweep did is not chosen
+    CPC_CK(cudaMemcpy(&gave_up, ctr.p + SWEEPS, sizeof(unsigned), cudaMemcpyDeviceToHost));
+    return gave_up ? 1e30f : best;
 }
 
 void level_apply(Handle& h, int l, int op, const double* x, double* y) {
@@ -1377,7 +1382,16 @@ double sweep_time_us(Handle& h, int l, int reps) {
         CPC_CK(cudaEventElapsedTime(&ms, e0, e1));
         best = std::min(best, ms);
     }
+    int gave_up = 0;
+    CPC_CK(cudaMemcpy(&gave_up, &h.state.p->gave_up, sizeof(int), cudaMemcpyDeviceToHost));
+    report_gave_up(h, gave_up);
     return 1000.0 * best / reps;
+}
+
+void report_gave_up(Handle& h, int gave_up) {
+    if (!gave_up) return;
+    CPC_CK(cudaMemsetAsync(&h.state.p->gave_up, 0, sizeof(int), h.s));
+    fail(CPC_ETIMEOUT, "a wait for a row of a sweep or triangular solve gave up, in this call or in an application before it");
 }
 
 void destroy_graphs(Handle& h) {
@@ -1467,11 +1481,11 @@ void solve_pcg(Handle& h, const double* b, double* x, double tol, int maxit, int
     if (!h.gexec[which]) build_solve_graph(h, which);
     cudaStream_t s = h.s;
     const int n = h.n;
-    // parameters for this run, then the graph
+    // parameters for this run (all but gave_up, its last member), then the graph
     PcgState init{};
     init.tol = tol;
     init.maxit = maxit;
-    CPC_CK(cudaMemcpyAsync(h.state.p, &init, sizeof(PcgState), cudaMemcpyHostToDevice, s));
+    CPC_CK(cudaMemcpyAsync(h.state.p, &init, offsetof(PcgState, gave_up), cudaMemcpyHostToDevice, s));
     CPC_CK(cudaMemcpyAsync(h.b.p, b, sizeof(double) * n, cudaMemcpyDeviceToDevice, s));
     CPC_CK(cudaGraphLaunch(h.gexec[which], s));
     CPC_CK(cudaMemcpyAsync(x, h.x.p, sizeof(double) * n, cudaMemcpyDeviceToDevice, s));
@@ -1480,7 +1494,7 @@ void solve_pcg(Handle& h, const double* b, double* x, double tol, int maxit, int
     CPC_CK(cudaStreamSynchronize(s));
     *iters = out.k;
     *status = out.status;
-    if (out.gave_up) fail(CPC_ETIMEOUT, "a dependent row was not reached in time");
+    report_gave_up(h, out.gave_up);
     if (res_hist && hist_cap > 0) {
         const int cnt = std::min(std::min(hist_cap, out.k + 1), HIST_CAP);
         CPC_CK(cudaMemcpy(res_hist, h.hist.p, sizeof(double) * cnt, cudaMemcpyDeviceToHost));

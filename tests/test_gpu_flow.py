@@ -164,3 +164,31 @@ def test_sweeps_of_more_chunks_than_the_gpu_holds_keep_their_launches():
     assert i["n"] // i["ncolours"] <= 24000 and i["n"] / (s.level_layout(2)["C"] * i["ncolours"]) > 0.75 * 2432
     by_colours = sum(2 * s.level_info(l)["ncolours"] - 1 + 3 for l in (1, 2))
     assert s.solve_launches()[0] >= 5 + 2 * (7 + by_colours + 1)
+
+
+@pytest.mark.parametrize("precision", ["fp64", "fp32"])
+def test_a_wait_that_gives_up_is_reported_once(precision):
+    """With one poll a wait, rows of later wavefronts give up at once (the first of them start together): the
+    launches end, the result holds NaN, the next call that synchronises says so, and nothing is left behind."""
+    p = inputs.small_3d(40, 36, 20, seed=92)
+    s = solver(p, precision=precision)
+    b = torch.tensor(inputs.random_vector(p.n, 93), device=DEV)
+    z = s.apply(b)
+    x, iters, status, _ = s.solve(b, tol=1e-8)
+    for call in (lambda: s.solve(b, tol=1e-8), lambda: s.sweep_time_us(1)):
+        s.set_wait_polls(1)
+        assert bool(torch.isnan(s.apply(b)).any())
+        s.set_wait_polls(0)
+        with pytest.raises(cpc.CpcError) as e:
+            call()
+        assert e.value.code == 6
+        assert torch.equal(s.apply(b), z)
+        again = s.solve(b, tol=1e-8)
+        assert torch.equal(again[0], x) and again[1:3] == (iters, status)
+    s.set_wait_polls(1)
+    with pytest.raises(cpc.CpcError) as e:
+        s.solve(b, tol=1e-8)
+    assert e.value.code == 6
+    s.set_wait_polls(0)
+    again = s.solve(b, tol=1e-8)
+    assert torch.equal(again[0], x) and again[1:3] == (iters, status)
