@@ -171,7 +171,7 @@ struct Entries {
 
 // acc[j] += sum_w a_w x[col_w][j] over entries w0, w0 + step, ... of a row, U entries' gathers in flight
 // together and the next entries' columns beside them; m holds the first ones, loaded by the caller before it
-// waits for x.  Padding (-1) and marked columns (LATER) load nothing and add 0.  (With each batch's columns
+// waits for x.  Padding (-1) and marked columns (below -1) load nothing and add 0.  (With each batch's columns
 // loaded before its own gathers a row cost two trips through L2 per batch and one more after the wait:
 // 64 solves and adjoints at 1M 220 -> 203 ms, 28 at 433k cells 63.6 -> 53.2, a block solve of 12 22.9 -> 20.7.)
 template <int J, int R, int U, class VT, class MT, class XT>
@@ -182,7 +182,7 @@ __device__ __forceinline__ void brow(const int* __restrict__ col, const MT* __re
         VT xv[U][J];
 #pragma unroll
         for (int u = 0; u < U; ++u) {
-            if ((unsigned)m.c[u] < (unsigned)LATER) {
+            if (takes(m.c[u])) {
                 ldv<J>(x + L::at(m.c[u]), xv[u]);
             } else {
 #pragma unroll

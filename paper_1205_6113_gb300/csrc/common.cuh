@@ -135,8 +135,13 @@ enum VType { VT_F64 = 0, VT_F32 = 1, VT_BF16 = 2 };
 
 // An FP64 smoother layout keeps a row's entries of earlier and of later groups apart (Sell::cmid).  In an
 // FP32 one they stay in column order, so that a sum is rounded the same whichever of them it takes, and
-// Sell::fcol marks the columns of later groups with this bit: a sweep from a zero guess skips them.
-constexpr int LATER = 1 << 30;
+// Sell::fcol holds the columns of later groups below -1 (padding is -1 in both): a sweep from a zero guess
+// takes the columns from 0 on, any other takes all but the padding.
+__host__ __device__ constexpr int mark_later(int col) { return -2 - col; }
+__host__ __device__ constexpr bool is_later(int c) { return c < -1; }
+__host__ __device__ constexpr int marked_col(int c) { return c < -1 ? -2 - c : c; }
+// Whether a sum over col, or over fcol from a zero guess, takes the entry.
+__host__ __device__ constexpr bool takes(int c) { return c >= 0; }
 
 struct DiaOff {
     int o[8];
@@ -161,7 +166,7 @@ struct Sell {
     // group in [cmid[k], cptr[k+1]).  lanes_lo / lanes_up: most entries one lane holds of each part.
     int lanes_lo = 0, lanes_up = 0;
     DBuf<int> perm, cptr, cmid, col;
-    DBuf<int> fcol;                    // FP32 smoother copy: col with the columns of later groups marked
+    DBuf<int> fcol;                    // FP32 smoother copy: col with the columns of later groups marked (mark_later)
     DBuf<double> val, diag, dinv;      // FP64 copy (always); dinv = 1 / diag (split diagonal only)
     DBuf<float> val32, diag32, dinv32; // FP32 copy (mixed precision)
     DBuf<__nv_bfloat16> val16;         // BF16 copy of off-diagonals (coarse levels, mode 2)

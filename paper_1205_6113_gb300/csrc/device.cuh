@@ -68,7 +68,7 @@ inline void launch(void (*k)(KArgs...), int grid, int block, cudaStream_t s, Arg
 
 // One batch of exactly M entries per lane (entries o, o + 32, ... with oo < e; the others load
 // nothing and add 0): loads, then (WAIT) the wait and the caller's hook, then the gathers, then the
-// products in entry order.  Padding (-1) and marked columns (LATER) load nothing and add 0.
+// products in entry order.  Padding (-1) and marked columns (below -1) load nothing and add 0.
 template <int M, bool WAIT, class VT, class MT, class XT, class H>
 __device__ __forceinline__ void sell_batch(const int* __restrict__ col, const MT* __restrict__ val, int o, int e,
                                            const XT* x, VT& acc, H& after_wait) {
@@ -85,7 +85,7 @@ __device__ __forceinline__ void sell_batch(const int* __restrict__ col, const MT
         after_wait();           // the caller's own loads of predecessor data, in flight with the gathers
     }
 #pragma unroll
-    for (int u = 0; u < M; ++u) xv[u] = (unsigned)c[u] < (unsigned)LATER ? Cv<VT>::f(x[c[u]]) : VT(0);
+    for (int u = 0; u < M; ++u) xv[u] = takes(c[u]) ? Cv<VT>::f(x[c[u]]) : VT(0);
 #pragma unroll
     for (int u = 0; u < M; ++u) acc += v[u] * xv[u];
 }

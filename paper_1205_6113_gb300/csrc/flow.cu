@@ -104,20 +104,17 @@ struct FlowBatch {
         }
     }
     // The same over a row whose entries keep their order: the new values of one part, the old ones of
-    // the other, told apart by LATER.  MODE FLOW_FWD0 takes no old ones (they are zero).
+    // the other, told apart by the mark.  MODE FLOW_FWD0 takes no old ones (they are zero).
     template <int MODE>
     __device__ __forceinline__ void add_mixed(const VT* xo, const VT* xn, VT& acc, int* err, int polls) {
         using U = Unset<VT>;
         typename U::B b[M];
-        auto from = [&](int u) {
-            const bool later = c[u] & LATER;
-            return (later == (MODE == FLOW_BWD) ? xn : xo) + (c[u] & ~LATER);
-        };
+        auto on = [&](int u) { return MODE == FLOW_FWD0 ? takes(c[u]) : c[u] != -1; };
+        auto from = [&](int u) { return on(u) ? (is_later(c[u]) == (MODE == FLOW_BWD) ? xn : xo) + marked_col(c[u]) : xn; };
 #pragma unroll
         for (int u = 0; u < M; ++u) {
-            if (c[u] < 0 || (MODE == FLOW_FWD0 && (c[u] & LATER))) c[u] = -1;
             b[u] = 0;
-            flow_ld(b[u], c[u] >= 0 ? from(u) : xn, c[u] >= 0);
+            flow_ld(b[u], from(u), on(u));
         }
         for (int spin = 0;; ++spin) {
             bool miss = false;
@@ -131,7 +128,7 @@ struct FlowBatch {
                 break;
             }
 #pragma unroll
-            for (int u = 0; u < M; ++u) flow_ld(b[u], c[u] >= 0 ? from(u) : xn, b[u] == U::bits);
+            for (int u = 0; u < M; ++u) flow_ld(b[u], from(u), b[u] == U::bits);
         }
 #pragma unroll
         for (int u = 0; u < M; ++u) acc += v[u] * flow_val(b[u]);

@@ -1581,7 +1581,7 @@ __global__ void k_flag_later(int nslots, int C, const int* perm, const int* cptr
     const int i = perm[s], k = s / C;
     for (int e = cptr[k] + s % C; e < cptr[k + 1]; e += C) {
         const int j = col[e];
-        fcol[e] = i >= 0 && j >= 0 && key[j] > key[i] ? j | LATER : j;
+        fcol[e] = i >= 0 && j >= 0 && key[j] > key[i] ? mark_later(j) : j;
     }
 }
 

@@ -239,7 +239,7 @@ __global__ void __launch_bounds__(SELL_TPB) k_spmv_dia(DV<MT, DT> A, const XT* x
 // with the view's diagonal field holding 1 / a_ii (a multiply instead of an FP64 division).
 // Rows of one colour are not coupled, so they update in parallel exactly as in sequential order.
 // LOW: in a forward sweep from a zero guess the rows of later colours are still zero, so only the
-// entries of earlier colours are taken: up to cmid in FP64, those not marked LATER in FP32.
+// entries of earlier colours are taken: up to cmid in FP64, those not marked later in FP32.
 template <class MT, class DT, class FT, class VT, int U, bool LOW>
 __global__ void __launch_bounds__(SELL_TPB) k_gs(SV<MT, DT> A, const int* __restrict__ cmid, int c0, int c1, const FT* f,
                                                  VT* x) {

@@ -1,0 +1,34 @@
+"""Rules of the SELL layouts that need no GPU, compiled for the host from the library's own header."""
+import os
+import shutil
+import subprocess
+
+import pytest
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+NVCC = shutil.which("nvcc") or "/usr/local/cuda/bin/nvcc"
+
+
+def run(tmp_path, body):
+    src, exe = tmp_path / "t.cu", tmp_path / "t"
+    src.write_text('#include "common.cuh"\n#include <cstdint>\n#include <cstdio>\nusing namespace cpc;\n'
+                   "#define OK(c) if (!(c)) { std::printf(\"%%d: %%s\\n\", __LINE__, #c); return 1; }\n"
+                   "int main() {\n%s\nreturn 0;\n}\n" % body)
+    subprocess.run([NVCC, "-std=c++17", "-O1", "--expt-relaxed-constexpr", "-I", os.path.join(ROOT, "paper_1205_6113_gb300", "csrc"), str(src),
+                    "-o", str(exe)], check=True)
+    r = subprocess.run([str(exe)], capture_output=True, text=True)
+    assert r.returncode == 0, r.stdout
+
+
+@pytest.mark.skipif(not os.path.exists(NVCC), reason="no nvcc")
+def test_columns_and_their_marks_take_every_int32(tmp_path):
+    """A column up to the last of the largest matrix is taken as it is; marked, it is skipped from a zero
+    guess and found again; padding is neither."""
+    run(tmp_path, """
+    for (int64_t j : {0ll, 1ll, (1ll << 30) - 1, 1ll << 30, (1ll << 30) + 1, (1ll << 31) - 2}) {
+        const int c = (int)j, m = mark_later(c);
+        OK(takes(c) && !is_later(c) && marked_col(c) == c && c != -1)
+        OK(!takes(m) && is_later(m) && marked_col(m) == c && m != -1)
+    }
+    OK(!takes(-1) && !is_later(-1))
+""")
