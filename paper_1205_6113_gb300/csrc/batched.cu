@@ -417,7 +417,7 @@ __global__ void __launch_bounds__(CWARPS * 32) kb_coarse_seq(int n, const AT* __
     using L = Cols<J, R>;
     constexpr int KP = L::KP, ROWS = CWARPS * R * SROWS, TPB = CWARPS * 32;
     constexpr int FPT = (CTILE * KP + TPB - 1) / TPB, APT = (ROWS * CTILE + TPB - 1) / TPB;
-    __shared__ VT fs[CTILE * KP];
+    __shared__ __align__(16) VT fs[CTILE * KP];          // read by ldv, up to 16 bytes at a time
     __shared__ VT as[ROWS][CTILE + 1];
     pdl_launch_dependents();
     const int t = threadIdx.x, b0 = blockIdx.x * ROWS;
@@ -1054,7 +1054,7 @@ enum { KF_BAD = 0, KF_DONE, KF_COUNT };
 template <int KP, class UT>
 __global__ void __launch_bounds__(KK_TPB) kk_gram(int n, const UT* U, const double* V, double* __restrict__ part) {
     constexpr int T = KP / 4, NT = T * (T + 1) / 2, GROUPS = KK_TPB / NT, ROWS = KK_ELEMS / KP;
-    extern __shared__ double ksm[];
+    extern __shared__ __align__(16) double ksm[];
     double* us = ksm;                      // [ROWS][KP]
     double* vs = ksm + KK_ELEMS;           // [ROWS][KP]
     const int t = threadIdx.x, grp = t / NT;
@@ -1140,7 +1140,7 @@ __global__ void __launch_bounds__(256) kk_gram_sum(int G, int Kp, const double* 
 // With copy_to, W is copied there afterwards (gamma_old <- gamma_new).
 __global__ void __launch_bounds__(KK_TPB) kk_solve(int K, int Kp, const double* S, const double* W,
                                                    double* __restrict__ out, double* copy_to, int* flag) {
-    extern __shared__ double ksm[];
+    extern __shared__ __align__(16) double ksm[];
     double* L = ksm;                       // [K][K]
     double* Y = ksm + K * K;               // [K][K]
     __shared__ int bad;
@@ -1221,7 +1221,7 @@ __global__ void __launch_bounds__(BTPB) kk_update(int n, int K, double* __restri
     using L = Cols<J, R>;
     constexpr int Kp = L::KP;
     if (flag[KF_BAD]) return;              // a K x K solve failed: keep the last good iterate
-    extern __shared__ double ksm[];
+    extern __shared__ __align__(16) double ksm[];
     double* al = ksm;                      // [Kp][Kp]
     double* ws = ksm + Kp * Kp;            // [BWARPS R][Kp]
     for (int e = threadIdx.x; e < Kp * Kp; e += BTPB) al[e] = alpha[e];
@@ -1274,7 +1274,7 @@ __global__ void __launch_bounds__(BTPB) kk_pupdate(int n, int K, const ZT* Z, do
     using L = Cols<J, R>;
     constexpr int Kp = L::KP;
     if (flag[KF_BAD]) return;
-    extern __shared__ double ksm[];
+    extern __shared__ __align__(16) double ksm[];
     for (int e = threadIdx.x; e < Kp * Kp; e += BTPB) ksm[e] = beta[e];
     __syncthreads();
     for (int i0 = (blockIdx.x * BWARPS + (threadIdx.x >> 5)) * R; i0 < n; i0 += gridDim.x * BWARPS * R) {

@@ -32,3 +32,15 @@ def test_columns_and_their_marks_take_every_int32(tmp_path):
     }
     OK(!takes(-1) && !is_later(-1))
 """)
+
+
+def test_shared_arrays_of_vector_loads_are_aligned():
+    """ldv reads up to 16 bytes at a time: every shared array that it reads is declared so."""
+    import re
+    text = open(os.path.join(ROOT, "paper_1205_6113_gb300", "csrc", "batched.cu")).read()
+    shared = dict((name, decl) for decl, name in re.findall(r"((?:extern )?__shared__ [^;\n]*?\b(\w+)\[)", text))
+    alias = dict(re.findall(r"double\* (\w+) = (ksm)\b", text))
+    read = {alias.get(a, a) for a in re.findall(r"\bldv<\w+>\((\w+)", text)} & set(shared)
+    assert read == {"fs", "ksm"}
+    decls = [d for d in re.findall(r"(?:extern )?__shared__ [^;\n]*", text) if re.search(r"\b(fs|ksm)\[", d)]
+    assert len(decls) == 5 and all("__align__(16)" in d for d in decls), decls
