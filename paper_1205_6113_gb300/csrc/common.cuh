@@ -143,6 +143,9 @@ __host__ __device__ constexpr int marked_col(int c) { return c < -1 ? -2 - c : c
 // Whether a sum over col, or over fcol from a zero guess, takes the entry.
 __host__ __device__ constexpr bool takes(int c) { return c >= 0; }
 
+// Whether chunks of so many entries, padding included, can be addressed by the 32-bit offsets of a Sell.
+constexpr bool sell_fits(int64_t entries) { return entries <= INT32_MAX; }
+
 struct DiaOff {
     int o[8];
 };

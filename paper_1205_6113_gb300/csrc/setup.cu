@@ -1656,6 +1656,13 @@ __global__ void k_recip(int n, const double* d, double* r) {
     if (i < n) r[i] = 1.0 / d[i];
 }
 
+__global__ void k_sum_int(const int* a, int n, unsigned long long* out) {
+    unsigned long long m = 0;
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) m += (unsigned long long)a[i];
+    for (int o = 16; o > 0; o >>= 1) m += __shfl_xor_sync(0xffffffffu, m, o);
+    if ((threadIdx.x & 31) == 0 && m > 0) atomicAdd(out, m);
+}
+
 // Chunk height for rows of average length avg: 32 / G rows per warp with G lanes sharing a row,
 // G the largest power of two <= avg / 4 (1..8), so that a row costs one round of loads.
 int choose_chunk(double avg) {
@@ -1666,10 +1673,11 @@ int choose_chunk(double avg) {
 
 // Fill a Sell of chunk height C from CSR rows in the slot order `slots` (device, nslots entries).
 // key (device, may be null): the rows' group (by_col: the columns' group); splits each chunk by it
-// (Sell::cmid).
-void build_sell(const int* ptr, const int* col, const double* val, const DBuf<int>& slots, int nslots,
+// (Sell::cmid).  Padding counts: chunks whose entries exceed the layout's 32-bit offsets are an error, or with
+// may_halve give false, for the caller to take half the chunk height (1 has no padding).
+bool build_sell(const int* ptr, const int* col, const double* val, const DBuf<int>& slots, int nslots,
                 const std::vector<int>& seg, int C, int mode, bool split_diag, const int* imap, Sell& S,
-                cudaStream_t s, const int* key = nullptr, bool by_col = false) {
+                cudaStream_t s, const int* key = nullptr, bool by_col = false, bool may_halve = false) {
     S.nslots = nslots;
     S.C = C;
     S.nchunks = nslots / C;
@@ -1683,6 +1691,16 @@ void build_sell(const int* ptr, const int* col, const double* val, const DBuf<in
     int wm[3];
     CPC_CK(cudaMemcpyAsync(wm, wmax.get(), sizeof wm, cudaMemcpyDeviceToHost, s));
     S.nelem = d2h(S.cptr.p + S.nchunks, s);
+    if (!sell_fits((int64_t)S.nchunks * wm[0])) {              // may exceed: count in 64 bits
+        Tmp<unsigned long long> total(1, s);
+        CPC_CK(cudaMemsetAsync(total.get(), 0, sizeof(unsigned long long), s));
+        k_sum_int<<<std::min(nblk(S.nchunks), 304), TPB, 0, s>>>(width.get(), S.nchunks, total.get());
+        CPC_LAUNCH_CK();
+        if (!sell_fits((int64_t)d2h(total.get(), s))) {
+            if (may_halve && C > 1) return false;
+            fail(CPC_ESETUP, "a matrix layout exceeds 32-bit offsets");
+        }
+    }
     S.lanes = (wm[0] + 31) / 32;
     S.lanes_lo = (wm[1] + 31) / 32;
     S.lanes_up = (wm[2] + 31) / 32;
@@ -1701,6 +1719,7 @@ void build_sell(const int* ptr, const int* col, const double* val, const DBuf<in
         k_recip<<<nblk(nslots), TPB, 0, s>>>(nslots, S.diag.p, S.dinv.p);
     }
     CPC_LAUNCH_CK();
+    return true;
 }
 
 // The offset's place in a table of 8 (EMPTY = INT_MIN: no offset can be INT_MIN); false when it is full.
@@ -2570,13 +2589,16 @@ void setup_level_sells(Level& L, cudaStream_t s, bool last, bool tune, bool fp64
         std::vector<int> seg;
         auto group = [&](int C) { grouped_slots(L.n, L.colour.p, L.ncolours, C, s, slots, nslots, seg); };
         auto build = [&](int C, Sell& out) {
-            build_sell(L.A.ptr.p, L.A.col.p, L.A.val.p, slots, nslots, seg, C, SELL_OFFDIAG, true, nullptr, out, s,
-                       fp64 ? L.colour.p : nullptr);
+            const bool fits = build_sell(L.A.ptr.p, L.A.col.p, L.A.val.p, slots, nslots, seg, C, SELL_OFFDIAG, true,
+                                         nullptr, out, s, fp64 ? L.colour.p : nullptr, false, true);
             CPC_CK(cudaStreamSynchronize(s));
+            return fits;
         };
         auto build_grouped = [&](int C, Sell& out) {
-            group(C);
-            build(C, out);
+            for (;; C /= 2) {
+                group(C);
+                if (build(C, out)) return;
+            }
         };
         int ca = choose_chunk((double)(L.A.nnz - L.n) / std::max(1, L.n)), widest = 0;
         group(ca);
@@ -2586,8 +2608,8 @@ void setup_level_sells(Level& L, cudaStream_t s, bool last, bool tune, bool fp64
         // (level 1 at 8.4M: 300 -> 264 us a sweep).
         const bool many = !tune && fp64 && ca < 32 && widest > 4 * GS_RESIDENT_WARPS;
         if (many) group(ca *= 2);
-        build(ca, L.S);
-        if (!tune && !many && ca < 32) {
+        if (!build(ca, L.S)) build_grouped(ca / 2, L.S);
+        if (!tune && !many && ca < 32 && L.S.C == ca) {
             // One wave: a colour step whose blocks do not all fit on the GPU at once runs in two waves, and
             // only the first wave's matrix loads overlap the previous step.  If the widest colour needs more
             // blocks than fit (by the registers of the batch width) and twice the chunk height would fit,
@@ -2603,7 +2625,8 @@ void setup_level_sells(Level& L, cudaStream_t s, bool last, bool tune, bool fp64
             for (int C : {ca / 2, ca * 2}) {
                 if (C < 4 || C > 32) continue;
                 Sell cand;
-                build_grouped(C, cand);
+                group(C);
+                if (!build(C, cand)) continue;
                 const float t = time_gs_sweep(cand, L.n);
                 if (t < 0.97f * best) {
                     best = t;
@@ -2624,10 +2647,12 @@ void setup_level_sells(Level& L, cudaStream_t s, bool last, bool tune, bool fp64
         DBuf<int> rs;
         int rn = 0;
         std::vector<int> rseg;
-        const int cr = choose_chunk((double)L.R.nnz / std::max(1, L.R.n));
-        natural_slots(L.R.n, cr, s, rs, rn, rseg);
-        build_sell(L.R.ptr.p, L.R.col.p, L.R.val.p, rs, rn, rseg, cr, SELL_ALL, false, nullptr, L.SR, s,
-                   rb && fp64 ? L.colour.p : nullptr, true);
+        for (int cr = choose_chunk((double)L.R.nnz / std::max(1, L.R.n));; cr /= 2) {
+            natural_slots(L.R.n, cr, s, rs, rn, rseg);
+            if (build_sell(L.R.ptr.p, L.R.col.p, L.R.val.p, rs, rn, rseg, cr, SELL_ALL, false, nullptr, L.SR, s,
+                           rb && fp64 ? L.colour.p : nullptr, true, true))
+                break;
+        }
         CPC_CK(cudaStreamSynchronize(s));
     }
 }

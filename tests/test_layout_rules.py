@@ -44,3 +44,13 @@ def test_shared_arrays_of_vector_loads_are_aligned():
     assert read == {"fs", "ksm"}
     decls = [d for d in re.findall(r"(?:extern )?__shared__ [^;\n]*", text) if re.search(r"\b(fs|ksm)\[", d)]
     assert len(decls) == 5 and all("__align__(16)" in d for d in decls), decls
+
+
+@pytest.mark.skipif(not os.path.exists(NVCC), reason="no nvcc")
+def test_layouts_stay_within_their_offsets(tmp_path):
+    """Two paddings per chunk can carry a layout past 32-bit offsets where one did not; the count that decides
+    is taken in 64 bits (67,108,864 chunks of 32 entries are one entry too many)."""
+    run(tmp_path, """
+    OK(sell_fits(0) && sell_fits(INT32_MAX) && !sell_fits((int64_t)INT32_MAX + 1))
+    OK(!sell_fits((int64_t)67108864 * 32) && sell_fits((int64_t)67108863 * 32))
+""")
