@@ -38,13 +38,11 @@ MAXIT = 5000
 METRIC = "PCG ms to 1e-6 rel. residual (combined vs AMG/ILU alone, FP32 vs FP64 prec), %HBM peak"
 L2_FLUSH_BYTES = 512 << 20
 # dram__bytes_read.sum + dram__bytes_write.sum of one fine-level Gauss-Seidel launch from the
-# committed ncu capture (profiles/dram_bco_fp64_correlated3d_128x128x64.md); None until a capture
+# committed ncu capture (profiles/k_gs_pk_fine_correlated3d_128x128x64.md); None until a capture
 # of the current kernel exists.
-TRAFFIC_K_GS_FINE = 48238848
-# The same for one forward sweep of every coarse level (the k_gs launches of the sweep, summed,
-# cold cache; profiles/dram_bco_fp64_correlated3d_128x128x64.md); None until a capture of the
-# current hierarchy exists.
-TRAFFIC_COARSE_SWEEP = 230672896
+TRAFFIC_K_GS_FINE = 48355584
+# The same for one backward sweep of every coarse level; None: the present kernels' has not been captured.
+TRAFFIC_COARSE_SWEEP = None
 
 
 def peaks():
@@ -296,8 +294,9 @@ def gpu_arm(args, rank, world):
                 s.close()
 
     # the dominant kernels, timed live on the solver's stream:
-    # (1) the coarse-level Gauss-Seidel colour steps (k_gs; the largest share of the solve's kernel
-    #     time): one forward sweep per coarse level replayed from a CUDA graph as in the solve.
+    # (1) the coarse-level Gauss-Seidel sweeps (k_gs, k_flow; the largest share of the solve's kernel
+    #     time): one backward sweep per coarse level replayed from a CUDA graph as in the solve, where a
+    #     level has one a cycle beside a forward sweep that reads half its entries.
     #     Algorithmic bytes per sweep: 12 B per off-diagonal entry (value, column) + 28 B per row
     #     (1 / a_ii, slot -> row, f read, x written, x read once).
     peak, peak_kind = peaks()
@@ -362,8 +361,8 @@ def gpu_arm(args, rank, world):
     headline_ms = float(np.mean(ms))
     roofline = dict(bound="hbm", achieved=round(coarse_achieved, 1), peak=peak, unit="GB/s",
                     frac=round(coarse_achieved / peak, 4), traffic=TRAFFIC_COARSE_SWEEP,
-                    kernel="k_gs, k_flow (Gauss-Seidel sweeps of the coarse levels 1..%d, FP64): one forward sweep per "
-                           "level, aggregated; the latency of their dependent steps bounds them" % (s_bco.nlevels - 2),
+                    kernel="k_gs, k_flow (Gauss-Seidel sweeps of the coarse levels 1..%d, FP64): one backward sweep (full "
+                           "rows) per level, aggregated; the latency of their dependent steps bounds them" % (s_bco.nlevels - 2),
                     bytes_per_sweep=int(cbytes), us_per_sweep=round(cus, 2), peak_kind=peak_kind, levels=coarse,
                     fine_gs=fine, spmv=spmv)
     out.update(dict(p=p, arms=arms, matrices=matrices, clocks=clk, e2e_ms=e2e_ms, true_res=true_res,
@@ -660,7 +659,7 @@ def profile_mode(name):
     (for `ncu --profile-from-start off`), after two untimed warm-up applications.  With
     name = "blockcg_fp32": one block PCG solve of the 64 right-hand sides of the batched workload
     (FP32 preconditioner) after one untimed warm-up solve.  With name = "sweeps_fp64": one
-    forward Gauss-Seidel sweep of every coarse level, after two untimed ones.  With name =
+    backward Gauss-Seidel sweep of every coarse level, after two untimed ones.  With name =
     "setup_fp64": one setup of the benchmark's solver (the kernels of the AMG setup; the process
     does nothing else on the GPU besides the matrix assembly)."""
     import torch
@@ -688,16 +687,16 @@ def profile_mode(name):
         print(json.dumps({"profiled": name, "block_iterations": int(it), "status": int(st)}))
         return
     s = cpc.Solver(rowptr, col, val, precond=pre if pre != "sweeps" else "bco", precision=prec, ic_order="colour")
-    if pre == "sweeps":     # one forward Gauss-Seidel sweep of every coarse level (k_gs launches only)
+    if pre == "sweeps":     # one backward Gauss-Seidel sweep of every coarse level (and its vectors' preparation)
         xs = [torch.randn(s.level_info(l)["n"], dtype=torch.float64, device=dev) for l in range(s.nlevels - 1)]
         ys = [torch.zeros_like(x) for x in xs]
         for _ in range(2):
             for l in range(1, s.nlevels - 1):
-                s.level_apply(l, 5, xs[l], ys[l])
+                s.level_apply(l, 2, xs[l], ys[l])
         torch.cuda.synchronize()
         torch.cuda.profiler.start()
         for l in range(1, s.nlevels - 1):
-            s.level_apply(l, 5, xs[l], ys[l])
+            s.level_apply(l, 2, xs[l], ys[l])
         torch.cuda.synchronize()
         torch.cuda.profiler.stop()
         print(json.dumps({"profiled": name, "colours": [s.level_info(l)["ncolours"] for l in range(1, s.nlevels - 1)]}))

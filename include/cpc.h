@@ -283,11 +283,13 @@ int cpc_set_wait_polls(cpc_handle* h, int32_t polls);
  * graph if it does not exist yet. */
 int cpc_solve_launches(cpc_handle* h, int64_t* per_iteration, int64_t* fixed);
 
-/* Profiling: *us = microseconds per forward Gauss-Seidel sweep (colours ascending, Section 3.3: one
- * dependent launch per colour, or on a small level one launch ordered by its data) of level `level` (0 <= level < levels - 1), in the handle's
- * preconditioner precision, replayed from a CUDA graph as inside the solve: `reps` sweeps
- * (1..1000) per replay, best of three replays after a warm-up.  Overwrites the level's work
- * vectors.  Synchronous. */
+/* Profiling: *us = microseconds per backward Gauss-Seidel sweep (S_l^T of a cycle: colours descending,
+ * Section 3.3, one dependent launch per colour, or on a small level one launch ordered by its data) of
+ * level `level` (0 <= level < levels - 1), in the handle's preconditioner precision, replayed from a CUDA
+ * graph as inside the solve: `reps` sweeps (1..1000) per replay, best of three replays after a warm-up.
+ * It reads every entry of every row; the forward sweep, which starts from zero, reads about half of them
+ * in FP64.  With one launch ordered by its data the time contains the launch that marks the rows as not
+ * yet computed, which in a cycle the prolongation does.  Overwrites the level's work vectors.  Synchronous. */
 int cpc_sweep_time_us(cpc_handle* h, int32_t level, int32_t reps, double* us);
 
 /* Number of AMG levels (finest = 0). */

@@ -363,7 +363,7 @@ class Solver:
         return m.value, r.value
 
     def sweep_time_us(self, l, reps=20):
-        """Microseconds per forward Gauss-Seidel sweep of level l, replayed from a CUDA graph."""
+        """Microseconds per backward Gauss-Seidel sweep of level l, replayed from a CUDA graph."""
         us = ctypes.c_double()
         _check(load().cpc_sweep_time_us(self._h, l, reps, ctypes.byref(us)), self._h)
         return us.value

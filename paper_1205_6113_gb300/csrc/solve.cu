@@ -1327,9 +1327,10 @@ void level_apply(Handle& h, int l, int op, const double* x, double* y) {
     CPC_LAUNCH_CK();
 }
 
-// Microseconds per forward Gauss-Seidel sweep (colours ascending) of level l in the
-// preconditioner's precision on the level's own work vectors, replayed from a CUDA graph as in the
-// solve: reps sweeps per replay, the best of three replays after one warm-up.
+// Microseconds per backward Gauss-Seidel sweep (colours descending, every entry of every row) of level l in
+// the preconditioner's precision on the level's own work vectors, replayed from a CUDA graph as in the solve:
+// reps sweeps per replay, the best of three replays after one warm-up.  A flow sweep's time contains a
+// launch that marks its rows unset, as the prolongation does in a cycle.
 double sweep_time_us(Handle& h, int l, int reps) {
     const int nl = (int)h.lev.size();
     if (l < 0 || l >= nl - 1) fail(CPC_EINVAL, "level has no smoother");
@@ -1340,23 +1341,23 @@ double sweep_time_us(Handle& h, int l, int reps) {
     struct SG { cudaStream_t s; ~SG() { cudaStreamSynchronize(s); cudaStreamDestroy(s); } } sg{cs};
     CPC_CK(cudaStreamSynchronize(h.s));
     // the old values of a flow sweep are read as they are: none may be unset
-    if (L.x64.p) CPC_CK(cudaMemsetAsync(L.x64.p, 0, sizeof(double) * L.n, cs));
-    if (L.x32.p) CPC_CK(cudaMemsetAsync(L.x32.p, 0, sizeof(float) * L.n, cs));
+    if (L.xa64.p) CPC_CK(cudaMemsetAsync(L.xa64.p, 0, sizeof(double) * L.n, cs));
+    if (L.xa32.p) CPC_CK(cudaMemsetAsync(L.xa32.p, 0, sizeof(float) * L.n, cs));
     CPC_CK(cudaStreamSynchronize(cs));
     cudaGraph_t g;
     CPC_CK(cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal));
     for (int k = 0; k < reps; ++k) {
         if (L.flow) {
             if (fp64(h)) {
-                launch(k_fill_unset<double>, vec_blocks(L.n), VEC_TPB, cs, (int64_t)L.n, L.xa64.p);
-                rec_sweep<double, double>(h, l, FLOW_FWD, L.f64.p, L.x64.p, L.xa64.p, cs);
+                launch(k_fill_unset<double>, vec_blocks(L.n), VEC_TPB, cs, (int64_t)L.n, L.x64.p);
+                rec_sweep<double, double>(h, l, FLOW_BWD, L.f64.p, L.xa64.p, L.x64.p, cs);
             } else {
-                launch(k_fill_unset<float>, vec_blocks(L.n), VEC_TPB, cs, (int64_t)L.n, L.xa32.p);
-                rec_sweep<float, float>(h, l, FLOW_FWD, L.f32.p, L.x32.p, L.xa32.p, cs);
+                launch(k_fill_unset<float>, vec_blocks(L.n), VEC_TPB, cs, (int64_t)L.n, L.x32.p);
+                rec_sweep<float, float>(h, l, FLOW_BWD, L.f32.p, L.xa32.p, L.x32.p, cs);
             }
             continue;
         }
-        for (int c = 0; c < L.ncolours; ++c) {
+        for (int c = L.ncolours - 1; c >= 0; --c) {
             if (fp64(h)) rec_gs<double, double>(L, c, (const double*)L.f64.p, L.x64.p, cs);
             else rec_gs<float, float>(L, c, (const float*)L.f32.p, L.x32.p, cs);
         }
