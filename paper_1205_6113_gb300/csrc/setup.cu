@@ -1585,6 +1585,12 @@ __global__ void k_flag_later(int nslots, int C, const int* perm, const int* cptr
     }
 }
 
+void mark_columns(Sell& S, const int* key, cudaStream_t s) {
+    S.fcol.alloc(S.nelem);
+    k_flag_later<<<nblk(S.nslots), TPB, 0, s>>>(S.nslots, S.C, S.perm.p, S.cptr.p, S.col.p, key, S.fcol.p);
+    CPC_LAUNCH_CK();
+}
+
 // Slot order from a per-row group key (colour or level): rows sorted by (key, row), each group
 // padded to a multiple of the chunk height C.  Returns the chunk boundaries of the groups in seg.
 // The first row of each group among the sorted keys (-1 where the group has none): no counting by atomics,
@@ -1661,6 +1667,11 @@ __global__ void k_sum_int(const int* a, int n, unsigned long long* out) {
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) m += (unsigned long long)a[i];
     for (int o = 16; o > 0; o >>= 1) m += __shfl_xor_sync(0xffffffffu, m, o);
     if ((threadIdx.x & 31) == 0 && m > 0) atomicAdd(out, m);
+}
+
+// Storage of a level's smoother values.
+VType level_vtype(int prec, int l) {
+    return prec == CPC_PREC_FP64 ? VT_F64 : prec == CPC_PREC_FP32_BF16 && l > 0 ? VT_BF16 : VT_F32;
 }
 
 // Chunk height for rows of average length avg: 32 / G rows per warp with G lanes sharing a row,
@@ -2581,7 +2592,8 @@ void setup_ic_rb(Handle& h, bool colour_ic, cudaStream_t s) {
 // (within 4..32) around the row-length rule, each is timed on a forward Gauss-Seidel sweep replayed
 // from a graph (time_gs_sweep), and a candidate replaces the rule's layout only when it is more
 // than 3% faster.  C sets the threads per row (32 / C) of every kernel on that copy.
-void setup_level_sells(Level& L, cudaStream_t s, bool last, bool tune, bool fp64) {
+void setup_level_sells(Level& L, cudaStream_t s, bool last, bool tune, VType vt) {
+    const bool fp64 = vt == VT_F64;
     // colour-grouped A_l (Gauss-Seidel and residual)
     if (!last) {
         DBuf<int> slots;
@@ -2621,13 +2633,21 @@ void setup_level_sells(Level& L, cudaStream_t s, bool last, bool tune, bool fp64
             if ((widest + 3) / 4 > per_sm * sms && (widest / 2 + 4) / 4 <= 6 * sms) build_grouped(2 * ca, L.S);
         }
         if (tune) {
-            float best = time_gs_sweep(L.S, L.n);
+            auto time = [&](Sell& S) {                          // in the values and by the launches of the solve
+                if (!fp64) {
+                    sell_lowp(S, vt, s);
+                    mark_columns(S, L.colour.p, s);
+                    CPC_CK(cudaStreamSynchronize(s));
+                }
+                return time_gs_sweep(S, L.n, vt);
+            };
+            float best = time(L.S);
             for (int C : {ca / 2, ca * 2}) {
                 if (C < 4 || C > 32) continue;
                 Sell cand;
                 group(C);
                 if (!build(C, cand)) continue;
-                const float t = time_gs_sweep(cand, L.n);
+                const float t = time(cand);
                 if (t < 0.97f * best) {
                     best = t;
                     L.S = std::move(cand);
@@ -2969,7 +2989,7 @@ void setup_handle(Handle& h, const cpc_csr& in) {
     {
         AllocOn layouts_alloc(s3);
         for (int l = 0; l < nl; ++l) setup_level_sells(h.lev[l], s3, l == nl - 1, h.opt.autotune == 1 && l > 0,
-                                                          h.opt.precision == CPC_PREC_FP64);
+                                                          level_vtype(h.opt.precision, l));
         // fine A in natural order for the SpMVs
         DBuf<int> slots;
         int nslots = 0;
@@ -3068,7 +3088,7 @@ void setup_handle(Handle& h, const cpc_csr& in) {
     const int prec = h.opt.precision;
     for (int l = 0; l < nl; ++l) {
         Level& L = h.lev[l];
-        L.vt = prec == CPC_PREC_FP64 ? VT_F64 : (prec == CPC_PREC_FP32_BF16 && l > 0 ? VT_BF16 : VT_F32);
+        L.vt = level_vtype(prec, l);
         if (l < nl - 1) {
             sell_lowp(L.S, L.vt, s);
             sell_lowp(L.SP, L.vt == VT_BF16 ? VT_F32 : L.vt, s);
@@ -3091,12 +3111,7 @@ void setup_handle(Handle& h, const cpc_csr& in) {
             if (L.vt == VT_F64) L.xa64.alloc(n);
             else L.xa32.alloc(n);
         }
-        if (l < nl - 1 && !L.skip_zeros() && !L.red_black) {
-            L.S.fcol.alloc(L.S.nelem);
-            k_flag_later<<<nblk(L.S.nslots), TPB, 0, s>>>(L.S.nslots, L.S.C, L.S.perm.p, L.S.cptr.p, L.S.col.p, L.colour.p,
-                                                          L.S.fcol.p);
-            CPC_LAUNCH_CK();
-        }
+        if (l < nl - 1 && !L.skip_zeros() && !L.red_black) mark_columns(L.S, L.colour.p, s);
     }
     if (prec != CPC_PREC_FP64) {
         sell_lowp(h.Anat, VT_F32, s);

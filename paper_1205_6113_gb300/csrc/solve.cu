@@ -1202,29 +1202,30 @@ void spmv_fine(Handle& h, const double* x, double* y, cudaStream_t s) {
     CPC_LAUNCH_CK();
 }
 
-float time_gs_sweep(const Sell& S, int n) {
+template <class MT, class VT>
+static float time_sweep(const Sell& S, int n, VType vt, const SV<MT, VT>& v) {
     AllocOn plain(nullptr);                 // f and x are used on cs, not on a setup stream
     cudaStream_t cs;
     CPC_CK(cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking));
     struct SG { cudaStream_t s; ~SG() { cudaStreamSynchronize(s); cudaStreamDestroy(s); } } sg{cs};
     constexpr int SWEEPS = 4;
-    DBuf<double> f, x, xa;
+    DBuf<VT> f, x, xa;
     DBuf<unsigned> ctr;                     // a counter per launch and their error word
     f.alloc(n);
     x.alloc(n);
     xa.alloc(n);
     ctr.alloc(SWEEPS + 1);
-    CPC_CK(cudaMemsetAsync(f.p, 0, sizeof(double) * n, cs));
-    CPC_CK(cudaMemsetAsync(x.p, 0, sizeof(double) * n, cs));
+    CPC_CK(cudaMemsetAsync(f.p, 0, sizeof(VT) * n, cs));
+    CPC_CK(cudaMemsetAsync(x.p, 0, sizeof(VT) * n, cs));
     CPC_CK(cudaMemsetAsync(ctr.p, 0, sizeof(unsigned) * ctr.n, cs));
     CPC_CK(cudaStreamSynchronize(cs));
-    const bool flow = S.cmid.p && gs_by_flow(S, n, VT_F64);   // (an FP32 layout is timed by launches)
+    const bool flow = gs_by_flow(S, n, vt);
     cudaGraph_t g;
     CPC_CK(cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal));
     for (int k = 0; k < SWEEPS; ++k) {      // the launches of the solve's sweeps
         if (flow) {
-            launch(k_fill_unset<double>, vec_blocks(n), VEC_TPB, cs, (int64_t)n, xa.p);
-            rec_flow<double, double>(FLOW_FWD, S, VT_F64, f.p, x.p, xa.p, nullptr, nullptr, ctr.p + k, (int*)(ctr.p + SWEEPS), 0, cs);
+            launch(k_fill_unset<VT>, vec_blocks(n), VEC_TPB, cs, (int64_t)n, xa.p);
+            rec_flow<VT, VT>(FLOW_FWD, S, vt, f.p, x.p, xa.p, nullptr, nullptr, ctr.p + k, (int*)(ctr.p + SWEEPS), 0, cs);
             continue;
         }
         for (size_t c = 0; c + 1 < S.seg.size(); ++c) {
@@ -1232,9 +1233,8 @@ float time_gs_sweep(const Sell& S, int n) {
             if (c1 <= c0) continue;
             const int w = gs_block_warps(c1 - c0);
             with_u_gs(S.lanes, c1 - c0, [&](auto u) {
-                launch(k_gs<double, double, double, double, decltype(u)::value, false>, (c1 - c0 + w - 1) / w, 32 * w, cs,
-                       view(S, (const double*)S.val.p, (const double*)S.dinv.p), (const int*)S.cmid.p, c0, c1,
-                       (const double*)f.p, x.p);
+                launch(k_gs<MT, VT, VT, VT, decltype(u)::value, false>, (c1 - c0 + w - 1) / w, 32 * w, cs, v,
+                       (const int*)S.cmid.p, c0, c1, (const VT*)f.p, x.p);
             });
         }
     }
@@ -1262,6 +1262,12 @@ float time_gs_sweep(const Sell& S, int n) {
     unsigned gave_up = 0;                   // a layout whose sweep did is not chosen
     CPC_CK(cudaMemcpy(&gave_up, ctr.p + SWEEPS, sizeof(unsigned), cudaMemcpyDeviceToHost));
     return gave_up ? 1e30f : best;
+}
+
+float time_gs_sweep(const Sell& S, int n, VType vt) {
+    if (vt == VT_F64) return time_sweep(S, n, vt, view(S, (const double*)S.val.p, (const double*)S.dinv.p));
+    if (vt == VT_BF16) return time_sweep(S, n, vt, view(S, (const __nv_bfloat16*)S.val16.p, (const float*)S.dinv32.p));
+    return time_sweep(S, n, vt, view(S, (const float*)S.val32.p, (const float*)S.dinv32.p));
 }
 
 void level_apply(Handle& h, int l, int op, const double* x, double* y) {

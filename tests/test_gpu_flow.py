@@ -192,3 +192,18 @@ def test_a_wait_that_gives_up_is_reported_once(precision):
     s.set_wait_polls(0)
     again = s.solve(b, tol=1e-8)
     assert torch.equal(again[0], x) and again[1:3] == (iters, status)
+
+
+@pytest.mark.parametrize("precision", ["fp32", "fp32_bf16"])
+def test_chunk_heights_are_timed_on_the_sweeps_that_run(precision):
+    """Autotuned layouts in FP32 modes, level 1 swept by colour launches and the others by flow: sound, and a
+    solve in as many iterations as with the rule's heights, to one (the rounding of the sums differs)."""
+    p = inputs.small_3d(128, 128, 64, seed=99)
+    b = torch.tensor(inputs.random_vector(p.n, 100), device=DEV)
+    s, t = (solver(p, precision=precision, ic_order="colour", autotune=a) for a in (True, False))
+    c = s.check_layouts()
+    assert c.pop("layouts") == 3 * (s.nlevels - 1) + 3 and not any(c.values())
+    x, iters, status, _ = s.solve(b, tol=1e-8)
+    _, rule, _, _ = t.solve(b, tol=1e-8)
+    assert status == 0 and abs(iters - rule) <= 1
+    assert float((b - s.spmv(x)).norm() / b.norm()) <= 2e-8
