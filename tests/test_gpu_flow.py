@@ -207,3 +207,33 @@ def test_chunk_heights_are_timed_on_the_sweeps_that_run(precision):
     _, rule, _, _ = t.solve(b, tol=1e-8)
     assert status == 0 and abs(iters - rule) <= 1
     assert float((b - s.spmv(x)).norm() / b.norm()) <= 2e-8
+
+
+@pytest.mark.parametrize("precision", ["fp64", "fp32"])
+def test_one_handle_takes_batched_calls_of_every_kind(precision):
+    """The batched graph is kept by padded width and kind and replayed: on one handle, calls of other
+    right-hand sides, widths within one padding and across paddings, tolerances, limits and kinds give what
+    a fresh handle gives, to the bit."""
+    p = inputs.small_3d(19, 17, 9, seed=97)
+    make = lambda: solver(p, coarse_max=64, ic_order="colour", precision=precision)      # noqa: E731
+
+    def call(s, kind, K, tol, maxit):
+        B = torch.tensor(np.ascontiguousarray(inputs.batch_rhs(p.n, K, cells_per_rhs=4, seed=98 + K).T), device=DEV)
+        if kind == "block":
+            X, it, _, st = s.solve_block(B, tol=tol, maxit=maxit)
+            return [X], [it, st]
+        if kind == "adjoint":
+            X, L, itf, ita = s.solve_batched_adjoint(B, tol=tol, maxit=maxit)
+            return [X, L], [itf.tolist(), ita.tolist()]
+        X, it, st = s.solve_batched(B, tol=tol, maxit=maxit)
+        return [X], [it.tolist(), st.tolist()]
+
+    s = make()
+    for args in [("batched", 16, 1e-6, 100), ("batched", 9, 1e-8, 100), ("adjoint", 9, 1e-6, 100), ("block", 12, 1e-6, 100),
+                 ("batched", 16, 1e-8, 3), ("batched", 12, 1e-8, 100), ("adjoint", 40, 1e-8, 100), ("adjoint", 33, 1e-6, 100),
+                 ("block", 33, 1e-6, 100), ("batched", 5, 1e-6, 100), ("batched", 16, 1e-6, 100)]:
+        fresh = make()
+        (tensors, numbers), (want, count) = call(s, *args), call(fresh, *args)
+        assert numbers == count, args
+        assert all(torch.equal(a, b) for a, b in zip(tensors, want)), args
+        fresh.close()
