@@ -169,8 +169,11 @@ void record_precond(Handle& h, int which, const double* r, void* z, cudaStream_t
 void apply_precond(Handle& h, int which, const double* r, double* z);
 // Whether the sweeps of a level of n rows run as flow launches (flow.cu).
 bool gs_by_flow(const Sell& S, int n, VType vt);
-// Warps resident at once at the colour steps' occupancy (8 blocks of 4 warps on each of 152 SMs).
-constexpr int GS_RESIDENT_WARPS = 152 * 32;
+// Blocks of four warps (a chunk each) of the FP64 colour step that the GPU holds at once, for an operator whose
+// lanes hold at most `lanes` entries; and warps, at the batch of 12 (8 blocks an SM).
+constexpr int GS_WARPS_PER_BLOCK = 4;
+int gs_resident_blocks(int lanes);
+int gs_resident_warps();
 // Marks the n elements of p unset (flow.cuh).
 template <class VT> void fill_unset(VT* p, int64_t n, cudaStream_t s);
 void spmv_fine(Handle& h, const double* x, double* y, cudaStream_t s);

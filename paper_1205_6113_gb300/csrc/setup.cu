@@ -32,6 +32,7 @@ namespace {
 
 constexpr uint32_t COLOUR_SEED = 0x5bd1e995u;
 constexpr int TPB = 256;
+constexpr int SMS = 152;             // multiprocessors of the part: grids of a few blocks on each
 
 // Published MurmurHash3 32-bit finaliser (a bijection): tie-break weights.
 __device__ __forceinline__ uint32_t fmix32(uint32_t h) {
@@ -718,7 +719,7 @@ void spgemm(const Csr& A, const Csr& B, Csr& C, cudaStream_t s) {
     Tmp<int64_t> cnt(n + 1, s), off(n + 1, s), mx(1, s);
     k_prod_count<<<nblk(n + 1), TPB, 0, s>>>(n, A.ptr.p, A.col.p, B.ptr.p, cnt.get());
     CPC_CK(cudaMemsetAsync(mx.get(), 0, sizeof(int64_t), s));
-    k_max_i64<<<std::min(nblk(n), 304), TPB, 0, s>>>(cnt.get(), n, mx.get());
+    k_max_i64<<<std::min(nblk(n), 2 * SMS), TPB, 0, s>>>(cnt.get(), n, mx.get());
     exclusive_scan(cnt.get(), off.get(), n + 1, s);
     CPC_LAUNCH_CK();
     const int64_t most = d2h(mx.get(), s);
@@ -1705,7 +1706,7 @@ bool build_sell(const int* ptr, const int* col, const double* val, const DBuf<in
     if (!sell_fits((int64_t)S.nchunks * wm[0])) {              // may exceed: count in 64 bits
         Tmp<unsigned long long> total(1, s);
         CPC_CK(cudaMemsetAsync(total.get(), 0, sizeof(unsigned long long), s));
-        k_sum_int<<<std::min(nblk(S.nchunks), 304), TPB, 0, s>>>(width.get(), S.nchunks, total.get());
+        k_sum_int<<<std::min(nblk(S.nchunks), 2 * SMS), TPB, 0, s>>>(width.get(), S.nchunks, total.get());
         CPC_LAUNCH_CK();
         if (!sell_fits((int64_t)d2h(total.get(), s))) {
             if (may_halve && C > 1) return false;
@@ -1788,7 +1789,7 @@ void build_dia(int n, const int* ptr, const int* col, const double* val, Sell& S
     Tmp<int> table(8, s), over(1, s);
     k_fill_int<<<1, 32, 0, s>>>(table.get(), 8, INT_MIN);
     CPC_CK(cudaMemsetAsync(over.get(), 0, sizeof(int), s));
-    k_dia_offsets<<<std::min(nblk(n), 1216), TPB, 0, s>>>(n, ptr, col, table.get(), over.get());
+    k_dia_offsets<<<std::min(nblk(n), 8 * SMS), TPB, 0, s>>>(n, ptr, col, table.get(), over.get());
     CPC_LAUNCH_CK();
     int t[8];
     CPC_CK(cudaMemcpyAsync(t, table.get(), sizeof(t), cudaMemcpyDeviceToHost, s));
@@ -2618,19 +2619,18 @@ void setup_level_sells(Level& L, cudaStream_t s, bool last, bool tune, VType vt)
         // FP64 issue bounds a colour that takes many waves of warps, and adding the partial sums of a row's
         // lanes costs as much of it as a few entries: twice the chunk height, half the lanes per row
         // (level 1 at 8.4M: 300 -> 264 us a sweep).
-        const bool many = !tune && fp64 && ca < 32 && widest > 4 * GS_RESIDENT_WARPS;
+        const bool many = !tune && fp64 && ca < 32 && widest > 4 * gs_resident_warps();
         if (many) group(ca *= 2);
         if (!build(ca, L.S)) build_grouped(ca / 2, L.S);
         if (!tune && !many && ca < 32 && L.S.C == ca) {
             // One wave: a colour step whose blocks do not all fit on the GPU at once runs in two waves, and
             // only the first wave's matrix loads overlap the previous step.  If the widest colour needs more
-            // blocks than fit (by the registers of the batch width) and twice the chunk height would fit,
-            // take twice the chunk height (level 1 at 1M, FP64: 55 -> 49 us a sweep).
-            int sms = 0, dev = 0;
-            CPC_CK(cudaGetDevice(&dev));
-            CPC_CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-            const int per_sm = L.S.lanes <= 4 ? 16 : L.S.lanes <= 6 ? 12 : L.S.lanes <= 8 ? 9 : L.S.lanes <= 12 ? 8 : 6;
-            if ((widest + 3) / 4 > per_sm * sms && (widest / 2 + 4) / 4 <= 6 * sms) build_grouped(2 * ca, L.S);
+            // blocks than fit and twice the chunk height would fit, take twice the chunk height (level 1 at 1M,
+            // FP64: 55 -> 49 us a sweep).  The FP64 kernel's blocks count in FP32 modes too: the heights are then
+            // the same, and with them the order of every sum, whatever the registers of an FP32 kernel.
+            const int W = GS_WARPS_PER_BLOCK;
+            if ((widest + W - 1) / W > gs_resident_blocks(L.S.lanes) && (widest / 2 + W) / W <= gs_resident_blocks(16))
+                build_grouped(2 * ca, L.S);
         }
         if (tune) {
             auto time = [&](Sell& S) {                          // in the values and by the launches of the solve

@@ -22,7 +22,7 @@ namespace cpc {
 
 namespace {
 
-constexpr int WPB = 4;                   // warps (= SELL chunks) per block
+constexpr int WPB = GS_WARPS_PER_BLOCK;  // warps (= SELL chunks) per block
 constexpr int SELL_TPB = WPB * 32;
 constexpr int VEC_TPB = 256;
 
@@ -35,6 +35,13 @@ void with_u(int lanes, F&& f) {
     else f(std::integral_constant<int, 8>{});
 }
 
+// As with_u, with batches of up to 16.
+template <class F>
+void with_u16(int lanes, F&& f) {
+    if (lanes <= 8) with_u(lanes, f);
+    else if (lanes <= 12) f(std::integral_constant<int, 12>{});
+    else f(std::integral_constant<int, 16>{});
+}
 // As with_u for the Gauss-Seidel colour steps, with batches of up to 16: a colour step lasts as long
 // as its widest chunk, and one batch per lane keeps it to one round of dependent gathers (level 1 at
 // 1M: 49 us a sweep, 67 with batches of 8).  A step of several waves of warps is bound by what it
@@ -42,9 +49,8 @@ void with_u(int lanes, F&& f) {
 // The products are added in the same entry order whatever the batch, so the results do not change.
 template <class F>
 void with_u_gs(int lanes, int chunks, F&& f) {
-    if (lanes <= 8 || chunks > 4 * GS_RESIDENT_WARPS) with_u(lanes, f);
-    else if (lanes <= 12) f(std::integral_constant<int, 12>{});
-    else f(std::integral_constant<int, 16>{});
+    if (chunks > 4 * gs_resident_warps()) with_u(lanes, f);
+    else with_u16(lanes, f);
 }
 
 // Calls f(std::integral_constant<int, ND>{}) with the padded diagonal count (4, 6 or 8).
@@ -1393,6 +1399,22 @@ double sweep_time_us(Handle& h, int l, int reps) {
     CPC_CK(cudaMemcpy(&gave_up, &h.state.p->gave_up, sizeof(int), cudaMemcpyDeviceToHost));
     report_gave_up(h, gave_up);
     return 1000.0 * best / reps;
+}
+
+int gs_resident_blocks(int lanes) {
+    int dev = 0, sms = 0, per_sm = 0;
+    CPC_CK(cudaGetDevice(&dev));
+    CPC_CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    with_u16(lanes, [&](auto u) {
+        CPC_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(
+            &per_sm, k_gs<double, double, double, double, decltype(u)::value, false>, SELL_TPB, 0));
+    });
+    return std::max(1, sms * per_sm);
+}
+
+int gs_resident_warps() {
+    static const int warps = GS_WARPS_PER_BLOCK * gs_resident_blocks(12);
+    return warps;
 }
 
 void report_gave_up(Handle& h, int gave_up) {

@@ -237,3 +237,16 @@ def test_one_handle_takes_batched_calls_of_every_kind(precision):
         assert numbers == count, args
         assert all(torch.equal(a, b) for a, b in zip(tensors, want)), args
         fresh.close()
+
+
+def test_chunk_heights_do_not_depend_on_the_precision():
+    """The rule for the chunk height of a widest colour that takes two waves of blocks goes by the FP64 kernel's
+    occupancy: 8 entries to a lane leave 9 blocks of four chunks on an SM.  FP32 modes take the same heights, so
+    that every sum keeps its order (a colour of many waves, in FP64 alone, is left out by the sizes)."""
+    sms = torch.cuda.get_device_properties(DEV).multi_processor_count
+    for shape in [(61, 53, 37), (112, 112, 56), (128, 128, 64)]:
+        p = inputs.small_3d(*shape, seed=101)
+        hs = [solver(p, precision=q) for q in ("fp64", "fp32", "fp32_bf16")]
+        for l in range(1, hs[0].nlevels - 1):
+            if hs[0].level_info(l)["n"] // hs[0].level_info(l)["ncolours"] < 4 * 8 * 4 * sms:
+                assert len({s.level_layout(l)["C"] for s in hs}) == 1, (shape, l)
