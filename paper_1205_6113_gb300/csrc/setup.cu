@@ -2593,7 +2593,7 @@ void setup_ic_rb(Handle& h, bool colour_ic, cudaStream_t s) {
 // (within 4..32) around the row-length rule, each is timed on a forward Gauss-Seidel sweep replayed
 // from a graph (time_gs_sweep), and a candidate replaces the rule's layout only when it is more
 // than 3% faster.  C sets the threads per row (32 / C) of every kernel on that copy.
-void setup_level_sells(Level& L, cudaStream_t s, bool last, bool tune, VType vt) {
+void setup_level_sells(Level& L, cudaStream_t s, bool last, bool tune, VType vt, bool dia) {
     const bool fp64 = vt == VT_F64;
     // colour-grouped A_l (Gauss-Seidel and residual)
     if (!last) {
@@ -2654,9 +2654,9 @@ void setup_level_sells(Level& L, cudaStream_t s, bool last, bool tune, VType vt)
                 }
             }
         }
-        // On a two-colour level the red rows of P come first and the red columns of R make the first part:
-        // the cycle reads no others there (rec_vcycle).
-        const bool rb = L.ncolours == 2;     // (R in FP64 only: FP32 sums keep their order)
+        // On a red-black level (two colours in diagonal form) the red rows of P come first and the red columns
+        // of R make the first part: the cycle reads no others there (rec_vcycle).
+        const bool rb = dia && L.ncolours == 2;     // (R in FP64 only: FP32 sums keep their order)
         DBuf<int> ps;
         int pn = 0;
         std::vector<int> pseg;
@@ -2988,8 +2988,6 @@ void setup_handle(Handle& h, const cpc_csr& in) {
     CPC_CK(cudaStreamWaitEvent(s3, ph[1], 0));
     {
         AllocOn layouts_alloc(s3);
-        for (int l = 0; l < nl; ++l) setup_level_sells(h.lev[l], s3, l == nl - 1, h.opt.autotune == 1 && l > 0,
-                                                          level_vtype(h.opt.precision, l));
         // fine A in natural order for the SpMVs
         DBuf<int> slots;
         int nslots = 0;
@@ -2998,6 +2996,9 @@ void setup_handle(Handle& h, const cpc_csr& in) {
         build_sell(h.lev[0].A.ptr.p, h.lev[0].A.col.p, h.lev[0].A.val.p, slots, nslots, seg, CHUNK, SELL_OFFDIAG,
                    true, nullptr, h.Anat, s3);
         build_dia(h.n, h.lev[0].A.ptr.p, h.lev[0].A.col.p, h.lev[0].A.val.p, h.Anat, s3);
+        for (int l = 0; l < nl; ++l)
+            setup_level_sells(h.lev[l], s3, l == nl - 1, h.opt.autotune == 1 && l > 0, level_vtype(h.opt.precision, l),
+                              l == 0 && h.Anat.ndiag > 0);
         if (nl > 1) build_dia(h.n, h.lev[0].A.ptr.p, h.lev[0].A.col.p, h.lev[0].A.val.p, h.lev[0].S, s3, true);
         CPC_CK(cudaStreamSynchronize(s3));
     }

@@ -250,3 +250,27 @@ def test_chunk_heights_do_not_depend_on_the_precision():
         for l in range(1, hs[0].nlevels - 1):
             if hs[0].level_info(l)["n"] // hs[0].level_info(l)["ncolours"] < 4 * 8 * 4 * sms:
                 assert len({s.level_layout(l)["C"] for s in hs}) == 1, (shape, l)
+
+
+def test_two_colours_without_diagonals():
+    """A grid in a random order: two colours, no diagonal form, so whole rows of P and R.  The same as the
+    oracle's application up to the rounding of the sums (a relative 1e-11, as for the other layouts)."""
+    import oracle as O
+    A = O.tpfa_problem(inputs.small_3d(40, 36, 1, seed=102))
+    n = A.rowptr.size - 1
+    new = np.random.default_rng(103).permutation(n)
+    rows = new[np.repeat(np.arange(n), np.diff(A.rowptr))]
+    o = np.lexsort((new[A.col], rows))
+    ptr = np.concatenate(([0], np.cumsum(np.bincount(rows, minlength=n)))).astype(np.int32)
+    csr = ptr, new[A.col][o].astype(np.int32), A.val[o]
+    orc = O.Oracle(O.Csr(n, *csr), coarse_max=64)
+    s = cpc.Solver(*csr, coarse_max=64)
+    assert s.level_info(0)["ncolours"] == 2 and s.level_layout(0)["ndiag"] == 0
+    r = inputs.random_vector(n, 104)
+    for which, op in (("bco", O.BCO), ("amg", O.STILDE)):
+        z, ref = s.apply(torch.tensor(r, device=DEV), which).cpu().numpy(), orc.apply(op, r)
+        assert np.linalg.norm(z - ref) / np.linalg.norm(ref) < 1e-11
+    B = torch.tensor(np.stack((r, 2.0 * r), 1), device=DEV)
+    X, it, st = s.solve_batched(B, tol=1e-10)
+    x, iters, _, _ = s.solve(B[:, 0].contiguous(), tol=1e-10)
+    assert not st.any() and it[0] == it[1] == iters and float((X[:, 0] - x).norm() / x.norm()) <= 1e-11
