@@ -312,7 +312,8 @@ int cpc_level_layout(const cpc_handle* h, int32_t level, int64_t* info);
  * (host) receives: [0] indices out of range (slot rows, chunk pointers, columns, diagonal offsets,
  * group boundaries); [1] rows missing from or repeated in a layout; [2] pairs of coupled rows
  * (a_ij != 0) in one Gauss-Seidel colour group, which one launch would update in parallel
- * (Section 3.3); [3] IC(0) factor entries whose row's triangular-solve level is not after its
+ * (Section 3.3), and entries of the smoother copy (or of a split restriction) on the wrong side of
+ * earlier and later colours; [3] IC(0) factor entries whose row's triangular-solve level is not after its
  * column's (Algorithm 3.1); [4] the number of layouts checked.  All but [4] are 0 for a sound
  * handle.  Synchronises the stream; allocates temporary device memory.
  */

@@ -7,7 +7,9 @@
 //   [1] coverage: a row missing from or repeated in a layout (every layout holds each of its rows
 //       exactly once);
 //   [2] Gauss-Seidel races: two rows coupled in A_l (a_ij != 0, i != j) in one colour group of the
-//       smoother layout, whose rows one launch updates in parallel (Section 3.3);
+//       smoother layout, whose rows one launch updates in parallel (Section 3.3); or an entry that a
+//       sweep would read on the wrong side: in the part, or with the mark, of columns of earlier
+//       (later) groups while its column's group is not;
 //   [3] triangular-solve races: an entry of the IC(0) factor whose row's level is not after its
 //       column's (forward levels for j < i, backward levels for j > i; Algorithm 3.1).
 // Every index is bounds-checked here before it is used.
@@ -67,6 +69,28 @@ __global__ void k_chk_entries(int nchunks, int C, int64_t nelem, int ncols, cons
             const int c = col[e];
             if (c < -1 || c >= ncols) atomicAdd(&cnt[C_RANGE], 1ull);
         }
+}
+
+// Sides of the entries (common.cuh): cmid splits the chunks by the groups of row and column, or (by_col) by whether
+// the column's group is the first; fcol marks the columns of later groups.  Only entries and rows in range
+// are looked at (the others are counted above).
+__global__ void k_chk_sides(int nslots, int C, int nrows, int ncols, int64_t nelem, const int* perm, const int* cptr,
+                            const int* cmid, const int* col, const int* fcol, const int* grp, bool by_col,
+                            unsigned long long* cnt) {
+    for (int s = blockIdx.x * blockDim.x + threadIdx.x; s < nslots; s += gridDim.x * blockDim.x) {
+        const int i = perm[s], k = s / C, a = cptr[k], b = cptr[k + 1];
+        if (i < 0 || i >= nrows || a < 0 || a > b || b > nelem) continue;
+        for (int64_t e = a + s % C; e < b; e += C) {
+            const int c = col[e];
+            if (c < 0 || c >= ncols) {
+                if (fcol && fcol[e] != c) atomicAdd(&cnt[C_GS_RACE], 1ull);
+                continue;
+            }
+            const int gr = by_col ? 1 : grp[i];
+            if (cmid && !part_holds(e < cmid[k], gr, grp[c])) atomicAdd(&cnt[C_GS_RACE], 1ull);
+            if (fcol && !mark_holds(fcol[e], c, gr, grp[c])) atomicAdd(&cnt[C_GS_RACE], 1ull);
+        }
+    }
 }
 
 __global__ void k_chk_seen(int n, const int* seen, int exact, unsigned long long* cnt) {
@@ -133,6 +157,14 @@ struct Checker {
         CPC_CK(cudaStreamSynchronize(s));
         bump(C_LAYOUTS);
     }
+    // The sides of S's entries, where it has any; grp: the columns' groups (and, unless by_col, the rows').
+    void sides(const Sell& S, int nrows, int ncols, const int* grp, bool by_col) {
+        if (!S.cmid.p && !S.fcol.p) return;
+        k_chk_sides<<<cblk(S.nslots), CTPB, 0, s>>>(S.nslots, S.C, nrows, ncols, S.nelem, S.perm.p, S.cptr.p, S.cmid.p,
+                                                    S.col.p, S.fcol.p, grp, by_col, cnt.p);
+        CPC_LAUNCH_CK();
+        CPC_CK(cudaStreamSynchronize(s));
+    }
     void bump(int k) {
         unsigned long long v = 0;
         CPC_CK(cudaMemcpyAsync(&v, cnt.p + k, sizeof(v), cudaMemcpyDeviceToHost, s));
@@ -155,11 +187,13 @@ void check_layouts(Handle& h, int64_t* counts) {
         const int nc = h.lev[l + 1].n;
         Tmp<int> grp(L.n, s);
         ck.sell(L.S, L.n, L.n, true, grp.get());
+        ck.sides(L.S, L.n, L.n, grp.get(), false);
         k_chk_pairs<<<cblk(L.n), CTPB, 0, s>>>(L.n, L.A.ptr.p, L.A.col.p, grp.get(), grp.get(), 0, nullptr, ck.cnt.p);
         CPC_LAUNCH_CK();
         CPC_CK(cudaStreamSynchronize(s));
         ck.sell(L.SP, L.n, nc, true);
         ck.sell(L.SR, nc, L.n, true);
+        ck.sides(L.SR, nc, L.n, grp.get(), true);
     }
     ck.sell(h.Anat, h.n, h.n, true);
     if (h.Aic.n == h.n && h.L.nslots > 0) {

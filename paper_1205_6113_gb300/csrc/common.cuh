@@ -143,6 +143,14 @@ __host__ __device__ constexpr int marked_col(int c) { return c < -1 ? -2 - c : c
 // Whether a sum over col, or over fcol from a zero guess, takes the entry.
 __host__ __device__ constexpr bool takes(int c) { return c >= 0; }
 
+// Whether an entry stands on its side of a smoother layout, in a row of group gr and a column of group gc: in
+// the first part (low) if and only if the column's group is earlier; fc, its place in fcol, the column c itself,
+// marked if and only if the group is later.
+__host__ __device__ constexpr bool part_holds(bool low, int gr, int gc) { return low == (gc < gr); }
+__host__ __device__ constexpr bool mark_holds(int fc, int c, int gr, int gc) {
+    return fc != -1 && marked_col(fc) == c && is_later(fc) == (gc > gr);
+}
+
 // Whether chunks of so many entries, padding included, can be addressed by the 32-bit offsets of a Sell.
 constexpr bool sell_fits(int64_t entries) { return entries <= INT32_MAX; }
 

@@ -53,3 +53,15 @@ def test_layouts_full_size():
         nl = s.nlevels
         s.close()
         assert c == dict(out_of_range=0, coverage=0, gs_races=0, triangular_races=0, layouts=3 * (nl - 1) + 3)
+
+
+@pytest.mark.parametrize("precision", ["fp64", "fp32", "fp32_bf16"])
+@pytest.mark.parametrize("name", ["tpfa_colour_ic", "tpfa_natural_gs", "mhfem", "ragged_1d"])
+def test_sides_are_sound_in_every_precision(name, precision):
+    """The parts of the FP64 smoother copies and of the red-black R, and the marked columns of the FP32 ones."""
+    make, kw = CASES[name]
+    A = make()
+    s = cpc.Solver(A.rowptr, A.col, A.val, precision=precision, **kw)
+    c = s.check_layouts()
+    assert c.pop("layouts") == 3 * (s.nlevels - 1) + 3 and not any(c.values()), c
+    s.close()

@@ -54,3 +54,21 @@ def test_layouts_stay_within_their_offsets(tmp_path):
     OK(sell_fits(0) && sell_fits(INT32_MAX) && !sell_fits((int64_t)INT32_MAX + 1))
     OK(!sell_fits((int64_t)67108864 * 32) && sell_fits((int64_t)67108863 * 32))
 """)
+
+
+@pytest.mark.skipif(not os.path.exists(NVCC), reason="no nvcc")
+def test_sides_of_entries_are_told_apart(tmp_path):
+    """The layout checker's rules on sound and planted entries: the part of earlier groups, the mark of later
+    ones, a column that is not the entry's, an entry dropped as padding."""
+    run(tmp_path, """
+    for (int gr = 0; gr < 3; ++gr)
+        for (int gc = 0; gc < 3; ++gc) {
+            if (gc == gr) continue;
+            OK(part_holds(gc < gr, gr, gc) && !part_holds(gc > gr, gr, gc))
+            for (int c : {0, 7, 1 << 30}) {
+                const int right = gc > gr ? mark_later(c) : c, wrong = gc > gr ? c : mark_later(c);
+                OK(mark_holds(right, c, gr, gc) && !mark_holds(wrong, c, gr, gc))
+                OK(!mark_holds(-1, c, gr, gc) && !mark_holds(right, c + 1, gr, gc))
+            }
+        }
+""")
