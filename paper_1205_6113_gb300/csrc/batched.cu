@@ -1040,7 +1040,7 @@ __global__ void kb_adjoint_rhs(int64_t nk, double* __restrict__ b, const double*
 // ------------------------------------------------------------------------------------------------
 constexpr int KK_TPB = 256;
 constexpr int KK_ELEMS = 2048;            // elements of U (and of V) staged per step of kk_gram
-constexpr int KK_GRID = 152 * 2;          // blocks of kk_gram / kk_update / kk_colnorm (fixed)
+constexpr int KK_GRID = 152 * 2;          // blocks of kk_init / kk_gram / kk_update / kk_pupdate (fixed)
 enum { KM_PQ = 0, KM_GAMMA, KM_GAMMA_NEW, KM_ALPHA, KM_BETA, KM_COUNT };
 enum { KV_BNORM = 0, KV_RES, KV_COUNT };
 enum { KF_BAD = 0, KF_DONE, KF_COUNT };
