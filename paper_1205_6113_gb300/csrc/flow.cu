@@ -273,7 +273,8 @@ int flow_resident(int lanes) {
 // lane takes 16 entries at a time): once they are not all resident a flow waits for its own chunks.  Launches and
 // flow, us a full sweep, at chunks a colour per resident warp: FP64 0.83 68 and 57, 0.94 76 and 70, 1.02 59 and
 // 53, 1.12 75 and 77, 1.49 67 and 85, 2.6 103 and 161 (with the sweep from zero, half a row, two cycles at 1.12
-// 1,884 and 1,858, at 1.25 2,048 and 2,042, at 1.40 2,217 and 2,225); FP32, which polls every entry of a row, 0.42
+// 1,884 and 1,858, at 1.25 2,048 and 2,042, at 1.40 2,217 and 2,225; with at most 8 entries to a lane, at 1.32
+// 1,838 and 1,773, at 1.58 2,192 and 2,151); FP32, which polls every entry of a row, 0.42
 // 19 and 16, 0.66 47 and 42, 0.71 46 and 45, 0.84 46 and 54, 1.25 36 and 59, 2.0 52 and 115, and 83 and 109 at
 // 0.55 with 30 entries to a lane, two batches.
 bool gs_by_flow(const Sell& S, int n, VType vt) {
@@ -281,7 +282,7 @@ bool gs_by_flow(const Sell& S, int n, VType vt) {
     const int g = std::max(1, (int)S.seg.size() - 1), lanes = sweep_lanes(S, vt == VT_F64);
     if (n / g > FLOW_ROWS) return false;
     const double per = (double)S.nchunks / g;
-    if (vt == VT_F64) return per <= 1.25 * flow_resident<double, double>(lanes);
+    if (vt == VT_F64) return per <= (lanes <= 8 ? 1.6 : 1.25) * flow_resident<double, double>(lanes);
     const int res = vt == VT_BF16 ? flow_resident<__nv_bfloat16, float>(lanes) : flow_resident<float, float>(lanes);
     return per * std::max(1.0, lanes / 16.0) <= 0.75 * res;
 }
